@@ -1,19 +1,39 @@
-// bf16 x bf16 -> fp32 GEMM on the 5th-generation tensor cores (tcgen05) with the four fused
-// epilogues of the DiT block.
+// bf16 x bf16 -> fp32 GEMM on the 5th-generation tensor cores (tcgen05) with the fused epilogues of
+// the DiT block.
 //
 //   acc[b, i, n] = sum_k A[b, i, k] * W[n, k]          (both operands K-major)
 //
-// Structure of one CTA (persistent, one per SM, 192 threads):
-//   warp 0    TMA producer: 128 x 64 tiles of A and BN x 64 tiles of W into a ring of
-//             shared-memory stages (128-byte swizzle), completion on mbarriers
-//   warp 1    owns TMEM; one thread issues tcgen05.mma (M = 128, N = BN, K = 16) into one of
-//             two fp32 accumulators in TMEM and commits stage releases / accumulator-ready
-//   warps 2-5 epilogue: tcgen05.ld the finished accumulator (thread = output row), apply the
-//             epilogue in fp32 and store; runs while the next tile's main loop fills the
-//             other accumulator
-// A row's result depends only on (row, N, K): the K loop always runs in the same order and the
-// tile shape is chosen from N alone, so outputs are bit-identical however rows are chunked.
-#include <type_traits>
+// One kernel, two forms.  A persistent grid of 192-thread CTAs walks over output tiles:
+//   PAIR    CTA pairs (two neighbouring SMs) share one 256 x 256 tile.  Each CTA loads its own 128
+//           rows of A and one half (128 rows) of the W tile, so a stage costs 32 KB of shared-memory
+//           fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
+//           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows x 256 columns in the TMEM of
+//           each CTA.
+//   single  one CTA per 128 x BN tile.
+//
+//   warp 0    TMA producer: tiles of A and W into a ring of shared-memory stages (128-byte swizzle)
+//   warp 1    owns TMEM; converged warp, one elected lane issues tcgen05.mma into one of two fp32
+//             accumulators in TMEM and commits stage releases / accumulator-ready
+//   warps 2-5 epilogue (thread = output row) of the finished accumulator, while the next tile's main
+//             loop fills the other one
+// Barriers of the pair form:
+//   full[s]        barrier of the even CTA: its producer expects the bytes of both CTAs, and both
+//                  CTAs' loads complete on it (an expect-tx arrival sent from the peer CTA for every
+//                  stage halved the speed of the whole loop)
+//   empty[s]       one barrier per CTA, released for both by a multicast commit
+//   tmem_full[a]   one barrier per CTA, same commit form
+//   tmem_empty[a]  barrier of the even CTA: the four epilogue warps of both CTAs arrive
+//
+// The epilogue must not wait for global memory: bias and gate of the tile go to shared memory, the
+// residual arrives by TMA in 32-column chunks and the rotation angles in registers, all requested
+// while the main loop still runs, and the results leave through shared memory by TMA stores.  With
+// plain loads in the chunk loop a 256-column tile took 11 000 (GELU) to 16 000 cycles (RMSNorm + RoPE,
+// gated) whatever the shape -- 1300 to 3500 cycles of load latency per chunk -- which is 6 to 8 us at the
+// end of every launch.
+//
+// A row's result depends only on (row, N, K): every form accumulates K in the same order, 16 at a
+// time, so outputs are bit-identical however rows are chunked and whichever tile is chosen.
+#include <algorithm>
 
 #include "kernels.h"
 #include "sm100.cuh"
@@ -21,31 +41,43 @@
 namespace xema {
 using namespace sm100;
 
-constexpr int BM = 128;
+namespace {
+constexpr int BM = 128;          // rows per CTA
 constexpr int BK = 64;
 constexpr int GEMM_THREADS = 192;
 constexpr int GROUP_M = 8;
 constexpr int A_TILE_BYTES = BM * BK * 2;
+constexpr int PAIR_BN = 256;
+constexpr int CHUNK = 32;        // columns per epilogue step
+constexpr int BUF_BYTES = 4096;  // one staging buffer: 32 rows x 32 columns of fp32, or of bf16 in its first half
 
-template <int BN>
+template <int EPI>
+constexpr bool kGated = EPI == XEMA_EPI_GATE_RES_F32 || EPI == XEMA_EPI_GATE_RES_BF16;
+
+template <int EPI, int BN, bool PAIR>
 struct GemmCfg {
-  static constexpr int B_TILE_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = A_TILE_BYTES + B_TILE_BYTES;
-  static constexpr int STAGES = (BN == 256) ? 4 : 6;
+  static constexpr int W_ROWS = PAIR ? BN / 2 : BN;            // rows of W a CTA loads per stage
+  static constexpr int STAGE_BYTES = A_TILE_BYTES + W_ROWS * BK * 2;
+  // staging buffers per epilogue warp: the gated epilogues keep residual chunks in flight
+  static constexpr int RING = kGated<EPI> ? 4 : 2;
+  static constexpr int RING_BYTES = 4 * RING * BUF_BYTES;
+  static constexpr int STAGES = kGated<EPI> ? 5 : 6;
+  static constexpr int OFF_RING = STAGES * STAGE_BYTES;
+  static constexpr int OFF_BIAS = OFF_RING + RING_BYTES;       // float [BN]: bias
+  static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
+  static constexpr int OFF_BAR = OFF_GATE + (kGated<EPI> ? BN * 4 : 512);
+  static constexpr int SMEM_BYTES = OFF_BAR + 384;
   static constexpr int TMEM_COLS = 2 * BN;
-  static constexpr int BAR_BYTES = 256;
-  static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + BAR_BYTES;
+  static_assert((2 * STAGES + 4 + 4 * RING) * 8 + 8 <= 384, "barrier area");
+  static_assert(SMEM_BYTES <= 232448, "shared memory of one SM");
 };
 
 struct GemmParams {
   const __nv_bfloat16* bias;
-  void* out;
-  long long ldo, out_batch_rows;
-  const void* resid;
-  long long ldr, resid_batch_rows;
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K;
+  int resid_batch;                  // 1: the residual has a batch dimension, 0: the same rows for every element
   unsigned int* status;
   // XEMA_EPI_BIAS_NORM_ROPE only: heads that start below column norm_cols get RMSNorm * gain
   // and RoPE in the epilogue (a thread owns whole rows, hence whole heads, of the tile)
@@ -60,244 +92,33 @@ __device__ __forceinline__ float gelu_tanh_f(float z) {
   return 0.5f * z * (1.f + tanh_approx(u));
 }
 
-template <int EPI>
-__device__ __forceinline__ void epilogue_chunk(const GemmParams& p, int b, int row, int n0, const uint32_t (&r)[32]) {
-  // bias and gate are the same for every row of the tile: broadcast loads
-  float v[32];
-  const uint4* bp = reinterpret_cast<const uint4*>(p.bias + n0);
+// ---- staging buffers: row = lane, 16-byte pieces swizzled as the TMA boxes expect them ---------
+// fp32: 128-byte rows, 128-byte swizzle; bf16: 64-byte rows, 64-byte swizzle.
+__device__ __forceinline__ uint8_t* piece_f32(uint8_t* buf, int lane, int q) { return buf + lane * 128 + ((q ^ (lane & 7)) << 4); }
+__device__ __forceinline__ uint8_t* piece_b16(uint8_t* buf, int lane, int q) {
+  return buf + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4);
+}
+__device__ __forceinline__ void put_b16(uint8_t* buf, int lane, const float (&v)[CHUNK]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint4 bb = __ldg(bp + q);
-    v[8 * q + 0] = __uint_as_float(r[8 * q + 0]) + bf16_lo(bb.x);
-    v[8 * q + 1] = __uint_as_float(r[8 * q + 1]) + bf16_hi(bb.x);
-    v[8 * q + 2] = __uint_as_float(r[8 * q + 2]) + bf16_lo(bb.y);
-    v[8 * q + 3] = __uint_as_float(r[8 * q + 3]) + bf16_hi(bb.y);
-    v[8 * q + 4] = __uint_as_float(r[8 * q + 4]) + bf16_lo(bb.z);
-    v[8 * q + 5] = __uint_as_float(r[8 * q + 5]) + bf16_hi(bb.z);
-    v[8 * q + 6] = __uint_as_float(r[8 * q + 6]) + bf16_lo(bb.w);
-    v[8 * q + 7] = __uint_as_float(r[8 * q + 7]) + bf16_hi(bb.w);
-  }
-  if (row >= p.rows) return;
-  const size_t orow = ((size_t)b * p.out_batch_rows + row) * p.ldo + n0;
-  if constexpr (EPI == XEMA_EPI_BIAS || EPI == XEMA_EPI_BIAS_GELU) {
-    if constexpr (EPI == XEMA_EPI_BIAS_GELU) {
-#pragma unroll
-      for (int t = 0; t < 32; ++t) v[t] = gelu_tanh_f(v[t]);
-    }
-    uint4* op = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + orow);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      op[q] = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                         pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
-  } else {
-    const float4* gp = reinterpret_cast<const float4*>(p.gate + (size_t)b * p.gate_stride + n0);
-    const size_t rrow = ((size_t)b * p.resid_batch_rows + row) * p.ldr + n0;
-    if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
-      // out fp32 = resid(bf16) + gate * v
-      const uint4* rp = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.resid) + rrow);
-      float4* op = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + orow);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 x = __ldg(rp + q);
-        const float4 g0 = __ldg(gp + 2 * q), g1 = __ldg(gp + 2 * q + 1);
-        op[2 * q] = make_float4(fmaf(g0.x, v[8 * q + 0], bf16_lo(x.x)), fmaf(g0.y, v[8 * q + 1], bf16_hi(x.x)),
-                                fmaf(g0.z, v[8 * q + 2], bf16_lo(x.y)), fmaf(g0.w, v[8 * q + 3], bf16_hi(x.y)));
-        op[2 * q + 1] = make_float4(fmaf(g1.x, v[8 * q + 4], bf16_lo(x.z)), fmaf(g1.y, v[8 * q + 5], bf16_hi(x.z)),
-                                    fmaf(g1.z, v[8 * q + 6], bf16_lo(x.w)), fmaf(g1.w, v[8 * q + 7], bf16_hi(x.w)));
-      }
-    } else {
-      // out bf16 = resid(fp32) + gate * v
-      const float4* rp = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.resid) + rrow);
-      uint4* op = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + orow);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 x0 = __ldg(rp + 2 * q), x1 = __ldg(rp + 2 * q + 1);
-        const float4 g0 = __ldg(gp + 2 * q), g1 = __ldg(gp + 2 * q + 1);
-        op[q] = make_uint4(
-            pack_bf16x2(fmaf(g0.x, v[8 * q + 0], x0.x), fmaf(g0.y, v[8 * q + 1], x0.y)),
-            pack_bf16x2(fmaf(g0.z, v[8 * q + 2], x0.z), fmaf(g0.w, v[8 * q + 3], x0.w)),
-            pack_bf16x2(fmaf(g1.x, v[8 * q + 4], x1.x), fmaf(g1.y, v[8 * q + 5], x1.y)),
-            pack_bf16x2(fmaf(g1.z, v[8 * q + 6], x1.z), fmaf(g1.w, v[8 * q + 7], x1.w)));
-      }
-    }
-  }
+  for (int q = 0; q < 4; ++q)
+    *reinterpret_cast<uint4*>(piece_b16(buf, lane, q)) =
+        make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
+                   pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
 }
 
-// The two gated epilogues for one 32-column chunk of a warp's 32 rows, with coalesced global
-// accesses.  In the accumulator a thread owns a row, so a warp-wide 16-byte access would touch 32
-// different rows -- 32 separate lines per instruction, eight store instructions and four to eight
-// residual loads per chunk; the load/store unit then takes longer over a tile's epilogue (30 000
-// cycles measured) than the tensor pipe over the next tile's main loop (22 000).  Here the accumulator
-// goes through a per-warp shared-memory tile (rows padded to 36 floats) and comes back
-// transposed: eight lanes cover the 32 columns of one row, a warp instruction covers four whole
-// rows, and residual, gate and output are accessed a full row segment at a time.
-constexpr int STAGE_LD = 36;                         // floats per staged row (16-byte aligned, conflict-light)
-constexpr int STAGE_FLOATS = 32 * STAGE_LD;          // per warp
-template <int EPI>
-struct GatedResid {
-  typename std::conditional<EPI == XEMA_EPI_GATE_RES_F32, uint2, float4>::type x[8];
-  float4 gate;   // of the lane's four columns
-  uint2 bias;    // four bf16
-};
-// Requests what a lane needs for one chunk besides the accumulator: the residual values of its
-// four columns in eight rows, and the gate and bias of those columns.
-template <int EPI>
-__device__ __forceinline__ void gated_load_resid(const GemmParams& p, int b, int row0, int n0, int lane, GatedResid<EPI>& rs) {
-  const int c4 = (lane & 7) * 4;
-  const int rbase = row0 + (lane >> 3);
-  rs.gate = __ldg(reinterpret_cast<const float4*>(p.gate + (size_t)b * p.gate_stride + n0 + c4));
-  rs.bias = __ldg(reinterpret_cast<const uint2*>(p.bias + n0 + c4));
+// Accumulator chunk + bias (broadcast reads of the tile's bias in shared memory).
+__device__ __forceinline__ void load_chunk(uint32_t t_addr, const float* bias, float (&v)[CHUNK]) {
+  tmem_ld32(t_addr, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+  float4 bb[CHUNK / 4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = rbase + 4 * i;
-    if (row < p.rows) {
-      const size_t rrow = ((size_t)b * p.resid_batch_rows + row) * p.ldr + n0 + c4;
-      if constexpr (EPI == XEMA_EPI_GATE_RES_F32)
-        rs.x[i] = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(p.resid) + rrow));
-      else
-        rs.x[i] = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.resid) + rrow));
-    }
-  }
-}
-template <int EPI>
-__device__ __forceinline__ void epilogue_chunk_gated(const GemmParams& p, int b, int row0, int n0, const uint32_t (&r)[32],
-                                                     float* stage, int lane, const GatedResid<EPI>& rs) {
-  {
-    // the raw accumulator row of this thread into the tile
-    uint4* sp = reinterpret_cast<uint4*>(stage + lane * STAGE_LD);
+  for (int q = 0; q < CHUNK / 4; ++q) bb[q] = reinterpret_cast<const float4*>(bias)[q];
+  tmem_ld_wait_on(*reinterpret_cast<uint32_t(*)[32]>(&v[0]));
 #pragma unroll
-    for (int q = 0; q < 8; ++q) sp[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-  }
-  __syncwarp();
-  const int c4 = (lane & 7) * 4;                     // this lane's four columns of the chunk
-  const float4 g = rs.gate;
-  const float4 bs = make_float4(bf16_lo(rs.bias.x), bf16_hi(rs.bias.x), bf16_lo(rs.bias.y), bf16_hi(rs.bias.y));
-  const int rbase = row0 + (lane >> 3);
-  float4 v[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 a = *reinterpret_cast<const float4*>(stage + (4 * i + (lane >> 3)) * STAGE_LD + c4);
-    v[i] = make_float4(a.x + bs.x, a.y + bs.y, a.z + bs.z, a.w + bs.w);
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = rbase + 4 * i;
-    if (row < p.rows) {
-      const size_t orow = ((size_t)b * p.out_batch_rows + row) * p.ldo + n0 + c4;
-      if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + orow) =
-            make_float4(fmaf(g.x, v[i].x, bf16_lo(rs.x[i].x)), fmaf(g.y, v[i].y, bf16_hi(rs.x[i].x)),
-                        fmaf(g.z, v[i].z, bf16_lo(rs.x[i].y)), fmaf(g.w, v[i].w, bf16_hi(rs.x[i].y)));
-      } else {
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + orow) =
-            make_uint2(pack_bf16x2(fmaf(g.x, v[i].x, rs.x[i].x), fmaf(g.y, v[i].y, rs.x[i].y)),
-                       pack_bf16x2(fmaf(g.z, v[i].z, rs.x[i].z), fmaf(g.w, v[i].w, rs.x[i].w)));
-      }
-    }
-  }
-  __syncwarp();                                      // the tile is free for the next chunk
-}
-
-// One head (DH columns starting at n0) of this thread's row: acc + bias, RMSNorm over the head,
-// gain, rotation of adjacent pairs by the token's angles, bf16 store.
-template <int DH>
-__device__ __forceinline__ void epilogue_head_norm_rope(const GemmParams& p, int b, int row, int n0, uint32_t t_cols) {
-  float v[DH];
-#pragma unroll
-  for (int ch = 0; ch < DH / 32; ++ch)
-    tmem_ld32(t_cols + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[ch * 32]));
-  tmem_ld_wait();
-  if (row >= p.rows) return;
-  float ss = 0.f;
-#pragma unroll
-  for (int q = 0; q < DH / 8; ++q) {
-    const uint4 bb = __ldg(reinterpret_cast<const uint4*>(p.bias + n0) + q);
-    v[8 * q + 0] += bf16_lo(bb.x); v[8 * q + 1] += bf16_hi(bb.x);
-    v[8 * q + 2] += bf16_lo(bb.y); v[8 * q + 3] += bf16_hi(bb.y);
-    v[8 * q + 4] += bf16_lo(bb.z); v[8 * q + 5] += bf16_hi(bb.z);
-    v[8 * q + 6] += bf16_lo(bb.w); v[8 * q + 7] += bf16_hi(bb.w);
-#pragma unroll
-    for (int t = 0; t < 8; ++t) ss = fmaf(v[8 * q + t], v[8 * q + t], ss);
-  }
-  const float rstd = rsqrtf(ss * (1.f / DH) + p.rms_eps) * p.norm_out_scale;
-  const float4* rp = reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * DH);
-  uint4* op = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) +
-                                       ((size_t)b * p.out_batch_rows + row) * p.ldo + n0);
-#pragma unroll
-  for (int q = 0; q < DH / 8; ++q) {
-    const uint4 gg = __ldg(reinterpret_cast<const uint4*>(p.norm_gain) + q);
-    const float gn[8] = {bf16_lo(gg.x), bf16_hi(gg.x), bf16_lo(gg.y), bf16_hi(gg.y),
-                         bf16_lo(gg.z), bf16_hi(gg.z), bf16_lo(gg.w), bf16_hi(gg.w)};
-    const float4 cs0 = __ldg(rp + 2 * q), cs1 = __ldg(rp + 2 * q + 1);
-    const float cosv[4] = {cs0.x, cs0.z, cs1.x, cs1.z};
-    const float sinv[4] = {cs0.y, cs0.w, cs1.y, cs1.w};
-    float y[8];
-#pragma unroll
-    for (int pr = 0; pr < 4; ++pr) {
-      const float a = v[8 * q + 2 * pr] * rstd * gn[2 * pr];
-      const float c = v[8 * q + 2 * pr + 1] * rstd * gn[2 * pr + 1];
-      y[2 * pr] = a * cosv[pr] - c * sinv[pr];
-      y[2 * pr + 1] = a * sinv[pr] + c * cosv[pr];
-    }
-    op[q] = make_uint4(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]), pack_bf16x2(y[4], y[5]), pack_bf16x2(y[6], y[7]));
-  }
-}
-
-// The finished BN-wide accumulator row of one thread (TMEM address t_addr) -> global memory.
-// `stage`: the warp's shared-memory tile for the coalesced form of the gated epilogues, or null
-// (every thread then reads and writes its own row directly).
-template <int BN, int EPI>
-__device__ __forceinline__ void epilogue_row(const GemmParams& p, int b, int row, int n_base, uint32_t t_addr,
-                                             float* stage = nullptr) {
-  if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
-    // head by head; heads at or beyond norm_cols (the V half of a KV product) get the bias only
-#pragma unroll 1
-    for (int hc = 0; hc < BN; hc += p.head_dim) {
-      const int n0 = n_base + hc;
-      if (n0 < p.norm_cols) {
-        if (p.head_dim == 64) epilogue_head_norm_rope<64>(p, b, row, n0, t_addr + hc);
-        else epilogue_head_norm_rope<128>(p, b, row, n0, t_addr + hc);
-      } else {
-#pragma unroll 1
-        for (int ch = 0; ch < p.head_dim / 32; ++ch) {
-          uint32_t r[32];
-          tmem_ld32(t_addr + hc + ch * 32, r);
-          tmem_ld_wait();
-          epilogue_chunk<XEMA_EPI_BIAS>(p, b, row, n0 + ch * 32, r);
-        }
-      }
-    }
-  } else {
-    if constexpr (EPI == XEMA_EPI_GATE_RES_F32 || EPI == XEMA_EPI_GATE_RES_BF16) {
-      if (stage) {
-        // coalesced form; the residual of chunk c+1 is requested before chunk c is worked on, and
-        // all loads of a chunk are in flight together (one memory round trip per chunk, covered)
-        const int lane = threadIdx.x & 31;
-        const int row0 = row - lane;
-        GatedResid<EPI> ra, rb;
-        gated_load_resid<EPI>(p, b, row0, n_base, lane, ra);
-#pragma unroll 1
-        for (int ch = 0; ch < BN / 32; ch += 2) {
-          uint32_t r[32];
-          gated_load_resid<EPI>(p, b, row0, n_base + (ch + 1) * 32, lane, rb);
-          tmem_ld32(t_addr + ch * 32, r);
-          tmem_ld_wait();
-          epilogue_chunk_gated<EPI>(p, b, row0, n_base + ch * 32, r, stage, lane, ra);
-          if (ch + 2 < BN / 32) gated_load_resid<EPI>(p, b, row0, n_base + (ch + 2) * 32, lane, ra);
-          tmem_ld32(t_addr + (ch + 1) * 32, r);
-          tmem_ld_wait();
-          epilogue_chunk_gated<EPI>(p, b, row0, n_base + (ch + 1) * 32, r, stage, lane, rb);
-        }
-        return;
-      }
-    }
-#pragma unroll 1
-    for (int ch = 0; ch < BN / 32; ++ch) {
-      uint32_t r[32];
-      tmem_ld32(t_addr + ch * 32, r);
-      tmem_ld_wait();
-      epilogue_chunk<EPI>(p, b, row, n_base + ch * 32, r);
-    }
+  for (int q = 0; q < CHUNK / 4; ++q) {
+    v[4 * q + 0] += bb[q].x;
+    v[4 * q + 1] += bb[q].y;
+    v[4 * q + 2] += bb[q].z;
+    v[4 * q + 3] += bb[q].w;
   }
 }
 
@@ -319,204 +140,208 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, int m_tiles, int n_til
   return c;
 }
 
-template <int BN, int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                 const GemmParams p) {
-  using Cfg = GemmCfg<BN>;
-  constexpr int STAGES = Cfg::STAGES;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* bar_base = smem + STAGES * Cfg::STAGE_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(bar_base);
-  uint64_t* empty = full + STAGES;
-  uint64_t* tmem_full = empty + STAGES;
-  uint64_t* tmem_empty = tmem_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + 2);
-  volatile uint32_t* abort_flag = tmem_slot + 1;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tiles = (p.rows + BM - 1) / BM;
-  const int n_tiles = p.N / BN;
-  const int k_blocks = p.K / BK;
-  const int total_tiles = p.batch * m_tiles * n_tiles;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&tmem_full[s], 1);
-      mbar_init(&tmem_empty[s], 4);
-    }
-    *abort_flag = 0;
-    fence_mbar_init();
-    prefetch_tmap(&map_a);
-    prefetch_tmap(&map_w);
-  }
-  if (warp == 1) {
-    tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
-        const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
-          uint8_t* sb = sa + A_TILE_BYTES;
-          mbar_expect_tx(&full[stage], Cfg::STAGE_BYTES);
-          tma_load_3d(sa, &map_a, &full[stage], kb * BK, c.mt * BM, c.b);
-          tma_load_3d(sb, &map_w, &full[stage], kb * BK, c.nt * BN, 0);
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
-        }
-      }
-      if (!ok) {
-        // gave up: let the copies already issued land before the CTA leaves
-        for (int s = 0; s < STAGES; ++s) {
-          const int st = (stage + s) % STAGES;                 // oldest outstanding first
-          const uint32_t ph = (st < stage) ? phase : (phase ^ 1);
-          volatile uint32_t dummy = 0;
-          mbar_wait(&full[st], ph, &dummy);
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    // The whole warp walks the loop and waits together; one elected lane issues.  (A lone
-    // thread of a diverged warp issues MMAs markedly slower than the tensor pipe retires them.)
-    {
-      constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, false, false);
-      // Descriptors are built once and advanced by adding constants (the start-address field
-      // counts 16-byte units and never carries out of its 14 bits inside shared memory).
-      const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-      const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + A_TILE_BYTES), 16, 1024);
-      auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
-        return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
-      };
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
-        if (!(ok = wait_all(&tmem_empty[acc], acc_phase ^ 1))) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
-        uint32_t accumulate = 0;
-#pragma unroll 1
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = wait_all(&full[stage], phase))) break;
-          tc_fence_after();
-          if (elect_one()) {
-            const uint64_t soff = (uint64_t)(stage * (Cfg::STAGE_BYTES >> 4));
-            const uint64_t da = a_desc0 + soff, db = b_desc0 + soff;
-            mma_ss(d_tmem, da, db, idesc, accumulate);
-            mma_ss(d_tmem, da + 2, db + 2, idesc, 1);
-            mma_ss(d_tmem, da + 4, db + 4, idesc, 1);
-            mma_ss(d_tmem, da + 6, db + 6, idesc, 1);
-            mma_commit(&empty[stage]);
-          }
-          __syncwarp();
-          accumulate = 1;
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
-        }
-        if (!ok) break;
-        if (elect_one()) mma_commit(&tmem_full[acc]);
-        __syncwarp();
-        if (++acc == 2) { acc = 0; acc_phase ^= 1; }
-      }
-    }
-  } else {
-    // ---------------- epilogue ----------------
-    const int quad = warp & 3;           // TMEM lanes [32*quad, 32*quad + 32) belong to this warp
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
-      const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
-      ok = mbar_wait(&tmem_full[acc], acc_phase, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      const int row = c.mt * BM + quad * 32 + lane;
-      const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * BN;
-      epilogue_row<BN, EPI>(p, c.b, row, c.nt * BN, t_addr);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tmem_empty[acc]);
-      if (++acc == 2) { acc = 0; acc_phase ^= 1; }
-    }
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
-  }
-  if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
-}
-
-
-// ---------------------------------------------------------------------------------------------
-// CTA-pair variant (N a multiple of 256): two CTAs on neighbouring SMs share one 256 x 256
-// output tile.  Each CTA loads its own 128 rows of A and one half (128 rows) of the W tile, so a
-// stage costs 32 KB of shared-memory fill per SM instead of 48 KB and every MMA reads 8 KB of
-// operands per SM instead of 12 KB; the even CTA issues tcgen05.mma.cta_group::2 (M = 256),
-// which accumulates 128 rows x 256 columns in the TMEM of each CTA.
-//   full[s]        barrier of the even CTA: its producer expects the bytes of both CTAs, and
-//                  both CTAs' loads complete on it (an expect-tx arrival sent from the peer
-//                  CTA for every stage halved the speed of the whole loop)
-//   empty[s]       one barrier per CTA, released for both by a multicast commit
-//   tmem_full[a]   one barrier per CTA, same commit form
-//   tmem_empty[a]  barrier of the even CTA: the four epilogue warps of both CTAs arrive
-// The K loop and the per-instruction summation are the same for every row, so results do not
-// depend on how rows are chunked.
-constexpr int PAIR_BN = 256;
-constexpr int PAIR_STAGES = 6;
-constexpr int PAIR_B_HALF_BYTES = (PAIR_BN / 2) * BK * 2;
-constexpr int PAIR_STAGE_BYTES = A_TILE_BYTES + PAIR_B_HALF_BYTES;
-constexpr int PAIR_STAGE_TILE_BYTES = 4 * STAGE_FLOATS * 4;      // one transposition tile per epilogue warp
-constexpr int PAIR_SMEM_BYTES = 1024 + PAIR_STAGES * PAIR_STAGE_BYTES + 256 + PAIR_STAGE_TILE_BYTES;
-constexpr int PAIR_TMEM_COLS = 2 * PAIR_BN;
 // Limit of one drain wait after a give-up (about 50 ms): long enough for any copy in flight,
-// short enough that six of them in a row stay far below the limit of a regular wait.
+// short enough that several of them in a row stay far below the limit of a regular wait.
 constexpr long long kDrainLimitCycles = 100000000ll;
 
-template <int EPI>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
-gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                      const GemmParams p) {
-  constexpr int STAGES = PAIR_STAGES;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* bar_base = smem + STAGES * PAIR_STAGE_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(bar_base);
+// One epilogue warp: its staging ring and the chunks of one tile.
+template <int EPI, int BN, bool PAIR>
+struct Epilogue {
+  using Cfg = GemmCfg<EPI, BN, PAIR>;
+  static constexpr int RING = Cfg::RING;
+  const GemmParams& p;
+  const CUtensorMap* map_out;
+  const CUtensorMap* map_res;
+  uint8_t* ring;          // [RING][BUF_BYTES]
+  uint64_t* rbar;         // [RING] residual chunk has arrived
+  const float* bias;      // [BN], shared memory
+  const float* gate;      // [BN] (gated) or the RMSNorm gain
+  volatile uint32_t* abort_flag;
+  int lane;
+  uint32_t used = 0;      // chunks worked on so far (buffer = used % RING)
+  uint32_t asked = 0;     // residual chunks requested so far
+
+  __device__ __forceinline__ void request(int b, int row0, int n0) {   // whole warp; lane 0 acts
+    if (lane == 0) {
+      uint64_t* bar = rbar + asked % RING;
+      mbar_expect_tx(bar, EPI == XEMA_EPI_GATE_RES_F32 ? BUF_BYTES / 2 : BUF_BYTES);
+      tma_load_3d(ring + (asked % RING) * BUF_BYTES, map_res, bar, n0, row0, p.resid_batch ? b : 0);
+    }
+    __syncwarp();
+    ++asked;
+  }
+  // The chunk in buffer used % RING is complete in shared memory: send it off.
+  __device__ __forceinline__ void send(uint8_t* buf, int b, int row0, int n0) {
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_3d(map_out, buf, n0, row0, b);
+      bulk_commit();
+    }
+    ++used;
+  }
+  // Buffer for the next chunk of an epilogue without residual: its earlier store has been read.
+  __device__ __forceinline__ uint8_t* next_buf() {
+    if (lane == 0) bulk_wait_read<RING - 1>();
+    __syncwarp();
+    return ring + (used % RING) * BUF_BYTES;
+  }
+
+  __device__ __forceinline__ bool gated_tile(int b, int row0, int n_base, uint32_t t_addr) {
+#pragma unroll 1
+    for (int ch = 0; ch < BN / CHUNK; ++ch) {
+      uint8_t* buf = ring + (used % RING) * BUF_BYTES;
+      if (!mbar_wait_warp(rbar + used % RING, (used / RING) & 1u, abort_flag)) return false;
+      float v[CHUNK];
+      load_chunk(t_addr + ch * CHUNK, bias + ch * CHUNK, v);
+      const float4* g = reinterpret_cast<const float4*>(gate + ch * CHUNK);
+      if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
+        // out fp32 = resid(bf16) + gate * v
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 x = *reinterpret_cast<const uint4*>(piece_b16(buf, lane, q));
+          const float4 g0 = g[2 * q], g1 = g[2 * q + 1];
+          v[8 * q + 0] = fmaf(g0.x, v[8 * q + 0], bf16_lo(x.x));
+          v[8 * q + 1] = fmaf(g0.y, v[8 * q + 1], bf16_hi(x.x));
+          v[8 * q + 2] = fmaf(g0.z, v[8 * q + 2], bf16_lo(x.y));
+          v[8 * q + 3] = fmaf(g0.w, v[8 * q + 3], bf16_hi(x.y));
+          v[8 * q + 4] = fmaf(g1.x, v[8 * q + 4], bf16_lo(x.z));
+          v[8 * q + 5] = fmaf(g1.y, v[8 * q + 5], bf16_hi(x.z));
+          v[8 * q + 6] = fmaf(g1.z, v[8 * q + 6], bf16_lo(x.w));
+          v[8 * q + 7] = fmaf(g1.w, v[8 * q + 7], bf16_hi(x.w));
+        }
+      } else {
+        // out bf16 = resid(fp32) + gate * v
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float4 x = *reinterpret_cast<const float4*>(piece_f32(buf, lane, q));
+          const float4 gg = g[q];
+          v[4 * q + 0] = fmaf(gg.x, v[4 * q + 0], x.x);
+          v[4 * q + 1] = fmaf(gg.y, v[4 * q + 1], x.y);
+          v[4 * q + 2] = fmaf(gg.z, v[4 * q + 2], x.z);
+          v[4 * q + 3] = fmaf(gg.w, v[4 * q + 3], x.w);
+        }
+      }
+      __syncwarp();                                    // every lane has read its residual row
+      if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(piece_f32(buf, lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      } else {
+        put_b16(buf, lane, v);
+      }
+      send(buf, b, row0, n_base + ch * CHUNK);
+      // the buffer of the chunk before this one takes the next residual once its store has been read
+      if (ch > 0 && ch - 1 + RING < BN / CHUNK) {
+        if (lane == 0) bulk_wait_read<1>();
+        __syncwarp();
+        request(b, row0, n_base + (ch - 1 + RING) * CHUNK);
+      }
+    }
+    return true;
+  }
+
+  __device__ __forceinline__ void plain_chunk(int b, int row0, int n_base, int col, uint32_t t_addr) {
+    float v[CHUNK];
+    uint8_t* buf = next_buf();
+    load_chunk(t_addr + col, bias + col, v);
+    if constexpr (EPI == XEMA_EPI_BIAS_GELU) {
+#pragma unroll
+      for (int t = 0; t < CHUNK; ++t) v[t] = gelu_tanh_f(v[t]);
+    }
+    put_b16(buf, lane, v);
+    send(buf, b, row0, n_base + col);
+  }
+
+  // 16 angles (32 columns) of one row of the rotation table
+  __device__ __forceinline__ void load_angles(const float4* rp, float4 (&cs)[8]) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) cs[q] = __ldg(rp + q);
+  }
+  // acc + bias, RMSNorm over each head, gain, rotation of adjacent pairs by the token's angles.
+  // First the head norms from a pass over the accumulator, then 32 columns of every head per
+  // step, so that a row's angles are loaded once per tile and not once per head.
+  template <int DH>
+  __device__ __forceinline__ void norm_rope_tile(int b, int row0, int n_base, uint32_t t_addr, float4 (&cs)[8]) {
+    constexpr int HEADS = BN / DH;
+    const int norm_heads = min(HEADS, max(0, (p.norm_cols - n_base) / DH));
+    float rstd[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int h = 0; h < norm_heads; ++h) {
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < DH; c += CHUNK) {
+        float v[CHUNK];
+        load_chunk(t_addr + h * DH + c, bias + h * DH + c, v);
+#pragma unroll
+        for (int t = 0; t < CHUNK; t += 4) {
+          s0 = fmaf(v[t], v[t], s0);
+          s1 = fmaf(v[t + 1], v[t + 1], s1);
+          s2 = fmaf(v[t + 2], v[t + 2], s2);
+          s3 = fmaf(v[t + 3], v[t + 3], s3);
+        }
+      }
+      const float r = rsqrtf(((s0 + s1) + (s2 + s3)) * (1.f / DH) + p.rms_eps) * p.norm_out_scale;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rstd[i] = h == i ? r : rstd[i];
+    }
+    const int row = min(row0 + lane, p.rows - 1);
+    const float4* rp = reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * DH);
+#pragma unroll 1
+    for (int c = 0; c < DH; c += CHUNK) {
+#pragma unroll 1
+      for (int h = 0; h < HEADS; ++h) {
+        const int col = h * DH + c;
+        if (h >= norm_heads) {                     // the V half of a K | V product gets the bias only
+          plain_chunk(b, row0, n_base, col, t_addr);
+          continue;
+        }
+        const float r = h == 0 ? rstd[0] : h == 1 ? rstd[1] : h == 2 ? rstd[2] : rstd[3];
+        float v[CHUNK];
+        uint8_t* buf = next_buf();
+        load_chunk(t_addr + col, bias + col, v);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float4 g = reinterpret_cast<const float4*>(gate + c)[q];
+          const float a0 = v[4 * q + 0] * r * g.x, c0 = v[4 * q + 1] * r * g.y;
+          const float a1 = v[4 * q + 2] * r * g.z, c1 = v[4 * q + 3] * r * g.w;
+          v[4 * q + 0] = a0 * cs[q].x - c0 * cs[q].y;
+          v[4 * q + 1] = a0 * cs[q].y + c0 * cs[q].x;
+          v[4 * q + 2] = a1 * cs[q].z - c1 * cs[q].w;
+          v[4 * q + 3] = a1 * cs[q].w + c1 * cs[q].z;
+        }
+        put_b16(buf, lane, v);
+        send(buf, b, row0, n_base + col);
+      }
+      if (c + CHUNK < DH && norm_heads > 0) load_angles(rp + (c + CHUNK) / 4, cs);
+    }
+  }
+};
+
+template <int EPI, int BN, bool PAIR>
+__device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_out,
+                                          const CUtensorMap& map_res, const GemmParams& p) {
+  using Cfg = GemmCfg<EPI, BN, PAIR>;
+  constexpr int STAGES = Cfg::STAGES, RING = Cfg::RING;
+  constexpr bool GATED = kGated<EPI>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
   uint64_t* empty = full + STAGES;
   uint64_t* tmem_full = empty + STAGES;
   uint64_t* tmem_empty = tmem_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + 2);
+  uint64_t* res_full = tmem_empty + 2;               // [4][RING]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_full + 4 * RING);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();            // 0: even CTA (issues the MMAs), 1: its peer
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int m_tiles = (p.rows + 2 * BM - 1) / (2 * BM);   // tiles of 256 rows
-  const int n_tiles = p.N / PAIR_BN;
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0;   // 0: even CTA (issues the MMAs), 1: its peer
+  const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x, n_workers = PAIR ? gridDim.x >> 1 : gridDim.x;
+  constexpr int TM = PAIR ? 2 * BM : BM;                // rows per tile
+  const int m_tiles = (p.rows + TM - 1) / TM;
+  const int n_tiles = p.N / BN;
   const int k_blocks = p.K / BK;
-  const int total_tiles = p.batch * m_tiles * n_tiles;
+  const bool aligned = (smem_u32(smem) & 1023u) == 0;   // the swizzled tiles need a 1024-byte aligned base
+  const int total_tiles = aligned ? p.batch * m_tiles * n_tiles : 0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -525,21 +350,32 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&tmem_full[s], 1);
-      mbar_init(&tmem_empty[s], 8);
+      mbar_init(&tmem_empty[s], PAIR ? 8 : 4);
     }
-    *abort_flag = 0;
+    if (GATED)
+      for (int s = 0; s < 4 * RING; ++s) mbar_init(&res_full[s], 1);
+    *abort_flag = aligned ? 0u : 1u;
     fence_mbar_init();
     prefetch_tmap(&map_a);
     prefetch_tmap(&map_w);
+    prefetch_tmap(&map_out);
+    if (GATED) prefetch_tmap(&map_res);
   }
   if (warp == 1) {
-    tmem_alloc_pair(tmem_slot, PAIR_TMEM_COLS);
-    tmem_relinquish_pair();
+    if (PAIR) {
+      tmem_alloc_pair(tmem_slot, Cfg::TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
-  cluster_arrive();      // both CTAs' barriers exist before anything arrives on them remotely
-  cluster_wait();
+  if (PAIR) {
+    cluster_arrive();      // both CTAs' barriers exist before anything arrives on them remotely
+    cluster_wait();
+  }
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -549,33 +385,40 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
+      for (int tile = worker; ok && tile < total_tiles; tile += n_workers) {
         const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          uint8_t* sa = smem + stage * PAIR_STAGE_BYTES;
+          uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
           uint8_t* sb = sa + A_TILE_BYTES;
-          const uint32_t full0 = mapa_shared(smem_u32(&full[stage]), 0);
-          if (rank == 0) mbar_expect_tx(&full[stage], 2 * PAIR_STAGE_BYTES);
-          tma_load_3d_pair(sa, &map_a, full0, kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
-          tma_load_3d_pair(sb, &map_w, full0, kb * BK, c.nt * PAIR_BN + (int)rank * (PAIR_BN / 2), 0);
+          if constexpr (PAIR) {
+            const uint32_t full0 = mapa_shared(smem_u32(&full[stage]), 0);
+            if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::STAGE_BYTES);
+            tma_load_3d_pair(sa, &map_a, full0, kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
+            tma_load_3d_pair(sb, &map_w, full0, kb * BK, c.nt * BN + (int)rank * (BN / 2), 0);
+          } else {
+            mbar_expect_tx(&full[stage], Cfg::STAGE_BYTES);
+            tma_load_3d(sa, &map_a, &full[stage], kb * BK, c.mt * BM, c.b);
+            tma_load_3d(sb, &map_w, &full[stage], kb * BK, c.nt * BN, 0);
+          }
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
-      // Tail: the same waits as for STAGES further fills, without filling.  They return once the
-      // commits that release this CTA's last fills (arrivals multicast by the even CTA) have
+      // Tail (pair): the same waits as for STAGES further fills, without filling.  They return once
+      // the commits that release this CTA's last fills (arrivals multicast by the even CTA) have
       // landed here, so none of them can reach this CTA's barriers after it has left.
-      for (int s = 0; ok && s < STAGES; ++s) {
-        ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag);
-        if (++stage == STAGES) { stage = 0; phase ^= 1; }
+      if constexpr (PAIR) {
+        for (int s = 0; ok && s < STAGES; ++s) {
+          ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag);
+          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+        }
       }
       if (!ok) {
-        // Gave up.  Copies already issued must land before either CTA leaves: all of them
-        // complete on the even CTA's full[] barriers, so the even CTA waits (bounded, and
-        // without looking at the abort flag) for the latest fill of every stage, which covers
-        // the bytes of both CTAs wherever both issued; the closing cluster barrier then keeps
-        // the peer until that is done.  A short settling time on both CTAs covers loads of a
-        // stage that only one of the two CTAs still issued.
+        // Gave up.  Copies already issued must land before a CTA leaves.  Pair: all of them complete
+        // on the even CTA's full[] barriers, so the even CTA waits (bounded, and without looking
+        // at the abort flag) for the latest fill of every stage, which covers the bytes of both CTAs
+        // wherever both issued; the closing cluster barrier then keeps the peer until that is done.
+        // A short settling time covers loads of a stage that only one of the two CTAs still issued.
         if (rank == 0) {
           for (int s = 0; s < STAGES; ++s) {
             const int st = (stage + s) % STAGES;                 // oldest outstanding first
@@ -588,9 +431,13 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer (even CTA only; converged warp, one elected lane) ----------------
+    // ---------------- MMA issuer (pair: even CTA only) ----------------
+    // The whole warp walks the loop and waits together; one elected lane issues.  (A lone
+    // thread of a diverged warp issues MMAs markedly slower than the tensor pipe retires them.)
     if (rank == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, PAIR_BN, false, false);
+      constexpr uint32_t idesc = idesc_bf16_f32(TM, BN, false, false);
+      // Descriptors are built once and advanced by adding constants (the start-address field
+      // counts 16-byte units and never carries out of its 14 bits inside shared memory).
       const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
       const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + A_TILE_BYTES), 16, 1024);
       auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
@@ -601,87 +448,164 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
-        // the peer's epilogue warps arrive on this barrier from their own CTA: cluster-scope acquire
+      for (int tile = worker; ok && tile < total_tiles; tile += n_workers) {
+        // pair: the peer's epilogue warps arrive from their own CTA, hence the cluster-scope acquire
         if (!(ok = __all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[acc], acc_phase ^ 1, abort_flag)))) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * PAIR_BN;
+        const uint32_t d_tmem = tmem_base + acc * BN;
         uint32_t accumulate = 0;
 #pragma unroll 1
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = wait_all(&full[stage], phase))) break;
           tc_fence_after();
           if (elect_one()) {
-            const uint64_t soff = (uint64_t)(stage * (PAIR_STAGE_BYTES >> 4));
+            const uint64_t soff = (uint64_t)(stage * (Cfg::STAGE_BYTES >> 4));
             const uint64_t da = a_desc0 + soff, db = b_desc0 + soff;
-            mma_ss_pair(d_tmem, da, db, idesc, accumulate);
-            mma_ss_pair(d_tmem, da + 2, db + 2, idesc, 1);
-            mma_ss_pair(d_tmem, da + 4, db + 4, idesc, 1);
-            mma_ss_pair(d_tmem, da + 6, db + 6, idesc, 1);
-            mma_commit_pair(&empty[stage]);
+            if constexpr (PAIR) {
+              mma_ss_pair(d_tmem, da, db, idesc, accumulate);
+              mma_ss_pair(d_tmem, da + 2, db + 2, idesc, 1);
+              mma_ss_pair(d_tmem, da + 4, db + 4, idesc, 1);
+              mma_ss_pair(d_tmem, da + 6, db + 6, idesc, 1);
+              mma_commit_pair(&empty[stage]);
+            } else {
+              mma_ss(d_tmem, da, db, idesc, accumulate);
+              mma_ss(d_tmem, da + 2, db + 2, idesc, 1);
+              mma_ss(d_tmem, da + 4, db + 4, idesc, 1);
+              mma_ss(d_tmem, da + 6, db + 6, idesc, 1);
+              mma_commit(&empty[stage]);
+            }
           }
           __syncwarp();
           accumulate = 1;
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        if (elect_one()) mma_commit_pair(&tmem_full[acc]);
+        if (elect_one()) {
+          if (PAIR) mma_commit_pair(&tmem_full[acc]);
+          else mma_commit(&tmem_full[acc]);
+        }
         __syncwarp();
         if (++acc == 2) { acc = 0; acc_phase ^= 1; }
       }
     }
   } else {
-    // ---------------- epilogue (both CTAs, each its own 128 rows) ----------------
-    const int quad = warp & 3;
+    // ---------------- epilogue (pair: each CTA its own 128 rows) ----------------
+    const int quad = warp & 3;           // TMEM lanes [32*quad, 32*quad + 32) belong to this warp
+    float* s_bias = reinterpret_cast<float*>(smem + Cfg::OFF_BIAS);
+    float* s_gate = reinterpret_cast<float*>(smem + Cfg::OFF_GATE);
+    Epilogue<EPI, BN, PAIR> ep{p, &map_out, &map_res, smem + Cfg::OFF_RING + quad * RING * BUF_BYTES, res_full + quad * RING,
+                               s_bias, s_gate, abort_flag, lane};
+    const int et = threadIdx.x - 64;     // 0..127
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
+    if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
+      if (et < p.head_dim) s_gate[et] = __bfloat162float(p.norm_gain[et]);   // read after the tile's barrier
+    }
+    for (int tile = worker; tile < total_tiles; tile += n_workers) {
+      // The four warps meet (the previous tile's bias and gate are no longer read) and agree on going
+      // on: a warp that gave up a wait still comes here, so that nobody waits for it.
+      if (!(ok = named_barrier_and(1, 128, ok))) break;
       const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
-      ok = mbar_wait(&tmem_full[acc], acc_phase, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
+      const int row0 = (c.mt * (TM / BM) + (int)rank) * BM + quad * 32;
+      const int n_base = c.nt * BN;
+      const bool live = row0 < p.rows;   // rows past the end: nothing to read or store
+      // everything the tile needs besides its accumulator, requested while the main loop runs
+      if constexpr (GATED) {
+        if (lane == 0) bulk_wait_read<0>();
+        __syncwarp();
+        if (live)
+          for (int ch = 0; ch < (RING < BN / CHUNK ? RING : BN / CHUNK); ++ch) ep.request(c.b, row0, n_base + ch * CHUNK);
+      }
+      float4 cs[8];
+      if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
+        if (live && n_base < p.norm_cols) {
+          const int row = min(row0 + lane, p.rows - 1);
+          ep.load_angles(reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * p.head_dim), cs);
+        }
+      }
+      for (int i = et * 2; i < BN; i += 256) {
+        const uint32_t bb = __ldg(reinterpret_cast<const uint32_t*>(p.bias + n_base + i));
+        *reinterpret_cast<float2*>(s_bias + i) = make_float2(bf16_lo(bb), bf16_hi(bb));
+        if constexpr (GATED)
+          *reinterpret_cast<float2*>(s_gate + i) =
+              __ldg(reinterpret_cast<const float2*>(p.gate + (size_t)c.b * p.gate_stride + n_base + i));
+      }
+      named_barrier(1, 128);
+      ok = mbar_wait_warp(&tmem_full[acc], acc_phase, abort_flag);
       tc_fence_after();
-      const int row = (c.mt * 2 + (int)rank) * BM + quad * 32 + lane;
-      const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * PAIR_BN;
-      epilogue_row<PAIR_BN, EPI>(p, c.b, row, c.nt * PAIR_BN, t_addr,
-                                 reinterpret_cast<float*>(bar_base + 256) + quad * STAGE_FLOATS);
+      const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * BN;
+      if (live && ok) {
+        if constexpr (GATED) {
+          ok = ep.gated_tile(c.b, row0, n_base, t_addr);
+        } else if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
+          if (p.head_dim == 64) ep.template norm_rope_tile<64>(c.b, row0, n_base, t_addr, cs);
+          else if constexpr (BN >= 128) ep.template norm_rope_tile<128>(c.b, row0, n_base, t_addr, cs);
+        } else {
+#pragma unroll 1
+          for (int col = 0; col < BN; col += CHUNK) ep.plain_chunk(c.b, row0, n_base, col, t_addr);
+        }
+      }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tmem_empty[acc]), 0));
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(mapa_shared(smem_u32(&tmem_empty[acc]), 0));
+        else mbar_arrive(&tmem_empty[acc]);
+      }
       if (++acc == 2) { acc = 0; acc_phase ^= 1; }
     }
+    if (GATED && !ok) {
+      // gave up: the residual chunks already requested must land before the CTA leaves
+      for (uint32_t i = ep.asked > (uint32_t)RING ? ep.asked - RING : 0; i < ep.asked; ++i) {
+        volatile uint32_t dummy = 0;
+        mbar_wait_slow(ep.rbar + i % RING, (i / RING) & 1u, &dummy, kDrainLimitCycles);
+      }
+    }
+    if (lane == 0) bulk_wait<0>();       // this warp's stores are complete
+    __syncwarp();
   }
 
-  // Neither CTA leaves (or frees TMEM) while the other may still read its shared memory, write
+  // Pair: neither CTA leaves (or frees TMEM) while the other may still read its shared memory, write
   // its TMEM or arrive on its barriers.
   tc_fence_before();
   __syncthreads();
-  cluster_arrive();
-  cluster_wait();
+  if (PAIR) {
+    cluster_arrive();
+    cluster_wait();
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc_pair(tmem_base, PAIR_TMEM_COLS);
+    if (PAIR) tmem_dealloc_pair(tmem_base, Cfg::TMEM_COLS);
+    else tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
   }
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
 }
 
+template <int EPI, int BN>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
+                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmParams p) {
+  gemm_body<EPI, BN, false>(map_a, map_w, map_out, map_res, p);
+}
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
+gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
+                      const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
+                      const GemmParams p) {
+  gemm_body<EPI, PAIR_BN, true>(map_a, map_w, map_out, map_res, p);
+}
+
 // ---------------------------------------------------------------------------------------------
-static GemmParams make_params(const GemmLaunch& g) {
+GemmParams make_params(const GemmLaunch& g) {
   GemmParams p;
   p.bias = (const __nv_bfloat16*)g.bias;
-  p.out = g.out;
-  p.ldo = g.ldo;
-  p.out_batch_rows = g.out_batch_rows;
-  p.resid = g.resid;
-  p.ldr = g.ldr;
-  p.resid_batch_rows = g.resid_batch_rows;
   p.gate = g.gate;
   p.gate_stride = g.gate_stride;
   p.batch = g.batch;
   p.rows = g.rows;
   p.N = g.N;
   p.K = g.K;
+  p.resid_batch = g.resid_batch_rows != 0;
   p.status = g.status;
   p.norm_gain = (const __nv_bfloat16*)g.norm_gain;
   p.rope = g.rope;
@@ -693,25 +617,24 @@ static GemmParams make_params(const GemmLaunch& g) {
   return p;
 }
 
-template <int BN, int EPI>
-static int launch_gemm_t(const GemmLaunch& g, cudaStream_t stream) {
-  using Cfg = GemmCfg<BN>;
+template <int EPI, int BN>
+int launch_single(const GemmLaunch& g, cudaStream_t stream) {
+  using Cfg = GemmCfg<EPI, BN, false>;
   static PerDeviceInt attr_done;
-  auto kern = gemm_bf16_kernel<BN, EPI>;
+  auto kern = gemm_bf16_kernel<EPI, BN>;
   if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
-  const GemmParams p = make_params(g);
-  const int m_tiles = (g.rows + BM - 1) / BM;
-  const long long tiles = (long long)g.batch * m_tiles * (g.N / BN);
+  const long long tiles = (long long)g.batch * ((g.rows + BM - 1) / BM) * (g.N / BN);
   const int grid = (int)std::min<long long>(tiles, sm_count());
-  kern<<<grid, GEMM_THREADS, Cfg::SMEM_BYTES, stream>>>(g.map_a, g.map_w, p);
+  kern<<<grid, GEMM_THREADS, Cfg::SMEM_BYTES, stream>>>(g.map_a, g.map_w, g.map_out, g.map_res, make_params(g));
   return check_launch();
 }
 
 template <int EPI>
-static int launch_gemm_pair_t(const GemmLaunch& g, cudaStream_t stream) {
+int launch_pair(const GemmLaunch& g, cudaStream_t stream) {
+  using Cfg = GemmCfg<EPI, PAIR_BN, true>;
   static PerDeviceInt attr_done;
   auto kern = gemm_bf16_pair_kernel<EPI>;
-  if (int rc = ensure_smem_attr(kern, PAIR_SMEM_BYTES, attr_done)) return rc;
+  if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
   // A persistent grid must be resident all at once: ask how many CTA pairs fit on the device
   // (SMs are handed out to clusters in hardware groups, so it can be fewer than SMs / 2).
   static PerDeviceInt pairs_cache;
@@ -721,7 +644,7 @@ static int launch_gemm_pair_t(const GemmLaunch& g, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (sm_count() / 2), 1, 1);
     cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = PAIR_SMEM_BYTES;
+    cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
@@ -738,42 +661,31 @@ static int launch_gemm_pair_t(const GemmLaunch& g, cudaStream_t stream) {
     max_pairs = std::min(n, sm_count() / 2);
     pairs_cache.set(dev, max_pairs);
   }
-  const GemmParams p = make_params(g);
-  const int m_tiles = (g.rows + 2 * BM - 1) / (2 * BM);
-  const long long tiles = (long long)g.batch * m_tiles * (g.N / PAIR_BN);
+  const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / PAIR_BN);
   const int pairs = (int)std::min<long long>(tiles, max_pairs);
-  kern<<<2 * pairs, GEMM_THREADS, PAIR_SMEM_BYTES, stream>>>(g.map_a, g.map_w, p);
+  kern<<<2 * pairs, GEMM_THREADS, Cfg::SMEM_BYTES, stream>>>(g.map_a, g.map_w, g.map_out, g.map_res, make_params(g));
   return check_launch();
 }
 
-static int launch_gemm_pair(const GemmLaunch& g, cudaStream_t stream) {
-  switch (g.epilogue) {
-    case XEMA_EPI_BIAS: return launch_gemm_pair_t<XEMA_EPI_BIAS>(g, stream);
-    case XEMA_EPI_BIAS_GELU: return launch_gemm_pair_t<XEMA_EPI_BIAS_GELU>(g, stream);
-    case XEMA_EPI_GATE_RES_F32: return launch_gemm_pair_t<XEMA_EPI_GATE_RES_F32>(g, stream);
-    case XEMA_EPI_GATE_RES_BF16: return launch_gemm_pair_t<XEMA_EPI_GATE_RES_BF16>(g, stream);
-    case XEMA_EPI_BIAS_NORM_ROPE: return launch_gemm_pair_t<XEMA_EPI_BIAS_NORM_ROPE>(g, stream);
-    default: return XEMA_EINVAL;
-  }
+template <int EPI>
+int launch_epi(const GemmLaunch& g, cudaStream_t stream) {
+  if (g.block_n == 256) return launch_pair<EPI>(g, stream);
+  if (g.block_n == 128) return launch_single<EPI, 128>(g, stream);
+  return XEMA_EINVAL;
 }
 
-template <int BN>
-static int launch_gemm_bn(const GemmLaunch& g, cudaStream_t stream) {
-  switch (g.epilogue) {
-    case XEMA_EPI_BIAS: return launch_gemm_t<BN, XEMA_EPI_BIAS>(g, stream);
-    case XEMA_EPI_BIAS_GELU: return launch_gemm_t<BN, XEMA_EPI_BIAS_GELU>(g, stream);
-    case XEMA_EPI_GATE_RES_F32: return launch_gemm_t<BN, XEMA_EPI_GATE_RES_F32>(g, stream);
-    case XEMA_EPI_GATE_RES_BF16: return launch_gemm_t<BN, XEMA_EPI_GATE_RES_BF16>(g, stream);
-    case XEMA_EPI_BIAS_NORM_ROPE: return launch_gemm_t<BN, XEMA_EPI_BIAS_NORM_ROPE>(g, stream);
-    default: return XEMA_EINVAL;
-  }
-}
+}  // namespace
 
 int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
   if (g.rows == 0 || g.batch == 0) return XEMA_OK;
-  if (g.block_n == 256) return launch_gemm_pair(g, stream);
-  if (g.block_n == 128) return launch_gemm_bn<128>(g, stream);
-  return XEMA_EINVAL;
+  switch (g.epilogue) {
+    case XEMA_EPI_BIAS: return launch_epi<XEMA_EPI_BIAS>(g, stream);
+    case XEMA_EPI_BIAS_GELU: return launch_epi<XEMA_EPI_BIAS_GELU>(g, stream);
+    case XEMA_EPI_GATE_RES_F32: return launch_epi<XEMA_EPI_GATE_RES_F32>(g, stream);
+    case XEMA_EPI_GATE_RES_BF16: return launch_epi<XEMA_EPI_GATE_RES_BF16>(g, stream);
+    case XEMA_EPI_BIAS_NORM_ROPE: return launch_epi<XEMA_EPI_BIAS_NORM_ROPE>(g, stream);
+    default: return XEMA_EINVAL;
+  }
 }
 
 int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw) {
@@ -792,12 +704,20 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
   if (mis(a) || mis(w) || mis(g->bias) || mis(g->out) || (g->resid && mis(g->resid)) || (g->gate && mis(g->gate)))
     return XEMA_EALIGN;
-  // tile width from N alone, so the arithmetic of a row never depends on how rows are chunked
   g->block_n = (g->N % 256 == 0) ? 256 : 128;
-  int rc = encode_tmap_bf16(&g->map_a, a, g->K, g->rows > 0 ? g->rows : 1, g->batch, lda, a_batch_rows, BM);
+  const long long rows = g->rows > 0 ? g->rows : 1;
+  int rc = encode_tmap_bf16(&g->map_a, a, g->K, rows, g->batch, lda, a_batch_rows, BM);
   if (rc) return rc;
-  // the pair kernel (N % 256 == 0) loads the W tile as two 128-row halves, one per CTA
-  return encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, 128);
+  // the pair form loads its W tile as two 128-row halves, one per CTA
+  rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, 128);
+  if (rc) return rc;
+  // results leave, and residuals arrive, as boxes of 32 columns x 32 rows
+  rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, g->N, rows, g->batch, g->ldo,
+                         g->out_batch_rows);
+  if (rc || !gated) return rc;
+  const bool per_batch = g->resid_batch_rows != 0;
+  return encode_tmap_box32(&g->map_res, g->resid, g->epilogue == XEMA_EPI_GATE_RES_BF16, g->N, rows,
+                           per_batch ? g->batch : 1, g->ldr, g->resid_batch_rows);
 }
 
 }  // namespace xema

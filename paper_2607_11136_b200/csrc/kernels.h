@@ -58,11 +58,17 @@ int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void*
 // columns read as zero.
 int encode_tmap_bf16(CUtensorMap* out, const void* base, long long cols, long long rows, long long batch,
                      long long ld, long long batch_rows, int box_rows);
+// bf16 or fp32 tensor viewed the same way; box = 32 columns x 32 rows x 1, swizzled over its
+// 64-byte (bf16) or 128-byte (fp32) rows.
+int encode_tmap_box32(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
+                      long long ld, long long batch_rows);
 
 // ---- GEMM ------------------------------------------------------------------------------------
 struct GemmLaunch {
   CUtensorMap map_a;   // [batch][rows][K], box 64 x 128
-  CUtensorMap map_w;   // [1][N][K],       box 64 x block_n
+  CUtensorMap map_w;   // [1][N][K],       box 64 x 128
+  CUtensorMap map_out; // [batch][rows][N], box 32 x 32
+  CUtensorMap map_res; // the same for the residual (gated epilogues)
   const void* bias;    // bf16 [N]
   void* out;
   long long ldo, out_batch_rows;
@@ -79,7 +85,7 @@ struct GemmLaunch {
   float rms_eps;
   float norm_out_scale;   // the normalised, rotated heads are multiplied by this before rounding (1 = as they are)
 };
-// Fills map_a / map_w / block_n from plain pointers.
+// Fills the descriptors and block_n (tile width) from plain pointers.
 int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw);
 int launch_gemm(const GemmLaunch& g, cudaStream_t stream);
 

@@ -65,26 +65,40 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-int encode_tmap_bf16(CUtensorMap* out, const void* base, long long cols, long long rows, long long batch,
-                     long long ld, long long batch_rows, int box_rows) {
+static int encode_tmap(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
+                       long long ld, long long batch_rows, int box_cols, int box_rows, CUtensorMapSwizzle swizzle) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return XEMA_ECUDA;
-  if (cols < 64 || rows < 1 || batch < 1 || ld < cols || box_rows < 1 || box_rows > 256) return XEMA_EINVAL;
-  if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return XEMA_EALIGN;
-  if (batch > 1 && batch_rows < rows) return XEMA_EINVAL;
+  const int elem = f32 ? 4 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch};
-  long long bstride = (batch_rows > 0 ? batch_rows : rows) * ld * 2;
-  cuuint64_t strides[2] = {(cuuint64_t)(ld * 2), (cuuint64_t)bstride};
-  cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, 1u};
+  long long bstride = (batch_rows > 0 ? batch_rows : rows) * ld * elem;
+  cuuint64_t strides[2] = {(cuuint64_t)(ld * elem), (cuuint64_t)bstride};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1u};
   cuuint32_t estr[3] = {1u, 1u, 1u};
-  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+  CUresult r = fn(out, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base),
+                  dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     t_last_cuda_error = (int)r;
     return XEMA_ECUDA;
   }
   return XEMA_OK;
+}
+
+int encode_tmap_bf16(CUtensorMap* out, const void* base, long long cols, long long rows, long long batch,
+                     long long ld, long long batch_rows, int box_rows) {
+  if (cols < 64 || rows < 1 || batch < 1 || ld < cols || box_rows < 1 || box_rows > 256) return XEMA_EINVAL;
+  if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return XEMA_EALIGN;
+  if (batch > 1 && batch_rows < rows) return XEMA_EINVAL;
+  return encode_tmap(out, base, false, cols, rows, batch, ld, batch_rows, 64, box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+int encode_tmap_box32(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
+                      long long ld, long long batch_rows) {
+  if (cols < 32 || rows < 1 || batch < 1 || ld < cols) return XEMA_EINVAL;
+  if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return XEMA_EALIGN;
+  return encode_tmap(out, base, f32, cols, rows, batch, ld, batch_rows, 32, 32,
+                     f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 // ---------------------------------------------------------------------------------------------

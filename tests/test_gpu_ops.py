@@ -140,6 +140,22 @@ def test_gemm_epilogues(epi, B, rows, N, K):
         assert_bf16_close(got, ref, ("gemm", epi, B, rows, N, K), atol_rms=2e-3 if epi == xb.EPI_BIAS_GELU else 2e-4)
 
 
+@pytest.mark.parametrize("epi", [0, 1, 2, 3])
+@pytest.mark.parametrize("rows", [1, 31, 33, 127, 160, 225, 257])
+def test_gemm_epilogue_row_edges(epi, rows):
+    """Rows that end inside, at and just past a warp's 32 and a tile's 128 / 256 rows, in both tile
+    forms (N = 384: one CTA per tile, N = 512: CTA pairs), two batch elements: the results leave in
+    boxes of 32 rows x 32 columns, and rows past the end must stay untouched (checked by
+    _gemm_case).  Tolerances as in test_gemm_epilogues: half a bf16 spacing of the output, 1e-4 of
+    RMS for fp32 sums of K = 192 products."""
+    for N in (384, 512):
+        got, ref = _gemm_case(np.random.default_rng(300 + rows + epi), 2, rows, N, 192, epi)
+        if epi == xb.EPI_GATE_RES_F32:
+            assert_close(got, ref, ("gemm edges", epi, rows, N), rel=1e-4, cos=0.9999999)
+        else:
+            assert_bf16_close(got, ref, ("gemm edges", epi, rows, N), atol_rms=2e-3 if epi == xb.EPI_BIAS_GELU else 2e-4)
+
+
 def test_gemm_many_tiles_persistent():
     """More tiles than SMs so every CTA runs several tiles through both TMEM accumulators."""
     rng = np.random.default_rng(7)
