@@ -119,6 +119,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (threadIdx.x == 0) grid_dep_launch();
+  grid_dep_wait();
   const uint32_t tmem_o = tmem_base + Cfg::TMEM_O;
 
   if (warp == 0) {
@@ -397,7 +399,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 }
 
 template <int DH>
-static int launch_attention_t(const AttnLaunch& a, cudaStream_t stream) {
+static int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   using Cfg = AttnCfg<DH>;
   static PerDeviceInt attr_done;
   auto kern = attention_kernel<DH>;
@@ -413,14 +415,13 @@ static int launch_attention_t(const AttnLaunch& a, cudaStream_t stream) {
   p.scale = a.q_scale * 0.6931471805599453f;        // ... and times this = natural exponents (for lse)
   p.status = a.status;
   dim3 grid((a.rows + ATT_BM - 1) / ATT_BM, a.heads, a.batch);
-  kern<<<grid, ATT_THREADS, Cfg::SMEM_BYTES, stream>>>(a.map_q, a.map_k, a.map_v, p);
-  return check_launch();
+  return launch_kernel(kern, grid, ATT_THREADS, Cfg::SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
 }
 
-int launch_attention(const AttnLaunch& a, cudaStream_t stream) {
+int launch_attention(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   if (a.rows == 0 || a.batch == 0) return XEMA_OK;
-  if (a.head_dim == 64) return launch_attention_dh64(a, stream);
-  if (a.head_dim == 128) return launch_attention_t<128>(a, stream);
+  if (a.head_dim == 64) return launch_attention_dh64(a, stream, chained);
+  if (a.head_dim == 128) return launch_attention_t<128>(a, stream, chained);
   return XEMA_EINVAL;
 }
 

@@ -231,6 +231,8 @@ attention_dh64_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (threadIdx.x == 0) grid_dep_launch();
+  grid_dep_wait();
 
   // ---- per-role state that lives across the sweeps ------------------------------------------
   // producer and MMA warp: rings of K and V stages
@@ -594,7 +596,7 @@ attention_dh64_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
 }
 
-int launch_attention_dh64(const AttnLaunch& a, cudaStream_t stream) {
+int launch_attention_dh64(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   static PerDeviceInt attr_done;
   if (int rc = ensure_smem_attr(attention_dh64_kernel, SMEM_BYTES, attr_done)) return rc;
   Attn64Params p;
@@ -609,8 +611,7 @@ int launch_attention_dh64(const AttnLaunch& a, cudaStream_t stream) {
   p.gain_q = (const __nv_bfloat16*)a.gain_q;
   p.gain_k = (const __nv_bfloat16*)a.gain_k;
   dim3 grid((a.rows + TILES * BM - 1) / (TILES * BM), a.heads, a.batch);
-  attention_dh64_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(a.map_q, a.map_k, a.map_v, p);
-  return check_launch();
+  return launch_kernel(attention_dh64_kernel, grid, THREADS, SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
 }
 
 }  // namespace xema

@@ -2,6 +2,7 @@
 // per-head RMSNorm + RoPE.  128-bit coalesced accesses, one warp per token row, warp-shuffle
 // reductions, fp32 arithmetic on bf16 storage.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 #include "sm100.cuh"
@@ -10,6 +11,10 @@ namespace xema {
 
 using sm100::bf16_hi;
 using sm100::bf16_lo;
+using sm100::grid_dep_launch;
+using sm100::grid_dep_wait;
+using sm100::ld_f4;
+using sm100::ld_u4;
 using sm100::pack_bf16x2;
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -26,9 +31,11 @@ constexpr int kModWarps = 8;
 constexpr int kModMaxBatch = 8;
 
 __global__ void __launch_bounds__(kModWarps * 32)
-mod_gemv_kernel(const __nv_bfloat16* __restrict__ temb, const __nv_bfloat16* __restrict__ w,
-                const __nv_bfloat16* __restrict__ bias, float* __restrict__ mod, int batch, int Dt, int n_out) {
+mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w,
+                const __nv_bfloat16* __restrict__ bias, float* mod, int batch, int Dt, int n_out) {
   extern __shared__ float s_e[];  // [batch][Dt]
+  grid_dep_launch();
+  grid_dep_wait();
   for (int i = threadIdx.x; i < batch * Dt; i += blockDim.x) {
     float z = __bfloat162float(temb[i]);
     s_e[i] = z / (1.f + __expf(-z));
@@ -66,58 +73,95 @@ mod_gemv_kernel(const __nv_bfloat16* __restrict__ temb, const __nv_bfloat16* __r
 }
 
 int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream) {
+               cudaStream_t stream, bool chained) {
   if (batch < 1 || Dt < 8 || (Dt & 7) || n_out < 1) return XEMA_EINVAL;
   size_t smem = (size_t)batch * Dt * sizeof(float);
   if (smem > 48 * 1024) return XEMA_EINVAL;
   int blocks = (n_out + kModWarps - 1) / kModWarps;
-  mod_gemv_kernel<<<blocks, kModWarps * 32, smem, stream>>>(
-      (const __nv_bfloat16*)temb, (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
-  return check_launch();
+  return launch_kernel(mod_gemv_kernel, dim3(blocks), kModWarps * 32, smem, stream, chained, (const __nv_bfloat16*)temb,
+                       (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
 }
 
 // ---------------------------------------------------------------------------------------
-// out = LN(in) * (1 + scale) + shift, one warp per row, the row held in registers.
+// out = LN(in) * (1 + scale) + shift, one warp per row: no block-wide barrier, the whole row is in
+// flight at once (NV 16-byte loads per lane) and stays in registers for the mean, the centred sum of
+// squares and the result.  Bound by HBM for many rows, by the latency of load, two reductions and
+// store for few.
 // bf16 input: lane reads 8 elements (16 B) per step; fp32 input: 4 elements (16 B) per step.
 // NV = steps per row (compile-time so the row stays in registers); NV == 0 selects the
-// generic variant that re-reads the row instead.
+// generic variant for rows wider than 4096, which re-reads the row instead.
 // ---------------------------------------------------------------------------------------
 constexpr int kLnWarps = 4;
 
 template <bool IN_F32>
 struct LnIo {
   static constexpr int EPV = IN_F32 ? 4 : 8;  // elements per lane per step
-  __device__ static __forceinline__ void load(const void* row, int idx, float (&f)[EPV]) {
+  using Raw = typename std::conditional<IN_F32, float4, uint4>::type;
+  __device__ static __forceinline__ Raw load(const void* row, int idx) {
+    if constexpr (IN_F32) return ld_f4(reinterpret_cast<const float4*>(row) + idx);
+    else return ld_u4(reinterpret_cast<const uint4*>(row) + idx);
+  }
+  __device__ static __forceinline__ void unpack(const Raw& v, float (&f)[EPV]) {
     if constexpr (IN_F32) {
-      float4 v = __ldg(reinterpret_cast<const float4*>(row) + idx);
       f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
     } else {
-      uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + idx);
       f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
       f[4] = bf16_lo(v.z); f[5] = bf16_hi(v.z); f[6] = bf16_lo(v.w); f[7] = bf16_hi(v.w);
     }
   }
   __device__ static __forceinline__ void store(__nv_bfloat16* row, int idx, const float (&f)[EPV]) {
-    if constexpr (IN_F32) {
-      uint2 v = make_uint2(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]));
-      reinterpret_cast<uint2*>(row)[idx] = v;
-    } else {
-      uint4 v = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]),
-                           pack_bf16x2(f[6], f[7]));
-      reinterpret_cast<uint4*>(row)[idx] = v;
+    if constexpr (IN_F32)
+      reinterpret_cast<uint2*>(row)[idx] = make_uint2(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]));
+    else
+      reinterpret_cast<uint4*>(row)[idx] = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]),
+                                                      pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+  }
+  // sum of a lane's elements of one step; the same of their squares once the mean is off
+  __device__ static __forceinline__ float sum(const float (&f)[EPV]) {
+    float s = (f[0] + f[1]) + (f[2] + f[3]);
+    if constexpr (!IN_F32) s += (f[4] + f[5]) + (f[6] + f[7]);
+    return s;
+  }
+  __device__ static __forceinline__ float centre(float (&f)[EPV], float mean) {
+#pragma unroll
+    for (int t = 0; t < EPV; ++t) f[t] -= mean;
+    float s = fmaf(f[0], f[0], f[1] * f[1]) + fmaf(f[2], f[2], f[3] * f[3]);
+    if constexpr (!IN_F32) s += fmaf(f[4], f[4], f[5] * f[5]) + fmaf(f[6], f[6], f[7] * f[7]);
+    return s;
+  }
+  // scale and shift of one step
+  struct Mod {
+    float4 a[EPV / 4], c[EPV / 4];
+  };
+  __device__ static __forceinline__ void load_mod(const float* sc, const float* sh, int idx, Mod& m) {
+#pragma unroll
+    for (int q = 0; q < EPV / 4; ++q) {
+      m.a[q] = ld_f4(sc + idx * EPV + 4 * q);
+      m.c[q] = ld_f4(sh + idx * EPV + 4 * q);
+    }
+  }
+  __device__ static __forceinline__ void modulate(float (&f)[EPV], float mean, float rstd, const Mod& m) {
+#pragma unroll
+    for (int q = 0; q < EPV / 4; ++q) {
+      f[4 * q + 0] = fmaf((f[4 * q + 0] - mean) * rstd, 1.f + m.a[q].x, m.c[q].x);
+      f[4 * q + 1] = fmaf((f[4 * q + 1] - mean) * rstd, 1.f + m.a[q].y, m.c[q].y);
+      f[4 * q + 2] = fmaf((f[4 * q + 2] - mean) * rstd, 1.f + m.a[q].z, m.c[q].z);
+      f[4 * q + 3] = fmaf((f[4 * q + 3] - mean) * rstd, 1.f + m.a[q].w, m.c[q].w);
     }
   }
 };
 
 template <bool IN_F32, int NV>
 __global__ void __launch_bounds__(kLnWarps * 32)
-ln_modulate_kernel(const void* __restrict__ in, long long in_batch_rows, __nv_bfloat16* __restrict__ out,
-                   const float* __restrict__ shift, const float* __restrict__ scale, long long mod_stride,
-                   int batch, int rows, int D, float eps) {
+ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, const float* shift, const float* scale,
+                   long long mod_stride, int batch, int rows, int D, float eps) {
   using Io = LnIo<IN_F32>;
   constexpr int EPV = Io::EPV;
+  grid_dep_launch();
+  grid_dep_wait();
   const int lane = threadIdx.x & 31;
   const long long total = (long long)batch * rows;
+  const float inv_d = 1.f / (float)D;
   const long long r = (long long)blockIdx.x * kLnWarps + (threadIdx.x >> 5);
   if (r >= total) return;
   const int b = (int)(r / rows);
@@ -127,198 +171,87 @@ ln_modulate_kernel(const void* __restrict__ in, long long in_batch_rows, __nv_bf
   __nv_bfloat16* dst = out + (size_t)r * D;
   const float* sh = shift + (size_t)b * mod_stride;
   const float* sc = scale + (size_t)b * mod_stride;
-  const int nv = D / (32 * EPV);
-  const float inv_d = 1.f / (float)D;
 
   if constexpr (NV > 0) {
-    float x[NV][EPV];
+    typename Io::Raw raw[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) raw[v] = Io::load(src, v * 32 + lane);
+    typename Io::Mod m[2];
+    Io::load_mod(sc, sh, lane, m[0]);
+    float f[EPV];
     float s = 0.f;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      Io::load(src, v * 32 + lane, x[v]);
-#pragma unroll
-      for (int t = 0; t < EPV; ++t) s += x[v][t];
+      Io::unpack(raw[v], f);
+      s += Io::sum(f);
     }
     const float mean = warp_sum(s) * inv_d;
     float q = 0.f;
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int t = 0; t < EPV; ++t) {
-        x[v][t] -= mean;
-        q = fmaf(x[v][t], x[v][t], q);
-      }
+    for (int v = 0; v < NV; ++v) {
+      Io::unpack(raw[v], f);
+      q += Io::centre(f, mean);
+    }
     const float rstd = rsqrtf(warp_sum(q) * inv_d + eps);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const int e0 = (v * 32 + lane) * EPV;
-      float y[EPV];
-#pragma unroll
-      for (int t4 = 0; t4 < EPV; t4 += 4) {
-        float4 a = __ldg(reinterpret_cast<const float4*>(sc + e0 + t4));
-        float4 c = __ldg(reinterpret_cast<const float4*>(sh + e0 + t4));
-        y[t4 + 0] = fmaf(x[v][t4 + 0] * rstd, 1.f + a.x, c.x);
-        y[t4 + 1] = fmaf(x[v][t4 + 1] * rstd, 1.f + a.y, c.y);
-        y[t4 + 2] = fmaf(x[v][t4 + 2] * rstd, 1.f + a.z, c.z);
-        y[t4 + 3] = fmaf(x[v][t4 + 3] * rstd, 1.f + a.w, c.w);
-      }
-      Io::store(dst, v * 32 + lane, y);
+      if (v + 1 < NV) Io::load_mod(sc, sh, (v + 1) * 32 + lane, m[(v + 1) & 1]);
+      Io::unpack(raw[v], f);
+      Io::modulate(f, mean, rstd, m[v & 1]);
+      Io::store(dst, v * 32 + lane, f);
     }
   } else {
+    const int nv = D / (32 * EPV);
+    float f[EPV];
     float s = 0.f;
     for (int v = 0; v < nv; ++v) {
-      float x[EPV];
-      Io::load(src, v * 32 + lane, x);
-#pragma unroll
-      for (int t = 0; t < EPV; ++t) s += x[t];
+      Io::unpack(Io::load(src, v * 32 + lane), f);
+      s += Io::sum(f);
     }
     const float mean = warp_sum(s) * inv_d;
     float q = 0.f;
     for (int v = 0; v < nv; ++v) {
-      float x[EPV];
-      Io::load(src, v * 32 + lane, x);
-#pragma unroll
-      for (int t = 0; t < EPV; ++t) {
-        float c = x[t] - mean;
-        q = fmaf(c, c, q);
-      }
+      Io::unpack(Io::load(src, v * 32 + lane), f);
+      q += Io::centre(f, mean);
     }
     const float rstd = rsqrtf(warp_sum(q) * inv_d + eps);
     for (int v = 0; v < nv; ++v) {
-      float x[EPV], y[EPV];
-      Io::load(src, v * 32 + lane, x);
-      const int e0 = (v * 32 + lane) * EPV;
-#pragma unroll
-      for (int t = 0; t < EPV; ++t) y[t] = fmaf((x[t] - mean) * rstd, 1.f + __ldg(sc + e0 + t), __ldg(sh + e0 + t));
-      Io::store(dst, v * 32 + lane, y);
-    }
-  }
-}
-
-// Wide rows (D a multiple of 1024): one 128-thread block per row, 8 consecutive features per
-// thread and step.  A thread then holds only D/128 values, so many more warps are resident and
-// enough loads are in flight to cover the HBM latency; the two reductions go through shared
-// memory.  Same arithmetic as above (mean, then centred sum of squares).
-constexpr int kLnRowThreads = 128;
-
-__device__ __forceinline__ float block_sum_128(float v, float* red, int phase) {
-  v = warp_sum(v);
-  float* slot = red + phase * 4;
-  if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = v;
-  __syncthreads();
-  return (slot[0] + slot[1]) + (slot[2] + slot[3]);
-}
-
-template <bool IN_F32, int VPT>
-__global__ void __launch_bounds__(kLnRowThreads)
-ln_modulate_row_kernel(const void* __restrict__ in, long long in_batch_rows, __nv_bfloat16* __restrict__ out,
-                       const float* __restrict__ shift, const float* __restrict__ scale, long long mod_stride,
-                       int batch, int rows, int D, float eps) {
-  __shared__ float red[16];
-  const long long total = (long long)batch * rows;
-  const float inv_d = 1.f / (float)D;
-  int parity = 0;
-  for (long long r = blockIdx.x; r < total; r += gridDim.x, parity ^= 2) {
-    const int b = (int)(r / rows);
-    const int i = (int)(r - (long long)b * rows);
-    const size_t in_elem = ((size_t)b * in_batch_rows + i) * D;
-    const float* sh = shift + (size_t)b * mod_stride;
-    const float* sc = scale + (size_t)b * mod_stride;
-    float x[VPT][8];
-    float s = 0.f;
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const int e0 = (v * kLnRowThreads + threadIdx.x) * 8;
-      if constexpr (IN_F32) {
-        const float4* p = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(in) + in_elem + e0);
-        const float4 a = __ldg(p), c = __ldg(p + 1);
-        x[v][0] = a.x; x[v][1] = a.y; x[v][2] = a.z; x[v][3] = a.w;
-        x[v][4] = c.x; x[v][5] = c.y; x[v][6] = c.z; x[v][7] = c.w;
-      } else {
-        const uint4 u = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(in) + in_elem + e0));
-        x[v][0] = bf16_lo(u.x); x[v][1] = bf16_hi(u.x); x[v][2] = bf16_lo(u.y); x[v][3] = bf16_hi(u.y);
-        x[v][4] = bf16_lo(u.z); x[v][5] = bf16_hi(u.z); x[v][6] = bf16_lo(u.w); x[v][7] = bf16_hi(u.w);
-      }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) s += x[v][t];
-    }
-    const float mean = block_sum_128(s, red, parity) * inv_d;
-    float q = 0.f;
-#pragma unroll
-    for (int v = 0; v < VPT; ++v)
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        x[v][t] -= mean;
-        q = fmaf(x[v][t], x[v][t], q);
-      }
-    const float rstd = rsqrtf(block_sum_128(q, red, parity + 1) * inv_d + eps);
-    __nv_bfloat16* dst = out + (size_t)r * D;
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const int e0 = (v * kLnRowThreads + threadIdx.x) * 8;
-      const float4 a0 = __ldg(reinterpret_cast<const float4*>(sc + e0)), a1 = __ldg(reinterpret_cast<const float4*>(sc + e0 + 4));
-      const float4 c0 = __ldg(reinterpret_cast<const float4*>(sh + e0)), c1 = __ldg(reinterpret_cast<const float4*>(sh + e0 + 4));
-      const float y0 = fmaf(x[v][0] * rstd, 1.f + a0.x, c0.x), y1 = fmaf(x[v][1] * rstd, 1.f + a0.y, c0.y);
-      const float y2 = fmaf(x[v][2] * rstd, 1.f + a0.z, c0.z), y3 = fmaf(x[v][3] * rstd, 1.f + a0.w, c0.w);
-      const float y4 = fmaf(x[v][4] * rstd, 1.f + a1.x, c1.x), y5 = fmaf(x[v][5] * rstd, 1.f + a1.y, c1.y);
-      const float y6 = fmaf(x[v][6] * rstd, 1.f + a1.z, c1.z), y7 = fmaf(x[v][7] * rstd, 1.f + a1.w, c1.w);
-      *reinterpret_cast<uint4*>(dst + e0) =
-          make_uint4(pack_bf16x2(y0, y1), pack_bf16x2(y2, y3), pack_bf16x2(y4, y5), pack_bf16x2(y6, y7));
+      typename Io::Mod m;
+      Io::unpack(Io::load(src, v * 32 + lane), f);
+      Io::load_mod(sc, sh, v * 32 + lane, m);
+      Io::modulate(f, mean, rstd, m);
+      Io::store(dst, v * 32 + lane, f);
     }
   }
 }
 
 template <bool IN_F32>
 static int launch_ln_t(const void* in, long long in_batch_rows, void* out, const float* shift, const float* scale,
-                       long long mod_stride, int batch, int rows, int D, float eps, cudaStream_t stream) {
-  constexpr int EPV = LnIo<IN_F32>::EPV;
+                       long long mod_stride, int batch, int rows, int D, float eps, cudaStream_t stream, bool chained) {
+  constexpr int PER = IN_F32 ? 2 : 1;                  // steps per 256 columns
   const long long total = (long long)batch * rows;
-  if (D % 1024 == 0 && D / 1024 <= 4) {
-    // 16 resident blocks per SM cover the whole GPU; rows beyond that are taken in a stride loop
-    const unsigned grid = (unsigned)std::min<long long>(total, 148LL * 16);
-    auto* o2 = (__nv_bfloat16*)out;
-#define XEMA_LNROW_CASE(N)                                                                                       \
-  case N:                                                                                                        \
-    ln_modulate_row_kernel<IN_F32, N><<<grid, kLnRowThreads, 0, stream>>>(in, in_batch_rows, o2, shift, scale,   \
-                                                                           mod_stride, batch, rows, D, eps);     \
-    break;
-    switch (D / 1024) {
-      XEMA_LNROW_CASE(1)
-      XEMA_LNROW_CASE(2)
-      XEMA_LNROW_CASE(3)
-      XEMA_LNROW_CASE(4)
-    }
-#undef XEMA_LNROW_CASE
-    return check_launch();
-  }
   const unsigned blocks = (unsigned)((total + kLnWarps - 1) / kLnWarps);
-  const int nv = D / (32 * EPV);
-  auto* o = (__nv_bfloat16*)out;
-#define XEMA_LN_CASE(N)                                                                                      \
-  case N:                                                                                                    \
-    ln_modulate_kernel<IN_F32, N><<<blocks, kLnWarps * 32, 0, stream>>>(in, in_batch_rows, o, shift, scale,  \
-                                                                         mod_stride, batch, rows, D, eps);   \
-    break;
-  switch (nv) {
-    XEMA_LN_CASE(2)
-    XEMA_LN_CASE(4)
-    XEMA_LN_CASE(12)
-    XEMA_LN_CASE(24)
-    default:
-      ln_modulate_kernel<IN_F32, 0><<<blocks, kLnWarps * 32, 0, stream>>>(in, in_batch_rows, o, shift, scale,
-                                                                           mod_stride, batch, rows, D, eps);
-  }
+  auto run = [&](auto kern) {
+    return launch_kernel(kern, dim3(blocks), kLnWarps * 32, 0, stream, chained, in, in_batch_rows, (__nv_bfloat16*)out, shift,
+                         scale, mod_stride, batch, rows, D, eps);
+  };
+  switch (D / 256) {
+#define XEMA_LN_CASE(N) case N: return run(ln_modulate_kernel<IN_F32, N * PER>);
+    XEMA_LN_CASE(1) XEMA_LN_CASE(2) XEMA_LN_CASE(3) XEMA_LN_CASE(4) XEMA_LN_CASE(5) XEMA_LN_CASE(6)
+    XEMA_LN_CASE(7) XEMA_LN_CASE(8) XEMA_LN_CASE(9) XEMA_LN_CASE(10) XEMA_LN_CASE(11) XEMA_LN_CASE(12)
+    XEMA_LN_CASE(13) XEMA_LN_CASE(14) XEMA_LN_CASE(15) XEMA_LN_CASE(16)
 #undef XEMA_LN_CASE
-  return check_launch();
+    default: return run(ln_modulate_kernel<IN_F32, 0>);
+  }
 }
 
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
-                       cudaStream_t stream) {
+                       cudaStream_t stream, bool chained) {
   if (batch < 1 || rows < 0 || D < 256 || (D % 256)) return XEMA_EINVAL;
   if (rows == 0) return XEMA_OK;
-  return in_is_f32 ? launch_ln_t<true>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream)
-                   : launch_ln_t<false>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream);
+  return in_is_f32 ? launch_ln_t<true>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained)
+                   : launch_ln_t<false>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -378,6 +378,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
   }
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (threadIdx.x == 0) grid_dep_launch();
 
   if (warp == 0) {
     // ---------------- TMA producer (one per CTA) ----------------
@@ -385,22 +386,40 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      auto load_a = [&](int st, const TileCoord& c, int kb) {
+        uint8_t* sa = smem + st * Cfg::STAGE_BYTES;
+        if constexpr (PAIR)
+          tma_load_3d_pair(sa, &map_a, mapa_shared(smem_u32(&full[st]), 0), kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
+        else
+          tma_load_3d(sa, &map_a, &full[st], kb * BK, c.mt * BM, c.b);
+      };
+      auto load_w = [&](int st, const TileCoord& c, int kb) {   // with the stage's expected bytes
+        uint8_t* sb = smem + st * Cfg::STAGE_BYTES + A_TILE_BYTES;
+        if constexpr (PAIR) {
+          if (rank == 0) mbar_expect_tx(&full[st], 2 * Cfg::STAGE_BYTES);
+          tma_load_3d_pair(sb, &map_w, mapa_shared(smem_u32(&full[st]), 0), kb * BK, c.nt * BN + (int)rank * (BN / 2), 0);
+        } else {
+          mbar_expect_tx(&full[st], Cfg::STAGE_BYTES);
+          tma_load_3d(sb, &map_w, &full[st], kb * BK, c.nt * BN, 0);
+        }
+      };
+      // The weights of the first stages do not depend on earlier launches (see launch_kernel): they
+      // are requested before the wait for those, the activations after it.
+      const int early = worker < total_tiles ? min(STAGES, k_blocks) : 0;
+      if (early > 0) {
+        const TileCoord c = tile_coord(worker, m_tiles, n_tiles);
+        for (int kb = 0; kb < early; ++kb) load_w(kb, c, kb);
+        grid_dep_wait();
+        for (int kb = 0; kb < early; ++kb) load_a(kb, c, kb);
+        if (early == STAGES) phase = 1;
+        else stage = early;
+      }
       for (int tile = worker; ok && tile < total_tiles; tile += n_workers) {
         const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = tile == worker ? early : 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
-          uint8_t* sb = sa + A_TILE_BYTES;
-          if constexpr (PAIR) {
-            const uint32_t full0 = mapa_shared(smem_u32(&full[stage]), 0);
-            if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::STAGE_BYTES);
-            tma_load_3d_pair(sa, &map_a, full0, kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
-            tma_load_3d_pair(sb, &map_w, full0, kb * BK, c.nt * BN + (int)rank * (BN / 2), 0);
-          } else {
-            mbar_expect_tx(&full[stage], Cfg::STAGE_BYTES);
-            tma_load_3d(sa, &map_a, &full[stage], kb * BK, c.mt * BM, c.b);
-            tma_load_3d(sb, &map_w, &full[stage], kb * BK, c.nt * BN, 0);
-          }
+          load_w(stage, c, kb);
+          load_a(stage, c, kb);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
@@ -502,6 +521,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
       if (et < p.head_dim) s_gate[et] = __bfloat162float(p.norm_gain[et]);   // read after the tile's barrier
     }
+    grid_dep_wait();
     for (int tile = worker; tile < total_tiles; tile += n_workers) {
       // The four warps meet (the previous tile's bias and gate are no longer read) and agree on going
       // on: a warp that gave up a wait still comes here, so that nobody waits for it.
@@ -529,7 +549,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
         *reinterpret_cast<float2*>(s_bias + i) = make_float2(bf16_lo(bb), bf16_hi(bb));
         if constexpr (GATED)
           *reinterpret_cast<float2*>(s_gate + i) =
-              __ldg(reinterpret_cast<const float2*>(p.gate + (size_t)c.b * p.gate_stride + n_base + i));
+              ld_f2(p.gate + (size_t)c.b * p.gate_stride + n_base + i);
       }
       named_barrier(1, 128);
       ok = mbar_wait_warp(&tmem_full[acc], acc_phase, abort_flag);
@@ -618,19 +638,19 @@ GemmParams make_params(const GemmLaunch& g) {
 }
 
 template <int EPI, int BN>
-int launch_single(const GemmLaunch& g, cudaStream_t stream) {
+int launch_single(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   using Cfg = GemmCfg<EPI, BN, false>;
   static PerDeviceInt attr_done;
   auto kern = gemm_bf16_kernel<EPI, BN>;
   if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
   const long long tiles = (long long)g.batch * ((g.rows + BM - 1) / BM) * (g.N / BN);
   const int grid = (int)std::min<long long>(tiles, sm_count());
-  kern<<<grid, GEMM_THREADS, Cfg::SMEM_BYTES, stream>>>(g.map_a, g.map_w, g.map_out, g.map_res, make_params(g));
-  return check_launch();
+  return launch_kernel(kern, dim3(grid), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out, g.map_res,
+                       make_params(g));
 }
 
 template <int EPI>
-int launch_pair(const GemmLaunch& g, cudaStream_t stream) {
+int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   using Cfg = GemmCfg<EPI, PAIR_BN, true>;
   static PerDeviceInt attr_done;
   auto kern = gemm_bf16_pair_kernel<EPI>;
@@ -663,27 +683,27 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream) {
   }
   const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / PAIR_BN);
   const int pairs = (int)std::min<long long>(tiles, max_pairs);
-  kern<<<2 * pairs, GEMM_THREADS, Cfg::SMEM_BYTES, stream>>>(g.map_a, g.map_w, g.map_out, g.map_res, make_params(g));
-  return check_launch();
+  return launch_kernel(kern, dim3(2 * pairs), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out,
+                       g.map_res, make_params(g));
 }
 
 template <int EPI>
-int launch_epi(const GemmLaunch& g, cudaStream_t stream) {
-  if (g.block_n == 256) return launch_pair<EPI>(g, stream);
-  if (g.block_n == 128) return launch_single<EPI, 128>(g, stream);
+int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
+  if (g.block_n == 256) return launch_pair<EPI>(g, stream, chained);
+  if (g.block_n == 128) return launch_single<EPI, 128>(g, stream, chained);
   return XEMA_EINVAL;
 }
 
 }  // namespace
 
-int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
+int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   if (g.rows == 0 || g.batch == 0) return XEMA_OK;
   switch (g.epilogue) {
-    case XEMA_EPI_BIAS: return launch_epi<XEMA_EPI_BIAS>(g, stream);
-    case XEMA_EPI_BIAS_GELU: return launch_epi<XEMA_EPI_BIAS_GELU>(g, stream);
-    case XEMA_EPI_GATE_RES_F32: return launch_epi<XEMA_EPI_GATE_RES_F32>(g, stream);
-    case XEMA_EPI_GATE_RES_BF16: return launch_epi<XEMA_EPI_GATE_RES_BF16>(g, stream);
-    case XEMA_EPI_BIAS_NORM_ROPE: return launch_epi<XEMA_EPI_BIAS_NORM_ROPE>(g, stream);
+    case XEMA_EPI_BIAS: return launch_epi<XEMA_EPI_BIAS>(g, stream, chained);
+    case XEMA_EPI_BIAS_GELU: return launch_epi<XEMA_EPI_BIAS_GELU>(g, stream, chained);
+    case XEMA_EPI_GATE_RES_F32: return launch_epi<XEMA_EPI_GATE_RES_F32>(g, stream, chained);
+    case XEMA_EPI_GATE_RES_BF16: return launch_epi<XEMA_EPI_GATE_RES_BF16>(g, stream, chained);
+    case XEMA_EPI_BIAS_NORM_ROPE: return launch_epi<XEMA_EPI_BIAS_NORM_ROPE>(g, stream, chained);
     default: return XEMA_EINVAL;
   }
 }

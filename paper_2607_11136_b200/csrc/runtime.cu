@@ -161,21 +161,22 @@ struct xema_plan {
   }
 };
 
-static int issue(const xema_plan* pl, const Op& op, cudaStream_t st) {
+// `chained`: the launch right before this one in the stream is the op before it (see launch_kernel).
+static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained) {
   const xema_config& c = pl->cfg;
   switch (op.kind) {
     case OP_MOD:
-      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st);
+      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained);
     case OP_LN:
       return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale,
-                                6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st);
+                                6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st, chained);
     case OP_ROPE:
       return launch_rmsnorm_rope(op.rope_x, op.rope_ld, op.rope_batch_rows, op.rope_g, pl->rope, op.pos0, op.batch,
                                  op.rows, c.heads, c.head_dim, c.rms_eps, st);
     case OP_GEMM:
-      return launch_gemm(op.gemm, st);
+      return launch_gemm(op.gemm, st, chained);
     case OP_ATTN:
-      return launch_attention(op.attn, st);
+      return launch_attention(op.attn, st, chained);
     case OP_FUSED:
       return XEMA_OK;
   }
@@ -187,9 +188,11 @@ static int run_ops(const xema_plan* pl, size_t first, size_t n, void* stream) {
   if (!pl->bound) return XEMA_ESTATE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   n = std::min(n, pl->ops.size());
+  bool chained = false;
   for (size_t i = first; i < n; ++i) {
-    int rc = issue(pl, pl->ops[i], st);
+    int rc = issue(pl, pl->ops[i], st, chained);
     if (rc) return rc;
+    chained = chained || pl->ops[i].kind != OP_FUSED;
   }
   return XEMA_OK;
 }
@@ -664,16 +667,20 @@ int xema_forward_host(const xema_plan* plan, const void* hid_in_host, const void
 
   // ---- launches, with the waits for input pieces and the copies of finished output pieces
   size_t k_in = 0, k_out = 0;
+  bool chained = false;
   for (size_t i = 0; i < n; ++i) {
     if (split_in && k_in < in_ops.size() && i == in_ops[k_in]) {
       if (in_ready[k_in] && (e = cudaStreamWaitEvent(st, in_ready[k_in], 0)) != cudaSuccess) return fail(e);
+      if (in_ready[k_in]) chained = false;
       ++k_in;
     }
-    int rc = issue(plan, ops[i], st);
+    int rc = issue(plan, ops[i], st, chained);
     if (rc) return rc;
+    chained = chained || ops[i].kind != OP_FUSED;
     if (split_out && k_out < out_ops.size() && i == out_ops[k_out]) {
       const Op& o = ops[i];
       const bool last = (k_out + 1 == out_ops.size());
+      chained = false;
       if (!last) {
         cudaEvent_t ev = plan->copy_events[next_event++];
         if ((e = cudaEventRecord(ev, st)) != cudaSuccess || (e = cudaStreamWaitEvent(cs, ev, 0)) != cudaSuccess) return fail(e);

@@ -162,6 +162,32 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   }
 }
 
+// ---- programmatic dependent launch -----------------------------------------------------------
+// A kernel launched with LaunchChained may start while the launch before it still runs.  It has to
+// call grid_dep_wait() in every thread that reads what earlier launches wrote (or overwrites what
+// they read), before it does; the wait returns when everything before it in the stream has
+// completed.  grid_dep_launch() lets the next launch start once every CTA of this grid has called
+// it (or has left) -- only after the CTA holds its TMEM, so that a later kernel's CTA can never sit
+// on columns that an earlier one still needs.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Loads of what an earlier launch wrote: a read-only (__ldg) load may be moved above the wait.
+__device__ __forceinline__ uint4 ld_u4(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_f4(const void* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ld_f2(const void* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
 // ---- CTA pairs (thread-block cluster of two) -------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;

@@ -56,6 +56,30 @@ def test_ln_modulate(D, in_f32):
     assert_bf16_close(from_dev_bf16(out), ref, "ln", atol_rms=1e-4)
 
 
+@pytest.mark.parametrize("D", [256, 1024, 2304, 4096, 4352])
+@pytest.mark.parametrize("rows", [1, 3, 5])
+def test_ln_modulate_widths(D, rows):
+    """Every kind of row the kernel has an instance for: one step per lane, odd step counts, the
+    widest row kept in registers and one beyond it, with rows that do not fill a block's warps.
+    The result is rounded to bf16 once; 1e-4 of RMS covers the fp32 sums over D terms."""
+    rng = np.random.default_rng(5 + D)
+    B = 2
+    for in_f32 in (0, 1):
+        xf32 = (rng.standard_normal((B, rows, D), dtype=np.float32) * 2 + 0.5).astype(np.float32)
+        bits = bf16_bits(xf32)
+        x_dev = torch.from_numpy(xf32).to(DEV) if in_f32 else to_dev(bits)
+        xf = xf32.astype(np.float64) if in_f32 else bits_to_f64(bits)
+        mod = rng.standard_normal((B, 2 * D), dtype=np.float32) * 0.3
+        mod_dev = torch.from_numpy(mod).to(DEV)
+        out = torch.empty(B, rows, D, dtype=torch.int16, device=DEV)
+        xb.xema_op_ln_modulate(x_dev.data_ptr(), in_f32, rows, out.data_ptr(), mod_dev.data_ptr(),
+                               mod_dev.data_ptr() + D * 4, 2 * D, B, rows, D, 1e-6)
+        torch.cuda.synchronize()
+        m64 = mod.astype(np.float64)
+        ref = ob.layer_norm(xf, 1e-6) * (1 + m64[:, None, D:]) + m64[:, None, :D]
+        assert_bf16_close(from_dev_bf16(out), ref, ("ln widths", D, rows, in_f32), atol_rms=1e-4)
+
+
 @pytest.mark.parametrize("name", ["tiny", "flux"])
 def test_rmsnorm_rope(name):
     t = template(name)
