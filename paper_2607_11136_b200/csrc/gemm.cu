@@ -9,7 +9,7 @@
 //           fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
 //           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows x 256 columns in the TMEM of
 //           each CTA.
-//   single  one CTA per 128 x BN tile.
+//   single  one CTA per 128 x 128 or 128 x 64 tile, for problems that would leave SMs idle otherwise.
 //
 //   warp 0    TMA producer: tiles of A and W into a ring of shared-memory stages (128-byte swizzle)
 //   warp 1    owns TMEM; converged warp, one elected lane issues tcgen05.mma into one of two fp32
@@ -56,12 +56,18 @@ constexpr bool kGated = EPI == XEMA_EPI_GATE_RES_F32 || EPI == XEMA_EPI_GATE_RES
 
 template <int EPI, int BN, bool PAIR>
 struct GemmCfg {
-  static constexpr int W_ROWS = PAIR ? BN / 2 : BN;            // rows of W a CTA loads per stage
-  static constexpr int STAGE_BYTES = A_TILE_BYTES + W_ROWS * BK * 2;
+  static constexpr int W_ROWS = PAIR ? BN / 2 : BN;            // rows of W a CTA loads per K block
+  static constexpr int W_TILE_BYTES = W_ROWS * BK * 2;
+  // K blocks of 64 per stage.  A single CTA's K block is short (128 to 256 cycles of MMA), and with a
+  // stage per block the barrier round of each one takes longer than that: 8888 x 12288 x 3072 with
+  // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block, 72 B/clk of fill).
+  static constexpr int KSUB = PAIR ? 1 : 2;
+  static constexpr int STAGE_BYTES = KSUB * (A_TILE_BYTES + W_TILE_BYTES);
+  static constexpr int OFF_W = KSUB * A_TILE_BYTES;            // in a stage
   // staging buffers per epilogue warp: the gated epilogues keep residual chunks in flight
-  static constexpr int RING = kGated<EPI> ? 4 : 2;
+  static constexpr int RING = kGated<EPI> && PAIR ? 4 : 2;
   static constexpr int RING_BYTES = 4 * RING * BUF_BYTES;
-  static constexpr int STAGES = kGated<EPI> ? 5 : 6;
+  static constexpr int STAGES = PAIR ? (kGated<EPI> ? 5 : 6) : 196608 / STAGE_BYTES;
   static constexpr int OFF_RING = STAGES * STAGE_BYTES;
   static constexpr int OFF_BIAS = OFF_RING + RING_BYTES;       // float [BN]: bias
   static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
@@ -322,7 +328,7 @@ template <int EPI, int BN, bool PAIR>
 __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_out,
                                           const CUtensorMap& map_res, const GemmParams& p) {
   using Cfg = GemmCfg<EPI, BN, PAIR>;
-  constexpr int STAGES = Cfg::STAGES, RING = Cfg::RING;
+  constexpr int STAGES = Cfg::STAGES, RING = Cfg::RING, KSUB = Cfg::KSUB;
   constexpr bool GATED = kGated<EPI>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
@@ -339,7 +345,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
   constexpr int TM = PAIR ? 2 * BM : BM;                // rows per tile
   const int m_tiles = (p.rows + TM - 1) / TM;
   const int n_tiles = p.N / BN;
-  const int k_blocks = p.K / BK;
+  const int k_blocks = p.K / BK, k_stages = (k_blocks + KSUB - 1) / KSUB;
   const bool aligned = (smem_u32(smem) & 1023u) == 0;   // the swizzled tiles need a 1024-byte aligned base
   const int total_tiles = aligned ? p.batch * m_tiles * n_tiles : 0;
 
@@ -382,44 +388,62 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
 
   if (warp == 0) {
     // ---------------- TMA producer (one per CTA) ----------------
-    if (lane == 0) {
+    {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      auto load_a = [&](int st, const TileCoord& c, int kb) {
+      // ks: stage-sized step along K; the last one may hold fewer K blocks
+      auto load_a = [&](int st, const TileCoord& c, int ks) {
         uint8_t* sa = smem + st * Cfg::STAGE_BYTES;
-        if constexpr (PAIR)
-          tma_load_3d_pair(sa, &map_a, mapa_shared(smem_u32(&full[st]), 0), kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
-        else
-          tma_load_3d(sa, &map_a, &full[st], kb * BK, c.mt * BM, c.b);
+#pragma unroll
+        for (int u = 0; u < KSUB; ++u) {
+          const int kb = ks * KSUB + u;
+          if (KSUB > 1 && kb >= k_blocks) break;
+          if constexpr (PAIR)
+            tma_load_3d_pair(sa, &map_a, mapa_shared(smem_u32(&full[st]), 0), kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
+          else
+            tma_load_3d(sa + u * A_TILE_BYTES, &map_a, &full[st], kb * BK, c.mt * BM, c.b);
+        }
       };
-      auto load_w = [&](int st, const TileCoord& c, int kb) {   // with the stage's expected bytes
-        uint8_t* sb = smem + st * Cfg::STAGE_BYTES + A_TILE_BYTES;
+      auto load_w = [&](int st, const TileCoord& c, int ks) {   // with the stage's expected bytes
+        uint8_t* sb = smem + st * Cfg::STAGE_BYTES + Cfg::OFF_W;
         if constexpr (PAIR) {
           if (rank == 0) mbar_expect_tx(&full[st], 2 * Cfg::STAGE_BYTES);
-          tma_load_3d_pair(sb, &map_w, mapa_shared(smem_u32(&full[st]), 0), kb * BK, c.nt * BN + (int)rank * (BN / 2), 0);
+          tma_load_3d_pair(sb, &map_w, mapa_shared(smem_u32(&full[st]), 0), ks * BK, c.nt * BN + (int)rank * (BN / 2), 0);
         } else {
-          mbar_expect_tx(&full[st], Cfg::STAGE_BYTES);
-          tma_load_3d(sb, &map_w, &full[st], kb * BK, c.nt * BN, 0);
+          mbar_expect_tx(&full[st], min(KSUB, k_blocks - ks * KSUB) * (A_TILE_BYTES + Cfg::W_TILE_BYTES));
+#pragma unroll
+          for (int u = 0; u < KSUB; ++u) {
+            const int kb = ks * KSUB + u;
+            if (KSUB > 1 && kb >= k_blocks) break;
+            tma_load_3d(sb + u * Cfg::W_TILE_BYTES, &map_w, &full[st], kb * BK, c.nt * BN, 0);
+          }
         }
       };
       // The weights of the first stages do not depend on earlier launches (see launch_kernel): they
       // are requested before the wait for those, the activations after it.
-      const int early = worker < total_tiles ? min(STAGES, k_blocks) : 0;
+      const int early = worker < total_tiles ? min(STAGES, k_stages) : 0;
       if (early > 0) {
         const TileCoord c = tile_coord(worker, m_tiles, n_tiles);
-        for (int kb = 0; kb < early; ++kb) load_w(kb, c, kb);
+        if (elect_one())
+          for (int kb = 0; kb < early; ++kb) load_w(kb, c, kb);
+        __syncwarp();
         grid_dep_wait();
-        for (int kb = 0; kb < early; ++kb) load_a(kb, c, kb);
+        if (elect_one())
+          for (int kb = 0; kb < early; ++kb) load_a(kb, c, kb);
+        __syncwarp();
         if (early == STAGES) phase = 1;
         else stage = early;
       }
       for (int tile = worker; ok && tile < total_tiles; tile += n_workers) {
         const TileCoord c = tile_coord(tile, m_tiles, n_tiles);
-        for (int kb = tile == worker ? early : 0; kb < k_blocks; ++kb) {
-          if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          load_w(stage, c, kb);
-          load_a(stage, c, kb);
+        for (int kb = tile == worker ? early : 0; kb < k_stages; ++kb) {
+          if (!(ok = mbar_wait_warp(&empty[stage], phase ^ 1, abort_flag))) break;
+          if (elect_one()) {
+            load_w(stage, c, kb);
+            load_a(stage, c, kb);
+          }
+          __syncwarp();
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
@@ -428,7 +452,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
       // landed here, so none of them can reach this CTA's barriers after it has left.
       if constexpr (PAIR) {
         for (int s = 0; ok && s < STAGES; ++s) {
-          ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag);
+          ok = mbar_wait_warp(&empty[stage], phase ^ 1, abort_flag);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
@@ -438,7 +462,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
         // at the abort flag) for the latest fill of every stage, which covers the bytes of both CTAs
         // wherever both issued; the closing cluster barrier then keeps the peer until that is done.
         // A short settling time covers loads of a stage that only one of the two CTAs still issued.
-        if (rank == 0) {
+        if (rank == 0 && lane == 0) {
           for (int s = 0; s < STAGES; ++s) {
             const int st = (stage + s) % STAGES;                 // oldest outstanding first
             const uint32_t ph = (st < stage) ? phase : (phase ^ 1);
@@ -458,10 +482,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
       // Descriptors are built once and advanced by adding constants (the start-address field
       // counts 16-byte units and never carries out of its 14 bits inside shared memory).
       const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-      const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + A_TILE_BYTES), 16, 1024);
-      auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
-        return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
-      };
+      const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + Cfg::OFF_W), 16, 1024);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -474,8 +495,8 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
         const uint32_t d_tmem = tmem_base + acc * BN;
         uint32_t accumulate = 0;
 #pragma unroll 1
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = wait_all(&full[stage], phase))) break;
+        for (int ks = 0; ks < k_stages; ++ks) {
+          if (!(ok = mbar_wait_warp(&full[stage], phase, abort_flag))) break;
           tc_fence_after();
           if (elect_one()) {
             const uint64_t soff = (uint64_t)(stage * (Cfg::STAGE_BYTES >> 4));
@@ -487,10 +508,15 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
               mma_ss_pair(d_tmem, da + 6, db + 6, idesc, 1);
               mma_commit_pair(&empty[stage]);
             } else {
-              mma_ss(d_tmem, da, db, idesc, accumulate);
-              mma_ss(d_tmem, da + 2, db + 2, idesc, 1);
-              mma_ss(d_tmem, da + 4, db + 4, idesc, 1);
-              mma_ss(d_tmem, da + 6, db + 6, idesc, 1);
+#pragma unroll
+              for (int u = 0; u < KSUB; ++u) {
+                if (KSUB > 1 && ks * KSUB + u >= k_blocks) break;
+                const uint64_t ua = da + (uint64_t)(u * (A_TILE_BYTES >> 4)), ub = db + (uint64_t)(u * (Cfg::W_TILE_BYTES >> 4));
+                mma_ss(d_tmem, ua, ub, idesc, u > 0 ? 1 : accumulate);
+                mma_ss(d_tmem, ua + 2, ub + 2, idesc, 1);
+                mma_ss(d_tmem, ua + 4, ub + 4, idesc, 1);
+                mma_ss(d_tmem, ua + 6, ub + 6, idesc, 1);
+              }
               mma_commit(&empty[stage]);
             }
           }
@@ -691,9 +717,39 @@ template <int EPI>
 int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   if (g.block_n == 256) return launch_pair<EPI>(g, stream, chained);
   if (g.block_n == 128) return launch_single<EPI, 128>(g, stream, chained);
-  return XEMA_EINVAL;
+  return launch_single<EPI, 64>(g, stream, chained);
 }
 
+
+// Tile for a problem: the one with the shortest estimated time, waves x K blocks x cycles per K block
+// plus the last tile's epilogue.  Cycles as measured (B200, 1.9 GHz): a 256 x 256 pair tile runs at its
+// math time, 512 per K block, with all SMs busy and nearer 600 in the latency of a short loop; a
+// 128 x 128 tile takes 490-550 and a 128 x 64 tile 335 -- a CTA fills shared memory at about 70 B/clk
+// whatever its tile -- so the smaller tiles are slower per flop and pay only where the larger ones
+// leave SMs idle: 1101 x 1536 x 6144 39.2 / 30.9 / 39.3 us (256 / 128 / 64), 333 x 1024 x 4096 28.8 / 22.0 / 16.5,
+// 288 x 512 x 2048 18.6 / 13.5 / 12.1, but 4444 x 3072 x 3072 58.4 / 74.7 / 106.
+// The bits of a row do not depend on the choice.
+int pick_tile(const GemmLaunch& g) {
+  struct Tile {
+    int block_n, rows, workers_per_sm_x2, cycles, epilogue;
+  };
+  static const Tile tiles[] = {{256, 2 * BM, 1, 600, 4000}, {128, BM, 2, 520, 2500}, {64, BM, 2, 340, 1500}};
+  const long long k_blocks = g.K / BK;
+  long long best = 0;
+  int pick = 0;
+  for (const Tile& t : tiles) {
+    if (g.N % t.block_n) continue;
+    if (g.epilogue == XEMA_EPI_BIAS_NORM_ROPE && t.block_n < g.head_dim) continue;   // whole heads only
+    const long long n = (long long)g.batch * ((g.rows + t.rows - 1) / t.rows) * (g.N / t.block_n);
+    const long long workers = std::max(1, sm_count() * t.workers_per_sm_x2 / 2);
+    const long long cost = (n + workers - 1) / workers * k_blocks * t.cycles + t.epilogue;
+    if (!pick || cost < best) {
+      best = cost;
+      pick = t.block_n;
+    }
+  }
+  return pick;
+}
 }  // namespace
 
 int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained) {
@@ -724,12 +780,12 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
   if (mis(a) || mis(w) || mis(g->bias) || mis(g->out) || (g->resid && mis(g->resid)) || (g->gate && mis(g->gate)))
     return XEMA_EALIGN;
-  g->block_n = (g->N % 256 == 0) ? 256 : 128;
+  g->block_n = pick_tile(*g);
   const long long rows = g->rows > 0 ? g->rows : 1;
   int rc = encode_tmap_bf16(&g->map_a, a, g->K, rows, g->batch, lda, a_batch_rows, BM);
   if (rc) return rc;
   // the pair form loads its W tile as two 128-row halves, one per CTA
-  rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, 128);
+  rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, g->block_n == 64 ? 64 : 128);
   if (rc) return rc;
   // results leave, and residuals arrive, as boxes of 32 columns x 32 rows
   rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, g->N, rows, g->batch, g->ldo,

@@ -180,6 +180,36 @@ def test_gemm_epilogue_row_edges(epi, rows):
             assert_bf16_close(got, ref, ("gemm edges", epi, rows, N), atol_rms=2e-3 if epi == xb.EPI_BIAS_GELU else 2e-4)
 
 
+@pytest.mark.parametrize("N,K", [(512, 320), (1536, 64), (768, 448)])
+def test_gemm_tile_forms_give_the_same_bits(N, K):
+    """The tile (256 x 256 over a CTA pair, 128 x 128, 128 x 64) is chosen from the size of the
+    problem; a row's bits must not show it.  The same rows as a problem of their own (small tiles)
+    and inside one that fills the GPU (pairs), K with an odd number of 64-wide blocks (a stage
+    of the single-CTA forms holds two); the first also against the oracle."""
+    rng = np.random.default_rng(12 + N)
+    rows = 256 * (2 * 74 * 256 // N + 1)
+    a_dev, w_dev, b_dev = (to_dev(rand_bf16(rng, s, c)[0]) for s, c in (((rows, K), 1.0), ((N, K), 0.05), ((N,), 0.5)))
+    gate = torch.from_numpy(rng.standard_normal(N, dtype=np.float32)).to(DEV)
+    res = torch.from_numpy(rng.standard_normal((rows, N), dtype=np.float32)).to(DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+    def run(n, epi):
+        out = torch.zeros(n, N, dtype=torch.int16, device=DEV)
+        xb.xema_op_gemm(status=status.data_ptr(), a=a_dev.data_ptr(), lda=K, a_batch_rows=n, w=w_dev.data_ptr(), ldw=K,
+                        bias=b_dev.data_ptr(), out=out.data_ptr(), ldo=N, out_batch_rows=n, batch=1, rows=n, N=N, K=K,
+                        epilogue=epi, resid=res.data_ptr(), ldr=N, resid_batch_rows=n, gate=gate.data_ptr(), gate_stride=N)
+        return out
+
+    for epi in (xb.EPI_BIAS, xb.EPI_GATE_RES_BF16):
+        full = run(rows, epi)
+        for n in (100, 1300, 3000):
+            if n < rows:
+                assert torch.equal(run(n, epi), full[:n]), (epi, n)
+    _sync_status(status)
+    got, ref = _gemm_case(rng, 1, 100, N, K, xb.EPI_BIAS)
+    assert_bf16_close(got, ref, ("gemm small tile", N, K), atol_rms=2e-4)
+
+
 def test_gemm_many_tiles_persistent():
     """More tiles than SMs so every CTA runs several tiles through both TMEM accumulators."""
     rng = np.random.default_rng(7)
