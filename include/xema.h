@@ -272,6 +272,11 @@ int xema_plan_tensor_at(const xema_plan* plan, size_t i, xema_tensor* tensor, ui
 int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes,
                    const xema_block_weights* weights, const float* rope_dev, void* status_dev);
 
+/* Puts a forward call's inputs into the arena: hid0 from hid_dev [B, rows owned, D] bf16 and temb
+ * from temb_dev [B, Dt] bf16 (device, contiguous), in one launch (two plain copies where a
+ * pointer is not 16-byte aligned).  Enqueues on `stream`.  XEMA_ESTATE if the plan is unbound. */
+int xema_plan_set_inputs(const xema_plan* plan, const void* hid_dev, const void* temb_dev, void* stream);
+
 /* Enqueues the block (n_blocks must be 1) / all n_blocks blocks on `stream` (a cudaStream_t
  * passed as void*).  Input: the caller has written hid0 [B,S,D] bf16 and temb [B,Dt] bf16 at
  * their plan offsets; output: hid<n_blocks> [B,S,D] bf16 at its plan offset once the stream

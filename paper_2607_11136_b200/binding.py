@@ -23,7 +23,7 @@ EXPORTS = (
     "xema_phase_chunks_for_budget", "xema_pressure_ranges", "xema_trace_mitigated", "xema_mitigation_for_budget", "xema_rope_table",
     "xema_plan_create", "xema_plan_create_phases", "xema_plan_create_mitigated", "xema_plan_destroy",
     "xema_plan_info", "xema_plan_phase_chunks", "xema_plan_mitigation", "xema_plan_tensor",
-    "xema_plan_tensor_at", "xema_plan_bind", "xema_block_forward", "xema_step_forward",
+    "xema_plan_tensor_at", "xema_plan_bind", "xema_plan_set_inputs", "xema_block_forward", "xema_step_forward",
     "xema_block_forward_static",
     "xema_shard_rows", "xema_trace_sharded", "xema_plan_create_sharded", "xema_plan_shard", "xema_plan_gather_point", "xema_plan_create_guarded", "xema_plan_guard_bytes",
     "xema_plan_launch_count", "xema_forward_host", "xema_forward_prefix", "xema_forward_range", "xema_plan_op", "xema_op_mod", "xema_op_ln_modulate",
@@ -124,6 +124,7 @@ def lib() -> C.CDLL:
             "xema_plan_tensor": [vp, C.c_char_p, P(u64), P(u64)],
             "xema_plan_tensor_at": [vp, sz, P(xema_tensor), P(u64)],
             "xema_plan_bind": [vp, vp, u64, P(xema_block_weights), vp, vp],
+            "xema_plan_set_inputs": [vp, vp, vp, vp],
             "xema_block_forward": [vp, vp],
             "xema_step_forward": [vp, vp],
             "xema_forward_host": [vp, vp, vp, vp, vp],
@@ -445,6 +446,10 @@ class Plan:
 
     def launch_count(self) -> int:
         return lib().xema_plan_launch_count(self._h)
+
+    def set_inputs(self, hid: int, temb: int, stream: int = 0):
+        """Device pointers of the block input and the timestep embedding, copied into the arena."""
+        _check(lib().xema_plan_set_inputs(self._h, hid, temb, stream), "xema_plan_set_inputs")
 
     def block_forward(self, stream: int = 0):
         _check(lib().xema_block_forward(self._h, stream), "xema_block_forward")

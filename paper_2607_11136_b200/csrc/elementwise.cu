@@ -330,4 +330,38 @@ int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void*
   return check_launch();
 }
 
+// ---------------------------------------------------------------------------------------
+// Two contiguous copies in one launch (a forward call's inputs): 16 bytes per thread and step, four
+// loads in flight.  One launch instead of two memory copies takes 2-4 us off a call with small inputs;
+// bound by HBM for large ones.
+// ---------------------------------------------------------------------------------------
+constexpr int kCopyThreads = 256;
+
+__device__ __forceinline__ void copy_part(uint8_t* dst, const uint8_t* src, size_t bytes) {
+  const size_t n = bytes / 16, stride = (size_t)gridDim.x * kCopyThreads;
+  uint4* d = reinterpret_cast<uint4*>(dst);
+  const uint4* s = reinterpret_cast<const uint4*>(src);
+  for (size_t i = (size_t)blockIdx.x * kCopyThreads + threadIdx.x; i < n; i += 4 * stride) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + u * stride < n) v[u] = __ldcs(s + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + u * stride < n) d[i + u * stride] = v[u];
+  }
+}
+__global__ void __launch_bounds__(kCopyThreads)
+copy2_kernel(uint8_t* dst0, const uint8_t* src0, size_t n0, uint8_t* dst1, const uint8_t* src1, size_t n1) {
+  copy_part(dst0, src0, n0);
+  copy_part(dst1, src1, n1);
+}
+
+int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream) {
+  const size_t steps = (std::max(n0, n1) / 16 + 4 * kCopyThreads) / (4 * kCopyThreads);
+  const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>(steps, 1), (size_t)sm_count() * 8);
+  return launch_kernel(copy2_kernel, dim3(blocks), kCopyThreads, 0, stream, false, (uint8_t*)dst0, (const uint8_t*)src0, n0,
+                       (uint8_t*)dst1, (const uint8_t*)src1, n1);
+}
+
 }  // namespace xema

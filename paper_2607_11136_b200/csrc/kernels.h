@@ -80,6 +80,9 @@ int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, v
 int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void* g, const float* rope, int pos0,
                         int batch, int rows, int heads, int head_dim, float eps, cudaStream_t stream);
 
+// dst0 <- src0 (n0 bytes) and dst1 <- src1 (n1 bytes); pointers and sizes are multiples of 16 bytes.
+int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream);
+
 // ---- TMA descriptors (encoded on the host once per bound tensor) --------------------------
 // bf16 tensor viewed as [batch][rows][cols] with row stride ld and batch stride batch_rows*ld
 // (elements); box = 64 columns x box_rows rows x 1, 128-byte swizzle, out-of-range rows and

@@ -148,6 +148,8 @@ struct xema_plan {
   uint32_t n_ops;
   bool bound;
   uint8_t* arena;     // as given to xema_plan_bind
+  uint8_t *hid_in, *temb_in;   // the inputs' slots in it
+  long long own_rows; // token rows of the plan's shard
   const float* rope;
   std::vector<Op> ops;
   // xema_forward_host: a second stream and one event per piece of the first and last phase, so
@@ -562,7 +564,28 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
     }
   }
   if (plan->ops.size() != plan->n_ops) return XEMA_EINVAL;
+  plan->hid_in = at("hid", 0, -1);
+  plan->temb_in = at("temb", -1, -1);
+  plan->own_rows = S;
   plan->bound = true;
+  return XEMA_OK;
+}
+
+int xema_plan_set_inputs(const xema_plan* plan, const void* hid_dev, const void* temb_dev, void* stream) {
+  if (!plan || !hid_dev || !temb_dev) return XEMA_EINVAL;
+  if (!plan->bound) return XEMA_ESTATE;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const xema_config& c = plan->cfg;
+  const size_t hid_bytes = (size_t)2 * c.batch * (size_t)plan->own_rows * c.hidden;
+  const size_t temb_bytes = (size_t)2 * c.batch * c.temb_dim;
+  if (((reinterpret_cast<uintptr_t>(hid_dev) | reinterpret_cast<uintptr_t>(temb_dev)) & 15) == 0)
+    return launch_copy2(plan->hid_in, hid_dev, hid_bytes, plan->temb_in, temb_dev, temb_bytes, st);
+  cudaError_t e = cudaMemcpyAsync(plan->hid_in, hid_dev, hid_bytes, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(plan->temb_in, temb_dev, temb_bytes, cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) {
+    t_last_cuda_error = (int)e;
+    return XEMA_ECUDA;
+  }
   return XEMA_OK;
 }
 

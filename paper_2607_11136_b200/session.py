@@ -85,6 +85,10 @@ class BlockSession:
         self.plan.bind(self.arena.data_ptr(), self.arena.numel(), ptrs, self.rope.data_ptr(), self.status.data_ptr())
         self.seq_all = template.s_text + template.grid_t * template.grid_h * template.grid_w
         self.seq = self.plan.rows          # token rows of this session's tensors (all of them unless sharded)
+        hid = (template.batch, self.seq, template.hidden)
+        self._hid_in = self.view("hid0", torch.int16, hid)
+        self._temb = self.view("temb", torch.int16, (template.batch, template.temb_dim))
+        self._hid_out = self.view("hid%d" % template.n_blocks, torch.int16, hid)
 
     # ---- views into the arena ---------------------------------------------------------
     def view(self, name: str, dtype=torch.int16, shape=None) -> torch.Tensor:
@@ -95,28 +99,39 @@ class BlockSession:
             v = v[:n].view(*shape)
         return v
 
+    # The plan's addresses never change, so the views of the inputs and the output are made once
+    # (making one takes several microseconds, on a path that small blocks run in tens of them).
     def hid_in(self) -> torch.Tensor:
-        t = self.template
-        return self.view("hid0", torch.int16, (t.batch, self.seq, t.hidden))
+        return self._hid_in
 
     def temb(self) -> torch.Tensor:
-        t = self.template
-        return self.view("temb", torch.int16, (t.batch, t.temb_dim))
+        return self._temb
 
     def hid_out(self) -> torch.Tensor:
-        t = self.template
-        return self.view("hid%d" % t.n_blocks, torch.int16, (t.batch, self.seq, t.hidden))
+        return self._hid_out
 
     # ---- data movement ------------------------------------------------------------------
+    def _in_place(self, src, dst) -> bool:
+        """Whether the library can copy `src` as it stands."""
+        return (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.device == dst.device
+                and src.numel() == dst.numel() and src.is_contiguous() and torch._C._cuda_getDevice() == dst.get_device())
+
     def set_inputs(self, x_bits, temb_bits, non_blocking: bool = False):
         """x_bits / temb_bits: uint16 numpy arrays or int16 torch tensors (host or device)."""
-        for dst, src in ((self.hid_in(), x_bits), (self.temb(), temb_bits)):
+        if self._in_place(x_bits, self._hid_in) and self._in_place(temb_bits, self._temb):
+            self.plan.set_inputs(x_bits.data_ptr(), temb_bits.data_ptr(), self._raw_stream())
+            return
+        for dst, src in ((self._hid_in, x_bits), (self._temb, temb_bits)):
             if isinstance(src, np.ndarray):
                 src = torch.from_numpy(np.ascontiguousarray(src).view(np.int16))
             dst.copy_(src.view(dst.shape), non_blocking=non_blocking)
 
+    def _raw_stream(self) -> int:
+        """The current stream of the session's device as an address."""
+        return torch._C._cuda_getCurrentRawStream(self._hid_in.get_device())
+
     def forward(self, stream: Optional[torch.cuda.Stream] = None):
-        s = (stream or torch.cuda.current_stream(self.device)).cuda_stream
+        s = stream.cuda_stream if stream is not None else self._raw_stream()
         if self.template.n_blocks == 1:
             self.plan.block_forward(s)
         else:

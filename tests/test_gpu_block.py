@@ -507,3 +507,28 @@ def test_guard_bands_between_arena_neighbours_stay_intact(name, chunks):
         torch.Tensor.fill_ = real_fill
     assert damaged["done"] and bad and bad[0][:1] == (0,) and all(b[2] == "hid0" and b[3] == 1 for b in bad)
     assert len(bad) == hid0["death"]
+
+
+@pytest.mark.parametrize("batch,chunks", [(1, 1), (3, 2)])
+def test_set_inputs_takes_every_kind_of_source(batch, chunks):
+    """Device tensors that the copy kernel takes as they stand, ones it cannot take (not 16-byte
+    aligned, not contiguous), host tensors and arrays all leave the same bytes in the arena, and
+    nothing around the two slots changes."""
+    t = template("tiny", batch=batch)
+    x, temb = make_activations(t)
+    s = BlockSession(t, [make_block_weights(t, 0)], chunks=chunks)
+    xd = torch.from_numpy(x.view(np.int16)).to("cuda:0")
+    td = torch.from_numpy(temb.view(np.int16)).to("cuda:0")
+    odd = torch.zeros(xd.numel() + 1, dtype=torch.int16, device="cuda:0")[1:].view(xd.shape)
+    odd.copy_(xd)
+    strided = torch.zeros(*xd.shape[:2], 2 * xd.shape[2], dtype=torch.int16, device="cuda:0")[..., :xd.shape[2]]
+    strided.copy_(xd)
+    slots = torch.zeros_like(s.arena, dtype=torch.bool)
+    for name, like in (("hid0", xd), ("temb", td)):
+        off, _ = s.plan.tensor(name)
+        slots[off:off + 2 * like.numel()] = True
+    for src_x, src_t in ((xd, td), (xd.view(-1), td.view(-1)), (odd, td), (strided, td), (xd.cpu(), td), (x, temb)):
+        s.arena.fill_(0x5A)
+        s.set_inputs(src_x, src_t)
+        assert torch.equal(s.hid_in(), xd) and torch.equal(s.temb(), td)
+        assert bool((s.arena[~slots] == 0x5A).all())
