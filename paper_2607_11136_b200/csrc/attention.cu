@@ -1,25 +1,53 @@
 // Non-causal flash-style attention on tcgen05: o = softmax(q k^T / sqrt(dh)) v over all keys.
 //
-// One CTA owns one (batch, head, 128-query-row tile) and streams the keys in blocks of 64; its
-// workspace (shared memory and TMEM) depends on the query tile only, never on the number of
-// keys.  Two CTAs share an SM.  192 threads:
-//   warp 0    TMA producer: Q tile once, then K and V tiles through a ring of stages
-//   warp 1    owns TMEM; one thread issues S(j) = Q K(j)^T into one of two TMEM score buffers
-//             and O += P(j) V(j) with P read from TMEM
-//   warps 2-5 softmax: thread = query row.  Reads its score row from TMEM into registers,
-//             keeps the running max / sum in the exp2 domain, writes P(j) (bf16, two per
-//             column) in place over the score buffer it came from, rescales O in TMEM when the
-//             running max moved, and at the end normalises O and stores it.
-// Pipeline: the issuing thread's tcgen05 operations execute in order, so after P(j) is ready
-// it queues PV(j) and then S(j+2) into the buffer PV(j) frees; the softmax warps therefore
-// find S(j+1) waiting and depend on the tensor pipe again only in the rare iterations in which
-// a row's running max moved (O must then be at rest).  Shared memory carries only Q, K, V.
+// One persistent CTA per SM walks over work items of up to 256 query rows (two 128-row tiles) of one
+// (batch, head) and streams the keys in blocks of 128 from key 0.  Its workspace (shared memory and
+// TMEM) depends on the tile only, never on the number of keys.
 //
-// Every decision is taken per row (the running max only moves when it grows by more than 2^8
-// in the exp2 domain; multiplying the other rows by exactly 1 changes nothing), keys are
-// always visited from key 0 in blocks of 64, and nothing is split or reduced across CTAs, so
-// a query row's output bits do not depend on how the query rows are chunked or tiled.
+//   warp 0       TMA producer: both Q tiles of an item, then K and V blocks through two rings
+//   warps 1, 2   MMA issuers (converged warp, one elected lane issues): dh 64 warp 1 the scores and
+//                warp 2 the products, dh 128 warp 1 both.  Warp 1 also owns TMEM
+//   warp 3       idle (fills the warpgroup, so that softmax warp w reads TMEM lanes 32 * (w % 4))
+//   warps 4-19   softmax: two threads per score row, 64 scores each per block
+//
+// The softmax threads set the pace (an SM retires 16 exponentials per clock against 4 * dh flop each),
+// so their instruction stream is kept short:
+//
+//   * no running maximum, and in the normal pass no reference at all: q arrives multiplied by
+//     log2(e) / sqrt(dh) (the Q projection's epilogue does that before its one rounding to bf16), so a
+//     score leaves the tensor core as the exponent to base 2 of its unnormalised probability and
+//     p = 2^s is formed whatever its size -- fp32 sums and bf16 probabilities keep their relative
+//     precision from 2^-90 to 2^90 -- so O is never rescaled and the two threads of a row need not talk
+//     to each other inside the loop.  A row that leaves that range (a sum of 2^90 or more, or of 2^-90
+//     or less), or that hands the exponential polynomial an argument outside its range, is flagged, and
+//     its item is done again after the CTA's last item, in two more sweeps: one over the scores only,
+//     which decides again which rows were at fault and takes their true maximum, and one that repeats
+//     the pass with that maximum taken off the scores of those rows.  Rows that were not at fault
+//     repeat exactly what they did before, bit for bit;
+//   * a share of the exponentials is evaluated as a polynomial on the FMA pipe (see kPolyPairs);
+//   * one body for all blocks where there are few: the first time an SM runs a piece of code costs
+//     microseconds of instruction fetch, which a call with few keys pays in full.  Keys past the end get
+//     the score -119 (they add 2^-119 each to a row sum of at least 2^-90; their V rows are zero).
+//
+// TMEM, per tile 256 columns:
+//   dh  64: S [0,128), P [128,192) (bf16 pairs), O [192,256).  S(j+1) is issued as soon as the tile's
+//           threads hold S(j) in registers and runs while they work; P(j) is stored once
+//           O += P(j-1) V(j-1), which reads the same columns, has finished.
+//   dh 128: S [0,128), O [128,256); P(j) lies over S(j), each thread's over its own scores.  S(j+1) is
+//           queued behind O += P(j) V(j) in the tensor pipe; the two tiles run half a block apart, so
+//           one tile's burst of MMAs runs under the other's softmax.  One warp issues both: with a warp
+//           per tile the two bursts shared the pipe and both ended late (a block 3090 cycles against
+//           2690).  P goes over in two halves, so half of the product runs under the rest of the softmax.
+//
+// Measured (B200, inside the block): dh 64, 4444 x 17776 x 48 heads 933 us (with one CTA per 256 rows and code
+// copies for first and last blocks 970); power-capped 17776-token block 7.28 ms against 7.52.  dh 128, 17776 x
+// 17776 x 24 heads 3.03 ms = 1280 TFLOP/s (one tile per CTA, two CTAs per SM, 64-key blocks, running maximum: 3.40),
+// 4608 x 4608 x 24 heads 232 us (261).  288 x 288 x 8 heads 10.4 us (14.4), launches back to back.
+//
+// Every decision is per row and keys are always visited in the same order, so a row's bits do not
+// depend on how rows are tiled or chunked.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 #include "sm100.cuh"
@@ -27,383 +55,727 @@
 namespace xema {
 using namespace sm100;
 
-constexpr int ATT_BM = 128;      // query rows per CTA
-constexpr int ATT_BN = 64;       // keys per block
-constexpr int ATT_THREADS = 192;
-constexpr int Q_ATOM_BYTES = ATT_BM * 128;    // 128 rows x 64 bf16, one swizzled column block
-constexpr int KV_ATOM_BYTES = ATT_BN * 128;   // 64 keys x 64 bf16
-// Share of the exponentials evaluated as a polynomial on the FMA pipe instead of the MUFU: none
-// in this kernel (with 128-wide heads a share of 1/8 or 1/4 measured 4-7 % slower: the shape is
-// not bound by the exponent rate).
-constexpr int POLY_NUM = 0, POLY_DEN = 4;
+namespace {
+constexpr int BM = 128;          // rows per tile
+constexpr int TILES = 2;
+constexpr int BN = kAttnKeysPerBlock;   // keys per block (128)
+constexpr int ATOM_BYTES = 128 * 128;   // 128 rows x 64 bf16, one swizzled column block
+constexpr float DANGER = 1.2379400392853803e27f;   // 2^90
+constexpr float TINY = 8.077935669463161e-28f;     // 2^-90
+constexpr float PAST_END = -119.f;      // score of a key past the end of the sequence
+constexpr int MAX_ITEMS = 1024;         // items one CTA can keep a flag for
+constexpr int TPR = 2;           // softmax threads per score row
+constexpr int COLS = BN / TPR;   // scores per softmax thread and block ...
+constexpr int CH = COLS / 4;     // ... worked on in four chunks
+constexpr int SOFTMAX_THREADS = TILES * BM * TPR;
+constexpr int THREADS = 128 + SOFTMAX_THREADS;
+// Registers a thread: the compiler allots 96 to 640 threads; the helper warps give some back to the
+// softmax warps.  128 * HELPER + SOFTMAX_THREADS * SOFTMAX must stay within THREADS * 96, or the
+// request would wait for ever.
+constexpr int REG_HELPER = 64, REG_SOFTMAX = 104;
+static_assert(128 * REG_HELPER + SOFTMAX_THREADS * REG_SOFTMAX <= THREADS * 96, "register pool");
+// Which of a thread's 32 column pairs evaluate 2^x as a polynomial on the FMA pipe, one bit per pair; the
+// others use the MUFU.  Without any the MUFU sets the pace, with too many the issue slots do, and where
+// they stand decides how well the compiler interleaves the two pipes.  Measured inside the block (scores
+// bounded, see below) over 125 placements of 6 to 17 bits: dh 64, 4444 x 17776 x 48 heads 933 to 1177 us (this
+// one 933, the next best 945; 9 bits 1000 and more), dh 128, 4608 x 4608 x 24 heads 232 to 247 us (this one 232).
+// Power-capped, the dh 64 block of 17776 tokens takes 7.28 ms with this placement, 7.39-7.56 with three others.
+template <int DH>
+constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0xa2898818u;
+static_assert(BN == 128 && BM == 128, "the kernel is written for 128-key blocks of 128-row tiles");
 
 template <int DH>
-struct AttnCfg {
-  static constexpr int ATOMS = DH / 64;                        // 64-wide column blocks per tile
-  static constexpr int Q_BYTES = ATOMS * Q_ATOM_BYTES;
-  static constexpr int KV_BYTES = ATOMS * KV_ATOM_BYTES;       // one K or V tile
-  static constexpr int KV_STAGES = (DH == 64) ? 4 : 2;
+struct Cfg {
+  static constexpr bool ALIAS = DH == 128;                 // P over S; otherwise P has its own columns
+  static constexpr int ISSUERS = ALIAS ? 1 : 2;            // MMA-issuing warps (from warp 1)
+  static constexpr int ATOMS = DH / 64;
+  static constexpr int TILE_BYTES = ATOMS * ATOM_BYTES;    // a Q tile, or a K or V block
+  static constexpr int QBUF = DH == 64 ? 2 : 1;
+  static constexpr int KS = DH == 64 ? 5 : 2;              // K and V stages
+  static constexpr int VS = DH == 64 ? 5 : 3;
   static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + Q_BYTES;
-  static constexpr int OFF_V = OFF_K + KV_STAGES * KV_BYTES;
-  static constexpr int OFF_BAR = OFF_V + KV_STAGES * KV_BYTES;
-  static constexpr int SMEM_BYTES = OFF_BAR + 256;
-  // TMEM columns: two score buffers S0 [0,64), S1 [64,128) (P(j) overwrites the first 32
-  // columns of the buffer S(j) came from); O fp32 [128, 128+DH)
-  static constexpr int TMEM_O = 128;
-  static constexpr int TMEM_COLS = 256;
+  static constexpr int OFF_K = OFF_Q + QBUF * TILES * TILE_BYTES;
+  static constexpr int OFF_V = OFF_K + KS * TILE_BYTES;
+  static constexpr int OFF_BAR = OFF_V + VS * TILE_BYTES;
+  static constexpr int OFF_XCH = OFF_BAR + 512;            // float [TILES][2][BM]
+  static constexpr int SMEM_BYTES = OFF_XCH + TILES * 2 * BM * 4;
+  static_assert(SMEM_BYTES <= 232448, "shared memory of one SM");
+  static constexpr int TM_TILE = 256;
+  static constexpr int TM_P = ALIAS ? 0 : 128;
+  static constexpr int TM_O = ALIAS ? 128 : 192;
 };
 
 struct AttnParams {
   __nv_bfloat16* o;
   float* lse;
   int batch, rows, keys, heads;
-  float scale;        // 1/sqrt(dh)
-  float scale_log2;   // scale * log2(e)
+  int tiles;          // query tiles per work item (1 or 2)
+  int q_items;        // work items per (batch, head)
+  int items;
+  float q_scale;      // q k^T times this = exponents to base 2 (SCALED kernels only)
   unsigned int* status;
+  const __nv_bfloat16 *gain_q, *gain_k;   // RMSNorm gains behind q and k, or null (see AttnLaunch)
 };
 
-template <int DH>
-__global__ void __launch_bounds__(ATT_THREADS, 2)
+// 2^x for two values on the FMA pipe, as exp2_poly_f32x2 but without its clamp: the caller
+// guarantees -125 <= x <= 126.
+__device__ __forceinline__ f32x2 exp2_poly_unclamped(f32x2 x2) {
+  const f32x2 magic = make_float2(12582912.f, 12582912.f);
+  const f32x2 neg_magic = make_float2(-12582912.f, -12582912.f);
+  const f32x2 neg_one = make_float2(-1.f, -1.f);
+  const f32x2 t2 = add_f32x2(x2, magic);                 // integer part lands in the low mantissa bits
+  const f32x2 n2 = add_f32x2(t2, neg_magic);             // nearest integer as a float
+  const f32x2 r2 = fma_f32x2(n2, neg_one, x2);           // r = x - n
+  f32x2 p2 = fma_f32x2(make_float2(0.0551716685f, 0.0551716685f), r2, make_float2(0.242611125f, 0.242611125f));
+  p2 = fma_f32x2(p2, r2, make_float2(0.693260968f, 0.693260968f));
+  p2 = fma_f32x2(p2, r2, make_float2(0.999928057f, 0.999928057f));
+  return make_float2(__uint_as_float(__float_as_uint(p2.x) + (__float_as_uint(t2.x) << 23)),
+                     __uint_as_float(__float_as_uint(p2.y) + (__float_as_uint(t2.y) << 23)));
+}
+
+// p = 2^s for chunk CHUNK of a thread's score columns: packed bf16x2 words, the values added into
+// four packed partial sums.  The polynomial is only valid for arguments in [-125, 126].
+// CLAMP = false: it is used as it is and, with TRACK, `poly_abs` collects the largest magnitude handed
+// to it, for the caller to check afterwards (without TRACK the caller knows a bound on every score
+// beforehand).  CLAMP = true: arguments are clamped from below first (2^-125 stands in for zero);
+// wherever the unclamped form was valid the result has the same bits.
+template <int DH, int CHUNK, bool CLAMP, bool TRACK>
+__device__ __forceinline__ void exp_cols(const float (&s)[CH], uint32_t* pk, f32x2 (&ls2)[4], float& poly_abs) {
+#pragma unroll
+  for (int t = 0; t < CH; t += 2) {
+    const int pair = t >> 1;
+    f32x2 e2 = pack_f32x2(s[t], s[t + 1]);   // the scores come out of the tensor core as exponents
+    float e0, e1;
+    if (kPolyPairs<DH> >> (CHUNK * (CH / 2) + pair) & 1u) {
+      if (CLAMP) {
+        e2 = exp2_poly_f32x2(e2);
+      } else {
+        if (TRACK) poly_abs = max3(poly_abs, fabsf(e2.x), fabsf(e2.y));
+        e2 = exp2_poly_unclamped(e2);
+      }
+      unpack_f32x2(e2, e0, e1);
+    } else {
+      unpack_f32x2(e2, e0, e1);
+      e0 = ex2_approx(e0);
+      e1 = ex2_approx(e1);
+      e2 = pack_f32x2(e0, e1);
+    }
+    ls2[pair & 3] = add_f32x2(ls2[pair & 3], e2);
+    pk[pair] = pack_bf16x2(e0, e1);
+  }
+}
+// columns at or beyond `valid` (keys past the end of the sequence) get `value`
+__device__ __forceinline__ void mask_tail(float (&s)[CH], int valid, float value) {
+#pragma unroll
+  for (int t = 0; t < CH; ++t)
+    if (t >= valid) s[t] = value;
+}
+__device__ __forceinline__ float row_max(const float (&s)[CH]) {
+  float mx = max3(s[0], s[1], s[2]);
+#pragma unroll
+  for (int t = 3; t + 1 < CH; t += 2) mx = max3(mx, s[t], s[t + 1]);
+  return fmaxf(mx, s[CH - 1]);
+}
+__device__ __forceinline__ float sum_partials(const f32x2 (&ls2)[4]) {
+  const f32x2 a = add_f32x2(ls2[0], ls2[1]), b = add_f32x2(ls2[2], ls2[3]);
+  const f32x2 c = add_f32x2(a, b);
+  return c.x + c.y;
+}
+__device__ __forceinline__ void ld_scores(uint32_t addr, float (&s)[CH]) { tmem_ld16(addr, *reinterpret_cast<uint32_t(*)[CH]>(&s[0])); }
+__device__ __forceinline__ void wait_scores(float (&s)[CH]) { tmem_ld_wait_on(*reinterpret_cast<uint32_t(*)[CH]>(&s[0])); }
+
+// Sweeps of one item: the pass itself; the scores only (flags and true maxima); the repeat.
+enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
+
+template <int DH, bool SCALED>
+__global__ void __launch_bounds__(THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
-  using Cfg = AttnCfg<DH>;
-  constexpr int STAGES = Cfg::KV_STAGES;
+  using C = Cfg<DH>;
+  constexpr int KS = C::KS, VS = C::VS, QBUF = C::QBUF;
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
-  uint64_t* q_full = bars + 0;
-  uint64_t* k_full = bars + 1;    // [STAGES <= 4]
-  uint64_t* k_empty = bars + 5;
-  uint64_t* v_full = bars + 9;
-  uint64_t* v_empty = bars + 13;
-  uint64_t* s_full = bars + 17;   // [2] one per score buffer
-  uint64_t* p_full = bars + 19;   // [2]
-  uint64_t* pv_done = bars + 21;  // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 23);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
+  uint64_t* q_full = bars + 0;     // [QBUF]
+  uint64_t* q_empty = bars + 2;    // [QBUF] both tiles' last scores of the item are done
+  uint64_t* k_full = bars + 4;     // [KS <= 5]
+  uint64_t* k_empty = bars + 9;
+  uint64_t* v_full = bars + 14;    // [VS <= 5]
+  uint64_t* v_empty = bars + 19;
+  uint64_t* s_full = bars + 24;    // [TILES] S(j) of the tile is complete in TMEM
+  uint64_t* s_free = bars + 26;    // [TILES] every softmax thread of the tile holds S(j) in registers
+  uint64_t* p_half = bars + 28;    // [TILES] the first half of P(j) is complete in TMEM (ALIAS)
+  uint64_t* p_full = bars + 30;    // [TILES] P(j) is complete in TMEM
+  uint64_t* pv_done = bars + 32;   // [TILES] O += P(j) V(j) has finished (ALIAS: of an item's last block)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 34);
   volatile uint32_t* abort_flag = tmem_slot + 1;
+  uint32_t* gain_max = tmem_slot + 2;               // [2] bit patterns of max|gain_q|, max|gain_k|
+  volatile uint32_t* any_flag = tmem_slot + 4;
+  uint32_t* item_flag = tmem_slot + 5;              // [MAX_ITEMS / 32] one bit per item of this CTA
+  static_assert(34 * 8 + (5 + MAX_ITEMS / 32) * 4 <= 512, "barrier area");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int n_kv = (p.keys + ATT_BN - 1) / ATT_BN;
+  const int n_kv = (p.keys + BN - 1) / BN;
+  const int n_items = (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // of this CTA
 
   // The swizzled tiles need a 1024-byte aligned base; refuse to run otherwise.
   if ((smem_u32(smem) & 1023u) != 0) {
     if (threadIdx.x == 0 && p.status) atomicExch(p.status, 0x54310002u);
     return;
   }
-
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < QBUF; ++s) {
+      mbar_init(&q_full[s], 1);
+      mbar_init(&q_empty[s], 1);
+    }
+    for (int s = 0; s < KS; ++s) {
       mbar_init(&k_full[s], 1);
       mbar_init(&k_empty[s], 1);
+    }
+    for (int s = 0; s < VS; ++s) {
       mbar_init(&v_full[s], 1);
       mbar_init(&v_empty[s], 1);
     }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&s_full[s], 1);
-      mbar_init(&p_full[s], 4);
-      mbar_init(&pv_done[s], 1);
+    for (int t = 0; t < TILES; ++t) {
+      mbar_init(&s_full[t], 1);
+      mbar_init(&s_free[t], BM * TPR);   // every softmax thread of the tile arrives
+      mbar_init(&p_half[t], BM * TPR);
+      mbar_init(&p_full[t], BM * TPR);
+      mbar_init(&pv_done[t], 1);
     }
     *abort_flag = 0;
+    *any_flag = 0;
+    gain_max[0] = gain_max[1] = 0;
     fence_mbar_init();
     prefetch_tmap(&map_q);
     prefetch_tmap(&map_k);
     prefetch_tmap(&map_v);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
+    tmem_alloc(tmem_slot, 512);
     tmem_relinquish();
   }
+  if (warp == 3 && lane < MAX_ITEMS / 32) item_flag[lane] = 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if (threadIdx.x == 0) grid_dep_launch();
   grid_dep_wait();
-  const uint32_t tmem_o = tmem_base + Cfg::TMEM_O;
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      bool ok = true;
-      mbar_expect_tx(q_full, Cfg::Q_BYTES);
+  struct Item {
+    int row0, h, b;
+  };
+  auto item_at = [&](int i) {
+    const int w = (int)blockIdx.x + i * (int)gridDim.x;
+    Item it;
+    const int bh = w / p.q_items;
+    it.row0 = (w - bh * p.q_items) * p.tiles * BM;
+    it.b = bh / p.heads;
+    it.h = bh - it.b * p.heads;
+    return it;
+  };
+  auto tile_live = [&](const Item& it, int t) { return t < p.tiles && it.row0 + t * BM < p.rows; };
+
+  // ---- per-role state that lives across items and sweeps -------------------------------------
+  int k_st = 0, v_st = 0, q_st = 0;                 // ring positions (producer; each MMA warp)
+  uint32_t k_ph = 0, v_ph = 0, q_ph = 0;
+  int k_issued = 0, v_issued = 0, q_issued = 0;     // producer, for the drain after a give-up
+  uint32_t s_ph = 0, pv_ph = 0;                     // softmax: s_full, pv_done
+  bool ok = true;
+
+  auto k_next = [&]() { if (++k_st == KS) { k_st = 0; k_ph ^= 1; } };
+  auto v_next = [&]() { if (++v_st == VS) { v_st = 0; v_ph ^= 1; } };
+  auto q_next = [&]() { if (++q_st == QBUF) { q_st = 0; q_ph ^= 1; } };
+
+  // One item in one sweep, in the roles of the single-warp loops.
+  auto produce = [&](const Item& it, bool with_v) {   // warp 0, one lane
+    auto load = [&](uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int row0) {
+      mbar_expect_tx(bar, C::TILE_BYTES);
 #pragma unroll
-      for (int a = 0; a < Cfg::ATOMS; ++a)
-        tma_load_3d(smem + Cfg::OFF_Q + a * Q_ATOM_BYTES, &map_q, q_full, h * DH + a * 64, qt * ATT_BM, b);
-      int k_issued = 0, v_issued = 0;
-      int st = 0;
-      uint32_t ph = 0;
-      for (int j = 0; j < n_kv; ++j) {
-        if (!(ok = mbar_wait(&k_empty[st], ph ^ 1, abort_flag))) break;
-        mbar_expect_tx(&k_full[st], Cfg::KV_BYTES);
-#pragma unroll
-        for (int a = 0; a < Cfg::ATOMS; ++a)
-          tma_load_3d(smem + Cfg::OFF_K + st * Cfg::KV_BYTES + a * KV_ATOM_BYTES, &map_k, &k_full[st],
-                      h * DH + a * 64, j * ATT_BN, b);
-        k_issued = j + 1;
-        if (!(ok = mbar_wait(&v_empty[st], ph ^ 1, abort_flag))) break;
-        mbar_expect_tx(&v_full[st], Cfg::KV_BYTES);
-#pragma unroll
-        for (int a = 0; a < Cfg::ATOMS; ++a)
-          tma_load_3d(smem + Cfg::OFF_V + st * Cfg::KV_BYTES + a * KV_ATOM_BYTES, &map_v, &v_full[st],
-                      h * DH + a * 64, j * ATT_BN, b);
-        v_issued = j + 1;
-        if (++st == STAGES) { st = 0; ph ^= 1; }
-      }
-      if (!ok) {
-        // gave up: let the copies already issued land before the CTA leaves (the latest
-        // fill of each stage; older fills were consumed before their stage was reused)
-        volatile uint32_t dummy = 0;
-        mbar_wait(q_full, 0, &dummy);
-        for (int j = max(0, k_issued - STAGES); j < k_issued; ++j) {
-          dummy = 0;
-          mbar_wait(&k_full[j % STAGES], (uint32_t)(j / STAGES) & 1u, &dummy);
-        }
-        for (int j = max(0, v_issued - STAGES); j < v_issued; ++j) {
-          dummy = 0;
-          mbar_wait(&v_full[j % STAGES], (uint32_t)(j / STAGES) & 1u, &dummy);
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    // The whole warp runs this loop converged and one elected lane issues: descriptors and
-    // barrier addresses then stay warp-uniform values (a lone divergent thread would have to
-    // move every operand into the uniform datapath one by one, and its dependent instruction
-    // stream, not the tensor pipe, would bound the kernel).
-    constexpr uint32_t idesc_s = idesc_bf16_f32(ATT_BM, ATT_BN, false, false);   // S = Q K^T
-    constexpr uint32_t idesc_o = idesc_bf16_f32(ATT_BM, DH, false, true);        // O = P V, V is N-major
-    const uint64_t q_desc = smem_desc_sw128(smem_u32(smem + Cfg::OFF_Q), 16, 1024);
-    const uint64_t k_desc0 = smem_desc_sw128(smem_u32(smem + Cfg::OFF_K), 16, 1024);
-    // V tile: rows = keys (the MMA's K), 64 dh per 128-byte row, 16 keys = 2048 bytes; the
-    // second 64-wide dh block (dh = 128) starts one atom further (leading byte offset)
-    const uint64_t v_desc0 = smem_desc_sw128(smem_u32(smem + Cfg::OFF_V), KV_ATOM_BYTES, 1024);
-    int k_st = 0, v_st = 0;
-    uint32_t k_ph = 0, v_ph = 0;
-    auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
-      return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+      for (int a = 0; a < C::ATOMS; ++a) tma_load_3d(dst + a * ATOM_BYTES, m, bar, it.h * DH + a * 64, row0, it.b);
     };
-    auto issue_s = [&](int buf) -> bool {
-      if (!wait_all(&k_full[k_st], k_ph)) return false;
-      tc_fence_after();
-      if (elect_one()) {
-        const uint64_t k_desc = k_desc0 + (uint64_t)(k_st * (Cfg::KV_BYTES >> 4));
-        const uint32_t d = tmem_base + buf * ATT_BN;
-#pragma unroll
-        for (int k = 0; k < DH / 16; ++k)
-          mma_ss(d, q_desc + (uint64_t)(((k / 4) * Q_ATOM_BYTES + (k % 4) * 32) >> 4),
-                 k_desc + (uint64_t)(((k / 4) * KV_ATOM_BYTES + (k % 4) * 32) >> 4), idesc_s, k != 0);
-        mma_commit(&k_empty[k_st]);
-        mma_commit(&s_full[buf]);
-      }
-      __syncwarp();
-      if (++k_st == STAGES) { k_st = 0; k_ph ^= 1; }
-      return true;
+    auto load_k = [&](int j) {
+      if (!(ok = mbar_wait(&k_empty[k_st], k_ph ^ 1, abort_flag))) return;
+      load(smem + C::OFF_K + k_st * C::TILE_BYTES, &map_k, &k_full[k_st], j * BN);
+      ++k_issued;
+      k_next();
     };
-    bool ok = wait_all(q_full, 0);
-    if (ok) ok = issue_s(0);
-    if (ok && n_kv > 1) ok = issue_s(1);
+    load_k(0);
+    if (!ok || !(ok = mbar_wait(&q_empty[q_st], q_ph ^ 1, abort_flag))) return;
+    mbar_expect_tx(&q_full[q_st], p.tiles * C::TILE_BYTES);
+    for (int t = 0; t < p.tiles; ++t)
+#pragma unroll
+      for (int a = 0; a < C::ATOMS; ++a)
+        tma_load_3d(smem + C::OFF_Q + (q_st * TILES + t) * C::TILE_BYTES + a * ATOM_BYTES, &map_q, &q_full[q_st],
+                    it.h * DH + a * 64, it.row0 + t * BM, it.b);
+    ++q_issued;
+    q_next();
     for (int j = 0; ok && j < n_kv; ++j) {
-      const int buf = j & 1;
-      const uint32_t par = (uint32_t)(j >> 1) & 1u;
-      const bool more = j + 2 < n_kv;
-      // K(j+2) and V(j) were loaded stages ahead: check them while P(j) is still being made,
-      // so that nothing stands between P(j) becoming ready and the two products being queued
-      // (only with a deep ring: with two stages K(j+2) is requested too late for that)
-      constexpr bool kEarlyK = STAGES >= 4;
-      if (kEarlyK && more && !(ok = wait_all(&k_full[k_st], k_ph))) break;
-      if (!(ok = wait_all(&v_full[v_st], v_ph))) break;
-      // P(j) sits in TMEM over S(j) (and O has been rescaled if a running max moved)
-      if (!(ok = wait_all(&p_full[buf], par))) break;
-      tc_fence_after();
-      if (elect_one()) {
-        const uint64_t v_desc = v_desc0 + (uint64_t)(v_st * (Cfg::KV_BYTES >> 4));
-        const uint32_t sp_tmem = tmem_base + buf * ATT_BN;
-#pragma unroll
-        for (int kk = 0; kk < ATT_BN / 16; ++kk)             // 16 keys = 8 packed P columns
-          mma_ts(tmem_o, sp_tmem + kk * 8, v_desc + (uint64_t)(kk * (2048 >> 4)), idesc_o, (j | kk) != 0);
-        mma_commit(&v_empty[v_st]);
-        mma_commit(&pv_done[buf]);
+      if (j + 1 < n_kv) load_k(j + 1);
+      if (!ok) return;
+      if (with_v) {
+        if (!(ok = mbar_wait(&v_empty[v_st], v_ph ^ 1, abort_flag))) return;
+        load(smem + C::OFF_V + v_st * C::TILE_BYTES, &map_v, &v_full[v_st], j * BN);
+        ++v_issued;
+        v_next();
       }
-      if (!kEarlyK && more) {
-        if (!(ok = wait_all(&k_full[k_st], k_ph))) break;
-        tc_fence_after();
-      }
-      if (elect_one()) {
-        const uint32_t sp_tmem = tmem_base + buf * ATT_BN;
-        // S(j+2) reuses the buffer; it is queued behind PV(j), which reads P(j) from it
-        if (more) {
-          const uint64_t k_desc = k_desc0 + (uint64_t)(k_st * (Cfg::KV_BYTES >> 4));
-#pragma unroll
-          for (int k = 0; k < DH / 16; ++k)
-            mma_ss(sp_tmem, q_desc + (uint64_t)(((k / 4) * Q_ATOM_BYTES + (k % 4) * 32) >> 4),
-                   k_desc + (uint64_t)(((k / 4) * KV_ATOM_BYTES + (k % 4) * 32) >> 4), idesc_s, k != 0);
-          mma_commit(&k_empty[k_st]);
-          mma_commit(&s_full[buf]);
-        }
-      }
-      __syncwarp();
-      if (++v_st == STAGES) { v_st = 0; v_ph ^= 1; }
-      if (more && ++k_st == STAGES) { k_st = 0; k_ph ^= 1; }
     }
-  } else {
-    // ---------------- softmax / correction / epilogue ----------------
-    const int quad = warp & 3;
-    const int r = quad * 32 + lane;                       // query row inside the tile = TMEM lane
-    const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
-    float m_run = -INFINITY, l_run = 0.f;
-    bool ok = true;
-    // The score row of block j+1 is requested from TMEM at the end of iteration j, right after
-    // P(j) has been handed over; s[] always holds the block that is being worked on.
-    float s[ATT_BN];
-    ok = __all_sync(0xffffffffu, mbar_wait(&s_full[0], 0, abort_flag));
-    if (ok) {
-      tc_fence_after();
+  };
+
+  constexpr uint32_t idesc_s = idesc_bf16_f32(BM, BN, false, false);   // S = Q K^T
+  constexpr uint32_t idesc_o = idesc_bf16_f32(BM, DH, false, true);    // O = P V, V is N-major
+  // (descriptors: the low words, which hold the address; the high word is the same constant for all)
+  const uint32_t q_desc0 = smem_desc_lo(smem_u32(smem + C::OFF_Q), 16);
+  const uint32_t k_desc0 = smem_desc_lo(smem_u32(smem + C::OFF_K), 16);
+  // V block: rows = keys (the MMA's K), 64 dh per 128-byte row, 16 keys = 2048 bytes; the second
+  // 64-wide dh block (dh = 128) starts one atom further (leading byte offset)
+  const uint32_t v_desc0 = smem_desc_lo(smem_u32(smem + C::OFF_V), ATOM_BYTES);
+  // Scores of one block, tile t.
+  auto mma_scores = [&](int t) {   // elected lane
+    const uint32_t qd = q_desc0 + (q_st * TILES + t) * (C::TILE_BYTES >> 4);
+    const uint32_t kd = k_desc0 + k_st * (C::TILE_BYTES >> 4);
 #pragma unroll
-      for (int ch = 0; ch < ATT_BN / 32; ++ch)
-        tmem_ld32(tmem_base + lane_sel + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[ch * 32]));
+    for (int k = 0; k < DH / 16; ++k) {
+      const uint32_t off = ((k / 4) * ATOM_BYTES + (k % 4) * 32) >> 4;
+      mma_ss_lo(tmem_base + t * C::TM_TILE, qd + off, kd + off, idesc_s, k != 0);
     }
-    for (int j = 0; ok && j < n_kv; ++j) {
-      const int buf = j & 1;
-      const uint32_t s_tmem = tmem_base + lane_sel + buf * ATT_BN;
-      const uint32_t next_par = (uint32_t)((j + 1) >> 1) & 1u;
-      tmem_ld_wait();
-      // keys past the end exist only in the last block
-      const int valid = p.keys - j * ATT_BN;
-      if (valid < ATT_BN) {
+    mma_commit(&s_full[t]);
+  };
+  // Half of the product of one block: O += P V over 64 keys, 16 keys = 8 packed P columns per step.
+  // ALIAS: P of each 64-key half lies over its own scores, and the first
+  // (second) 32 keys of both halves are handed over together.
+  auto mma_product = [&](int t, int hf, bool init) {   // elected lane
+    const uint32_t d = tmem_base + t * C::TM_TILE;
+    const uint32_t vd = v_desc0 + v_st * (C::TILE_BYTES >> 4);
 #pragma unroll
-        for (int t = 0; t < ATT_BN; ++t)
-          if (t >= valid) s[t] = -INFINITY;
+    for (int i = 0; i < 4; ++i) {
+      const int kk = C::ALIAS ? (i >> 1) * 4 + hf * 2 + (i & 1) : hf * 4 + i;
+      const int col = C::ALIAS ? (kk >> 2) * 64 + (kk & 3) * 8 : kk * 8;
+      mma_ts_lo(d + C::TM_O, d + C::TM_P + col, vd + kk * (2048 >> 4), idesc_o, !init || i != 0);
+    }
+  };
+  auto wait_k = [&](bool first) {
+    if (first && !(ok = mbar_wait_warp(&q_full[q_st], q_ph, abort_flag))) return;
+    ok = mbar_wait_warp(&k_full[k_st], k_ph, abort_flag);
+    tc_fence_after();
+  };
+  auto wait_v = [&]() {
+    ok = mbar_wait_warp(&v_full[v_st], v_ph, abort_flag);
+    tc_fence_after();
+  };
+  auto wait_phase = [&](uint64_t* bar, uint32_t& ph) {
+    ok = mbar_wait_warp(bar, ph, abort_flag);
+    ph ^= 1;
+    tc_fence_after();
+  };
+  // whole warp: the block's (and the item's last) scores, or its products, are issued
+  auto k_done = [&](bool last) {
+    if (elect_one()) {
+      mma_commit(&k_empty[k_st]);
+      if (last) mma_commit(&q_empty[q_st]);
+    }
+    __syncwarp();
+    k_next();
+  };
+  auto v_done = [&]() {
+    if (elect_one()) mma_commit(&v_empty[v_st]);
+    __syncwarp();
+    v_next();
+  };
+  uint32_t s_free_ph[TILES] = {0, 0}, p_full_ph[TILES] = {0, 0}, p_half_ph[TILES] = {0, 0};
+  bool s_pending[TILES] = {false, false};     // scores issued whose release has not been waited for yet
+
+  // dh 64, and the score-only sweep: a warp for the scores ...
+  auto issue_scores = [&](const Item& it) {
+    for (int j = 0; j < n_kv; ++j) {
+      wait_k(j == 0);
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) {
+        if (!ok) return;
+        if (!tile_live(it, t)) continue;
+        if (s_pending[t]) wait_phase(&s_free[t], s_free_ph[t]);
+        if (!ok) return;
+        if (elect_one()) mma_scores(t);
+        __syncwarp();
+        s_pending[t] = true;
       }
-      // row max: independent chains of three-input max
-      float mx[4];
+      k_done(j == n_kv - 1);
+    }
+    q_next();
+  };
+  // ... and one for the products: neither stream waits for the other's barriers.
+  auto issue_products = [&](const Item& it) {
+    for (int j = 0; j < n_kv; ++j) {
+      wait_v();
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        mx[u] = max3(s[16 * u], s[16 * u + 1], s[16 * u + 2]);
-#pragma unroll
-        for (int t = 3; t < 15; t += 2) mx[u] = max3(mx[u], s[16 * u + t], s[16 * u + t + 1]);
-        mx[u] = fmaxf(mx[u], s[16 * u + 15]);
-      }
-      const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-      // the running max moves only when it grows by more than 2^8 (exp2 domain); per row
-      float m_new = m_run;
-      if (j == 0 || (m_blk - m_run) * p.scale_log2 > 8.f) m_new = m_blk;
-      const float alpha = (j == 0 || m_new == m_run) ? 1.f : ex2_approx((m_run - m_new) * p.scale_log2);
-      const float neg_m = -m_new * p.scale_log2;
-      // p = exp2(s * c - m * c) on pairs of columns with packed fp32x2 arithmetic; POLY_NUM of
-      // every POLY_DEN pairs (fixed column positions) evaluate 2^x as a polynomial on the FMA
-      // pipe, the rest on the MUFU; row sum in four independent packed partial sums
-      const f32x2 c2 = pack_f32x2(p.scale_log2, p.scale_log2);
-      const f32x2 nm2 = pack_f32x2(neg_m, neg_m);
-      f32x2 ls2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      uint32_t pk[ATT_BN / 2];
-#pragma unroll
-      for (int t = 0; t < ATT_BN; t += 2) {
-        const int pair = t >> 1;
-        f32x2 e2 = fma_f32x2(pack_f32x2(s[t], s[t + 1]), c2, nm2);
-        float e0, e1;
-        if ((pair % POLY_DEN) < POLY_NUM) {
-          e2 = exp2_poly_f32x2(e2);
-          unpack_f32x2(e2, e0, e1);
-        } else {
-          unpack_f32x2(e2, e0, e1);
-          e0 = ex2_approx(e0);
-          e1 = ex2_approx(e1);
-          e2 = pack_f32x2(e0, e1);
+      for (int t = 0; t < TILES; ++t) {
+        if (!ok) return;
+        if (!tile_live(it, t)) continue;
+        wait_phase(&p_full[t], p_full_ph[t]);
+        if (!ok) return;
+        if (elect_one()) {
+          mma_product(t, 0, j == 0);
+          mma_product(t, 1, false);
+          mma_commit(&pv_done[t]);
         }
-        ls2[pair & 3] = add_f32x2(ls2[pair & 3], e2);
-        pk[pair] = pack_bf16x2(e0, e1);
+        __syncwarp();
       }
-      float ls[4];
-      {
-        float a0, a1;
+      v_done();
+    }
+  };
+  // dh 128, one warp for both tiles: O += P(j) V(j) and S(j+1) of one tile go out in one piece, then
+  // those of the other.  (With a warp per tile the two bursts share the tensor pipe and both end late.)
+  auto issue_both = [&](const Item& it) {
+    const bool live[TILES] = {tile_live(it, 0), tile_live(it, 1)};
+    // (after a score-only sweep: its last scores are overwritten without asking)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          unpack_f32x2(ls2[u], a0, a1);
-          ls[u] = a0 + a1;
+    for (int t = 0; t < TILES; ++t) {
+      if (ok && s_pending[t]) wait_phase(&s_free[t], s_free_ph[t]);
+      s_pending[t] = false;
+    }
+    if (!ok) return;
+    wait_k(true);
+    if (!ok) return;
+    if (elect_one()) {
+#pragma unroll
+      for (int t = 0; t < TILES; ++t)
+        if (live[t]) mma_scores(t);
+    }
+    __syncwarp();
+    k_done(n_kv == 1);
+    for (int j = 0; j < n_kv; ++j) {
+      const bool more = j + 1 < n_kv;
+      wait_v();
+      if (!ok) return;
+#pragma unroll
+      for (int t = 0; t < TILES; ++t) {
+        if (!live[t]) continue;
+        wait_phase(&p_half[t], p_half_ph[t]);
+        if (!ok) return;
+        if (elect_one()) mma_product(t, 0, j == 0);
+        __syncwarp();
+        if (more && t == 0) wait_k(false);
+        if (!ok) return;
+        wait_phase(&p_full[t], p_full_ph[t]);
+        if (!ok) return;
+        if (elect_one()) {
+          mma_product(t, 1, false);
+          if (more) mma_scores(t);          // queued behind the product, which reads P from the same columns
+          else mma_commit(&pv_done[t]);
+        }
+        __syncwarp();
+      }
+      v_done();
+      if (more) k_done(j + 2 == n_kv);
+    }
+    q_next();
+  };
+
+  // ---- softmax threads -------------------------------------------------------------------------
+  const int tile = ((warp - 4) >> 3) & 1;
+  const int half = ((warp - 4) >> 2) & 1;
+  const int quad = warp & 3;                               // TMEM lanes [32 * quad, 32 * quad + 32)
+  const int r = quad * 32 + lane;                          // query row inside the tile = TMEM lane
+  const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + tile * C::TM_TILE;
+  const uint32_t s_tmem = t_lane + half * COLS;
+  const uint32_t p_tmem = t_lane + C::TM_P + half * (C::ALIAS ? COLS : COLS / 2);
+  const uint32_t o_tmem = t_lane + C::TM_O + half * (DH / TPR);
+  f32x2 ls2[4];
+  float poly_abs = 0.f, m_ref = 0.f, m_true = 0.f;
+  // The two warps that share 32 rows meet: all of them, with a vote on going on (a warp that gave up
+  // still comes here, so that the other does not wait for it) ...
+  const int pair_bar = 2 + tile * 4 + quad;
+  auto agree = [&]() { ok = named_barrier_and(pair_bar, 64, ok); };
+  // ... and one value from each of the two threads of a row; returns the partner's.
+  auto exchange = [&](float mine) -> float {
+    volatile float* xch = reinterpret_cast<volatile float*>(smem + C::OFF_XCH) + tile * 2 * BM;
+    named_barrier(pair_bar, 64);
+    xch[half * BM + r] = mine;
+    named_barrier(pair_bar, 64);
+    return xch[(half ^ 1) * BM + r];
+  };
+
+  // One key block: this thread's COLS scores in four chunks, the next on its way from TMEM.
+  auto run_block = [&](int j, auto mode_tag, auto masked_tag, auto track_tag) {
+    constexpr bool MASKED = decltype(masked_tag)::value;   // some keys of the block may lie past the end
+    constexpr Mode MODE = decltype(mode_tag)::value;
+    constexpr bool TRACK = decltype(track_tag)::value;
+    constexpr bool CLAMP = MODE == REPEAT;
+    ok = mbar_wait_warp(&s_full[tile], s_ph, abort_flag);
+    if (!ok) return;
+    tc_fence_after();
+    s_ph ^= 1;
+    const int valid = p.keys - j * BN - half * COLS;     // keys of this thread's columns that exist
+    auto adjust = [&](float(&s)[CH], int c) {
+      if (SCALED) {
+        const f32x2 c2 = make_float2(p.q_scale, p.q_scale);
+#pragma unroll
+        for (int t = 0; t < CH; t += 2) {
+          const f32x2 v = __fmul2_rn(pack_f32x2(s[t], s[t + 1]), c2);
+          s[t] = v.x;
+          s[t + 1] = v.y;
         }
       }
-      l_run = fmaf(l_run, alpha, (ls[0] + ls[1]) + (ls[2] + ls[3]));
-      m_run = m_new;
-      // rescale O where the max moved (rows that kept their max multiply by exactly 1); only
-      // then must PV(j-1) have finished
-      if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-        ok = mbar_wait(&pv_done[(j - 1) & 1], (uint32_t)((j - 1) >> 1) & 1u, abort_flag);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
-#pragma unroll 1
-        for (int ch = 0; ch < DH / 32; ++ch) {
-          uint32_t o[32];
-          tmem_ld32(tmem_o + lane_sel + ch * 32, o);
-          tmem_ld_wait();
-#pragma unroll
-          for (int t = 0; t < 32; ++t) o[t] = __float_as_uint(__uint_as_float(o[t]) * alpha);
-          tmem_st32(tmem_o + lane_sel + ch * 32, o);
-        }
+      if (MODE == PROBE) {
+        if (MASKED) mask_tail(s, valid - c * CH, -INFINITY);
+        m_true = fmaxf(m_true, row_max(s));
       }
-      // P(j) in place over this thread's score row: two bf16 per column, 32 columns
-      tmem_st32(s_tmem, pk);
+      if (MODE == REPEAT) {
+#pragma unroll
+        for (int t = 0; t < CH; ++t) s[t] -= m_ref;       // zero for the rows that were fine
+      }
+      if (MASKED) mask_tail(s, valid - c * CH, PAST_END);
+    };
+    uint32_t pk[2][COLS / 4];                          // packed probabilities, by halves
+    float b0[CH], b1[CH], b2[CH];
+    ld_scores(s_tmem, b0);
+    ld_scores(s_tmem + CH, b1);
+    ld_scores(s_tmem + 2 * CH, b2);
+    wait_scores(b0);
+    wait_scores(b1);
+    wait_scores(b2);
+    adjust(b0, 0);
+    exp_cols<DH, 0, CLAMP, TRACK>(b0, &pk[0][0], ls2, poly_abs);
+    ld_scores(s_tmem + 3 * CH, b0);
+    adjust(b1, 1);
+    exp_cols<DH, 1, CLAMP, TRACK>(b1, &pk[0][CH / 2], ls2, poly_abs);
+    wait_scores(b0);
+    if (C::ALIAS && MODE != PROBE) {
+      tmem_st16(p_tmem, pk[0]);                            // all scores are in registers
       tmem_st_wait();
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_full[buf]);
-      // request the next score row (S(j+1) was queued while this block was being worked on)
-      if (j + 1 < n_kv) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&s_full[buf ^ 1], next_par, abort_flag));
-        if (!ok) break;
+      mbar_arrive(&p_half[tile]);
+    } else {
+      tc_fence_before();
+      mbar_arrive(&s_free[tile]);                         // S(j) is in registers: S(j+1) may land
+    }
+    adjust(b2, 2);
+    exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[1][0], ls2, poly_abs);
+    adjust(b0, 3);
+    exp_cols<DH, 3, CLAMP, TRACK>(b0, &pk[1][CH / 2], ls2, poly_abs);
+    if (MODE == PROBE) return;
+    if (!C::ALIAS) {
+      if (j > 0) {                                        // the previous product reads the same columns
+        if (!mbar_peek(&pv_done[tile], pv_ph)) ok = mbar_wait_warp(&pv_done[tile], pv_ph, abort_flag);
+        if (!ok) return;
+        pv_ph ^= 1;
         tc_fence_after();
+      }
+      tmem_st16(p_tmem, pk[0]);
+    }
+    tmem_st16(p_tmem + COLS / 4, pk[1]);
+    tmem_st_wait();
+    tc_fence_before();
+    mbar_arrive(&p_full[tile]);
+  };
+  // Blocks without keys past the end.  With few of them they all take the masking form, so that
+  // only one body has to be fetched.
+  const int n_plain = p.keys / BN > 3 ? p.keys / BN : 0;
+  auto run_blocks = [&](auto mode_tag, auto track_tag) {
 #pragma unroll
-        for (int ch = 0; ch < ATT_BN / 32; ++ch)
-          tmem_ld32(tmem_base + lane_sel + (buf ^ 1) * ATT_BN + ch * 32,
-                    *reinterpret_cast<uint32_t(*)[32]>(&s[ch * 32]));
+    for (int i = 0; i < 4; ++i) ls2[i] = make_float2(0.f, 0.f);
+    poly_abs = 0.f;
+#pragma unroll 1
+    for (int j = 0; ok && j < n_plain; ++j) run_block(j, mode_tag, std::false_type{}, track_tag);
+#pragma unroll 1
+    for (int j = n_plain; ok && j < n_kv; ++j) run_block(j, mode_tag, std::true_type{}, track_tag);
+  };
+  using PassT = std::integral_constant<Mode, PASS>;
+  using ProbeT = std::integral_constant<Mode, PROBE>;
+  using RepeatT = std::integral_constant<Mode, REPEAT>;
+  // Sum of a row over its threads, and whether the row left the range.  Any probability of 2^90 or
+  // more shows in the sum: the sums only ever grow, and an overflowed one is infinite or not a number.
+  // At or below 2^-90 the row's scores lie so far below zero that the small terms were flushed away.
+  // The threads of the row decide the same (an infinity stands for a thread's own flag).
+  auto row_sum = [&](bool& flag) -> float {
+    const float l = sum_partials(ls2);
+    float seen = !(l < DANGER) || poly_abs > 120.f ? INFINITY : l;
+    const float other = exchange(seen);
+    seen += other;
+    flag = !(seen < DANGER) || !(seen > TINY);
+    return l + other;            // used only where nothing was flagged
+  };
+  // The accumulator is final once the item's last product has finished: normalise and store.
+  auto finish = [&](const Item& it, float l_row) {
+    ok = mbar_wait_warp(&pv_done[tile], pv_ph, abort_flag);
+    pv_ph ^= 1;
+    if (!ok) return;
+    tc_fence_after();
+    const int row = it.row0 + tile * BM + r;
+    const float inv_l = 1.f / l_row;
+    __nv_bfloat16* orow =
+        p.o + ((size_t)it.b * p.rows + row) * ((size_t)p.heads * DH) + (size_t)it.h * DH + half * (DH / TPR);
+#pragma unroll 1
+    for (int ch = 0; ch < DH / TPR / 32; ++ch) {
+      uint32_t o[32];
+      tmem_ld32(o_tmem + ch * 32, o);
+      tmem_ld_wait_on(o);
+      if (row < p.rows) {
+        uint4* dst = reinterpret_cast<uint4*>(orow + ch * 32);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          dst[q] = make_uint4(pack_bf16x2(__uint_as_float(o[8 * q + 0]) * inv_l, __uint_as_float(o[8 * q + 1]) * inv_l),
+                              pack_bf16x2(__uint_as_float(o[8 * q + 2]) * inv_l, __uint_as_float(o[8 * q + 3]) * inv_l),
+                              pack_bf16x2(__uint_as_float(o[8 * q + 4]) * inv_l, __uint_as_float(o[8 * q + 5]) * inv_l),
+                              pack_bf16x2(__uint_as_float(o[8 * q + 6]) * inv_l, __uint_as_float(o[8 * q + 7]) * inv_l));
       }
     }
-    if (ok) {
-      ok = mbar_wait(&pv_done[(n_kv - 1) & 1], (uint32_t)((n_kv - 1) >> 1) & 1u, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
-    }
-    if (ok) {
-      tc_fence_after();
-      const int row = qt * ATT_BM + r;
-      const float inv_l = 1.f / l_run;
-      __nv_bfloat16* orow = p.o + ((size_t)b * p.rows + row) * ((size_t)p.heads * DH) + (size_t)h * DH;
+    tc_fence_before();     // ordered before this thread's next hand-over, after which O is overwritten
+    if (p.lse && half == 0 && row < p.rows)
+      p.lse[((size_t)it.b * p.heads + it.h) * p.rows + row] = fmaf(m_ref, 0.6931471805599453f, logf(l_row));
+  };
+
+  // All threads meet after the first pass and agree on whether there is a second.
+  auto second_pass = [&]() -> bool {
+    tc_fence_before();
+    const bool go = named_barrier_and(0, THREADS, ok && !*abort_flag) && *any_flag;
+    tc_fence_after();
+    return go;
+  };
+  // Calls f(item) for every item of this CTA with a row that left the range.
+  auto for_flagged = [&](auto f) {
 #pragma unroll 1
-      for (int ch = 0; ch < DH / 32; ++ch) {
-        uint32_t o[32];
-        tmem_ld32(tmem_o + lane_sel + ch * 32, o);
-        tmem_ld_wait();
-        if (row < p.rows) {
-          uint4* dst = reinterpret_cast<uint4*>(orow + ch * 32);
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            dst[q] = make_uint4(pack_bf16x2(__uint_as_float(o[8 * q + 0]) * inv_l, __uint_as_float(o[8 * q + 1]) * inv_l),
-                                pack_bf16x2(__uint_as_float(o[8 * q + 2]) * inv_l, __uint_as_float(o[8 * q + 3]) * inv_l),
-                                pack_bf16x2(__uint_as_float(o[8 * q + 4]) * inv_l, __uint_as_float(o[8 * q + 5]) * inv_l),
-                                pack_bf16x2(__uint_as_float(o[8 * q + 6]) * inv_l, __uint_as_float(o[8 * q + 7]) * inv_l));
+    for (int i = 0; i < n_items; ++i) {
+      const uint32_t word = ((volatile uint32_t*)item_flag)[i >> 5];
+      if (word >> (i & 31) & 1) f(item_at(i));
+    }
+  };
+
+  // First pass over the CTA's items, then the flagged ones once more in two sweeps.
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_HELPER));
+    if (warp == 0) {
+      if (lane == 0)
+        for (int i = 0; ok && i < n_items; ++i) produce(item_at(i), true);
+      __syncwarp();
+      const bool again = second_pass();
+      if (lane == 0) {
+        if (again)
+          for_flagged([&](const Item& it) {
+#pragma unroll 1
+            for (int with_v = 0; ok && with_v < 2; ++with_v) produce(it, with_v != 0);
+          });
+        if (!ok) {
+          // gave up: let the copies already issued land before the CTA leaves (the latest fill of
+          // each stage; older fills were consumed before their stage was reused)
+          auto drain = [&](uint64_t* full, int issued, int stages) {
+            for (int i = max(0, issued - stages); i < issued; ++i) {
+              volatile uint32_t dummy = 0;
+              mbar_wait(&full[i % stages], (uint32_t)(i / stages) & 1u, &dummy);
+            }
+          };
+          drain(q_full, q_issued, QBUF);
+          drain(k_full, k_issued, KS);
+          drain(v_full, v_issued, VS);
         }
       }
-      if (p.lse && row < p.rows)
-        p.lse[((size_t)b * p.heads + h) * p.rows + row] = fmaf(m_run, p.scale, logf(l_run));
+      __syncwarp();
+    } else if (warp <= C::ISSUERS) {
+      auto issue = [&](const Item& it, Mode mode) {
+        if (C::ALIAS) {
+          if (mode == PROBE) issue_scores(it);
+          else issue_both(it);
+        } else if (warp == 1) {
+          issue_scores(it);
+        } else if (mode != PROBE) {
+          issue_products(it);
+        }
+      };
+      // one call site for all sweeps (the loops keep to the helper warps' registers)
+      bool again = false;
+      Mode mode = PASS;
+      for (int i = 0;;) {
+        if (again)
+          while (i < n_items && !(((volatile uint32_t*)item_flag)[i >> 5] >> (i & 31) & 1)) ++i;
+        if (!ok || i >= n_items) {
+          if (again || !second_pass()) break;
+          again = true;
+          mode = PROBE;
+          i = 0;
+          continue;
+        }
+        issue(item_at(i), mode);
+        if (mode == PROBE) {
+          mode = REPEAT;
+        } else {
+          ++i;
+          if (again) mode = PROBE;
+        }
+      }
+    } else {
+      second_pass();
     }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_SOFTMAX));
+    // With q and k out of an RMSNorm (gains g), a rotation and, for q, the factor
+    // log2(e) / sqrt(dh), a head of q has norm <= max|g_q| * log2(e) and a head of k norm <=
+    // sqrt(dh) * max|g_k|: every score lies within +-log2(e) * sqrt(dh) * max|g_q| * max|g_k|
+    // (plus the bf16 roundings, under half a percent).  Far inside the polynomial's range nothing
+    // needs to be tracked per score.
+    bool bounded = false;
+    if (!SCALED && p.gain_q && p.gain_k) {
+      const int ts = threadIdx.x - 128;
+      if (ts < DH) {
+        atomicMax(&gain_max[0], __float_as_uint(fabsf(__bfloat162float(p.gain_q[ts]))));
+        atomicMax(&gain_max[1], __float_as_uint(fabsf(__bfloat162float(p.gain_k[ts]))));
+      }
+      named_barrier(1, SOFTMAX_THREADS);
+      const float gq = __uint_as_float(*(volatile uint32_t*)&gain_max[0]);
+      const float gk = __uint_as_float(*(volatile uint32_t*)&gain_max[1]);
+      constexpr float factor = (DH == 64 ? 11.55f : 16.33f) * 1.01f;
+      bounded = gq * gk * factor < 100.f;    // false for a NaN gain
+    }
+    for (int i = 0; i < n_items; ++i) {
+      const Item it = item_at(i);
+      if (!tile_live(it, tile)) continue;
+      if (ok) {
+        if (bounded) run_blocks(PassT{}, std::false_type{});
+        else run_blocks(PassT{}, std::true_type{});
+      }
+      agree();
+      if (!ok) break;
+      bool flag;
+      const float l = row_sum(flag);
+      if (flag) {
+        *any_flag = 1;
+        atomicOr(&item_flag[i >> 5], 1u << (i & 31));
+      }
+      finish(it, l);
+    }
+    if (second_pass())
+      for_flagged([&](const Item& it) {
+        if (!tile_live(it, tile)) return;
+        bool flag = false;
+        m_true = -INFINITY;
+        if (ok) run_blocks(ProbeT{}, std::true_type{});
+        agree();
+        if (!ok) return;
+        row_sum(flag);
+        m_true = fmaxf(m_true, exchange(m_true));
+        m_ref = flag ? m_true : 0.f;
+        run_blocks(RepeatT{}, std::false_type{});
+        agree();
+        if (!ok) return;
+        finish(it, row_sum(flag));
+        m_ref = 0.f;
+      });
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
+    tmem_dealloc(tmem_base, 512);
   }
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
 }
 
-template <int DH>
-static int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
-  using Cfg = AttnCfg<DH>;
+template <int DH, bool SCALED>
+int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
+  using C = Cfg<DH>;
   static PerDeviceInt attr_done;
-  auto kern = attention_kernel<DH>;
-  if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
+  auto kern = attention_kernel<DH, SCALED>;
+  if (int rc = ensure_smem_attr(kern, C::SMEM_BYTES, attr_done)) return rc;
   AttnParams p;
   p.o = (__nv_bfloat16*)a.o;
   p.lse = a.lse;
@@ -411,17 +783,31 @@ static int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool cha
   p.rows = a.rows;
   p.keys = a.keys;
   p.heads = a.heads;
-  p.scale_log2 = a.q_scale;                         // scores times this = exponents to base 2
-  p.scale = a.q_scale * 0.6931471805599453f;        // ... and times this = natural exponents (for lse)
+  p.q_scale = a.q_scale;
   p.status = a.status;
-  dim3 grid((a.rows + ATT_BM - 1) / ATT_BM, a.heads, a.batch);
-  return launch_kernel(kern, grid, ATT_THREADS, Cfg::SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
+  p.gain_q = (const __nv_bfloat16*)a.gain_q;
+  p.gain_k = (const __nv_bfloat16*)a.gain_k;
+  const long long q_tiles = (a.rows + BM - 1) / BM, bh = (long long)a.heads * a.batch;
+  // two tiles per item share their K and V blocks; where every tile can have an SM of its own they
+  // are faster apart
+  p.tiles = q_tiles * bh <= sm_count() ? 1 : TILES;
+  p.q_items = (int)((q_tiles + p.tiles - 1) / p.tiles);
+  const long long items = p.q_items * bh;
+  if (items > (1ll << 30)) return XEMA_EINVAL;
+  p.items = (int)items;
+  // one CTA per SM (each takes all of TMEM); more only where a CTA could not keep a flag per item
+  const int grid = std::max((int)std::min<long long>(items, sm_count()), (int)((items + MAX_ITEMS - 1) / MAX_ITEMS));
+  return launch_kernel(kern, dim3(grid), THREADS, C::SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
 }
+}  // namespace
 
 int launch_attention(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   if (a.rows == 0 || a.batch == 0) return XEMA_OK;
-  if (a.head_dim == 64) return launch_attention_dh64(a, stream, chained);
-  if (a.head_dim == 128) return launch_attention_t<128>(a, stream, chained);
+  const bool scaled = a.q_scale != 1.f;
+  if (a.head_dim == 64)
+    return scaled ? launch_attention_t<64, true>(a, stream, chained) : launch_attention_t<64, false>(a, stream, chained);
+  if (a.head_dim == 128)
+    return scaled ? launch_attention_t<128, true>(a, stream, chained) : launch_attention_t<128, false>(a, stream, chained);
   return XEMA_EINVAL;
 }
 
@@ -435,13 +821,11 @@ int attn_prepare(AttnLaunch* a, const void* q, long long ldq, long long q_batch_
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
   if (mis(q) || mis(k) || mis(v) || mis(a->o)) return XEMA_EALIGN;
   const long long width = (long long)a->heads * a->head_dim;
-  int rc = encode_tmap_bf16(&a->map_q, q, width, a->rows > 0 ? a->rows : 1, a->batch, ldq, q_batch_rows, ATT_BM);
+  int rc = encode_tmap_bf16(&a->map_q, q, width, a->rows > 0 ? a->rows : 1, a->batch, ldq, q_batch_rows, BM);
   if (rc) return rc;
-  // keys per block (= rows of a K/V box): 128 in the head_dim 64 kernel, 64 in the general one
-  const int kv_box = (a->head_dim == 64) ? kAttnDh64KeysPerBlock : ATT_BN;
-  rc = encode_tmap_bf16(&a->map_k, k, width, a->keys, a->batch, ldkv, kv_batch_rows, kv_box);
+  rc = encode_tmap_bf16(&a->map_k, k, width, a->keys, a->batch, ldkv, kv_batch_rows, BN);
   if (rc) return rc;
-  return encode_tmap_bf16(&a->map_v, v, width, a->keys, a->batch, ldkv, kv_batch_rows, kv_box);
+  return encode_tmap_bf16(&a->map_v, v, width, a->keys, a->batch, ldkv, kv_batch_rows, BN);
 }
 
 }  // namespace xema

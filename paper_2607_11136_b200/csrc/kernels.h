@@ -143,7 +143,6 @@ struct AttnLaunch {
 int attn_prepare(AttnLaunch* a, const void* q, long long ldq, long long q_batch_rows, const void* k, const void* v,
                  long long ldkv, long long kv_batch_rows);
 int launch_attention(const AttnLaunch& a, cudaStream_t stream, bool chained = false);
-int launch_attention_dh64(const AttnLaunch& a, cudaStream_t stream, bool chained);   // two-tile kernel for head_dim 64
-constexpr int kAttnDh64KeysPerBlock = 128;                             // rows of its K/V TMA boxes
+constexpr int kAttnKeysPerBlock = 128;   // rows of the K/V TMA boxes
 
 }  // namespace xema

@@ -279,6 +279,74 @@ def test_attention(B, rows, keys, H, dh):
     assert np.abs(got_l - ref_l).max() < 2e-3
 
 
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("rows,keys", [(1, 1), (127, 64), (128, 65), (129, 127), (256, 129), (257, 511), (33, 512), (300, 513)])
+def test_attention_edges(rows, keys, dh):
+    """Rows and keys at the edges of 32-row warps, 128-row tiles, two-tile items, 64-key halves and
+    128-key blocks, on both sides of the block count from which whole blocks run without masking.
+    Tolerances as in test_attention."""
+    rng = np.random.default_rng(700 + rows + keys)
+    got_o, ref_o, got_l, ref_l = _attention_case(rng, 2, rows, keys, 3, dh)
+    assert_bf16_close(got_o, ref_o, ("attention edges", rows, keys, dh), atol_rms=1.5e-2, cos=0.9999)
+    assert np.abs(got_l - ref_l).max() < 2e-3
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+def test_attention_items_of_one_cta_with_flagged_rows(dh):
+    """More work items than SMs, so that CTAs run several; the scores of a few heads lie near +-260 (in
+    exponents to base 2), so first and later items of some CTAs have to be repeated against their rows'
+    maxima while the other items keep their results.  Tolerances as in
+    test_attention_dh64_scores_far_from_zero (lse relative to its size)."""
+    rng = np.random.default_rng(93 + dh)
+    rows, keys, H = 130, 300, 170
+    D = H * dh
+    far = {3: 260.0, 20: -260.0, 151: 260.0, 168: -260.0}
+    q = rng.standard_normal((1, rows, D))
+    kv = rng.standard_normal((1, keys, 2 * D))
+    u = np.ones(dh) / math.sqrt(dh)
+    a = 30.0
+    for h, offset in far.items():
+        c = slice(h * dh, (h + 1) * dh)
+        q[0, :, c] = a * u + 0.3 * rng.standard_normal((rows, dh))
+        kv[0, :, c] = offset * math.sqrt(dh) / 1.4426950408889634 / a * u + 0.3 * rng.standard_normal((keys, dh))
+    (qb, qf), kvb = _exponent_units(q, dh), bf16_bits(kv.astype(np.float32))
+    kvf = bits_to_f64(kvb)
+    q_dev, kv_dev = to_dev(qb), to_dev(kvb)
+    o = torch.zeros(1, rows, D, dtype=torch.int16, device=DEV)
+    lse = torch.zeros(1, H, rows, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    xb.xema_op_attention(q_dev.data_ptr(), D, rows, kv_dev.data_ptr(), kv_dev.data_ptr() + D * 2, 2 * D, keys,
+                         o.data_ptr(), lse.data_ptr(), 1, rows, keys, H, dh, status=status.data_ptr(), q_scale=1.0)
+    _sync_status(status)
+    got = from_dev_bf16(o)
+    for h in sorted(set(far) | {0, 2, 4, 19, 21, 147, 148, 150, 152, 167, 169}):
+        c = slice(h * dh, (h + 1) * dh)
+        ref_o, ref_l = ob.attention_head(qf[0, :, c], kvf[0, :, c], kvf[0, :, D + h * dh:D + (h + 1) * dh], 1 / math.sqrt(dh))
+        assert_bf16_close(got[0, :, c], ref_o, ("flagged items", dh, h), atol_rms=2.5e-2, cos=0.9998)
+        assert np.abs(lse.cpu().numpy()[0, h] - ref_l).max() < 2e-3 * max(1.0, np.abs(ref_l).max() / 10)
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+def test_attention_rows_do_not_depend_on_tiles_per_item(dh):
+    """500 rows of 60 heads run as items of two tiles, 211 of them as items of one: the same bits."""
+    rng = np.random.default_rng(94)
+    rows, keys, H = 500, 700, 60
+    D = H * dh
+    q_dev, kv_dev = to_dev(_exponent_units(rng.standard_normal((1, rows, D)), dh)[0]), to_dev(rand_bf16(rng, (1, keys, 2 * D))[0])
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+    def run(r0, n):
+        o = torch.zeros(n, D, dtype=torch.int16, device=DEV)
+        lse = torch.zeros(H, n, dtype=torch.float32, device=DEV)
+        xb.xema_op_attention(q_dev.data_ptr() + r0 * D * 2, D, n, kv_dev.data_ptr(), kv_dev.data_ptr() + D * 2, 2 * D, keys,
+                             o.data_ptr(), lse.data_ptr(), 1, n, keys, H, dh, status=status.data_ptr(), q_scale=1.0)
+        return o, lse
+
+    (o_all, l_all), (o_part, l_part) = run(0, rows), run(167, 211)
+    _sync_status(status)
+    assert torch.equal(o_all[167:167 + 211], o_part) and torch.equal(l_all[:, 167:167 + 211], l_part)
+
+
 def test_attention_peaked_scores():
     """Large |q| makes the softmax peaked and moves the running max by more than the lazy
     threshold between key blocks, so the O rescale path runs."""
