@@ -42,7 +42,7 @@
 // Measured (B200, inside the block): dh 64, 4444 x 17776 x 48 heads 933 us (with one CTA per 256 rows and code
 // copies for first and last blocks 970); power-capped 17776-token block 7.28 ms against 7.52.  dh 128, 17776 x
 // 17776 x 24 heads 3.03 ms = 1280 TFLOP/s (one tile per CTA, two CTAs per SM, 64-key blocks, running maximum: 3.40),
-// 4608 x 4608 x 24 heads 232 us (261).  288 x 288 x 8 heads 10.4 us (14.4), launches back to back.
+// 4608 x 4608 x 24 heads 228 us (261).  288 x 288 x 8 heads 10.4 us (14.4), launches back to back.
 //
 // Every decision is per row and keys are always visited in the same order, so a row's bits do not
 // depend on how rows are tiled or chunked.
@@ -78,10 +78,11 @@ static_assert(128 * REG_HELPER + SOFTMAX_THREADS * REG_SOFTMAX <= THREADS * 96, 
 // others use the MUFU.  Without any the MUFU sets the pace, with too many the issue slots do, and where
 // they stand decides how well the compiler interleaves the two pipes.  Measured inside the block (scores
 // bounded, see below) over 125 placements of 6 to 17 bits: dh 64, 4444 x 17776 x 48 heads 933 to 1177 us (this
-// one 933, the next best 945; 9 bits 1000 and more), dh 128, 4608 x 4608 x 24 heads 232 to 247 us (this one 232).
+// one 933, the next best 945; 9 bits 1000 and more), dh 128, 4608 x 4608 x 24 heads 232 to 247 us (this one within
+// one percent of the fastest).
 // Power-capped, the dh 64 block of 17776 tokens takes 7.28 ms with this placement, 7.39-7.56 with three others.
 template <int DH>
-constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0xa2898818u;
+constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0x22440924u;
 static_assert(BN == 128 && BM == 128, "the kernel is written for 128-key blocks of 128-row tiles");
 
 template <int DH>
@@ -183,6 +184,23 @@ __device__ __forceinline__ float sum_partials(const f32x2 (&ls2)[4]) {
 }
 __device__ __forceinline__ void ld_scores(uint32_t addr, float (&s)[CH]) { tmem_ld16(addr, *reinterpret_cast<uint32_t(*)[CH]>(&s[0])); }
 __device__ __forceinline__ void wait_scores(float (&s)[CH]) { tmem_ld_wait_on(*reinterpret_cast<uint32_t(*)[CH]>(&s[0])); }
+
+__device__ __forceinline__ uint4 shfl_xor_u4(uint4 v, int m) {
+  return make_uint4(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m),
+                    __shfl_xor_sync(0xffffffffu, v.z, m), __shfl_xor_sync(0xffffffffu, v.w, m));
+}
+// c[k] of lane i in every group of four lanes <- c[i] of the group's lane k
+__device__ __forceinline__ void transpose_4x4(uint4 (&c)[4], int lane) {
+  const bool odd = lane & 1, high = lane & 2;
+  const uint4 ra = shfl_xor_u4(odd ? c[0] : c[1], 1), rb = shfl_xor_u4(odd ? c[2] : c[3], 1);
+  const uint4 a0 = odd ? ra : c[0], a1 = odd ? c[1] : ra;     // column (lane & 1) of the pair's two rows
+  const uint4 b0 = odd ? rb : c[2], b1 = odd ? c[3] : rb;     // column (lane & 1) + 2
+  const uint4 r0 = shfl_xor_u4(high ? a0 : b0, 2), r1 = shfl_xor_u4(high ? a1 : b1, 2);
+  c[0] = high ? r0 : a0;
+  c[1] = high ? r1 : a1;
+  c[2] = high ? b0 : r0;
+  c[3] = high ? b1 : r1;
+}
 
 // Sweeps of one item: the pass itself; the scores only (flags and true maxima); the repeat.
 enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
@@ -603,21 +621,35 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     tc_fence_after();
     const int row = it.row0 + tile * BM + r;
     const float inv_l = 1.f / l_row;
-    __nv_bfloat16* orow =
-        p.o + ((size_t)it.b * p.rows + row) * ((size_t)p.heads * DH) + (size_t)it.h * DH + half * (DH / TPR);
+    // dh 128: four lanes hold 64 bytes of four rows; transposed among themselves, a store covers whole
+    // 64-byte pieces of eight rows instead of 16 bytes of 32, which keeps the load/store unit busy for
+    // 4000 cycles an item (4608 x 4608 x 24 heads 232 -> 228 us).  The dh 64 kernel gains the same on its
+    // short calls (1101 keys 22.4 -> 21.3 us) but its main loop then comes out 2-4 % slower, so it keeps the
+    // plain stores.
+    constexpr bool TRANSPOSE = DH == 128;
+    const int first_row = TRANSPOSE ? row & ~3 : row;
+    __nv_bfloat16* orow = p.o + ((size_t)it.b * p.rows + first_row) * ((size_t)p.heads * DH) + (size_t)it.h * DH +
+                          half * (DH / TPR) + (TRANSPOSE ? (lane & 3) * 8 : 0);
 #pragma unroll 1
     for (int ch = 0; ch < DH / TPR / 32; ++ch) {
       uint32_t o[32];
       tmem_ld32(o_tmem + ch * 32, o);
       tmem_ld_wait_on(o);
-      if (row < p.rows) {
-        uint4* dst = reinterpret_cast<uint4*>(orow + ch * 32);
+      uint4 c[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          dst[q] = make_uint4(pack_bf16x2(__uint_as_float(o[8 * q + 0]) * inv_l, __uint_as_float(o[8 * q + 1]) * inv_l),
-                              pack_bf16x2(__uint_as_float(o[8 * q + 2]) * inv_l, __uint_as_float(o[8 * q + 3]) * inv_l),
-                              pack_bf16x2(__uint_as_float(o[8 * q + 4]) * inv_l, __uint_as_float(o[8 * q + 5]) * inv_l),
-                              pack_bf16x2(__uint_as_float(o[8 * q + 6]) * inv_l, __uint_as_float(o[8 * q + 7]) * inv_l));
+      for (int q = 0; q < 4; ++q)
+        c[q] = make_uint4(pack_bf16x2(__uint_as_float(o[8 * q + 0]) * inv_l, __uint_as_float(o[8 * q + 1]) * inv_l),
+                          pack_bf16x2(__uint_as_float(o[8 * q + 2]) * inv_l, __uint_as_float(o[8 * q + 3]) * inv_l),
+                          pack_bf16x2(__uint_as_float(o[8 * q + 4]) * inv_l, __uint_as_float(o[8 * q + 5]) * inv_l),
+                          pack_bf16x2(__uint_as_float(o[8 * q + 6]) * inv_l, __uint_as_float(o[8 * q + 7]) * inv_l));
+      if (TRANSPOSE) {
+        transpose_4x4(c, lane);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (first_row + k < p.rows) *reinterpret_cast<uint4*>(orow + (size_t)k * p.heads * DH + ch * 32) = c[k];
+      } else if (row < p.rows) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) reinterpret_cast<uint4*>(orow + ch * 32)[k] = c[k];
       }
     }
     tc_fence_before();     // ordered before this thread's next hand-over, after which O is overwritten

@@ -25,48 +25,76 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // ---------------------------------------------------------------------------------------
 // mod[b, j] = sum_k silu(temb[b,k]) * w[j,k] + bias[j]
-// One warp per output feature j; silu(temb) for all batch elements sits in shared memory.
+// A warp takes kModRows output features at once: their weight rows are requested together, for up to
+// 512 inputs before the wait for earlier launches (the weights do not depend on them); silu(temb) for
+// all batch elements sits in shared memory.  Bound by the latency of one trip to HBM for one batch
+// element, by the reductions (five shuffles per feature and batch element) for several.
 // ---------------------------------------------------------------------------------------
 constexpr int kModWarps = 8;
-constexpr int kModMaxBatch = 8;
+constexpr int kModRows = 4;
+constexpr int kModMaxBatch = 4;     // batch elements per pass over the weights
 
 __global__ void __launch_bounds__(kModWarps * 32)
-mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w,
-                const __nv_bfloat16* __restrict__ bias, float* mod, int batch, int Dt, int n_out) {
+mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, const __nv_bfloat16* __restrict__ bias,
+                float* mod, int batch, int Dt, int n_out) {
   extern __shared__ float s_e[];  // [batch][Dt]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j0 = (blockIdx.x * kModWarps + warp) * kModRows;
+  const int n8 = Dt / 8;
+  auto weights = [&](int r, int k8) {
+    return (j0 + r < n_out && k8 < n8) ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)(j0 + r) * Dt) + k8)
+                                       : make_uint4(0u, 0u, 0u, 0u);
+  };
+  uint4 first[2][kModRows];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int r = 0; r < kModRows; ++r) first[u][r] = weights(r, u * 32 + lane);
   grid_dep_launch();
   grid_dep_wait();
   for (int i = threadIdx.x; i < batch * Dt; i += blockDim.x) {
-    float z = __bfloat162float(temb[i]);
+    const float z = __bfloat162float(*(const volatile __nv_bfloat16*)(temb + i));
     s_e[i] = z / (1.f + __expf(-z));
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = blockIdx.x * kModWarps + warp; j < n_out; j += gridDim.x * kModWarps) {
-    const uint4* wr = reinterpret_cast<const uint4*>(w + (size_t)j * Dt);
-    for (int b0 = 0; b0 < batch; b0 += kModMaxBatch) {
-      float acc[kModMaxBatch];
+  for (int b0 = 0; b0 < batch; b0 += kModMaxBatch) {
+    float acc[kModRows][kModMaxBatch];
 #pragma unroll
-      for (int b = 0; b < kModMaxBatch; ++b) acc[b] = 0.f;
-      for (int k8 = lane; k8 * 8 < Dt; k8 += 32) {
-        uint4 v = __ldg(wr + k8);
-        float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y),
-                      bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
+    for (int r = 0; r < kModRows; ++r)
 #pragma unroll
-        for (int b = 0; b < kModMaxBatch; ++b) {
-          if (b0 + b < batch) {
-            const float* e = s_e + (size_t)(b0 + b) * Dt + k8 * 8;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) acc[b] = fmaf(f[t], e[t], acc[b]);
-          }
-        }
-      }
+      for (int b = 0; b < kModMaxBatch; ++b) acc[r][b] = 0.f;
+    auto add = [&](const uint4 (&v)[kModRows], int k8) {
 #pragma unroll
       for (int b = 0; b < kModMaxBatch; ++b) {
-        if (b0 + b < batch) {
-          float s = warp_sum(acc[b]);
-          if (lane == 0) mod[(size_t)(b0 + b) * n_out + j] = s + __bfloat162float(bias[j]);
+        if (b0 + b >= batch || k8 >= n8) continue;
+        const float4 e0 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * Dt + k8 * 8);
+        const float4 e1 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * Dt + k8 * 8 + 4);
+#pragma unroll
+        for (int r = 0; r < kModRows; ++r) {
+          float a = acc[r][b];
+          a = fmaf(bf16_lo(v[r].x), e0.x, a); a = fmaf(bf16_hi(v[r].x), e0.y, a);
+          a = fmaf(bf16_lo(v[r].y), e0.z, a); a = fmaf(bf16_hi(v[r].y), e0.w, a);
+          a = fmaf(bf16_lo(v[r].z), e1.x, a); a = fmaf(bf16_hi(v[r].z), e1.y, a);
+          a = fmaf(bf16_lo(v[r].w), e1.z, a); a = fmaf(bf16_hi(v[r].w), e1.w, a);
+          acc[r][b] = a;
         }
+      }
+    };
+    add(first[0], lane);
+    add(first[1], 32 + lane);
+    for (int k8 = 64 + lane; k8 < n8; k8 += 32) {
+      uint4 v[kModRows];
+#pragma unroll
+      for (int r = 0; r < kModRows; ++r) v[r] = weights(r, k8);
+      add(v, k8);
+    }
+#pragma unroll
+    for (int b = 0; b < kModMaxBatch; ++b) {
+      if (b0 + b >= batch) continue;
+#pragma unroll
+      for (int r = 0; r < kModRows; ++r) {
+        const float sum = warp_sum(acc[r][b]);
+        if (lane == r && j0 + r < n_out) mod[(size_t)(b0 + b) * n_out + j0 + r] = sum + __bfloat162float(bias[j0 + r]);
       }
     }
   }
@@ -77,7 +105,7 @@ int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mo
   if (batch < 1 || Dt < 8 || (Dt & 7) || n_out < 1) return XEMA_EINVAL;
   size_t smem = (size_t)batch * Dt * sizeof(float);
   if (smem > 48 * 1024) return XEMA_EINVAL;
-  int blocks = (n_out + kModWarps - 1) / kModWarps;
+  const int blocks = (n_out + kModWarps * kModRows - 1) / (kModWarps * kModRows);
   return launch_kernel(mod_gemv_kernel, dim3(blocks), kModWarps * 32, smem, stream, chained, (const __nv_bfloat16*)temb,
                        (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
 }

@@ -501,6 +501,7 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       const uint8_t* hid_pc = hid + at_row(pc, D, 2);
       const uint8_t* kv_b = kv + pc.b0 * S_all * 2 * D * 2;      // keys and values of these batch elements
       ln_op(hid_pc, 0, h1b, pc, 1, "LN1B", ci);
+      bool q_follows_kv = false;      // no launch between KV and Q, both reading LN1A's output
       // With one piece in both phases LN1B recomputes what LN1A wrote.  When the layout put h1b
       // at h1a's address and nothing was born in between (KROPE allocates nothing, so the only
       // births since the KV op are h1b's own), those bytes are still there: the launch is elided.
@@ -519,6 +520,7 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
         }
         if (untouched && ta.bytes == tb.bytes) {
           plan->ops.back().kind = OP_FUSED;
+          q_follows_kv = true;
           plan->ops.back().flops = 0.0;
           plan->ops.back().bytes = 0.0;
         }
@@ -526,6 +528,11 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       int rc = gemm_op(h1b, D, n, w_qkv, D, b_qkv, q, D, n, nullptr, 0, 0, nullptr, pc, (int)D, (int)D,
                        XEMA_EPI_BIAS_NORM_ROPE, "Q", ci, w.g_q, (int)D, (int)(row0 + pc.r0), q_scale);
       if (rc) return rc;
+      if (q_follows_kv) {
+        // ops: ..., KV, KROPE (fused), LN1B (elided), Q
+        plan->ops[plan->ops.size() - 4].gemm.late_trigger = 1;
+        plan->ops.back().gemm.early_input = 1;
+      }
       Op o{};
       o.kind = OP_FUSED;
       tag(o, "QROPE", ci, 0.0, 0.0);

@@ -2,6 +2,7 @@
 table; the library gets raw pointers.  No arithmetic of the block happens here."""
 from __future__ import annotations
 
+import math
 from typing import Optional, Sequence
 
 import numpy as np
@@ -85,10 +86,11 @@ class BlockSession:
         self.plan.bind(self.arena.data_ptr(), self.arena.numel(), ptrs, self.rope.data_ptr(), self.status.data_ptr())
         self.seq_all = template.s_text + template.grid_t * template.grid_h * template.grid_w
         self.seq = self.plan.rows          # token rows of this session's tensors (all of them unless sharded)
-        hid = (template.batch, self.seq, template.hidden)
-        self._hid_in = self.view("hid0", torch.int16, hid)
-        self._temb = self.view("temb", torch.int16, (template.batch, template.temb_dim))
-        self._hid_out = self.view("hid%d" % template.n_blocks, torch.int16, hid)
+        self._hid_shape = (template.batch, self.seq, template.hidden)
+        self._temb_shape = (template.batch, template.temb_dim)
+        self._views = {}
+        self._out_name = "hid%d" % template.n_blocks
+        self._index = self.arena.get_device()
 
     # ---- views into the arena ---------------------------------------------------------
     def view(self, name: str, dtype=torch.int16, shape=None) -> torch.Tensor:
@@ -101,34 +103,41 @@ class BlockSession:
 
     # The plan's addresses never change, so the views of the inputs and the output are made once
     # (making one takes several microseconds, on a path that small blocks run in tens of them).
+    def _view_once(self, name: str, shape) -> torch.Tensor:
+        v = self._views.get(name)
+        if v is None:
+            v = self._views[name] = self.view(name, torch.int16, shape)
+        return v
+
     def hid_in(self) -> torch.Tensor:
-        return self._hid_in
+        return self._view_once("hid0", self._hid_shape)
 
     def temb(self) -> torch.Tensor:
-        return self._temb
+        return self._view_once("temb", self._temb_shape)
 
     def hid_out(self) -> torch.Tensor:
-        return self._hid_out
+        return self._view_once(self._out_name, self._hid_shape)
 
     # ---- data movement ------------------------------------------------------------------
-    def _in_place(self, src, dst) -> bool:
+    def _in_place(self, src, shape) -> bool:
         """Whether the library can copy `src` as it stands."""
-        return (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.device == dst.device
-                and src.numel() == dst.numel() and src.is_contiguous() and torch._C._cuda_getDevice() == dst.get_device())
+        return (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.get_device() == self._index
+                and src.numel() == math.prod(shape) and src.is_contiguous())
 
     def set_inputs(self, x_bits, temb_bits, non_blocking: bool = False):
         """x_bits / temb_bits: uint16 numpy arrays or int16 torch tensors (host or device)."""
-        if self._in_place(x_bits, self._hid_in) and self._in_place(temb_bits, self._temb):
+        if (self._in_place(x_bits, self._hid_shape) and self._in_place(temb_bits, self._temb_shape)
+                and torch._C._cuda_getDevice() == self._index):
             self.plan.set_inputs(x_bits.data_ptr(), temb_bits.data_ptr(), self._raw_stream())
             return
-        for dst, src in ((self._hid_in, x_bits), (self._temb, temb_bits)):
+        for dst, src in ((self.hid_in(), x_bits), (self.temb(), temb_bits)):
             if isinstance(src, np.ndarray):
                 src = torch.from_numpy(np.ascontiguousarray(src).view(np.int16))
             dst.copy_(src.view(dst.shape), non_blocking=non_blocking)
 
     def _raw_stream(self) -> int:
         """The current stream of the session's device as an address."""
-        return torch._C._cuda_getCurrentRawStream(self._hid_in.get_device())
+        return torch._C._cuda_getCurrentRawStream(self._index)
 
     def forward(self, stream: Optional[torch.cuda.Stream] = None):
         s = stream.cuda_stream if stream is not None else self._raw_stream()
