@@ -785,6 +785,11 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
   if (mis(a) || mis(w) || mis(g->bias) || mis(g->out) || (g->resid && mis(g->resid)) || (g->gate && mis(g->gate)))
     return XEMA_EALIGN;
+  g->a = a;
+  g->w = w;
+  g->lda = lda;
+  g->a_batch_rows = a_batch_rows;
+  g->ldw = ldw;
   g->block_n = pick_tile(*g);
   const long long rows = g->rows > 0 ? g->rows : 1;
   int rc = encode_tmap_bf16(&g->map_a, a, g->K, rows, g->batch, lda, a_batch_rows, BM);

@@ -108,6 +108,8 @@ struct GemmLaunch {
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K, epilogue, block_n;
+  const void *a, *w;   // operands as given to gemm_prepare
+  long long lda, a_batch_rows, ldw;
   unsigned int* status;
   // Two launches in a row that read the same input (KV and Q): the first lets the next one start only
   // after its own wait (late_trigger), that is with the input complete; the second, when chained to it,

@@ -131,6 +131,14 @@ struct Op {
   AttnLaunch attn;
 };
 
+// One step of xema_forward_host: a launch, or the arrival / departure of a piece of the block input /
+// output (`rows` x `width` bytes at byte offset `offset` of the tensor, rows `pitch` apart).
+struct HostStep {
+  enum Kind { LAUNCH, COPY_IN, COPY_OUT } kind;
+  Op op;
+  size_t offset, width, rows, pitch;
+};
+
 }  // namespace xema
 
 using namespace xema;
@@ -152,9 +160,11 @@ struct xema_plan {
   long long own_rows; // token rows of the plan's shard
   const float* rope;
   std::vector<Op> ops;
-  // xema_forward_host: a second stream and one event per piece of the first and last phase, so
-  // that the copies of one piece overlap the launches of its neighbours (made at the first call;
-  // concurrent calls on one plan share the arena and are the caller's error anyway)
+  // xema_forward_host: its launch and copy list, a second stream and events, so that the copies of one
+  // piece overlap the launches of its neighbours (made at the first call after a bind; concurrent
+  // calls on one plan share the arena and are the caller's error anyway)
+  mutable std::vector<HostStep> host_steps;
+  mutable int host_pieces_in = 0, host_pieces_out = 0;
   mutable cudaStream_t copy_stream = nullptr;
   mutable std::vector<cudaEvent_t> copy_events;
   ~xema_plan() {
@@ -344,6 +354,7 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
     return XEMA_EINVAL;
   plan->bound = false;
   plan->ops.clear();
+  plan->host_steps.clear();
   plan->rope = rope_dev;
   plan->arena = static_cast<uint8_t*>(arena_dev);
   uint8_t* arena = static_cast<uint8_t*>(arena_dev);
@@ -607,59 +618,203 @@ int xema_step_forward(const xema_plan* plan, void* stream) {
   return run_ops(plan, 0, plan->ops.size(), stream);
 }
 
-// One piece of a [B, rows, D] bf16 tensor (rows [r0, r0 + rows) of `batch` consecutive batch
-// elements, the first at `dev`) between the arena and the host copy of the whole tensor.
-static cudaError_t copy_piece(uint8_t* tensor_dev, uint8_t* tensor_host, const uint8_t* dev, int batch, int rows,
-                              long long row_elems, long long batch_rows, bool to_host, cudaStream_t st) {
-  const size_t off = (size_t)(dev - tensor_dev), pitch = (size_t)batch_rows * row_elems * 2,
-               width = (size_t)rows * row_elems * 2;
-  if (to_host)
-    return cudaMemcpy2DAsync(tensor_host + off, pitch, tensor_dev + off, pitch, width, batch, cudaMemcpyDeviceToHost, st);
-  return cudaMemcpy2DAsync(tensor_dev + off, pitch, tensor_host + off, pitch, width, batch, cudaMemcpyHostToDevice, st);
+// `op` for batch elements [b0, b0 + nb) and rows [r0, r0 + n) of those it covers (rows only where it
+// covers one batch element: an LN's output and a chunk's tensors are contiguous over both).
+static int sub_op(const xema_config& c, const Op& op, long long b0, int nb, long long r0, int n, Op* out) {
+  *out = op;
+  if (op.kind == OP_LN) {
+    const int elem = op.ln_in_f32 ? 4 : 2;
+    out->ln_in = static_cast<const uint8_t*>(op.ln_in) + (b0 * op.ln_in_batch_rows + r0) * c.hidden * elem;
+    out->ln_out = static_cast<uint8_t*>(op.ln_out) + (b0 * op.rows + r0) * c.hidden * 2;
+    out->shift = op.shift + b0 * 6 * c.hidden;
+    out->scale = op.scale + b0 * 6 * c.hidden;
+    out->rows = n;
+    out->batch = nb;
+    return XEMA_OK;
+  }
+  GemmLaunch& g = out->gemm;
+  const int out_elem = g.epilogue == XEMA_EPI_GATE_RES_F32 ? 4 : 2, res_elem = g.epilogue == XEMA_EPI_GATE_RES_BF16 ? 4 : 2;
+  g.out = static_cast<uint8_t*>(g.out) + (b0 * g.out_batch_rows + r0) * g.ldo * out_elem;
+  if (g.resid) g.resid = static_cast<const uint8_t*>(g.resid) + (b0 * g.resid_batch_rows + r0) * g.ldr * res_elem;
+  if (g.gate) g.gate += b0 * g.gate_stride;
+  g.rope_pos0 += (int)r0;
+  g.batch = nb;
+  g.rows = n;
+  return gemm_prepare(&g, static_cast<const uint8_t*>(g.a) + (b0 * g.a_batch_rows + r0) * g.lda * 2, g.lda, g.a_batch_rows, g.w,
+                      g.ldw);
+}
+
+// The pieces in which the work of an op on `batch` elements x `rows` token rows follows its copies:
+// single batch elements, or, for one element, rows that fill the GPU's CTA pairs with 256 x 256 tiles of
+// the D-wide products twice (3072 rows of 3072 columns on 74 pairs), or once where that gives less than two
+// pieces; with `fine_end` the last one is halved, because nothing hides its copy.  Copies under 4 MB are not
+// worth an event.
+static std::vector<std::pair<long long, long long>> host_pieces(const xema_config& c, int batch, int rows, bool fine_end) {
+  std::vector<std::pair<long long, long long>> out;      // [begin, end) in elements (batch > 1) or rows
+  const long long row_bytes = 2LL * c.hidden, total = batch > 1 ? batch : rows;
+  const long long unit_bytes = batch > 1 ? row_bytes * rows : row_bytes;
+  const long long least = std::max<long long>(1, (4ll << 20) / unit_bytes);
+  long long step = 1;
+  if (batch == 1) {
+    const long long wave = std::max(1, sm_count() / 2 / std::max(1, c.hidden / 256)) * 256ll;
+    step = rows >= 4 * wave ? 2 * wave : wave;
+    fine_end = fine_end && rows % step > wave;
+  } else {
+    fine_end = false;
+  }
+  step = std::max(step, least);
+  for (long long at = 0; at < total; at += step) out.push_back({at, std::min(total, at + step)});
+  if (out.size() > 1 && out.back().second - out.back().first < least) {   // a remnant joins its neighbour
+    out[out.size() - 2].second = total;
+    out.pop_back();
+  }
+  if (fine_end && out.back().second - out.back().first >= 2 * least) {
+    const long long b = out.back().first, e = out.back().second, mid = b + (e - b + 1) / 2 / 256 * 256;
+    if (mid > b && mid < e) {
+      out.back().second = mid;
+      out.push_back({mid, e});
+    }
+  }
+  return out;
+}
+
+// The launches of the plan with the first block's key/value phase cut so that it can follow the input's
+// arrival, and the last block's feed-forward phase so that the output can leave while it is made.  A row's
+// bits do not depend on how rows are cut, and every launch stays inside the tensors of its op; where the
+// order of the ops changes, the tensors involved are checked to be disjoint.
+static int build_host_steps(const xema_plan* plan) {
+  const xema_config& c = plan->cfg;
+  const std::vector<Op>& ops = plan->ops;
+  std::vector<HostStep> steps;
+  int n_in = 0, n_out = 0;
+  std::vector<bool> done(ops.size(), false);
+  uint8_t* out_dev = nullptr;
+  {
+    char name[32];
+    std::snprintf(name, sizeof(name), "hid%d", c.n_blocks);
+    auto it = plan->index.find(name);
+    if (it == plan->index.end()) return XEMA_EINVAL;
+    out_dev = plan->arena + plan->offsets[it->second];
+  }
+  const size_t row_bytes = (size_t)2 * c.hidden, hid_bytes = (size_t)2 * c.batch * plan->own_rows * c.hidden;
+  auto launch = [&](const Op& op) {
+    HostStep st{};
+    st.kind = HostStep::LAUNCH;
+    st.op = op;
+    steps.push_back(st);
+  };
+  auto launch_sub = [&](const Op& op, long long b0, int nb, long long r0, int n) {
+    HostStep st{};
+    st.kind = HostStep::LAUNCH;
+    const int rc = sub_op(c, op, b0, nb, r0, n, &st.op);
+    if (!rc) steps.push_back(st);
+    return rc;
+  };
+  // the tensor's rows that `batch` elements x `rows` rows at `dev` cover, elements `batch_rows` apart
+  auto copy = [&](HostStep::Kind kind, const uint8_t* tensor, const uint8_t* dev, int batch, int rows, long long batch_rows) {
+    HostStep st{};
+    st.kind = kind;
+    st.offset = (size_t)(dev - tensor);
+    st.width = (size_t)rows * row_bytes;
+    st.rows = (size_t)batch;
+    st.pitch = (size_t)batch_rows * row_bytes;
+    steps.push_back(st);
+    ++(kind == HostStep::COPY_IN ? n_in : n_out);
+  };
+  for (size_t i = 0; i < ops.size(); ++i) {
+    const Op& op = ops[i];
+    if (done[i] || op.kind == OP_FUSED) continue;
+    const bool first_ln = op.kind == OP_LN && op.block == 0 && !std::strcmp(op.name, "LN1A");
+    const bool last_ln = op.kind == OP_LN && op.block == c.n_blocks - 1 && !std::strcmp(op.name, "LN2");
+    if (!first_ln && !last_ln) {
+      launch(op);
+      continue;
+    }
+    const bool by_batch = op.batch > 1;
+    const bool last_chunk = op.chunk + 1 == plan->chunks[2];
+    for (auto& pc : host_pieces(c, op.batch, op.rows, last_ln && last_chunk)) {
+      const long long b0 = by_batch ? pc.first : 0, r0 = by_batch ? 0 : pc.first;
+      const int nb = by_batch ? (int)(pc.second - pc.first) : 1, n = by_batch ? op.rows : (int)(pc.second - pc.first);
+      int rc = XEMA_OK;
+      if (first_ln) {
+        // LN1A, KV and, where it reads LN1A's output too, Q
+        copy(HostStep::COPY_IN, plan->hid_in, static_cast<const uint8_t*>(op.ln_in) + (b0 * op.ln_in_batch_rows + r0) * row_bytes,
+             nb, n, op.ln_in_batch_rows);
+        rc = launch_sub(op, b0, nb, r0, n);
+        if (!rc) rc = launch_sub(ops[i + 1], b0, nb, r0, n);
+        done[i + 1] = true;
+        // (q's bytes are free during KV: whatever lives then lives at the Q op as well)
+        if (!rc && i + 4 < ops.size() && ops[i + 4].kind == OP_GEMM && ops[i + 4].gemm.early_input) {
+          rc = launch_sub(ops[i + 4], b0, nb, r0, n);
+          done[i + 4] = true;
+        }
+      } else {
+        // LN2, FFN1, FFN2.  The output is born at the first FFN2 and may lie where h2 of the first
+        // chunk was: then the chunk's LN2 and FFN1 stay whole and only FFN2 is cut.
+        const Op &ffn1 = ops[i + 1], &ffn2 = ops[i + 2];
+        const uint8_t* h2 = static_cast<const uint8_t*>(op.ln_out);
+        const bool apart = h2 + (size_t)op.batch * op.rows * row_bytes <= out_dev || out_dev + hid_bytes <= h2;
+        if (apart) {
+          rc = launch_sub(op, b0, nb, r0, n);
+          if (!rc) rc = launch_sub(ffn1, b0, nb, r0, n);
+        } else if (pc.first == 0) {
+          launch(op);
+          launch(ffn1);
+        }
+        if (!rc) rc = launch_sub(ffn2, b0, nb, r0, n);
+        if (!rc)
+          copy(HostStep::COPY_OUT, out_dev, static_cast<const uint8_t*>(steps.back().op.gemm.out), nb, n,
+               ffn2.gemm.out_batch_rows);
+        done[i + 1] = done[i + 2] = true;
+      }
+      if (rc) return rc;
+    }
+  }
+  plan->host_steps.swap(steps);
+  plan->host_pieces_in = n_in;
+  plan->host_pieces_out = n_out;
+  return XEMA_OK;
 }
 
 int xema_forward_host(const xema_plan* plan, const void* hid_in_host, const void* temb_host, void* hid_out_host,
                       void* stream) {
   if (!plan || !hid_in_host || !temb_host || !hid_out_host) return XEMA_EINVAL;
   if (!plan->bound) return XEMA_ESTATE;
+  if (plan->shard.P != 1) return XEMA_ESTATE;   // a shard's step needs the caller's exchange in the middle
   const xema_config& c = plan->cfg;
   char out_name[32];
   std::snprintf(out_name, sizeof(out_name), "hid%d", c.n_blocks);
-  auto i_in = plan->index.find("hid0"), i_temb = plan->index.find("temb"), i_out = plan->index.find(out_name);
-  if (i_in == plan->index.end() || i_temb == plan->index.end() || i_out == plan->index.end()) return XEMA_EINVAL;
+  auto i_out = plan->index.find(out_name);
+  if (i_out == plan->index.end()) return XEMA_EINVAL;
+  if (plan->host_steps.empty())
+    if (int rc = build_host_steps(plan)) return rc;
   // exact sizes (the planned sizes are rounded up to 256 bytes; the caller's buffers are not)
-  int64_t own_rows = 0;
-  if (shard_rows(c, plan->shard, nullptr, &own_rows)) return XEMA_EINVAL;
-  if (plan->shard.P != 1) return XEMA_ESTATE;   // a shard's step needs the caller's exchange in the middle
-  const size_t hid_bytes = (size_t)2 * c.batch * (size_t)own_rows * c.hidden;
   const size_t temb_bytes = (size_t)2 * c.batch * c.temb_dim;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  uint8_t* in_dev = plan->arena + plan->offsets[i_in->second];
+  uint8_t* in_dev = plan->hid_in;
   uint8_t* out_dev = plan->arena + plan->offsets[i_out->second];
-  uint8_t* in_host = static_cast<uint8_t*>(const_cast<void*>(hid_in_host));
+  const uint8_t* in_host = static_cast<const uint8_t*>(hid_in_host);
   uint8_t* out_host = static_cast<uint8_t*>(hid_out_host);
-  const std::vector<Op>& ops = plan->ops;
-  const size_t n = ops.size();
   cudaError_t e = cudaSuccess;
   auto fail = [&](cudaError_t err) {
     t_last_cuda_error = (int)err;
     return XEMA_ECUDA;
   };
+  auto move = [&](const HostStep& s, cudaStream_t on) {
+    uint8_t* dev = (s.kind == HostStep::COPY_IN ? in_dev : out_dev) + s.offset;
+    const void* src = s.kind == HostStep::COPY_IN ? (const void*)(in_host + s.offset) : dev;
+    void* dst = s.kind == HostStep::COPY_IN ? (void*)dev : out_host + s.offset;
+    const cudaMemcpyKind kind = s.kind == HostStep::COPY_IN ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+    if (s.rows == 1) return cudaMemcpyAsync(dst, src, s.width, kind, on);
+    return cudaMemcpy2DAsync(dst, s.pitch, src, s.pitch, s.width, s.rows, kind, on);
+  };
 
-  // The pieces of the first block's key/value phase read the input piece by piece (LN1A of piece c
-  // reads the rows of piece c only), and the pieces of the last block's feed-forward phase finish
-  // the output piece by piece (FFN2 of piece c).  With more than one piece in either phase the
-  // copies run on a second stream, ordered by events: the input of piece c + 1 arrives while
-  // piece c is worked on, the output of piece c leaves while piece c + 1 is worked on.  Bits do
-  // not depend on it.  With one piece the copy is a plain one on the caller's stream.
-  std::vector<size_t> in_ops, out_ops;      // LN1A launches of block 0, FFN2 launches of the last block
-  for (size_t i = 0; i < n; ++i) {
-    if (ops[i].kind == OP_LN && ops[i].block == 0 && !std::strcmp(ops[i].name, "LN1A")) in_ops.push_back(i);
-    if (ops[i].kind == OP_GEMM && ops[i].block == c.n_blocks - 1 && !std::strcmp(ops[i].name, "FFN2")) out_ops.push_back(i);
-  }
-  const bool row_major_out = !out_ops.empty() && ops[out_ops[0]].gemm.ldo == c.hidden;
-  const bool split_in = in_ops.size() > 1, split_out = out_ops.size() > 1 && row_major_out;
-  const size_t n_events = (split_in ? in_ops.size() : 0) + (split_out ? out_ops.size() : 0) + 1;
+  // Where the input or the output moves in more than one piece, its copies run on the plan's second
+  // stream, ordered by events: input piece k + 1 arrives while piece k is worked on, output piece k
+  // leaves while piece k + 1 is worked on.  Bits do not depend on it.  One piece is a plain copy on the
+  // caller's stream.
+  const bool split_in = plan->host_pieces_in > 1, split_out = plan->host_pieces_out > 1;
+  const size_t n_events = (split_in ? plan->host_pieces_in : 0) + (split_out ? plan->host_pieces_out : 0) + 2;
   if (split_in || split_out) {
     if (!plan->copy_stream && (e = cudaStreamCreateWithFlags(&plan->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
       return fail(e);
@@ -671,64 +826,44 @@ int xema_forward_host(const xema_plan* plan, const void* hid_in_host, const void
   }
   size_t next_event = 0;
   cudaStream_t cs = plan->copy_stream;
-
-  // ---- input
-  if ((e = cudaMemcpyAsync(plan->arena + plan->offsets[i_temb->second], temb_host, temb_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-    return fail(e);
-  std::vector<cudaEvent_t> in_ready(in_ops.size(), nullptr);
-  if (!split_in) {
-    if ((e = cudaMemcpyAsync(in_dev, in_host, hid_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess) return fail(e);
-  } else {
-    // the copy stream starts where the caller's stream stands (the arena may still be in use by
-    // work enqueued before this call)
-    cudaEvent_t start = plan->copy_events[next_event++];
-    if ((e = cudaEventRecord(start, st)) != cudaSuccess || (e = cudaStreamWaitEvent(cs, start, 0)) != cudaSuccess) return fail(e);
-    for (size_t k = 0; k < in_ops.size(); ++k) {
-      const Op& o = ops[in_ops[k]];
-      e = copy_piece(in_dev, in_host, static_cast<const uint8_t*>(o.ln_in), o.batch, o.rows, c.hidden, o.ln_in_batch_rows,
-                     false, k == 0 ? st : cs);
-      if (e != cudaSuccess) return fail(e);
-      if (k > 0) {
-        in_ready[k] = plan->copy_events[next_event++];
-        if ((e = cudaEventRecord(in_ready[k], cs)) != cudaSuccess) return fail(e);
-      }
-    }
-  }
-
-  // ---- launches, with the waits for input pieces and the copies of finished output pieces
-  size_t k_in = 0, k_out = 0;
-  bool chained = false;
-  for (size_t i = 0; i < n; ++i) {
-    if (split_in && k_in < in_ops.size() && i == in_ops[k_in]) {
-      if (in_ready[k_in] && (e = cudaStreamWaitEvent(st, in_ready[k_in], 0)) != cudaSuccess) return fail(e);
-      if (in_ready[k_in]) chained = false;
-      ++k_in;
-    }
-    int rc = issue(plan, ops[i], st, chained);
-    if (rc) return rc;
-    chained = chained || ops[i].kind != OP_FUSED;
-    if (split_out && k_out < out_ops.size() && i == out_ops[k_out]) {
-      const Op& o = ops[i];
-      const bool last = (k_out + 1 == out_ops.size());
-      chained = false;
-      if (!last) {
-        cudaEvent_t ev = plan->copy_events[next_event++];
-        if ((e = cudaEventRecord(ev, st)) != cudaSuccess || (e = cudaStreamWaitEvent(cs, ev, 0)) != cudaSuccess) return fail(e);
-      }
-      e = copy_piece(out_dev, out_host, static_cast<const uint8_t*>(o.gemm.out), o.gemm.batch, o.gemm.rows, c.hidden,
-                     o.gemm.out_batch_rows, true, last ? st : cs);
-      if (e != cudaSuccess) return fail(e);
-      ++k_out;
-    }
-  }
-  if (!split_out) {
-    if ((e = cudaMemcpyAsync(out_host, out_dev, hid_bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return fail(e);
-  }
-  if (split_in || split_out) {
-    // the caller's stream ends after everything the copy stream was given
+  // `later` continues after what `earlier` was given so far
+  auto order = [&](cudaStream_t earlier, cudaStream_t later) {
     cudaEvent_t ev = plan->copy_events[next_event++];
-    if ((e = cudaEventRecord(ev, cs)) != cudaSuccess || (e = cudaStreamWaitEvent(st, ev, 0)) != cudaSuccess) return fail(e);
+    cudaError_t err = cudaEventRecord(ev, earlier);
+    return err != cudaSuccess ? err : cudaStreamWaitEvent(later, ev, 0);
+  };
+
+  if ((e = cudaMemcpyAsync(plan->temb_in, temb_host, temb_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess) return fail(e);
+  std::vector<cudaEvent_t> arrived;
+  if (split_in) {
+    // the copy stream starts where the caller's stream stands (the arena may still be in use by work
+    // enqueued before this call)
+    if ((e = order(st, cs)) != cudaSuccess) return fail(e);
+    for (const HostStep& s : plan->host_steps) {
+      if (s.kind != HostStep::COPY_IN) continue;
+      arrived.push_back(plan->copy_events[next_event++]);
+      if ((e = move(s, cs)) != cudaSuccess || (e = cudaEventRecord(arrived.back(), cs)) != cudaSuccess) return fail(e);
+    }
   }
+  size_t k_in = 0;
+  bool chained = false;
+  for (const HostStep& s : plan->host_steps) {
+    if (s.kind == HostStep::LAUNCH) {
+      if (int rc = issue(plan, s.op, st, chained)) return rc;
+      chained = true;
+      continue;
+    }
+    chained = false;      // what follows is ordered after a copy or an event, not after a launch alone
+    if (s.kind == HostStep::COPY_IN) {
+      e = split_in ? cudaStreamWaitEvent(st, arrived[k_in++], 0) : move(s, st);
+    } else {
+      if (split_out) e = order(st, cs);
+      if (e == cudaSuccess) e = move(s, split_out ? cs : st);
+    }
+    if (e != cudaSuccess) return fail(e);
+  }
+  // the caller's stream ends after everything the copy stream was given
+  if ((split_in || split_out) && (e = order(cs, st)) != cudaSuccess) return fail(e);
   return XEMA_OK;
 }
 

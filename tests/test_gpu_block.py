@@ -6,7 +6,7 @@ import torch
 from oracle import block as ob
 from paper_2607_11136_b200 import binding as xb
 from paper_2607_11136_b200.session import BlockSession
-from xema_inputs import bits_to_f64, make_activations, make_block_weights, sample_rows, template
+from xema_inputs import weight_shapes, bits_to_f64, make_activations, make_block_weights, sample_rows, template
 
 from gpu_util import DEV, assert_bf16_close, assert_close, check_block_parity, expect_raw_bound
 
@@ -532,3 +532,33 @@ def test_set_inputs_takes_every_kind_of_source(batch, chunks):
         s.set_inputs(src_x, src_t)
         assert torch.equal(s.hid_in(), xd) and torch.equal(s.temb(), td)
         assert bool((s.arena[~slots] == 0x5A).all())
+
+
+@pytest.mark.parametrize("over,chunks", [({}, (1, 1, 1)), ({}, (1, 1, 2)), ({}, (2, 1, 3)), ({"batch": 2}, (1, 1, 1)),
+                                         ({"grid_t": 2, "hidden": 2048, "heads": 32, "head_dim": 64, "ffn": 4096}, (1, 2, 1)),
+                                         ({"n_blocks": 2}, (1, 1, 2))])
+def test_forward_host_moves_large_tensors_in_pieces(over, chunks):
+    """Inputs and outputs large enough for xema_forward_host to cut the first key/value and the last
+    feed-forward phase so that copies and launches overlap (by rows, by batch elements, inside chunks,
+    over two blocks): the bits of set_inputs + forward, twice in a row with the arena scribbled over."""
+    if "heads" in over:
+        over = dict(over, rope_dim_t=0, rope_dim_h=0, rope_dim_w=0)
+    t = template("flux", **over)
+    gen = torch.Generator(device="cuda:0").manual_seed(5)
+    weights = [{k: (torch.randn(shape, device="cuda:0", generator=gen) * 0.02 + (1.0 if k in ("g_q", "g_k") else 0.0)
+                    ).to(torch.bfloat16) for k, shape in weight_shapes(t).items()} for _ in range(t.n_blocks)]
+    x = torch.randn(t.batch, t.seq, t.hidden, device="cuda:0", generator=gen).to(torch.bfloat16).view(torch.int16)
+    temb = torch.randn(t.batch, t.temb_dim, device="cuda:0", generator=gen).to(torch.bfloat16).view(torch.int16)
+    s = BlockSession(t, weights, chunks=chunks)
+    s.set_inputs(x, temb)
+    s.forward()
+    want = s.hid_out().clone()
+    x_h, t_h = x.cpu().pin_memory(), temb.cpu().pin_memory()
+    y_h = torch.empty_like(x_h).pin_memory()
+    for fill in (0xFF, 0x00):
+        s.arena.fill_(fill)
+        y_h.zero_()
+        s.plan.forward_host(x_h.data_ptr(), t_h.data_ptr(), y_h.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        s.check_status()
+        assert torch.equal(y_h, want.cpu()), (over, chunks, fill)
