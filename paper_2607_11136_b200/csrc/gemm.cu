@@ -4,12 +4,12 @@
 //   acc[b, i, n] = sum_k A[b, i, k] * W[n, k]          (both operands K-major)
 //
 // One kernel, two forms.  A persistent grid of 192-thread CTAs walks over output tiles:
-//   PAIR    CTA pairs (two neighbouring SMs) share one 256 x 256 tile.  Each CTA loads its own 128
-//           rows of A and one half (128 rows) of the W tile, so a stage costs 32 KB of shared-memory
-//           fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
-//           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows x 256 columns in the TMEM of
-//           each CTA.
-//   single  one CTA per 128 x 128 or 128 x 64 tile, for problems that would leave SMs idle otherwise.
+//   PAIR    CTA pairs (two neighbouring SMs) share one 256 x 256 or 256 x 128 tile.  Each CTA loads its own
+//           128 rows of A and one half of the W tile, so a stage of the wide tile costs 32 KB of shared-
+//           memory fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
+//           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows in the TMEM of each CTA.
+//   single  one CTA per 128 x 128 or 128 x 64 tile.
+// pick_tile says which when.
 //
 //   warp 0    TMA producer: tiles of A and W into a ring of shared-memory stages (128-byte swizzle)
 //   warp 1    owns TMEM; converged warp, one elected lane issues tcgen05.mma into one of two fp32
@@ -47,7 +47,6 @@ constexpr int BK = 64;
 constexpr int GEMM_THREADS = 192;
 constexpr int GROUP_M = 8;
 constexpr int A_TILE_BYTES = BM * BK * 2;
-constexpr int PAIR_BN = 256;
 constexpr int CHUNK = 32;        // columns per epilogue step
 constexpr int BUF_BYTES = 4096;  // one staging buffer: 32 rows x 32 columns of fp32, or of bf16 in its first half
 
@@ -58,16 +57,16 @@ template <int EPI, int BN, bool PAIR>
 struct GemmCfg {
   static constexpr int W_ROWS = PAIR ? BN / 2 : BN;            // rows of W a CTA loads per K block
   static constexpr int W_TILE_BYTES = W_ROWS * BK * 2;
-  // K blocks of 64 per stage.  A single CTA's K block is short (128 to 256 cycles of MMA), and with a
-  // stage per block the barrier round of each one takes longer than that: 8888 x 12288 x 3072 with
+  // K blocks of 64 per stage.  The K block of a smaller tile is short (128 to 256 cycles of MMA), and
+  // with a stage per block the barrier round of each one takes longer than that: 8888 x 12288 x 3072 with
   // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block, 72 B/clk of fill).
-  static constexpr int KSUB = PAIR ? 1 : 2;
+  static constexpr int KSUB = BN == 256 ? 1 : 2;
   static constexpr int STAGE_BYTES = KSUB * (A_TILE_BYTES + W_TILE_BYTES);
   static constexpr int OFF_W = KSUB * A_TILE_BYTES;            // in a stage
   // staging buffers per epilogue warp: the gated epilogues keep residual chunks in flight
-  static constexpr int RING = kGated<EPI> && PAIR ? 4 : 2;
+  static constexpr int RING = kGated<EPI> && BN == 256 ? 4 : 2;
   static constexpr int RING_BYTES = 4 * RING * BUF_BYTES;
-  static constexpr int STAGES = PAIR ? (kGated<EPI> ? 5 : 6) : 196608 / STAGE_BYTES;
+  static constexpr int STAGES = BN == 256 ? (kGated<EPI> ? 5 : 6) : 196608 / STAGE_BYTES;
   static constexpr int OFF_RING = STAGES * STAGE_BYTES;
   static constexpr int OFF_BIAS = OFF_RING + RING_BYTES;       // float [BN]: bias
   static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
@@ -401,24 +400,26 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
           const int kb = ks * KSUB + u;
           if (KSUB > 1 && kb >= k_blocks) break;
           if constexpr (PAIR)
-            tma_load_3d_pair(sa, &map_a, mapa_shared(smem_u32(&full[st]), 0), kb * BK, (c.mt * 2 + (int)rank) * BM, c.b);
+            tma_load_3d_pair(sa + u * A_TILE_BYTES, &map_a, mapa_shared(smem_u32(&full[st]), 0), kb * BK,
+                             (c.mt * 2 + (int)rank) * BM, c.b);
           else
             tma_load_3d(sa + u * A_TILE_BYTES, &map_a, &full[st], kb * BK, c.mt * BM, c.b);
         }
       };
       auto load_w = [&](int st, const TileCoord& c, int ks) {   // with the stage's expected bytes
         uint8_t* sb = smem + st * Cfg::STAGE_BYTES + Cfg::OFF_W;
-        if constexpr (PAIR) {
-          if (rank == 0) mbar_expect_tx(&full[st], 2 * Cfg::STAGE_BYTES);
-          tma_load_3d_pair(sb, &map_w, mapa_shared(smem_u32(&full[st]), 0), ks * BK, c.nt * BN + (int)rank * (BN / 2), 0);
-        } else {
-          mbar_expect_tx(&full[st], min(KSUB, k_blocks - ks * KSUB) * (A_TILE_BYTES + Cfg::W_TILE_BYTES));
+        const int bytes = min(KSUB, k_blocks - ks * KSUB) * (A_TILE_BYTES + Cfg::W_TILE_BYTES);
+        if (!PAIR) mbar_expect_tx(&full[st], bytes);
+        else if (rank == 0) mbar_expect_tx(&full[st], 2 * bytes);
 #pragma unroll
-          for (int u = 0; u < KSUB; ++u) {
-            const int kb = ks * KSUB + u;
-            if (KSUB > 1 && kb >= k_blocks) break;
+        for (int u = 0; u < KSUB; ++u) {
+          const int kb = ks * KSUB + u;
+          if (KSUB > 1 && kb >= k_blocks) break;
+          if constexpr (PAIR)
+            tma_load_3d_pair(sb + u * Cfg::W_TILE_BYTES, &map_w, mapa_shared(smem_u32(&full[st]), 0), kb * BK,
+                             c.nt * BN + (int)rank * (BN / 2), 0);
+          else
             tma_load_3d(sb + u * Cfg::W_TILE_BYTES, &map_w, &full[st], kb * BK, c.nt * BN, 0);
-          }
         }
       };
       // The weights of the first stages do not depend on earlier launches (see launch_kernel): they
@@ -504,24 +505,21 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
           if (elect_one()) {
             const uint64_t soff = (uint64_t)(stage * (Cfg::STAGE_BYTES >> 4));
             const uint64_t da = a_desc0 + soff, db = b_desc0 + soff;
-            if constexpr (PAIR) {
-              mma_ss_pair(d_tmem, da, db, idesc, accumulate);
-              mma_ss_pair(d_tmem, da + 2, db + 2, idesc, 1);
-              mma_ss_pair(d_tmem, da + 4, db + 4, idesc, 1);
-              mma_ss_pair(d_tmem, da + 6, db + 6, idesc, 1);
-              mma_commit_pair(&empty[stage]);
-            } else {
+            auto mma = [&](uint64_t ad, uint64_t bd, uint32_t acc_in) {
+              if constexpr (PAIR) mma_ss_pair(d_tmem, ad, bd, idesc, acc_in);
+              else mma_ss(d_tmem, ad, bd, idesc, acc_in);
+            };
 #pragma unroll
-              for (int u = 0; u < KSUB; ++u) {
-                if (KSUB > 1 && ks * KSUB + u >= k_blocks) break;
-                const uint64_t ua = da + (uint64_t)(u * (A_TILE_BYTES >> 4)), ub = db + (uint64_t)(u * (Cfg::W_TILE_BYTES >> 4));
-                mma_ss(d_tmem, ua, ub, idesc, u > 0 ? 1 : accumulate);
-                mma_ss(d_tmem, ua + 2, ub + 2, idesc, 1);
-                mma_ss(d_tmem, ua + 4, ub + 4, idesc, 1);
-                mma_ss(d_tmem, ua + 6, ub + 6, idesc, 1);
-              }
-              mma_commit(&empty[stage]);
+            for (int u = 0; u < KSUB; ++u) {
+              if (KSUB > 1 && ks * KSUB + u >= k_blocks) break;
+              const uint64_t ua = da + (uint64_t)(u * (A_TILE_BYTES >> 4)), ub = db + (uint64_t)(u * (Cfg::W_TILE_BYTES >> 4));
+              mma(ua, ub, u > 0 ? 1 : accumulate);
+              mma(ua + 2, ub + 2, 1);
+              mma(ua + 4, ub + 4, 1);
+              mma(ua + 6, ub + 6, 1);
             }
+            if constexpr (PAIR) mma_commit_pair(&empty[stage]);
+            else mma_commit(&empty[stage]);
           }
           __syncwarp();
           accumulate = 1;
@@ -636,12 +634,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmParams p) {
   gemm_body<EPI, BN, false>(map_a, map_w, map_out, map_res, p);
 }
-template <int EPI>
+template <int EPI, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                       const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
                       const GemmParams p) {
-  gemm_body<EPI, PAIR_BN, true>(map_a, map_w, map_out, map_res, p);
+  gemm_body<EPI, BN, true>(map_a, map_w, map_out, map_res, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -680,11 +678,11 @@ int launch_single(const GemmLaunch& g, cudaStream_t stream, bool chained) {
                        make_params(g, chained));
 }
 
-template <int EPI>
+template <int EPI, int BN>
 int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
-  using Cfg = GemmCfg<EPI, PAIR_BN, true>;
+  using Cfg = GemmCfg<EPI, BN, true>;
   static PerDeviceInt attr_done;
-  auto kern = gemm_bf16_pair_kernel<EPI>;
+  auto kern = gemm_bf16_pair_kernel<EPI, BN>;
   if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
   // A persistent grid must be resident all at once: ask how many CTA pairs fit on the device
   // (SMs are handed out to clusters in hardware groups, so it can be fewer than SMs / 2).
@@ -712,7 +710,7 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
     max_pairs = std::min(n, sm_count() / 2);
     pairs_cache.set(dev, max_pairs);
   }
-  const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / PAIR_BN);
+  const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / BN);
   const int pairs = (int)std::min<long long>(tiles, max_pairs);
   return launch_kernel(kern, dim3(2 * pairs), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out,
                        g.map_res, make_params(g, chained));
@@ -720,40 +718,41 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 
 template <int EPI>
 int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
-  if (g.block_n == 256) return launch_pair<EPI>(g, stream, chained);
+  if (g.pair) return g.block_n == 256 ? launch_pair<EPI, 256>(g, stream, chained) : launch_pair<EPI, 128>(g, stream, chained);
   if (g.block_n == 128) return launch_single<EPI, 128>(g, stream, chained);
   return launch_single<EPI, 64>(g, stream, chained);
 }
 
 
-// Tile for a problem: the one with the shortest estimated time, waves x K blocks x cycles per K block
-// plus the last tile's epilogue.  Cycles as measured (B200, 1.9 GHz): a 256 x 256 pair tile runs at its
-// math time, 512 per K block, with all SMs busy and nearer 600 in the latency of a short loop; a
-// 128 x 128 tile takes 490-550 and a 128 x 64 tile 335 -- a CTA fills shared memory at about 70 B/clk
-// whatever its tile -- so the smaller tiles are slower per flop and pay only where the larger ones
-// leave SMs idle: 1101 x 1536 x 6144 39.2 / 30.9 / 39.3 us (256 / 128 / 64), 333 x 1024 x 4096 28.8 / 22.0 / 16.5,
-// 288 x 512 x 2048 18.6 / 13.5 / 12.1, but 4444 x 3072 x 3072 58.4 / 74.7 / 106.
+// Tile for a problem: the one with the shortest estimated time, waves x K blocks x nanoseconds per K
+// block plus what its last tile's epilogue adds.  Measured (B200, shapes from 288 x 512 x 2048 to 8888 x 12288 x
+// 3072): a K block takes 370-385 ns with 256 x 256 pair tiles, 212-270 with 256 x 128 pair tiles, 255-290 with
+// 128 x 128 and 172-211 with 128 x 64 -- a CTA fills shared memory at about 70 B/clk whatever its tile -- so a
+// smaller tile is slower per flop and pays only where the larger one leaves SMs idle.  us for 256 x 256 /
+// 256 x 128 / 128 x 128 / 128 x 64: 333 x 1024 x 4096 28.8 / 20.2 / 21.9 / 16.5, 1101 x 1536 x 6144 39.1 / 27.3 / 30.9 /
+// 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.
 // The bits of a row do not depend on the choice.
-int pick_tile(const GemmLaunch& g) {
+void pick_tile(GemmLaunch* g) {
   struct Tile {
-    int block_n, rows, workers_per_sm_x2, cycles, epilogue;
+    int pair, block_n, block_ns, epilogue_ns;
   };
-  static const Tile tiles[] = {{256, 2 * BM, 1, 600, 4000}, {128, BM, 2, 520, 2500}, {64, BM, 2, 340, 1500}};
-  const long long k_blocks = g.K / BK;
+  static const Tile tiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}};
+  const long long k_blocks = g->K / BK;
   long long best = 0;
-  int pick = 0;
+  g->block_n = 0;
   for (const Tile& t : tiles) {
-    if (g.N % t.block_n) continue;
-    if (g.epilogue == XEMA_EPI_BIAS_NORM_ROPE && t.block_n < g.head_dim) continue;   // whole heads only
-    const long long n = (long long)g.batch * ((g.rows + t.rows - 1) / t.rows) * (g.N / t.block_n);
-    const long long workers = std::max(1, sm_count() * t.workers_per_sm_x2 / 2);
-    const long long cost = (n + workers - 1) / workers * k_blocks * t.cycles + t.epilogue;
-    if (!pick || cost < best) {
+    if (g->N % t.block_n) continue;
+    if (g->epilogue == XEMA_EPI_BIAS_NORM_ROPE && t.block_n < g->head_dim) continue;   // whole heads only
+    const int rows = t.pair ? 2 * BM : BM;
+    const long long n = (long long)g->batch * ((g->rows + rows - 1) / rows) * (g->N / t.block_n);
+    const long long workers = std::max(1, t.pair ? sm_count() / 2 : sm_count());
+    const long long cost = (n + workers - 1) / workers * k_blocks * t.block_ns + t.epilogue_ns;
+    if (!g->block_n || cost < best) {
       best = cost;
-      pick = t.block_n;
+      g->block_n = t.block_n;
+      g->pair = t.pair;
     }
   }
-  return pick;
 }
 }  // namespace
 
@@ -790,12 +789,12 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   g->lda = lda;
   g->a_batch_rows = a_batch_rows;
   g->ldw = ldw;
-  g->block_n = pick_tile(*g);
+  pick_tile(g);
   const long long rows = g->rows > 0 ? g->rows : 1;
   int rc = encode_tmap_bf16(&g->map_a, a, g->K, rows, g->batch, lda, a_batch_rows, BM);
   if (rc) return rc;
-  // the pair form loads its W tile as two 128-row halves, one per CTA
-  rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, g->block_n == 64 ? 64 : 128);
+  // the pair forms load their W tile as two halves, one per CTA
+  rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, g->pair ? g->block_n / 2 : g->block_n);
   if (rc) return rc;
   // results leave, and residuals arrive, as boxes of 32 columns x 32 rows
   rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, g->N, rows, g->batch, g->ldo,

@@ -108,6 +108,7 @@ struct GemmLaunch {
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K, epilogue, block_n;
+  int pair;            // a CTA pair per tile (256 x block_n) or one CTA (128 x block_n)
   const void *a, *w;   // operands as given to gemm_prepare
   long long lda, a_batch_rows, ldw;
   unsigned int* status;

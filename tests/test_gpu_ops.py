@@ -180,9 +180,9 @@ def test_gemm_epilogue_row_edges(epi, rows):
             assert_bf16_close(got, ref, ("gemm edges", epi, rows, N), atol_rms=2e-3 if epi == xb.EPI_BIAS_GELU else 2e-4)
 
 
-@pytest.mark.parametrize("N,K", [(512, 320), (1536, 64), (768, 448)])
+@pytest.mark.parametrize("N,K", [(512, 320), (1536, 64), (768, 448), (1536, 1600)])
 def test_gemm_tile_forms_give_the_same_bits(N, K):
-    """The tile (256 x 256 over a CTA pair, 128 x 128, 128 x 64) is chosen from the size of the
+    """The tile (256 x 256 or 256 x 128 over a CTA pair, 128 x 128, 128 x 64) is chosen from the size of the
     problem; a row's bits must not show it.  The same rows as a problem of their own (small tiles)
     and inside one that fills the GPU (pairs), K with an odd number of 64-wide blocks (a stage
     of the single-CTA forms holds two); the first also against the oracle."""
