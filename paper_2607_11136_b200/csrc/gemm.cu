@@ -8,7 +8,7 @@
 //           128 rows of A and one half of the W tile, so a stage of the wide tile costs 32 KB of shared-
 //           memory fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
 //           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows in the TMEM of each CTA.
-//   single  one CTA per 128 x 128 or 128 x 64 tile.
+//   single  one CTA per 128 x 128, 128 x 64 or (gated epilogues, few rows) 128 x 32 tile.
 // pick_tile says which when.
 //
 //   warp 0    TMA producer: tiles of A and W into a ring of shared-memory stages (128-byte swizzle)
@@ -72,7 +72,7 @@ struct GemmCfg {
   static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
   static constexpr int OFF_BAR = OFF_GATE + (kGated<EPI> ? BN * 4 : 512);
   static constexpr int SMEM_BYTES = OFF_BAR + 384;
-  static constexpr int TMEM_COLS = 2 * BN;
+  static constexpr int TMEM_COLS = 2 * BN;   // a power of two from 32 on
   static_assert((2 * STAGES + 4 + 4 * RING) * 8 + 8 <= 384, "barrier area");
   static_assert(SMEM_BYTES <= 232448, "shared memory of one SM");
 };
@@ -720,7 +720,9 @@ template <int EPI>
 int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   if (g.pair) return g.block_n == 256 ? launch_pair<EPI, 256>(g, stream, chained) : launch_pair<EPI, 128>(g, stream, chained);
   if (g.block_n == 128) return launch_single<EPI, 128>(g, stream, chained);
-  return launch_single<EPI, 64>(g, stream, chained);
+  if (g.block_n == 64) return launch_single<EPI, 64>(g, stream, chained);
+  if constexpr (kGated<EPI>) return launch_single<EPI, 32>(g, stream, chained);
+  return XEMA_EINVAL;
 }
 
 
@@ -730,18 +732,21 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // 128 x 128 and 172-211 with 128 x 64 -- a CTA fills shared memory at about 70 B/clk whatever its tile -- so a
 // smaller tile is slower per flop and pays only where the larger one leaves SMs idle.  us for 256 x 256 /
 // 256 x 128 / 128 x 128 / 128 x 64: 333 x 1024 x 4096 28.8 / 20.2 / 21.9 / 16.5, 1101 x 1536 x 6144 39.1 / 27.3 / 30.9 /
-// 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.
+// 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.  128 x 32 exists for the
+// gated epilogues, whose products are narrow: 288 x 512 x 2048 12.1 -> 10.4 us, a step of 8 blocks of 333 tokens
+// x 1024 521 -> 500.
 // The bits of a row do not depend on the choice.
 void pick_tile(GemmLaunch* g) {
   struct Tile {
     int pair, block_n, block_ns, epilogue_ns;
   };
-  static const Tile tiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}};
+  static const Tile tiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}, {0, 32, 150, 400}};
   const long long k_blocks = g->K / BK;
   long long best = 0;
   g->block_n = 0;
   for (const Tile& t : tiles) {
     if (g->N % t.block_n) continue;
+    if (t.block_n < 64 && g->epilogue != XEMA_EPI_GATE_RES_F32 && g->epilogue != XEMA_EPI_GATE_RES_BF16) continue;
     if (g->epilogue == XEMA_EPI_BIAS_NORM_ROPE && t.block_n < g->head_dim) continue;   // whole heads only
     const int rows = t.pair ? 2 * BM : BM;
     const long long n = (long long)g->batch * ((g->rows + rows - 1) / rows) * (g->N / t.block_n);

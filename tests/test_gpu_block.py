@@ -562,3 +562,48 @@ def test_forward_host_moves_large_tensors_in_pieces(over, chunks):
         torch.cuda.synchronize()
         s.check_status()
         assert torch.equal(y_h, want.cpu()), (over, chunks, fill)
+
+
+def test_chained_launches_on_two_streams_and_threads():
+    """The launches of a call may start before the previous one has finished; two sessions driven by
+    two threads on streams of their own (their kernels share the SMs) and a captured graph must still
+    give the bits of a session that runs alone."""
+    import threading
+    cases = []
+    for over in ({}, {"grid_t": 6, "grid_h": 16, "grid_w": 17}):
+        t = template("tiny", **over)
+        s = BlockSession(t, [make_block_weights(t, 0)], chunks=1)
+        x, temb = make_activations(t)
+        xd, td = torch.from_numpy(x.view(np.int16)).to(DEV), torch.from_numpy(temb.view(np.int16)).to(DEV)
+        s.set_inputs(xd, td)
+        s.forward()
+        torch.cuda.synchronize()
+        cases.append((s, xd, td, s.hid_out().clone(), torch.cuda.Stream()))
+    wrong = []
+
+    def work(k):
+        s, xd, td, want, stream = cases[k]
+        torch.cuda.set_device(0)
+        with torch.cuda.stream(stream):
+            for i in range(40):
+                s.arena.fill_(i)
+                s.set_inputs(xd, td)
+                s.forward(stream)
+                if i % 8 == 7 and not torch.equal(s.hid_out(), want):
+                    wrong.append((k, i))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert not wrong
+    for s, xd, td, want, _ in cases:
+        s.set_inputs(xd, td)
+        g = s.capture()
+        for _ in range(3):
+            s.set_inputs(xd, td)
+            g.replay()
+            assert torch.equal(s.hid_out(), want)
+        s.check_status()
