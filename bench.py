@@ -75,9 +75,9 @@ def whole_job_tflops(flops_per_replica: float, world: int, ms: float) -> float:
 
 
 # DRAM traffic of one attention launch (dram__bytes_read.sum + dram__bytes_write.sum under ncu, see
-# profiles/attention_dh64_rows2222_keys17776_h48.md).  Captured inside this bench at the full 17776
+# profiles/attention_rows2222_keys17776_h48_d64.md).  Captured inside this bench at the full 17776
 # query rows: 422.9 MB (329.0 read + 93.9 written; algorithmic 440.3 -- q is still in L2 from the Q
-# projection).  Captured alone at 2222 rows: 266.6 MB (algorithmic 246.2), of which k and v (4*S*D
+# projection).  Captured alone at 2222 rows: 259.6-266.6 MB (algorithmic 246.2), of which k and v (4*S*D
 # bytes, independent of the number of query rows) are read once and the rest scales with the query
 # rows; other row counts are scaled from that capture.  Not measured in the timed run.
 def attention_traffic_bytes(t, rows: int) -> float:
@@ -482,8 +482,8 @@ def main():
         r["traffic"] = None
         if dom == "ATTN":
             r["traffic"] = attention_traffic_bytes(t, t.seq * t.n_blocks // d["launches"])
-            r["traffic_source"] = ("not measured in this run: dram__bytes_read.sum + dram__bytes_write.sum of one ncu "
-                                   "capture, see profiles/attention_dh64_*.md" if r["traffic"] else None)
+            r["traffic_source"] = ("not measured in this run: dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture, "
+                                   "see profiles/attention_rows2222_keys17776_h48_d64.md" if r["traffic"] else None)
         return r
 
     def breakdown_of(ops_t, step_ms_):
@@ -503,10 +503,11 @@ def main():
     dom = roofline["kernel"]
     if dom == "ATTN" and t.head_dim == 64 and clocks.get("sm_max_mhz"):
         # context: with 64-wide heads there is one exponential per 4 * 64 flop and an SM retires 16 ex2 per
-        # clock; three eighths of the exponentials run as a polynomial on the FMA pipe instead
+        # clock; seven sixteenths of the exponentials run as a polynomial on the FMA pipe instead
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         mufu = 16.0 * sms * clocks["sm_max_mhz"] * 1e6 * 4 * t.head_dim / 1e12
-        roofline["exp_rate_ceiling_tflops"] = {"all_on_mufu_at_max_clock": mufu, "five_eighths_on_mufu": mufu / 0.625}
+        roofline["exp_rate_ceiling_tflops"] = {"all_on_mufu_at_max_clock": mufu,
+                                               "nine_sixteenths_on_mufu": mufu / 0.5625}
     breakdown = breakdown_of(per_op, per_op_total_ms / args.steps)
     if sustained is not None:
         s_ops = sustained.pop("per_op_raw")
@@ -551,8 +552,8 @@ def main():
         # are NOT part of the budget, so it is the extra, not the value.
         "e2e": {"value": whole_job_tflops(flops, world, e2e_serial_ms), "unit": UNIT, "ms_per_step": e2e_serial_ms,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
-                "how": "xema_forward_host: pinned host -> arena, forward, arena -> pinned host; the output of a finished "
-                       "feed-forward piece is copied out while the next piece runs (plan-owned copy stream)",
+                "how": "xema_forward_host: pinned host -> arena, forward, arena -> pinned host; the first launches follow "
+                       "the pieces of the input, a finished feed-forward piece is copied out while the next one runs",
                 "device_bytes": sess.plan.peak_bytes, "fits_budget": budget is None or sess.plan.peak_bytes <= budget,
                 "pipelined": {"value": whole_job_tflops(flops, world, e2e_ms), "ms_per_step": e2e_ms,
                               "how": "BlockSession.run_pipelined: copies of neighbouring steps overlap compute",
