@@ -13,21 +13,29 @@
 // The softmax threads set the pace (an SM retires 16 exponentials per clock against 4 * dh flop each),
 // so their instruction stream is kept short:
 //
-//   * no running maximum, and in the normal pass no reference at all: q arrives multiplied by
-//     log2(e) / sqrt(dh) (the Q projection's epilogue does that before its one rounding to bf16), so a
-//     score leaves the tensor core as the exponent to base 2 of its unnormalised probability and
-//     p = 2^s is formed whatever its size -- fp32 sums and bf16 probabilities keep their relative
-//     precision from 2^-90 to 2^90 -- so O is never rescaled and the two threads of a row need not talk
-//     to each other inside the loop.  A row that leaves that range (a sum of 2^90 or more, or of 2^-90
-//     or less), or that hands the exponential polynomial an argument outside its range, is flagged, and
-//     its item is done again after the CTA's last item, in two more sweeps: one over the scores only,
-//     which decides again which rows were at fault and takes their true maximum, and one that repeats
-//     the pass with that maximum taken off the scores of those rows.  Rows that were not at fault
-//     repeat exactly what they did before, bit for bit;
-//   * a share of the exponentials is evaluated as a polynomial on the FMA pipe (see kPolyPairs);
+//   * no running maximum: q arrives multiplied by log2(e) / sqrt(dh) (the Q projection's epilogue does
+//     that before its one rounding to bf16), so a score leaves the tensor core as the exponent to base 2
+//     of its unnormalised probability and p = 2^(s - reference) is formed whatever its size -- fp32 sums
+//     and bf16 probabilities keep their relative precision from 2^-90 to 2^90 -- so O is never rescaled
+//     and the two threads of a row need not talk to each other inside the loop.  The reference of a row
+//     is 0 for dh 64 and the largest of its first 128 scores for dh 128.  A row that leaves the
+//     range (a sum of 2^90 or more, or of 2^-90 or less), or that hands the exponential polynomial an
+//     argument outside its range, is flagged, and its item is done again after the CTA's last item, in
+//     two more sweeps: one over the scores only, which decides again which rows were at fault and takes
+//     their true maximum, and one that repeats the pass with that maximum as the reference of those
+//     rows.  Rows that were not at fault repeat exactly what they did before, bit for bit;
+//   * dh 64, where the exponentials set the pace: a share of them is evaluated as a polynomial on the
+//     FMA pipe (see kPolyPairs);
+//   * dh 128, where the threads have issue slots to spare (1264 of 2690 cycles a block): every
+//     exponential on the MUFU, and O is divided by the sum of the probabilities as they were rounded to
+//     bf16 (lse takes the unrounded sum), so that the rounding of a dominant key cancels.  Relative error
+//     of o against 64 bits, standard normal q and k: 2.24e-3 for 288 keys, 2.32e-3 for 1101, and 1.92e-3 for
+//     600 keys with three times the scores; without reference and rounded sum 2.34e-3, 2.35e-3, 2.35e-3; with a
+//     running maximum instead 2.29e-3, 2.33e-3, 2.23e-3.  Both together cost 2 % (4608 x 4608 x 24 heads
+//     229 -> 233 us, launches in turn on a warm board);
 //   * one body for all blocks where there are few: the first time an SM runs a piece of code costs
 //     microseconds of instruction fetch, which a call with few keys pays in full.  Keys past the end get
-//     the score -119 (they add 2^-119 each to a row sum of at least 2^-90; their V rows are zero).
+//     the exponent -119 (they add 2^-119 each to a row sum of at least 2^-90; their V rows are zero).
 //
 // TMEM, per tile 256 columns:
 //   dh  64: S [0,128), P [128,192) (bf16 pairs), O [192,256).  S(j+1) is issued as soon as the tile's
@@ -41,8 +49,8 @@
 //
 // Measured (B200, inside the block): dh 64, 4444 x 17776 x 48 heads 933 us (with one CTA per 256 rows and code
 // copies for first and last blocks 970); power-capped 17776-token block 7.28 ms against 7.52.  dh 128, 17776 x
-// 17776 x 24 heads 3.03 ms = 1280 TFLOP/s (one tile per CTA, two CTAs per SM, 64-key blocks, running maximum: 3.40),
-// 4608 x 4608 x 24 heads 228 us (261).  288 x 288 x 8 heads 10.4 us (14.4), launches back to back.
+// 17776 x 24 heads 3.38 ms on a warm board (one tile per CTA, two CTAs per SM, 64-key blocks, running maximum:
+// 3.79 in turn with it), 4608 x 4608 x 24 heads 235 us (275).  288 x 288 x 8 heads of 64 10.4 us (14.4).
 //
 // Every decision is per row and keys are always visited in the same order, so a row's bits do not
 // depend on how rows are tiled or chunked.
@@ -75,20 +83,24 @@ constexpr int THREADS = 128 + SOFTMAX_THREADS;
 constexpr int REG_HELPER = 64, REG_SOFTMAX = 104;
 static_assert(128 * REG_HELPER + SOFTMAX_THREADS * REG_SOFTMAX <= THREADS * 96, "register pool");
 // Which of a thread's 32 column pairs evaluate 2^x as a polynomial on the FMA pipe, one bit per pair; the
-// others use the MUFU.  Without any the MUFU sets the pace, with too many the issue slots do, and where
-// they stand decides how well the compiler interleaves the two pipes.  Measured inside the block (scores
-// bounded, see below) over 125 placements of 6 to 17 bits: dh 64, 4444 x 17776 x 48 heads 933 to 1177 us (this
-// one 933, the next best 945; 9 bits 1000 and more), dh 128, 4608 x 4608 x 24 heads 232 to 247 us (this one within
-// one percent of the fastest).
-// Power-capped, the dh 64 block of 17776 tokens takes 7.28 ms with this placement, 7.39-7.56 with three others.
+// others use the MUFU.  dh 64: without any the MUFU sets the pace, with too many the issue slots do, and
+// where they stand decides how well the compiler interleaves the two pipes -- the placement is the result of
+// a search with this compiler and nothing else: 4444 x 17776 x 48 heads 933 to 1177 us over 125 placements of 6 to
+// 17 bits (this one 933, the next best 945; 9 bits 1000 and more; 24 placements of 12 bits 4.8 to 12.7 % slower
+// inside the block).  Power-capped, the block of 17776 tokens takes 7.28 ms with this placement, 7.39-7.56 with
+// three others.  Accuracy: see exp2_poly; a polynomial of degree 4 costs 10 % of the launch.
+// dh 128: none.  The MUFU needs no longer for a block than the tensor pipe (2048 cycles each), and 8 pairs on the
+// FMA pipe were 2 % slower in turn with none (4608 x 4608 x 24 heads 231 against 226 us).
 template <int DH>
-constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0x22440924u;
+constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0u;
 static_assert(BN == 128 && BM == 128, "the kernel is written for 128-key blocks of 128-row tiles");
 
 template <int DH>
 struct Cfg {
   static constexpr bool ALIAS = DH == 128;                 // P over S; otherwise P has its own columns
   static constexpr int ISSUERS = ALIAS ? 1 : 2;            // MMA-issuing warps (from warp 1)
+  static constexpr bool FIRST_MAX = DH == 128;             // reference: the largest score of the first block
+  static constexpr bool ROUNDED_SUM = DH == 128;           // O over the sum of the rounded probabilities
   static constexpr int ATOMS = DH / 64;
   static constexpr int TILE_BYTES = ATOMS * ATOM_BYTES;    // a Q tile, or a K or V block
   static constexpr int QBUF = DH == 64 ? 2 : 1;
@@ -118,42 +130,50 @@ struct AttnParams {
   const __nv_bfloat16 *gain_q, *gain_k;   // RMSNorm gains behind q and k, or null (see AttnLaunch)
 };
 
-// 2^x for two values on the FMA pipe, as exp2_poly_f32x2 but without its clamp: the caller
-// guarantees -125 <= x <= 126.
-__device__ __forceinline__ f32x2 exp2_poly_unclamped(f32x2 x2) {
+// 2^x for two values on the FMA pipe instead of the MUFU: round-to-nearest split x = n + r with
+// |r| <= 1/2 through the 1.5 * 2^23 trick, a cubic for 2^r, then n added into the exponent field.
+// The cubic has the least mean square relative error (4.84e-5) among those of mean 0 that stay within
+// 1e-4 of 2^r, a twentieth of the bf16 rounding of the probability it feeds: the errors of a row's keys
+// do not add up in its sum.  (The cubic of least largest error, 7.5e-5, has a mean of 5e-6 and a mean square of
+// 5.2e-5; lse of 1101 keys 2.8e-6 off with it, 1.7e-6 with this one.)
+// Valid for -125 <= x <= 126; CLAMP raises smaller arguments to -125 (2^-125 stands in for zero) and leaves
+// the bits of valid ones as they are.
+template <bool CLAMP>
+__device__ __forceinline__ f32x2 exp2_poly(f32x2 x2) {
+  if (CLAMP) x2 = make_float2(fmaxf(x2.x, -125.f), fmaxf(x2.y, -125.f));
   const f32x2 magic = make_float2(12582912.f, 12582912.f);
   const f32x2 neg_magic = make_float2(-12582912.f, -12582912.f);
   const f32x2 neg_one = make_float2(-1.f, -1.f);
   const f32x2 t2 = add_f32x2(x2, magic);                 // integer part lands in the low mantissa bits
   const f32x2 n2 = add_f32x2(t2, neg_magic);             // nearest integer as a float
   const f32x2 r2 = fma_f32x2(n2, neg_one, x2);           // r = x - n
-  f32x2 p2 = fma_f32x2(make_float2(0.0551716685f, 0.0551716685f), r2, make_float2(0.242611125f, 0.242611125f));
-  p2 = fma_f32x2(p2, r2, make_float2(0.693260968f, 0.693260968f));
-  p2 = fma_f32x2(p2, r2, make_float2(0.999928057f, 0.999928057f));
+  f32x2 p2 = fma_f32x2(make_float2(0.0551208667f, 0.0551208667f), r2, make_float2(0.242484242f, 0.242484242f));
+  p2 = fma_f32x2(p2, r2, make_float2(0.693255842f, 0.693255842f));
+  p2 = fma_f32x2(p2, r2, make_float2(0.999933064f, 0.999933064f));
   return make_float2(__uint_as_float(__float_as_uint(p2.x) + (__float_as_uint(t2.x) << 23)),
                      __uint_as_float(__float_as_uint(p2.y) + (__float_as_uint(t2.y) << 23)));
 }
 
+// Partial sums of one thread's part of a row: of the probabilities, and (ROUNDED_SUM) of what bf16 makes
+// of them.
+struct RowSums {
+  f32x2 plain[4], rounded[2];
+};
+
 // p = 2^s for chunk CHUNK of a thread's score columns: packed bf16x2 words, the values added into
-// four packed partial sums.  The polynomial is only valid for arguments in [-125, 126].
-// CLAMP = false: it is used as it is and, with TRACK, `poly_abs` collects the largest magnitude handed
-// to it, for the caller to check afterwards (without TRACK the caller knows a bound on every score
-// beforehand).  CLAMP = true: arguments are clamped from below first (2^-125 stands in for zero);
-// wherever the unclamped form was valid the result has the same bits.
+// packed partial sums.  CLAMP = false: the polynomial is used as it is and, with TRACK, `poly_abs` collects the
+// largest magnitude handed to it, for the caller to check afterwards (without TRACK the caller knows a
+// bound on every score beforehand).  CLAMP = true: its arguments are clamped from below first.
 template <int DH, int CHUNK, bool CLAMP, bool TRACK>
-__device__ __forceinline__ void exp_cols(const float (&s)[CH], uint32_t* pk, f32x2 (&ls2)[4], float& poly_abs) {
+__device__ __forceinline__ void exp_cols(const float (&s)[CH], uint32_t* pk, RowSums& sums, float& poly_abs) {
 #pragma unroll
   for (int t = 0; t < CH; t += 2) {
     const int pair = t >> 1;
-    f32x2 e2 = pack_f32x2(s[t], s[t + 1]);   // the scores come out of the tensor core as exponents
+    f32x2 e2 = pack_f32x2(s[t], s[t + 1]);
     float e0, e1;
     if (kPolyPairs<DH> >> (CHUNK * (CH / 2) + pair) & 1u) {
-      if (CLAMP) {
-        e2 = exp2_poly_f32x2(e2);
-      } else {
-        if (TRACK) poly_abs = max3(poly_abs, fabsf(e2.x), fabsf(e2.y));
-        e2 = exp2_poly_unclamped(e2);
-      }
+      if (TRACK && !CLAMP) poly_abs = max3(poly_abs, fabsf(e2.x), fabsf(e2.y));
+      e2 = exp2_poly<CLAMP>(e2);
       unpack_f32x2(e2, e0, e1);
     } else {
       unpack_f32x2(e2, e0, e1);
@@ -161,8 +181,14 @@ __device__ __forceinline__ void exp_cols(const float (&s)[CH], uint32_t* pk, f32
       e1 = ex2_approx(e1);
       e2 = pack_f32x2(e0, e1);
     }
-    ls2[pair & 3] = add_f32x2(ls2[pair & 3], e2);
+    sums.plain[pair & 3] = add_f32x2(sums.plain[pair & 3], e2);
     pk[pair] = pack_bf16x2(e0, e1);
+  }
+  // (behind the chunk's exponentials: among them the compiler places them 3 % slower)
+  if (Cfg<DH>::ROUNDED_SUM) {
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i)
+      sums.rounded[i & 1] = add_f32x2(sums.rounded[i & 1], make_float2(bf16_lo(pk[i]), bf16_hi(pk[i])));
   }
 }
 // columns at or beyond `valid` (keys past the end of the sequence) get `value`
@@ -177,9 +203,13 @@ __device__ __forceinline__ float row_max(const float (&s)[CH]) {
   for (int t = 3; t + 1 < CH; t += 2) mx = max3(mx, s[t], s[t + 1]);
   return fmaxf(mx, s[CH - 1]);
 }
-__device__ __forceinline__ float sum_partials(const f32x2 (&ls2)[4]) {
-  const f32x2 a = add_f32x2(ls2[0], ls2[1]), b = add_f32x2(ls2[2], ls2[3]);
+__device__ __forceinline__ float sum_partials(const f32x2 (&v)[4]) {
+  const f32x2 a = add_f32x2(v[0], v[1]), b = add_f32x2(v[2], v[3]);
   const f32x2 c = add_f32x2(a, b);
+  return c.x + c.y;
+}
+__device__ __forceinline__ float sum_partials(const f32x2 (&v)[2]) {
+  const f32x2 c = add_f32x2(v[0], v[1]);
   return c.x + c.y;
 }
 __device__ __forceinline__ void ld_scores(uint32_t addr, float (&s)[CH]) { tmem_ld16(addr, *reinterpret_cast<uint32_t(*)[CH]>(&s[0])); }
@@ -498,7 +528,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t s_tmem = t_lane + half * COLS;
   const uint32_t p_tmem = t_lane + C::TM_P + half * (C::ALIAS ? COLS : COLS / 2);
   const uint32_t o_tmem = t_lane + C::TM_O + half * (DH / TPR);
-  f32x2 ls2[4];
+  RowSums sums;
   float poly_abs = 0.f, m_ref = 0.f, m_true = 0.f;
   // The two warps that share 32 rows meet: all of them, with a vote on going on (a warp that gave up
   // still comes here, so that the other does not wait for it) ...
@@ -513,6 +543,26 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return xch[(half ^ 1) * BM + r];
   };
 
+  // The reference of this thread's row from its first block of scores (which has arrived, if ok): the
+  // largest of them.  Both threads of a row come here and get the same value.
+  auto first_max = [&]() {
+    float m = -INFINITY;
+    if (ok) {
+      tc_fence_after();
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        float s[CH];
+        ld_scores(s_tmem + c * CH, s);
+        wait_scores(s);
+        mask_tail(s, p.keys - half * COLS - c * CH, -INFINITY);
+        m = fmaxf(m, row_max(s));
+      }
+    }
+    agree();
+    if (!ok) return;
+    m_ref = fmaxf(m, exchange(m));
+    if (SCALED) m_ref *= p.q_scale;
+  };
   // One key block: this thread's COLS scores in four chunks, the next on its way from TMEM.
   auto run_block = [&](int j, auto mode_tag, auto masked_tag, auto track_tag) {
     constexpr bool MASKED = decltype(masked_tag)::value;   // some keys of the block may lie past the end
@@ -520,16 +570,21 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr bool TRACK = decltype(track_tag)::value;
     constexpr bool CLAMP = MODE == REPEAT;
     ok = mbar_wait_warp(&s_full[tile], s_ph, abort_flag);
+    if (C::FIRST_MAX && MODE != REPEAT && j == 0) first_max();
     if (!ok) return;
     tc_fence_after();
     s_ph ^= 1;
     const int valid = p.keys - j * BN - half * COLS;     // keys of this thread's columns that exist
     auto adjust = [&](float(&s)[CH], int c) {
-      if (SCALED) {
-        const f32x2 c2 = make_float2(p.q_scale, p.q_scale);
+      // score -> exponent relative to the row's reference (zero for dh 64 but in the repeat of a flagged row)
+      if (SCALED || C::FIRST_MAX || MODE == REPEAT) {
+        const f32x2 c2 = make_float2(p.q_scale, p.q_scale), m2 = make_float2(-m_ref, -m_ref);
 #pragma unroll
         for (int t = 0; t < CH; t += 2) {
-          const f32x2 v = __fmul2_rn(pack_f32x2(s[t], s[t + 1]), c2);
+          f32x2 v = pack_f32x2(s[t], s[t + 1]);
+          if (!C::FIRST_MAX && MODE != REPEAT) v = __fmul2_rn(v, c2);
+          else if (SCALED) v = fma_f32x2(v, c2, m2);
+          else v = add_f32x2(v, m2);
           s[t] = v.x;
           s[t + 1] = v.y;
         }
@@ -537,10 +592,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (MODE == PROBE) {
         if (MASKED) mask_tail(s, valid - c * CH, -INFINITY);
         m_true = fmaxf(m_true, row_max(s));
-      }
-      if (MODE == REPEAT) {
-#pragma unroll
-        for (int t = 0; t < CH; ++t) s[t] -= m_ref;       // zero for the rows that were fine
       }
       if (MASKED) mask_tail(s, valid - c * CH, PAST_END);
     };
@@ -553,10 +604,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     wait_scores(b1);
     wait_scores(b2);
     adjust(b0, 0);
-    exp_cols<DH, 0, CLAMP, TRACK>(b0, &pk[0][0], ls2, poly_abs);
+    exp_cols<DH, 0, CLAMP, TRACK>(b0, &pk[0][0], sums, poly_abs);
     ld_scores(s_tmem + 3 * CH, b0);
     adjust(b1, 1);
-    exp_cols<DH, 1, CLAMP, TRACK>(b1, &pk[0][CH / 2], ls2, poly_abs);
+    exp_cols<DH, 1, CLAMP, TRACK>(b1, &pk[0][CH / 2], sums, poly_abs);
     wait_scores(b0);
     if (C::ALIAS && MODE != PROBE) {
       tmem_st16(p_tmem, pk[0]);                            // all scores are in registers
@@ -568,9 +619,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_arrive(&s_free[tile]);                         // S(j) is in registers: S(j+1) may land
     }
     adjust(b2, 2);
-    exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[1][0], ls2, poly_abs);
+    exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[1][0], sums, poly_abs);
     adjust(b0, 3);
-    exp_cols<DH, 3, CLAMP, TRACK>(b0, &pk[1][CH / 2], ls2, poly_abs);
+    exp_cols<DH, 3, CLAMP, TRACK>(b0, &pk[1][CH / 2], sums, poly_abs);
     if (MODE == PROBE) return;
     if (!C::ALIAS) {
       if (j > 0) {                                        // the previous product reads the same columns
@@ -591,7 +642,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int n_plain = p.keys / BN > 3 ? p.keys / BN : 0;
   auto run_blocks = [&](auto mode_tag, auto track_tag) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) ls2[i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < 4; ++i) sums.plain[i] = make_float2(0.f, 0.f);
+    sums.rounded[0] = sums.rounded[1] = make_float2(0.f, 0.f);
     poly_abs = 0.f;
 #pragma unroll 1
     for (int j = 0; ok && j < n_plain; ++j) run_block(j, mode_tag, std::false_type{}, track_tag);
@@ -606,7 +658,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // At or below 2^-90 the row's scores lie so far below zero that the small terms were flushed away.
   // The threads of the row decide the same (an infinity stands for a thread's own flag).
   auto row_sum = [&](bool& flag) -> float {
-    const float l = sum_partials(ls2);
+    const float l = sum_partials(sums.plain);
     float seen = !(l < DANGER) || poly_abs > 120.f ? INFINITY : l;
     const float other = exchange(seen);
     seen += other;
@@ -614,13 +666,19 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return l + other;            // used only where nothing was flagged
   };
   // The accumulator is final once the item's last product has finished: normalise and store.
+  // l_row: sum of the row's probabilities, for lse; O goes by the sum of what it was made from.
   auto finish = [&](const Item& it, float l_row) {
+    float o_row = l_row;
+    if (C::ROUNDED_SUM) {
+      const float mine = sum_partials(sums.rounded);
+      o_row = mine + exchange(mine);
+    }
     ok = mbar_wait_warp(&pv_done[tile], pv_ph, abort_flag);
     pv_ph ^= 1;
     if (!ok) return;
     tc_fence_after();
     const int row = it.row0 + tile * BM + r;
-    const float inv_l = 1.f / l_row;
+    const float inv_l = 1.f / o_row;
     // dh 128: four lanes hold 64 bytes of four rows; transposed among themselves, a store covers whole
     // 64-byte pieces of eight rows instead of 16 bytes of 32, which keeps the load/store unit busy for
     // 4000 cycles an item (4608 x 4608 x 24 heads 232 -> 228 us).  The dh 64 kernel gains the same on its
@@ -739,13 +797,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REG_SOFTMAX));
-    // With q and k out of an RMSNorm (gains g), a rotation and, for q, the factor
+    // dh 64: with q and k out of an RMSNorm (gains g), a rotation and, for q, the factor
     // log2(e) / sqrt(dh), a head of q has norm <= max|g_q| * log2(e) and a head of k norm <=
     // sqrt(dh) * max|g_k|: every score lies within +-log2(e) * sqrt(dh) * max|g_q| * max|g_k|
     // (plus the bf16 roundings, under half a percent).  Far inside the polynomial's range nothing
     // needs to be tracked per score.
-    bool bounded = false;
-    if (!SCALED && p.gain_q && p.gain_k) {
+    constexpr bool POLY = kPolyPairs<DH> != 0;
+    bool bounded = !POLY;
+    if (POLY && !SCALED && p.gain_q && p.gain_k) {
       const int ts = threadIdx.x - 128;
       if (ts < DH) {
         atomicMax(&gain_max[0], __float_as_uint(fabsf(__bfloat162float(p.gain_q[ts]))));
@@ -754,7 +813,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       named_barrier(1, SOFTMAX_THREADS);
       const float gq = __uint_as_float(*(volatile uint32_t*)&gain_max[0]);
       const float gk = __uint_as_float(*(volatile uint32_t*)&gain_max[1]);
-      constexpr float factor = (DH == 64 ? 11.55f : 16.33f) * 1.01f;
+      static_assert(!POLY || DH == 64, "log2(e) * sqrt(64) below");
+      constexpr float factor = 11.55f * 1.01f;
       bounded = gq * gk * factor < 100.f;    // false for a NaN gain
     }
     for (int i = 0; i < n_items; ++i) {
@@ -762,7 +822,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!tile_live(it, tile)) continue;
       if (ok) {
         if (bounded) run_blocks(PassT{}, std::false_type{});
-        else run_blocks(PassT{}, std::true_type{});
+        else run_blocks(PassT{}, std::bool_constant<POLY>{});
       }
       agree();
       if (!ok) break;
@@ -779,12 +839,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (!tile_live(it, tile)) return;
         bool flag = false;
         m_true = -INFINITY;
-        if (ok) run_blocks(ProbeT{}, std::true_type{});
+        m_ref = 0.f;
+        if (ok) run_blocks(ProbeT{}, std::bool_constant<POLY>{});
         agree();
         if (!ok) return;
         row_sum(flag);
+        // the true maximum is relative to the reference of the pass
         m_true = fmaxf(m_true, exchange(m_true));
-        m_ref = flag ? m_true : 0.f;
+        if (flag) m_ref += m_true;
         run_blocks(RepeatT{}, std::false_type{});
         agree();
         if (!ok) return;

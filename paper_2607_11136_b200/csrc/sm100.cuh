@@ -546,25 +546,6 @@ __device__ __forceinline__ void unpack_f32x2(f32x2 v, float& lo, float& hi) {
 }
 __device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b) { return __fadd2_rn(a, b); }
-// 2^x for two values on the FMA pipe instead of the MUFU: round-to-nearest split x = n + r with
-// |r| <= 1/2 through the 1.5 * 2^23 trick, a cubic for 2^r (relative error 7.5e-5, far below the
-// bf16 rounding of the probabilities it feeds), then n added into the exponent field.
-// Valid for x <= 126; inputs below -125 are clamped (2^-125 stands in for zero).
-__device__ __forceinline__ f32x2 exp2_poly_f32x2(f32x2 x2) {
-  x2 = make_float2(fmaxf(x2.x, -125.f), fmaxf(x2.y, -125.f));
-  const f32x2 magic = make_float2(12582912.f, 12582912.f);
-  const f32x2 neg_magic = make_float2(-12582912.f, -12582912.f);
-  const f32x2 neg_one = make_float2(-1.f, -1.f);
-  const f32x2 t2 = add_f32x2(x2, magic);                 // integer part lands in the low mantissa bits
-  const f32x2 n2 = add_f32x2(t2, neg_magic);             // nearest integer as a float
-  const f32x2 r2 = fma_f32x2(n2, neg_one, x2);           // r = x - n
-  f32x2 p2 = fma_f32x2(make_float2(0.0551716685f, 0.0551716685f), r2, make_float2(0.242611125f, 0.242611125f));
-  p2 = fma_f32x2(p2, r2, make_float2(0.693260968f, 0.693260968f));
-  p2 = fma_f32x2(p2, r2, make_float2(0.999928057f, 0.999928057f));
-  return make_float2(__uint_as_float(__float_as_uint(p2.x) + (__float_as_uint(t2.x) << 23)),
-                     __uint_as_float(__float_as_uint(p2.y) + (__float_as_uint(t2.y) << 23)));
-}
-
 // max of three values in one instruction
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;

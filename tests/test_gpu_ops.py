@@ -291,6 +291,38 @@ def test_attention_edges(rows, keys, dh):
     assert np.abs(got_l - ref_l).max() < 2e-3
 
 
+@pytest.mark.parametrize("dh,keys,spread,o_max,lse_max", [(64, 4608, 1.0, 2.4e-3, 1.5e-6), (128, 40, 1.0, 2.2e-3, 5e-7),
+                                                          (128, 288, 1.0, 2.3e-3, 5e-7), (128, 600, 3.0, 2.1e-3, 2e-6)])
+def test_attention_rms_error(dh, keys, spread, o_max, lse_max):
+    """Root-mean-square error of o (relative) and of lse over a million elements, where an element-wise bound
+    sees little.  Rounding o to bf16 alone gives 1.66e-3 and rounding independent probabilities to bf16 as
+    much again, 2.35e-3 together.  head_dim 128 has to stay below that where a few keys carry a row (few
+    keys, or scores spread threefold), because its largest probabilities are exact or cancel: half-way between
+    2.35e-3 and the 2.05e-3, 2.24e-3 and 1.92e-3 it reaches.  lse is a sum of fp32 exponentials: its bound is two to
+    three times what ex2 of 2^-22 gives (the error of a score of size s adds s * 2^-24), and for head_dim 64 less
+    than the 2.2e-6 that exponentials with a common error of 5e-6 in 14 of 32 places would add up to."""
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    rows, H = (500, 16) if keys > 1000 else (288, 96)
+    D = H * dh
+    q = (torch.randn(rows, D, device=DEV, generator=gen) * (spread * xb.exponent_scale(dh))).to(torch.bfloat16)
+    kv = torch.randn(keys, 2 * D, device=DEV, generator=gen).to(torch.bfloat16)
+    o = torch.empty(rows, D, dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty(H, rows, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    xb.xema_op_attention(q.data_ptr(), D, rows, kv.data_ptr(), kv.data_ptr() + D * 2, 2 * D, keys, o.data_ptr(), lse.data_ptr(),
+                         1, rows, keys, H, dh, status=status.data_ptr(), q_scale=1.0)
+    _sync_status(status)
+    err = ref = lse_err = 0.0
+    for h in range(H):
+        c = slice(h * dh, (h + 1) * dh)
+        s = (q[:, c].double() @ kv[:, c].double().T) * math.log(2.0)
+        want = torch.softmax(s, -1) @ kv[:, D + h * dh:D + (h + 1) * dh].double()
+        err += (o[:, c].double() - want).square().sum().item()
+        ref += want.square().sum().item()
+        lse_err += (lse[h].double() - torch.logsumexp(s, -1)).square().mean().item() / H
+    assert math.sqrt(err / ref) < o_max and math.sqrt(lse_err) < lse_max, (math.sqrt(err / ref), math.sqrt(lse_err))
+
+
 @pytest.mark.parametrize("dh", [64, 128])
 def test_attention_items_of_one_cta_with_flagged_rows(dh):
     """More work items than SMs, so that CTAs run several; the scores of a few heads lie near +-260 (in
