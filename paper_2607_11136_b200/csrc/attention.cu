@@ -23,7 +23,8 @@
 //     argument outside its range, is flagged, and its item is done again after the CTA's last item, in
 //     two more sweeps: one over the scores only, which decides again which rows were at fault and takes
 //     their true maximum, and one that repeats the pass with that maximum as the reference of those
-//     rows.  Rows that were not at fault repeat exactly what they did before, bit for bit;
+//     rows.  Rows that were not at fault repeat exactly what they did before, bit for bit.  A score
+//     that is not a number makes its row's maximum one too, and with it the whole row;
 //   * dh 64, where the exponentials set the pace: a share of them is evaluated as a polynomial on the
 //     FMA pipe (see kPolyPairs);
 //   * dh 128, where the threads have issue slots to spare (1264 of 2690 cycles a block): every
@@ -93,6 +94,7 @@ static_assert(128 * REG_HELPER + SOFTMAX_THREADS * REG_SOFTMAX <= THREADS * 96, 
 // FMA pipe were 2 % slower in turn with none (4608 x 4608 x 24 heads 231 against 226 us).
 template <int DH>
 constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0u;
+static_assert(!(kPolyPairs<64> & 1u), "a row's first key goes through the MUFU, which keeps a NaN");
 static_assert(BN == 128 && BM == 128, "the kernel is written for 128-key blocks of 128-row tiles");
 
 template <int DH>
@@ -197,11 +199,12 @@ __device__ __forceinline__ void mask_tail(float (&s)[CH], int valid, float value
   for (int t = 0; t < CH; ++t)
     if (t >= valid) s[t] = value;
 }
+// (a NaN among the values is the result)
 __device__ __forceinline__ float row_max(const float (&s)[CH]) {
-  float mx = max3(s[0], s[1], s[2]);
+  float mx = max3_nan(s[0], s[1], s[2]);
 #pragma unroll
-  for (int t = 3; t + 1 < CH; t += 2) mx = max3(mx, s[t], s[t + 1]);
-  return fmaxf(mx, s[CH - 1]);
+  for (int t = 3; t + 1 < CH; t += 2) mx = max3_nan(mx, s[t], s[t + 1]);
+  return max3_nan(mx, s[CH - 1], s[CH - 1]);
 }
 __device__ __forceinline__ float sum_partials(const f32x2 (&v)[4]) {
   const f32x2 a = add_f32x2(v[0], v[1]), b = add_f32x2(v[2], v[3]);
@@ -555,12 +558,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ld_scores(s_tmem + c * CH, s);
         wait_scores(s);
         mask_tail(s, p.keys - half * COLS - c * CH, -INFINITY);
-        m = fmaxf(m, row_max(s));
+        const float mc = row_max(s);
+        m = max3_nan(m, mc, mc);
       }
     }
     agree();
     if (!ok) return;
-    m_ref = fmaxf(m, exchange(m));
+    const float other = exchange(m);
+    m_ref = max3_nan(m, other, other);
     if (SCALED) m_ref *= p.q_scale;
   };
   // One key block: this thread's COLS scores in four chunks, the next on its way from TMEM.
@@ -591,7 +596,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       if (MODE == PROBE) {
         if (MASKED) mask_tail(s, valid - c * CH, -INFINITY);
-        m_true = fmaxf(m_true, row_max(s));
+        const float m = row_max(s);
+        m_true = max3_nan(m_true, m, m);
       }
       if (MASKED) mask_tail(s, valid - c * CH, PAST_END);
     };
@@ -844,9 +850,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         agree();
         if (!ok) return;
         row_sum(flag);
-        // the true maximum is relative to the reference of the pass
-        m_true = fmaxf(m_true, exchange(m_true));
-        if (flag) m_ref += m_true;
+        // the true maximum, relative to the reference of the pass; where there is none (a NaN, an
+        // infinity) the row has no finite probabilities
+        const float other = exchange(m_true);
+        m_true = max3_nan(m_true, other, other);
+        if (flag) m_ref = fabsf(m_true) < INFINITY ? m_ref + m_true : NAN;
         run_blocks(RepeatT{}, std::false_type{});
         agree();
         if (!ok) return;

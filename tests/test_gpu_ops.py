@@ -324,6 +324,45 @@ def test_attention_rms_error(dh, keys, spread, o_max, lse_max):
 
 
 @pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("plain", [False, True])
+def test_attention_non_finite_keys_reach_their_rows(dh, plain):
+    """A key that holds a NaN makes every row of its head NaN, one that holds an infinity the rows whose score
+    for it is +infinity (the others give it probability 0), whichever place of a key block it has -- all
+    places between two multiples of 64 are tried, because different places take different exponentials.
+    Heads without such a key are not touched."""
+    rng = np.random.default_rng(15)
+    rows, keys, H = 140, 300, 66
+    D = H * dh
+    q, kv = rng.standard_normal((rows, D)), bf16_bits(rng.standard_normal((keys, 2 * D), dtype=np.float32))
+    qb, qf = (lambda b: (b, bits_to_f64(b)))(bf16_bits(q.astype(np.float32))) if plain else _exponent_units(q, dh)
+    for h in range(64):
+        at = 64 * (h % 4) + h
+        if at < keys:
+            kv[at, h * dh + 3] = 0x7FC0 if h % 2 else 0x7F80
+    kvf = bits_to_f64(kv)
+    q_dev, kv_dev = to_dev(qb), to_dev(kv)
+    o = torch.zeros(rows, D, dtype=torch.int16, device=DEV)
+    lse = torch.zeros(H, rows, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    xb.xema_op_attention(q_dev.data_ptr(), D, rows, kv_dev.data_ptr(), kv_dev.data_ptr() + D * 2, 2 * D, keys, o.data_ptr(),
+                         lse.data_ptr(), 1, rows, keys, H, dh, status=status.data_ptr(), q_scale=None if plain else 1.0)
+    _sync_status(status)
+    got, got_l = from_dev_bf16(o), lse.cpu().numpy()
+    for h in range(H):
+        c = slice(h * dh, (h + 1) * dh)
+        with np.errstate(invalid="ignore"):
+            s = qf[:, c] @ kvf[:, c].T / math.sqrt(dh)
+            bad = np.isnan(s).any(axis=1) | np.isposinf(s).any(axis=1)
+        assert np.array_equal(np.isnan(got[:, c]).all(axis=1), bad) and np.array_equal(np.isnan(got[:, c]).any(axis=1), bad), h
+        assert np.array_equal(np.isfinite(got_l[h]), ~bad), h
+        ok = ~bad
+        if ok.any():
+            e = np.exp(s[ok] - s[ok].max(axis=1, keepdims=True))
+            want = (e / e.sum(axis=1, keepdims=True)) @ kvf[:, D + h * dh:D + (h + 1) * dh]
+            assert_bf16_close(got[ok][:, c], want, ("non-finite keys", dh, h), atol_rms=1.5e-2, cos=0.9999)
+
+
+@pytest.mark.parametrize("dh", [64, 128])
 def test_attention_items_of_one_cta_with_flagged_rows(dh):
     """More work items than SMs, so that CTAs run several; the scores of a few heads lie near +-260 (in
     exponents to base 2), so first and later items of some CTAs have to be repeated against their rows'
