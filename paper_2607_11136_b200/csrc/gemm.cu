@@ -82,7 +82,6 @@ struct GemmParams {
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K;
-  int late_trigger, early_input;    // see GemmLaunch
   int resid_batch;                  // 1: the residual has a batch dimension, 0: the same rows for every element
   unsigned int* status;
   // XEMA_EPI_BIAS_NORM_ROPE only: heads that start below column norm_cols get RMSNorm * gain
@@ -384,7 +383,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
   }
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x == 0 && !p.late_trigger) grid_dep_launch();
+  if (threadIdx.x == 0) grid_dep_launch();
 
   if (warp == 0) {
     // ---------------- TMA producer (one per CTA) ----------------
@@ -430,11 +429,9 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
         if (elect_one())
           for (int kb = 0; kb < early; ++kb) load_w(kb, c, kb);
         __syncwarp();
-        if (!p.early_input) grid_dep_wait();
-        if (elect_one()) {
-          if (p.late_trigger) grid_dep_launch();
+        grid_dep_wait();
+        if (elect_one())
           for (int kb = 0; kb < early; ++kb) load_a(kb, c, kb);
-        }
         __syncwarp();
         if (early == STAGES) phase = 1;
         else stage = early;
@@ -643,7 +640,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 }
 
 // ---------------------------------------------------------------------------------------------
-GemmParams make_params(const GemmLaunch& g, bool chained) {
+GemmParams make_params(const GemmLaunch& g) {
   GemmParams p;
   p.bias = (const __nv_bfloat16*)g.bias;
   p.gate = g.gate;
@@ -652,8 +649,6 @@ GemmParams make_params(const GemmLaunch& g, bool chained) {
   p.rows = g.rows;
   p.N = g.N;
   p.K = g.K;
-  p.late_trigger = g.late_trigger;
-  p.early_input = chained && g.early_input;
   p.resid_batch = g.resid_batch_rows != 0;
   p.status = g.status;
   p.norm_gain = (const __nv_bfloat16*)g.norm_gain;
@@ -675,7 +670,7 @@ int launch_single(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   const long long tiles = (long long)g.batch * ((g.rows + BM - 1) / BM) * (g.N / BN);
   const int grid = (int)std::min<long long>(tiles, sm_count());
   return launch_kernel(kern, dim3(grid), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out, g.map_res,
-                       make_params(g, chained));
+                       make_params(g));
 }
 
 template <int EPI, int BN>
@@ -713,7 +708,7 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / BN);
   const int pairs = (int)std::min<long long>(tiles, max_pairs);
   return launch_kernel(kern, dim3(2 * pairs), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out,
-                       g.map_res, make_params(g, chained));
+                       g.map_res, make_params(g));
 }
 
 template <int EPI>

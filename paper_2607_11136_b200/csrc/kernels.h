@@ -112,11 +112,6 @@ struct GemmLaunch {
   const void *a, *w;   // operands as given to gemm_prepare
   long long lda, a_batch_rows, ldw;
   unsigned int* status;
-  // Two launches in a row that read the same input (KV and Q): the first lets the next one start only
-  // after its own wait (late_trigger), that is with the input complete; the second, when chained to it,
-  // loads the input without a wait (early_input) and runs on the SMs the first leaves idle.  Its
-  // epilogue waits for the first as always, so nothing later can overtake either.
-  int late_trigger, early_input;
   // XEMA_EPI_BIAS_NORM_ROPE: RMSNorm * gain + RoPE for the heads below column norm_cols
   const void* norm_gain;
   const float* rope;

@@ -127,6 +127,7 @@ struct Op {
   // shared
   int rows;
   int batch;          // batch elements this launch covers (OP_LN, OP_ROPE)
+  bool reads_ln1a;    // OP_GEMM Q: its input is LN1A's output (LN1B elided)
   GemmLaunch gemm;
   AttnLaunch attn;
 };
@@ -512,7 +513,7 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       const uint8_t* hid_pc = hid + at_row(pc, D, 2);
       const uint8_t* kv_b = kv + pc.b0 * S_all * 2 * D * 2;      // keys and values of these batch elements
       ln_op(hid_pc, 0, h1b, pc, 1, "LN1B", ci);
-      bool q_follows_kv = false;      // no launch between KV and Q, both reading LN1A's output
+      bool q_follows_kv = false;      // no launch between KV and Q, both read LN1A's output
       // With one piece in both phases LN1B recomputes what LN1A wrote.  When the layout put h1b
       // at h1a's address and nothing was born in between (KROPE allocates nothing, so the only
       // births since the KV op are h1b's own), those bytes are still there: the launch is elided.
@@ -539,11 +540,7 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       int rc = gemm_op(h1b, D, n, w_qkv, D, b_qkv, q, D, n, nullptr, 0, 0, nullptr, pc, (int)D, (int)D,
                        XEMA_EPI_BIAS_NORM_ROPE, "Q", ci, w.g_q, (int)D, (int)(row0 + pc.r0), q_scale);
       if (rc) return rc;
-      if (q_follows_kv) {
-        // ops: ..., KV, KROPE (fused), LN1B (elided), Q
-        plan->ops[plan->ops.size() - 4].gemm.late_trigger = 1;
-        plan->ops.back().gemm.early_input = 1;
-      }
+      plan->ops.back().reads_ln1a = q_follows_kv;     // ops: LN1A, KV, KROPE (fused), LN1B (elided), Q
       Op o{};
       o.kind = OP_FUSED;
       tag(o, "QROPE", ci, 0.0, 0.0);
@@ -744,7 +741,7 @@ static int build_host_steps(const xema_plan* plan) {
         if (!rc) rc = launch_sub(ops[i + 1], b0, nb, r0, n);
         done[i + 1] = true;
         // (q's bytes are free during KV: whatever lives then lives at the Q op as well)
-        if (!rc && i + 4 < ops.size() && ops[i + 4].kind == OP_GEMM && ops[i + 4].gemm.early_input) {
+        if (!rc && i + 4 < ops.size() && ops[i + 4].kind == OP_GEMM && ops[i + 4].reads_ln1a) {
           rc = launch_sub(ops[i + 4], b0, nb, r0, n);
           done[i + 4] = true;
         }
