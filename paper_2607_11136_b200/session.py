@@ -102,12 +102,13 @@ class BlockSession:
         return v
 
     # The plan's addresses never change, so the views of the inputs and the output are made once
-    # (making one takes several microseconds, on a path that small blocks run in tens of them).
+    # (making one takes several microseconds, on a path that small blocks run in tens of them).  A caller
+    # gets a tensor of its own over the same bytes, which it may reshape in place.
     def _view_once(self, name: str, shape) -> torch.Tensor:
         v = self._views.get(name)
         if v is None:
             v = self._views[name] = self.view(name, torch.int16, shape)
-        return v
+        return v.view(shape)
 
     def hid_in(self) -> torch.Tensor:
         return self._view_once("hid0", self._hid_shape)

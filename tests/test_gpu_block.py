@@ -534,6 +534,23 @@ def test_set_inputs_takes_every_kind_of_source(batch, chunks):
         assert bool((s.arena[~slots] == 0x5A).all())
 
 
+def test_views_of_inputs_and_output_belong_to_the_caller():
+    """Changing the shape of a returned view in place leaves later calls as they were."""
+    t = template("tiny")
+    x, temb = make_activations(t)
+    s = BlockSession(t, [make_block_weights(t, 0)], chunks=1)
+    s.set_inputs(x, temb)
+    s.forward()
+    want = s.output_bits()
+    for get in (s.hid_in, s.temb, s.hid_out):
+        shape = tuple(get().shape)
+        get().unsqueeze_(0).transpose_(1, 2)
+        assert tuple(get().shape) == shape and get().is_contiguous()
+    s.set_inputs(x, temb)
+    s.forward()
+    assert np.array_equal(s.output_bits(), want)
+
+
 @pytest.mark.parametrize("over,chunks", [({}, (1, 1, 1)), ({}, (1, 1, 2)), ({}, (2, 1, 3)), ({"batch": 2}, (1, 1, 1)),
                                          ({"grid_t": 2, "hidden": 2048, "heads": 32, "head_dim": 64, "ffn": 4096}, (1, 2, 1)),
                                          ({"n_blocks": 2}, (1, 1, 2))])
