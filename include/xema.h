@@ -274,7 +274,8 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes,
 
 /* Puts a forward call's inputs into the arena: hid0 from hid_dev [B, rows owned, D] bf16 and temb
  * from temb_dev [B, Dt] bf16 (device, contiguous), in one launch (two plain copies where a
- * pointer is not 16-byte aligned).  Enqueues on `stream`.  XEMA_ESTATE if the plan is unbound. */
+ * pointer is not 16-byte aligned).  A source may be its own slot in the arena; one that overlaps a
+ * slot otherwise is refused (XEMA_EINVAL).  Enqueues on `stream`.  XEMA_ESTATE if the plan is unbound. */
 int xema_plan_set_inputs(const xema_plan* plan, const void* hid_dev, const void* temb_dev, void* stream);
 
 /* Enqueues the block (n_blocks must be 1) / all n_blocks blocks on `stream` (a cudaStream_t

@@ -593,6 +593,16 @@ int xema_plan_set_inputs(const xema_plan* plan, const void* hid_dev, const void*
   const xema_config& c = plan->cfg;
   const size_t hid_bytes = (size_t)2 * c.batch * (size_t)plan->own_rows * c.hidden;
   const size_t temb_bytes = (size_t)2 * c.batch * c.temb_dim;
+  // The two copies run side by side and in no order of their pieces: a source may be its own slot, but
+  // must not overlap a slot otherwise.
+  auto overlaps = [](const void* src, size_t n, const uint8_t* slot, size_t m) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src), b = reinterpret_cast<uintptr_t>(slot);
+    return a < b + m && b < a + n;
+  };
+  if ((hid_dev != plan->hid_in && overlaps(hid_dev, hid_bytes, plan->hid_in, hid_bytes)) ||
+      (temb_dev != plan->temb_in && overlaps(temb_dev, temb_bytes, plan->temb_in, temb_bytes)) ||
+      overlaps(hid_dev, hid_bytes, plan->temb_in, temb_bytes) || overlaps(temb_dev, temb_bytes, plan->hid_in, hid_bytes))
+    return XEMA_EINVAL;
   if (((reinterpret_cast<uintptr_t>(hid_dev) | reinterpret_cast<uintptr_t>(temb_dev)) & 15) == 0)
     return launch_copy2(plan->hid_in, hid_dev, hid_bytes, plan->temb_in, temb_dev, temb_bytes, st);
   cudaError_t e = cudaMemcpyAsync(plan->hid_in, hid_dev, hid_bytes, cudaMemcpyDeviceToDevice, st);

@@ -91,6 +91,7 @@ class BlockSession:
         self._views = {}
         self._out_name = "hid%d" % template.n_blocks
         self._index = self.arena.get_device()
+        self._arena_range = (self.arena.data_ptr(), self.arena.data_ptr() + self.arena.numel())
 
     # ---- views into the arena ---------------------------------------------------------
     def view(self, name: str, dtype=torch.int16, shape=None) -> torch.Tensor:
@@ -121,9 +122,13 @@ class BlockSession:
 
     # ---- data movement ------------------------------------------------------------------
     def _in_place(self, src, shape) -> bool:
-        """Whether the library can copy `src` as it stands."""
-        return (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.get_device() == self._index
-                and src.numel() == math.prod(shape) and src.is_contiguous())
+        """Whether the library can copy `src` as it stands.  A source inside the arena is left to torch,
+        which refuses one that overlaps its destination in part."""
+        if not (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.get_device() == self._index
+                and src.numel() == math.prod(shape) and src.is_contiguous()):
+            return False
+        at = src.data_ptr()
+        return at + 2 * src.numel() <= self._arena_range[0] or at >= self._arena_range[1]
 
     def set_inputs(self, x_bits, temb_bits, non_blocking: bool = False):
         """x_bits / temb_bits: uint16 numpy arrays or int16 torch tensors (host or device)."""

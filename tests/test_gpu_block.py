@@ -534,6 +534,38 @@ def test_set_inputs_takes_every_kind_of_source(batch, chunks):
         assert bool((s.arena[~slots] == 0x5A).all())
 
 
+def test_set_inputs_refuses_sources_that_overlap_their_slots():
+    """Sources inside the arena: the slot itself is fine, bytes elsewhere are copied, a source that overlaps
+    a slot in part is refused and nothing is copied."""
+    t = template("tiny")
+    x, temb = make_activations(t)
+    s = BlockSession(t, [make_block_weights(t, 0)], chunks=1)
+    s.set_inputs(x, temb)
+    before = s.arena.clone()
+    s.set_inputs(s.hid_in(), s.temb())
+    assert torch.equal(s.arena, before)
+    (hid, _), (te, _) = s.plan.tensor("hid0"), s.plan.tensor("temb")
+    n = 2 * s.hid_in().numel()
+
+    def inside(at):
+        return s.arena[at:at + n].view(torch.int16).view(s.hid_in().shape)
+
+    apart = [at for at in range(0, s.arena.numel() - n, 256) if (at >= hid + n or at + n <= hid) and (at >= te + 1024 or at + n <= te)]
+    assert apart
+    s.set_inputs(inside(apart[0]), torch.from_numpy(temb.view(np.int16)).to(DEV))
+    assert torch.equal(s.hid_in(), inside(apart[0]))
+    before = s.arena.clone()
+    at = hid + 256 if hid + 256 + n <= s.arena.numel() else hid - 256
+    with pytest.raises(RuntimeError):
+        s.set_inputs(inside(at), s.temb())
+    base, stream = s.arena.data_ptr(), torch.cuda.current_stream().cuda_stream
+    for a, b in ((base + at, base + te), (base + hid, base + te + 256), (base + hid, base + hid + 512), (base + te, base + te)):
+        with pytest.raises(xb.XemaError) as e:
+            s.plan.set_inputs(a, b, stream)
+        assert e.value.status == xb.XEMA_EINVAL
+    assert torch.equal(s.arena, before)
+
+
 def test_views_of_inputs_and_output_belong_to_the_caller():
     """Changing the shape of a returned view in place leaves later calls as they were."""
     t = template("tiny")
