@@ -397,7 +397,8 @@ typedef struct xema_gemm_args {
   const void* bias;     /* device bf16 [N]                                                 */
   void* out;            /* device, row (b,i) at element (b*out_batch_rows + i)*ldo         */
   int64_t ldo, out_batch_rows;
-  const void* resid;    /* device, same row addressing with ldr / resid_batch_rows; or NULL */
+  const void* resid;    /* device, same row addressing with ldr / resid_batch_rows (0: one row for
+                           all / the same rows for every batch element); or NULL             */
   int64_t ldr, resid_batch_rows;
   const float* gate;    /* device fp32, gate[b*gate_stride + n]; or NULL                   */
   int64_t gate_stride;

@@ -82,7 +82,7 @@ struct GemmParams {
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K;
-  int resid_batch;                  // 1: the residual has a batch dimension, 0: the same rows for every element
+  int resid_batch, resid_rows;      // 1: the residual has a batch dimension / rows of its own, 0: the same for all
   unsigned int* status;
   // XEMA_EPI_BIAS_NORM_ROPE only: heads that start below column norm_cols get RMSNorm * gain
   // and RoPE in the epilogue (a thread owns whole rows, hence whole heads, of the tile)
@@ -163,6 +163,7 @@ struct Epilogue {
   const float* gate;      // [BN] (gated) or the RMSNorm gain
   volatile uint32_t* abort_flag;
   int lane;
+  int rlane;              // row of a residual chunk that belongs to this lane
   uint32_t used = 0;      // chunks worked on so far (buffer = used % RING)
   uint32_t asked = 0;     // residual chunks requested so far
 
@@ -170,7 +171,7 @@ struct Epilogue {
     if (lane == 0) {
       uint64_t* bar = rbar + asked % RING;
       mbar_expect_tx(bar, EPI == XEMA_EPI_GATE_RES_F32 ? BUF_BYTES / 2 : BUF_BYTES);
-      tma_load_3d(ring + (asked % RING) * BUF_BYTES, map_res, bar, n0, row0, p.resid_batch ? b : 0);
+      tma_load_3d(ring + (asked % RING) * BUF_BYTES, map_res, bar, n0, p.resid_rows ? row0 : 0, p.resid_batch ? b : 0);
     }
     __syncwarp();
     ++asked;
@@ -204,7 +205,7 @@ struct Epilogue {
         // out fp32 = resid(bf16) + gate * v
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const uint4 x = *reinterpret_cast<const uint4*>(piece_b16(buf, lane, q));
+          const uint4 x = *reinterpret_cast<const uint4*>(piece_b16(buf, rlane, q));
           const float4 g0 = g[2 * q], g1 = g[2 * q + 1];
           v[8 * q + 0] = fmaf(g0.x, v[8 * q + 0], bf16_lo(x.x));
           v[8 * q + 1] = fmaf(g0.y, v[8 * q + 1], bf16_hi(x.x));
@@ -219,7 +220,7 @@ struct Epilogue {
         // out bf16 = resid(fp32) + gate * v
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const float4 x = *reinterpret_cast<const float4*>(piece_f32(buf, lane, q));
+          const float4 x = *reinterpret_cast<const float4*>(piece_f32(buf, rlane, q));
           const float4 gg = g[q];
           v[4 * q + 0] = fmaf(gg.x, v[4 * q + 0], x.x);
           v[4 * q + 1] = fmaf(gg.y, v[4 * q + 1], x.y);
@@ -537,7 +538,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     float* s_bias = reinterpret_cast<float*>(smem + Cfg::OFF_BIAS);
     float* s_gate = reinterpret_cast<float*>(smem + Cfg::OFF_GATE);
     Epilogue<EPI, BN, PAIR> ep{p, &map_out, &map_res, smem + Cfg::OFF_RING + quad * RING * BUF_BYTES, res_full + quad * RING,
-                               s_bias, s_gate, abort_flag, lane};
+                               s_bias, s_gate, abort_flag, lane, p.resid_rows ? lane : 0};
     const int et = threadIdx.x - 64;     // 0..127
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -649,7 +650,8 @@ GemmParams make_params(const GemmLaunch& g) {
   p.rows = g.rows;
   p.N = g.N;
   p.K = g.K;
-  p.resid_batch = g.resid_batch_rows != 0;
+  p.resid_batch = g.resid_batch_rows * g.ldr != 0;
+  p.resid_rows = g.ldr != 0;
   p.status = g.status;
   p.norm_gain = (const __nv_bfloat16*)g.norm_gain;
   p.rope = g.rope;
@@ -780,6 +782,10 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
       return XEMA_EINVAL;
     if ((reinterpret_cast<uintptr_t>(g->norm_gain) & 15) || (reinterpret_cast<uintptr_t>(g->rope) & 15)) return XEMA_EALIGN;
   }
+  // Result rows lie behind one another; residual rows may be shared (ldr = 0: one row for all,
+  // resid_batch_rows = 0: the same rows for every batch element).
+  if ((g->rows > 1 && g->ldo < g->N) || (g->batch > 1 && (g->ldo < 1 || g->out_batch_rows < 1))) return XEMA_EINVAL;
+  if (gated && (g->ldr < 0 || g->resid_batch_rows < 0)) return XEMA_EINVAL;
   if ((lda & 7) || (ldw & 7) || (g->ldo & 7) || (gated && (g->ldr & 7))) return XEMA_EALIGN;
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
   if (mis(a) || mis(w) || mis(g->bias) || mis(g->out) || (g->resid && mis(g->resid)) || (g->gate && mis(g->gate)))
@@ -798,11 +804,11 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   if (rc) return rc;
   // results leave, and residuals arrive, as boxes of 32 columns x 32 rows
   rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, g->N, rows, g->batch, g->ldo,
-                         g->out_batch_rows);
+                         g->out_batch_rows * g->ldo);
   if (rc || !gated) return rc;
-  const bool per_batch = g->resid_batch_rows != 0;
-  return encode_tmap_box32(&g->map_res, g->resid, g->epilogue == XEMA_EPI_GATE_RES_BF16, g->N, rows,
-                           per_batch ? g->batch : 1, g->ldr, g->resid_batch_rows);
+  const long long resid_stride = g->resid_batch_rows * g->ldr;
+  return encode_tmap_box32(&g->map_res, g->resid, g->epilogue == XEMA_EPI_GATE_RES_BF16, g->N, g->ldr ? rows : 1,
+                           resid_stride ? g->batch : 1, g->ldr, resid_stride);
 }
 
 }  // namespace xema

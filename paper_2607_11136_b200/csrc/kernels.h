@@ -89,10 +89,11 @@ int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void
 // columns read as zero.
 int encode_tmap_bf16(CUtensorMap* out, const void* base, long long cols, long long rows, long long batch,
                      long long ld, long long batch_rows, int box_rows);
-// bf16 or fp32 tensor viewed the same way; box = 32 columns x 32 rows x 1, swizzled over its
-// 64-byte (bf16) or 128-byte (fp32) rows.
+// bf16 or fp32 tensor viewed the same way, its batch stride given in elements; box = 32 columns x 32 rows x 1,
+// swizzled over its 64-byte (bf16) or 128-byte (fp32) rows.  The row stride of a single row and the batch
+// stride of a single element are not looked at.
 int encode_tmap_box32(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
-                      long long ld, long long batch_rows);
+                      long long ld, long long batch_stride);
 
 // ---- GEMM ------------------------------------------------------------------------------------
 struct GemmLaunch {

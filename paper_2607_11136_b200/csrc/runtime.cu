@@ -66,13 +66,12 @@ static EncodeTiledFn encode_fn() {
 }
 
 static int encode_tmap(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
-                       long long ld, long long batch_rows, int box_cols, int box_rows, CUtensorMapSwizzle swizzle) {
+                       long long ld, long long batch_stride, int box_cols, int box_rows, CUtensorMapSwizzle swizzle) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return XEMA_ECUDA;
   const int elem = f32 ? 4 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch};
-  long long bstride = (batch_rows > 0 ? batch_rows : rows) * ld * elem;
-  cuuint64_t strides[2] = {(cuuint64_t)(ld * elem), (cuuint64_t)bstride};
+  cuuint64_t strides[2] = {(cuuint64_t)(ld * elem), (cuuint64_t)(batch_stride * elem)};
   cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1u};
   cuuint32_t estr[3] = {1u, 1u, 1u};
   CUresult r = fn(out, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base),
@@ -90,14 +89,18 @@ int encode_tmap_bf16(CUtensorMap* out, const void* base, long long cols, long lo
   if (cols < 64 || rows < 1 || batch < 1 || ld < cols || box_rows < 1 || box_rows > 256) return XEMA_EINVAL;
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return XEMA_EALIGN;
   if (batch > 1 && batch_rows < rows) return XEMA_EINVAL;
-  return encode_tmap(out, base, false, cols, rows, batch, ld, batch_rows, 64, box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+  return encode_tmap(out, base, false, cols, rows, batch, ld, (batch_rows > 0 ? batch_rows : rows) * ld, 64, box_rows,
+                     CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 int encode_tmap_box32(CUtensorMap* out, const void* base, bool f32, long long cols, long long rows, long long batch,
-                      long long ld, long long batch_rows) {
-  if (cols < 32 || rows < 1 || batch < 1 || ld < cols) return XEMA_EINVAL;
-  if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7)) return XEMA_EALIGN;
-  return encode_tmap(out, base, f32, cols, rows, batch, ld, batch_rows, 32, 32,
+                      long long ld, long long batch_stride) {
+  if (cols < 32 || (cols & 7) || rows < 1 || batch < 1) return XEMA_EINVAL;
+  if (rows == 1) ld = cols;
+  if (batch == 1) batch_stride = rows * ld;
+  if (ld < 1 || batch_stride < 1) return XEMA_EINVAL;
+  if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld & 7) || (batch_stride & 7)) return XEMA_EALIGN;
+  return encode_tmap(out, base, f32, cols, rows, batch, ld, batch_stride, 32, 32,
                      f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 

@@ -31,6 +31,28 @@ def test_struct_sizes_match_the_header():
     assert ctypes.sizeof(xb.xema_gemm_args) == 168
 
 
+def test_gemm_layouts_that_are_refused():
+    """Results whose rows or batch elements would lie over one another, and negative residual strides, are
+    refused before any CUDA call; rows that nothing strides over and shared residual rows are not."""
+    base = dict(a=256, lda=64, a_batch_rows=4, w=256, ldw=64, bias=256, out=256, ldo=128, out_batch_rows=4, resid=256,
+                ldr=128, resid_batch_rows=4, gate=256, gate_stride=128, batch=2, rows=4, N=128, K=64, epilogue=2)
+    for over, refused in ((dict(out_batch_rows=0), True), (dict(out_batch_rows=-4), True), (dict(ldo=64), True),
+                          (dict(ldr=-128), True), (dict(resid_batch_rows=-1), True),
+                          (dict(ldr=0), False), (dict(resid_batch_rows=0), False), (dict(ldr=0, resid_batch_rows=0), False),
+                          (dict(rows=1, batch=1, ldo=0, ldr=0, out_batch_rows=0), False)):
+        try:
+            # (a null stream; without a driver the descriptors cannot be made, which is another status)
+            args = xb.xema_gemm_args()
+            for k, v in {**base, **over}.items():
+                setattr(args, k, v)
+            args.rows = args.rows if refused else 0     # nothing to launch
+            xb._check(xb.lib().xema_op_gemm(ctypes.byref(args), None, None), "xema_op_gemm")
+            status = 0
+        except xb.XemaError as e:
+            status = e.status
+        assert (status == xb.XEMA_EINVAL) == refused, (over, status)
+
+
 def test_error_paths_without_gpu():
     assert xb.version().startswith("xema-b200")
     assert xb.strerror(0) == "ok" and "budget" in xb.strerror(xb.XEMA_EBUDGET)

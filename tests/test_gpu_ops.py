@@ -210,6 +210,40 @@ def test_gemm_tile_forms_give_the_same_bits(N, K):
     assert_bf16_close(got, ref, ("gemm small tile", N, K), atol_rms=2e-4)
 
 
+@pytest.mark.parametrize("epi", [xb.EPI_GATE_RES_F32, xb.EPI_GATE_RES_BF16])
+@pytest.mark.parametrize("rows,N", [(1, 256), (37, 384), (300, 512), (700, 1536)])
+def test_gemm_residual_rows_may_be_shared(epi, rows, N):
+    """ldr = 0: one residual row for all; resid_batch_rows = 0: the same rows for every batch element;
+    overlapping residual rows; one row with no row stride at all.  The same bits as with the residual
+    written out."""
+    rng = np.random.default_rng(60 + rows)
+    B, K = 2, 128
+    a_dev, w_dev, b_dev = (to_dev(rand_bf16(rng, s, c)[0]) for s, c in (((B, rows, K), 1.0), ((N, K), 0.05), ((N,), 0.5)))
+    gate = torch.from_numpy(rng.standard_normal((B, N), dtype=np.float32)).to(DEV)
+    f32 = epi == xb.EPI_GATE_RES_F32
+    flat = torch.from_numpy(rng.standard_normal(B * rows * N + N, dtype=np.float32)).to(DEV)
+    flat = flat.to(torch.bfloat16) if f32 else flat
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+    def run(resid, ldr, batch_rows, batch=B, ldo=N):
+        out = torch.zeros(B, rows, N, dtype=torch.float32 if f32 else torch.bfloat16, device=DEV)
+        xb.xema_op_gemm(status=status.data_ptr(), a=a_dev.data_ptr(), lda=K, a_batch_rows=rows, w=w_dev.data_ptr(), ldw=K,
+                        bias=b_dev.data_ptr(), out=out.data_ptr(), ldo=ldo, out_batch_rows=rows if batch > 1 else 0, batch=batch,
+                        rows=rows, N=N, K=K, epilogue=epi, resid=resid.data_ptr(), ldr=ldr, resid_batch_rows=batch_rows,
+                        gate=gate.data_ptr(), gate_stride=N)
+        return out
+
+    one_row = flat[:N].expand(B, rows, N).contiguous()
+    same_rows = flat[:rows * N].view(1, rows, N).expand(B, rows, N).contiguous()
+    assert torch.equal(run(flat, 0, rows), run(one_row, N, rows)) and torch.equal(run(flat, 0, 0), run(one_row, N, rows))
+    assert torch.equal(run(flat, N, 0), run(same_rows, N, rows))
+    windows = flat.as_strided((B, rows, N), (rows * 64, 64, 1)).contiguous()
+    assert torch.equal(run(flat, 64, rows), run(windows, N, rows))
+    if rows == 1:
+        assert torch.equal(run(flat, 0, 0, batch=1, ldo=0)[:1], run(flat, N, 1, batch=1)[:1])
+    _sync_status(status)
+
+
 def test_gemm_many_tiles_persistent():
     """More tiles than SMs so every CTA runs several tiles through both TMEM accumulators."""
     rng = np.random.default_rng(7)
