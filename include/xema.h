@@ -416,6 +416,13 @@ typedef struct xema_gemm_args {
   const float* rope;     /* device fp32 [tokens][head_dim/2][cos, sin]                      */
 } xema_gemm_args;
 int xema_op_gemm(const xema_gemm_args* args, void* status_dev, void* stream);
+/* For tests: the tile xema_op_gemm takes for these sizes on the current device (host only; pointers
+ * and strides are not looked at) -- *pair 1: 256 x *block_n over two SMs, 0: 128 x *block_n on one -- and the
+ * same product in a tile of the caller's choice ({1, 256}, {1, 128}, {0, 128}, {0, 64}, gated epilogues
+ * {0, 32}; XEMA_EINVAL where the problem cannot run in it).  The results are the same bits in all. */
+int xema_gemm_tile(const xema_gemm_args* args, int32_t* pair, int32_t* block_n);
+int xema_op_gemm_in_tile(const xema_gemm_args* args, int32_t pair, int32_t block_n, void* status_dev,
+                         void* stream);
 
 /* Non-causal attention of `rows` query rows against all `keys` keys, per (batch, head):
  * o = softmax(q k^T / sqrt(head_dim)) v, lse = log sum exp (natural log).

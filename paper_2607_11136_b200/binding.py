@@ -27,7 +27,7 @@ EXPORTS = (
     "xema_block_forward_static",
     "xema_shard_rows", "xema_trace_sharded", "xema_plan_create_sharded", "xema_plan_shard", "xema_plan_gather_point", "xema_plan_create_guarded", "xema_plan_guard_bytes",
     "xema_plan_launch_count", "xema_forward_host", "xema_forward_prefix", "xema_forward_range", "xema_plan_op", "xema_op_mod", "xema_op_ln_modulate",
-    "xema_op_rmsnorm_rope", "xema_op_gemm", "xema_op_attention", "xema_strerror",
+    "xema_op_rmsnorm_rope", "xema_op_gemm", "xema_gemm_tile", "xema_op_gemm_in_tile", "xema_op_attention", "xema_strerror",
     "xema_last_cuda_error", "xema_version", "xema_selftest_wait_timeout",
     "xema_pluggable_malloc", "xema_pluggable_free", "xema_pluggable_mode", "xema_pluggable_recorded",
     "xema_pluggable_set_plan", "xema_pluggable_step_begin", "xema_pluggable_stats",
@@ -137,6 +137,8 @@ def lib() -> C.CDLL:
             "xema_op_ln_modulate": [vp, i32, i64, vp, vp, vp, i64, i32, i32, i32, C.c_float, vp],
             "xema_op_rmsnorm_rope": [vp, i64, i64, vp, vp, i32, i32, i32, i32, i32, C.c_float, vp],
             "xema_op_gemm": [P(xema_gemm_args), vp, vp],
+            "xema_gemm_tile": [P(xema_gemm_args), P(i32), P(i32)],
+            "xema_op_gemm_in_tile": [P(xema_gemm_args), i32, i32, vp, vp],
             "xema_op_attention": [vp, i64, i64, vp, vp, i64, i64, vp, vp, i32, i32, i32, i32, i32, C.c_float, vp, vp],
             "xema_last_cuda_error": [],
             "xema_selftest_wait_timeout": [vp, i64, vp, vp],
@@ -515,10 +517,25 @@ def xema_op_rmsnorm_rope(x, ld, batch_rows, g, rope, pos0, batch, rows, heads, h
 
 
 def xema_op_gemm(status=None, stream=0, **kw):
+    _check(lib().xema_op_gemm(C.byref(_gemm_args(kw)), status, stream), "xema_op_gemm")
+
+
+def _gemm_args(kw) -> xema_gemm_args:
     a = xema_gemm_args()
     for k, v in kw.items():
         setattr(a, k, v)
-    _check(lib().xema_op_gemm(C.byref(a), status, stream), "xema_op_gemm")
+    return a
+
+
+def xema_gemm_tile(**kw):
+    """-> (pair, block_n): the tile xema_op_gemm takes for these sizes."""
+    pair, block_n = C.c_int32(), C.c_int32()
+    _check(lib().xema_gemm_tile(C.byref(_gemm_args(kw)), C.byref(pair), C.byref(block_n)), "xema_gemm_tile")
+    return pair.value, block_n.value
+
+
+def xema_op_gemm_in_tile(pair, block_n, status=None, stream=0, **kw):
+    _check(lib().xema_op_gemm_in_tile(C.byref(_gemm_args(kw)), pair, block_n, status, stream), "xema_op_gemm_in_tile")
 
 
 def exponent_scale(head_dim: int) -> float:

@@ -733,18 +733,23 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // gated epilogues, whose products are narrow: 288 x 512 x 2048 12.1 -> 10.4 us, a step of 8 blocks of 333 tokens
 // x 1024 521 -> 500.
 // The bits of a row do not depend on the choice.
+struct Tile {
+  int pair, block_n, block_ns, epilogue_ns;
+};
+constexpr Tile kTiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}, {0, 32, 150, 400}};
+
+bool tile_fits(const GemmLaunch& g, const Tile& t) {
+  if (g.N % t.block_n) return false;
+  if (t.block_n < 64 && g.epilogue != XEMA_EPI_GATE_RES_F32 && g.epilogue != XEMA_EPI_GATE_RES_BF16) return false;
+  return g.epilogue != XEMA_EPI_BIAS_NORM_ROPE || t.block_n >= g.head_dim;   // whole heads only
+}
+
 void pick_tile(GemmLaunch* g) {
-  struct Tile {
-    int pair, block_n, block_ns, epilogue_ns;
-  };
-  static const Tile tiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}, {0, 32, 150, 400}};
   const long long k_blocks = g->K / BK;
   long long best = 0;
   g->block_n = 0;
-  for (const Tile& t : tiles) {
-    if (g->N % t.block_n) continue;
-    if (t.block_n < 64 && g->epilogue != XEMA_EPI_GATE_RES_F32 && g->epilogue != XEMA_EPI_GATE_RES_BF16) continue;
-    if (g->epilogue == XEMA_EPI_BIAS_NORM_ROPE && t.block_n < g->head_dim) continue;   // whole heads only
+  for (const Tile& t : kTiles) {
+    if (!tile_fits(*g, t)) continue;
     const int rows = t.pair ? 2 * BM : BM;
     const long long n = (long long)g->batch * ((g->rows + rows - 1) / rows) * (g->N / t.block_n);
     const long long workers = std::max(1, t.pair ? sm_count() / 2 : sm_count());
@@ -755,6 +760,15 @@ void pick_tile(GemmLaunch* g) {
       g->pair = t.pair;
     }
   }
+}
+
+// The sizes and flags of a problem, without its pointers.
+int check_shape(const GemmLaunch& g) {
+  if (g.batch < 1 || g.rows < 0 || g.N < 128 || (g.N % 128) || g.K < 64 || (g.K % 64)) return XEMA_EINVAL;
+  if (g.epilogue < XEMA_EPI_BIAS || g.epilogue > XEMA_EPI_BIAS_NORM_ROPE) return XEMA_EINVAL;
+  if (g.epilogue != XEMA_EPI_BIAS_NORM_ROPE) return XEMA_OK;
+  if (g.head_dim != 64 && g.head_dim != 128) return XEMA_EINVAL;
+  return g.norm_cols < 0 || g.norm_cols > g.N || g.norm_cols % g.head_dim || g.N % 256 || g.rope_pos0 < 0 ? XEMA_EINVAL : XEMA_OK;
 }
 }  // namespace
 
@@ -770,16 +784,20 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained) {
   }
 }
 
-int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw) {
-  if (g->batch < 1 || g->rows < 0 || g->N < 128 || (g->N % 128) || g->K < 64 || (g->K % 64)) return XEMA_EINVAL;
-  if (g->epilogue < XEMA_EPI_BIAS || g->epilogue > XEMA_EPI_BIAS_NORM_ROPE) return XEMA_EINVAL;
+int gemm_tile(GemmLaunch* g) {
+  if (int rc = check_shape(*g)) return rc;
+  pick_tile(g);
+  return XEMA_OK;
+}
+
+int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw,
+                 const int* tile) {
+  if (int rc = check_shape(*g)) return rc;
   if (!a || !w || !g->bias || !g->out) return XEMA_EINVAL;
   const bool gated = g->epilogue == XEMA_EPI_GATE_RES_F32 || g->epilogue == XEMA_EPI_GATE_RES_BF16;
   if (gated && (!g->resid || !g->gate)) return XEMA_EINVAL;
   if (g->epilogue == XEMA_EPI_BIAS_NORM_ROPE) {
-    if (!g->norm_gain || !g->rope || (g->head_dim != 64 && g->head_dim != 128)) return XEMA_EINVAL;
-    if (g->norm_cols < 0 || g->norm_cols > g->N || g->norm_cols % g->head_dim || g->N % 256 || g->rope_pos0 < 0)
-      return XEMA_EINVAL;
+    if (!g->norm_gain || !g->rope) return XEMA_EINVAL;
     if ((reinterpret_cast<uintptr_t>(g->norm_gain) & 15) || (reinterpret_cast<uintptr_t>(g->rope) & 15)) return XEMA_EALIGN;
   }
   // Result rows lie behind one another; residual rows may be shared (ldr = 0: one row for all,
@@ -795,7 +813,17 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   g->lda = lda;
   g->a_batch_rows = a_batch_rows;
   g->ldw = ldw;
-  pick_tile(g);
+  if (!tile) {
+    pick_tile(g);
+  } else {
+    g->block_n = 0;
+    for (const Tile& t : kTiles)
+      if (t.pair == tile[0] && t.block_n == tile[1] && tile_fits(*g, t)) {
+        g->pair = t.pair;
+        g->block_n = t.block_n;
+      }
+    if (!g->block_n) return XEMA_EINVAL;
+  }
   const long long rows = g->rows > 0 ? g->rows : 1;
   int rc = encode_tmap_bf16(&g->map_a, a, g->K, rows, g->batch, lda, a_batch_rows, BM);
   if (rc) return rc;

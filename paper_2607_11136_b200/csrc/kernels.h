@@ -120,8 +120,12 @@ struct GemmLaunch {
   float rms_eps;
   float norm_out_scale;   // the normalised, rotated heads are multiplied by this before rounding (1 = as they are)
 };
-// Fills the descriptors and block_n (tile width) from plain pointers.
-int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw);
+// Fills the descriptors and the tile (pair, block_n) from plain pointers.  `tile`: {pair, block_n} to take instead
+// of the one estimated to be fastest, XEMA_EINVAL where the problem cannot run in it.
+int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw,
+                 const int* tile = nullptr);
+// The tile alone, on the host (GemmLaunch as for gemm_prepare): fills pair and block_n.
+int gemm_tile(GemmLaunch* g);
 int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained = false);
 
 // ---- attention -------------------------------------------------------------------------------

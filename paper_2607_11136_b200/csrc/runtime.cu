@@ -928,8 +928,7 @@ int xema_op_rmsnorm_rope(void* x, int64_t ld, int64_t batch_rows, const void* g,
                              reinterpret_cast<cudaStream_t>(stream));
 }
 
-int xema_op_gemm(const xema_gemm_args* a, void* status_dev, void* stream) {
-  if (!a) return XEMA_EINVAL;
+static GemmLaunch gemm_launch_of(const xema_gemm_args* a, void* status_dev) {
   GemmLaunch g{};
   g.bias = a->bias; g.out = a->out; g.ldo = a->ldo; g.out_batch_rows = a->out_batch_rows;
   g.resid = a->resid; g.ldr = a->ldr; g.resid_batch_rows = a->resid_batch_rows;
@@ -938,7 +937,32 @@ int xema_op_gemm(const xema_gemm_args* a, void* status_dev, void* stream) {
   g.norm_gain = a->norm_gain; g.rope = a->rope; g.rope_pos0 = a->rope_pos0; g.head_dim = a->head_dim;
   g.norm_cols = a->norm_cols; g.rms_eps = a->rms_eps; g.norm_out_scale = a->norm_out_scale;
   g.status = static_cast<unsigned int*>(status_dev);
+  return g;
+}
+
+int xema_op_gemm(const xema_gemm_args* a, void* status_dev, void* stream) {
+  if (!a) return XEMA_EINVAL;
+  GemmLaunch g = gemm_launch_of(a, status_dev);
   int rc = gemm_prepare(&g, a->a, a->lda, a->a_batch_rows, a->w, a->ldw);
+  if (rc) return rc;
+  return launch_gemm(g, reinterpret_cast<cudaStream_t>(stream));
+}
+
+int xema_gemm_tile(const xema_gemm_args* a, int32_t* pair, int32_t* block_n) {
+  if (!a || !pair || !block_n) return XEMA_EINVAL;
+  GemmLaunch g = gemm_launch_of(a, nullptr);
+  int rc = gemm_tile(&g);
+  if (rc) return rc;
+  *pair = g.pair;
+  *block_n = g.block_n;
+  return XEMA_OK;
+}
+
+int xema_op_gemm_in_tile(const xema_gemm_args* a, int32_t pair, int32_t block_n, void* status_dev, void* stream) {
+  if (!a) return XEMA_EINVAL;
+  GemmLaunch g = gemm_launch_of(a, status_dev);
+  const int tile[2] = {pair, block_n};
+  int rc = gemm_prepare(&g, a->a, a->lda, a->a_batch_rows, a->w, a->ldw, tile);
   if (rc) return rc;
   return launch_gemm(g, reinterpret_cast<cudaStream_t>(stream));
 }
