@@ -94,6 +94,7 @@ class BlockSession:
         self.seq = self.plan.rows          # token rows of this session's tensors (all of them unless sharded)
         self._hid_shape = (template.batch, self.seq, template.hidden)
         self._temb_shape = (template.batch, template.temb_dim)
+        self._hid_numel, self._temb_numel = math.prod(self._hid_shape), math.prod(self._temb_shape)
         self._views = {}
         self._out_name = "hid%d" % template.n_blocks
         self._index = self.arena.get_device()
@@ -127,20 +128,22 @@ class BlockSession:
         return self._view_once(self._out_name, self._hid_shape)
 
     # ---- data movement ------------------------------------------------------------------
-    def _in_place(self, src, shape) -> bool:
-        """Whether the library can copy `src` as it stands.  A source inside the arena is left to torch,
-        which refuses one that overlaps its destination in part."""
+    def _address(self, src, numel: int) -> int:
+        """Where `src` stands if the library can copy it as it is, else 0.  A source inside the arena is
+        left to torch, which refuses one that overlaps its destination in part."""
         if not (isinstance(src, torch.Tensor) and src.dtype == torch.int16 and src.get_device() == self._index
-                and src.numel() == math.prod(shape) and src.is_contiguous()):
-            return False
+                and src.numel() == numel and src.is_contiguous()):
+            return 0
         at = src.data_ptr()
-        return at + 2 * src.numel() <= self._arena_range[0] or at >= self._arena_range[1]
+        first, end = self._arena_range
+        return at if at + 2 * numel <= first or at >= end else 0
 
     def set_inputs(self, x_bits, temb_bits, non_blocking: bool = False):
         """x_bits / temb_bits: uint16 numpy arrays or int16 torch tensors (host or device)."""
-        if (self._in_place(x_bits, self._hid_shape) and self._in_place(temb_bits, self._temb_shape)
-                and _current_device() == self._index):
-            self.plan.set_inputs(x_bits.data_ptr(), temb_bits.data_ptr(), self._raw_stream())
+        x_at = self._address(x_bits, self._hid_numel)
+        temb_at = x_at and self._address(temb_bits, self._temb_numel)
+        if temb_at and _current_device() == self._index:
+            self.plan.set_inputs(x_at, temb_at, self._raw_stream())
             return
         for dst, src in ((self.hid_in(), x_bits), (self.temb(), temb_bits)):
             if isinstance(src, np.ndarray):
