@@ -732,7 +732,9 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.  128 x 32 exists for the
 // gated epilogues, whose products are narrow: 288 x 512 x 2048 12.1 -> 10.4 us, a step of 8 blocks of 333 tokens
 // x 1024 521 -> 500.
-// The bits of a row do not depend on the choice.
+// The 256 x 256 figure was taken under the power cap, as launches that need it run, the small tiles' at full clock, as
+// theirs do.  Pairs are counted as SMs / 2, all of which are resident on a B200 (74); where fewer fit, the launch
+// takes those and only the estimate is off.  The bits of a row do not depend on the choice.
 struct Tile {
   int pair, block_n, block_ns, epilogue_ns;
 };

@@ -98,7 +98,7 @@ int encode_tmap_box32(CUtensorMap* out, const void* base, bool f32, long long co
 // ---- GEMM ------------------------------------------------------------------------------------
 struct GemmLaunch {
   CUtensorMap map_a;   // [batch][rows][K], box 64 x 128
-  CUtensorMap map_w;   // [1][N][K],       box 64 x 128 (64 x 64 for the 64-column tile)
+  CUtensorMap map_w;   // [1][N][K],       box 64 x block_n (a pair: each CTA half of it)
   CUtensorMap map_out; // [batch][rows][N], box 32 x 32
   CUtensorMap map_res; // the same for the residual (gated epilogues)
   const void* bias;    // bf16 [N]

@@ -657,8 +657,8 @@ static int sub_op(const xema_config& c, const Op& op, long long b0, int nb, long
 // The pieces in which the work of an op on `batch` elements x `rows` token rows follows its copies:
 // single batch elements, or, for one element, rows that fill the GPU's CTA pairs with 256 x 256 tiles of
 // the D-wide products twice (3072 rows of 3072 columns on 74 pairs), or once where that gives less than two
-// pieces; with `fine_end` the last one is halved, because nothing hides its copy.  Copies under 4 MB are not
-// worth an event.
+// pieces; with `fine_end` a last piece of more than one such wave and less than two is halved, because nothing hides
+// its copy (whole pieces stay as they are).  Copies under 4 MB are not worth an event.
 static std::vector<std::pair<long long, long long>> host_pieces(const xema_config& c, int batch, int rows, bool fine_end) {
   std::vector<std::pair<long long, long long>> out;      // [begin, end) in elements (batch > 1) or rows
   const long long row_bytes = 2LL * c.hidden, total = batch > 1 ? batch : rows;
