@@ -53,7 +53,12 @@ constexpr int BUF_BYTES = 4096;  // one staging buffer: 32 rows x 32 columns of 
 template <int EPI>
 constexpr bool kGated = EPI == XEMA_EPI_GATE_RES_F32 || EPI == XEMA_EPI_GATE_RES_BF16;
 
-template <int EPI, int BN, bool PAIR>
+// The wide tile has room for five stages and a ring of four residual chunks per epilogue warp, or (DEEP) for six stages
+// and two chunks.  The sixth stage keeps the main loop fed over many tiles, the longer ring shortens the epilogue
+// of a CTA's last one: 5 + 4 against 6 + 2 with a bf16 residual, K = 3072, N = 3072, us: 4444 rows 76.3 / 77.9, 4608
+// 77.0 / 77.9, 8888 149.6 / 145.5, 17776 292 / 283, 36000 575 / 554.  With an fp32 residual (K = 12288) 6 + 2 is 0 to 2 %
+// slower at every size.
+template <int EPI, int BN, bool PAIR, bool DEEP = false>
 struct GemmCfg {
   static constexpr int W_ROWS = PAIR ? BN / 2 : BN;            // rows of W a CTA loads per K block
   static constexpr int W_TILE_BYTES = W_ROWS * BK * 2;
@@ -64,9 +69,9 @@ struct GemmCfg {
   static constexpr int STAGE_BYTES = KSUB * (A_TILE_BYTES + W_TILE_BYTES);
   static constexpr int OFF_W = KSUB * A_TILE_BYTES;            // in a stage
   // staging buffers per epilogue warp: the gated epilogues keep residual chunks in flight
-  static constexpr int RING = kGated<EPI> && BN == 256 ? 4 : 2;
+  static constexpr int RING = kGated<EPI> && BN == 256 && !DEEP ? 4 : 2;
   static constexpr int RING_BYTES = 4 * RING * BUF_BYTES;
-  static constexpr int STAGES = BN == 256 ? (kGated<EPI> ? 5 : 6) : 196608 / STAGE_BYTES;
+  static constexpr int STAGES = BN == 256 ? (kGated<EPI> && !DEEP ? 5 : 6) : 196608 / STAGE_BYTES;
   static constexpr int OFF_RING = STAGES * STAGE_BYTES;
   static constexpr int OFF_BIAS = OFF_RING + RING_BYTES;       // float [BN]: bias
   static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
@@ -150,9 +155,9 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, int m_tiles, int n_til
 constexpr long long kDrainLimitCycles = 100000000ll;
 
 // One epilogue warp: its staging ring and the chunks of one tile.
-template <int EPI, int BN, bool PAIR>
+template <int EPI, int BN, bool PAIR, bool DEEP>
 struct Epilogue {
-  using Cfg = GemmCfg<EPI, BN, PAIR>;
+  using Cfg = GemmCfg<EPI, BN, PAIR, DEEP>;
   static constexpr int RING = Cfg::RING;
   const GemmParams& p;
   const CUtensorMap* map_out;
@@ -324,10 +329,10 @@ struct Epilogue {
   }
 };
 
-template <int EPI, int BN, bool PAIR>
+template <int EPI, int BN, bool PAIR, bool DEEP>
 __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_out,
                                           const CUtensorMap& map_res, const GemmParams& p) {
-  using Cfg = GemmCfg<EPI, BN, PAIR>;
+  using Cfg = GemmCfg<EPI, BN, PAIR, DEEP>;
   constexpr int STAGES = Cfg::STAGES, RING = Cfg::RING, KSUB = Cfg::KSUB;
   constexpr bool GATED = kGated<EPI>;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -537,7 +542,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     const int quad = warp & 3;           // TMEM lanes [32*quad, 32*quad + 32) belong to this warp
     float* s_bias = reinterpret_cast<float*>(smem + Cfg::OFF_BIAS);
     float* s_gate = reinterpret_cast<float*>(smem + Cfg::OFF_GATE);
-    Epilogue<EPI, BN, PAIR> ep{p, &map_out, &map_res, smem + Cfg::OFF_RING + quad * RING * BUF_BYTES, res_full + quad * RING,
+    Epilogue<EPI, BN, PAIR, DEEP> ep{p, &map_out, &map_res, smem + Cfg::OFF_RING + quad * RING * BUF_BYTES, res_full + quad * RING,
                                s_bias, s_gate, abort_flag, lane, p.resid_rows ? lane : 0};
     const int et = threadIdx.x - 64;     // 0..127
     int acc = 0;
@@ -630,14 +635,14 @@ template <int EPI, int BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmParams p) {
-  gemm_body<EPI, BN, false>(map_a, map_w, map_out, map_res, p);
+  gemm_body<EPI, BN, false, false>(map_a, map_w, map_out, map_res, p);
 }
-template <int EPI, int BN>
+template <int EPI, int BN, bool DEEP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                       const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
                       const GemmParams p) {
-  gemm_body<EPI, BN, true>(map_a, map_w, map_out, map_res, p);
+  gemm_body<EPI, BN, true, DEEP>(map_a, map_w, map_out, map_res, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -675,11 +680,11 @@ int launch_single(const GemmLaunch& g, cudaStream_t stream, bool chained) {
                        make_params(g));
 }
 
-template <int EPI, int BN>
+template <int EPI, int BN, bool DEEP = false>
 int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
-  using Cfg = GemmCfg<EPI, BN, true>;
+  using Cfg = GemmCfg<EPI, BN, true, DEEP>;
   static PerDeviceInt attr_done;
-  auto kern = gemm_bf16_pair_kernel<EPI, BN>;
+  auto kern = gemm_bf16_pair_kernel<EPI, BN, DEEP>;
   if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
   // A persistent grid must be resident all at once: ask how many CTA pairs fit on the device
   // (SMs are handed out to clusters in hardware groups, so it can be fewer than SMs / 2).
@@ -715,13 +720,17 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 
 template <int EPI>
 int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
+  if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
+    // six stages from four tiles a pair on (5.7 of them at 8888 rows x 3072 columns are 3 % faster, 2.9 at 4608 1 % slower)
+    const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / 256);
+    if (g.pair && g.block_n == 256 && tiles > 4LL * (sm_count() / 2)) return launch_pair<EPI, 256, true>(g, stream, chained);
+  }
   if (g.pair) return g.block_n == 256 ? launch_pair<EPI, 256>(g, stream, chained) : launch_pair<EPI, 128>(g, stream, chained);
   if (g.block_n == 128) return launch_single<EPI, 128>(g, stream, chained);
   if (g.block_n == 64) return launch_single<EPI, 64>(g, stream, chained);
   if constexpr (kGated<EPI>) return launch_single<EPI, 32>(g, stream, chained);
   return XEMA_EINVAL;
 }
-
 
 // Tile for a problem: the one with the shortest estimated time, waves x K blocks x nanoseconds per K
 // block plus what its last tile's epilogue adds.  Measured (B200, shapes from 288 x 512 x 2048 to 8888 x 12288 x

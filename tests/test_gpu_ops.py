@@ -277,6 +277,36 @@ def test_gemm_residual_rows_may_be_shared(epi, rows, N):
     _sync_status(status)
 
 
+@pytest.mark.parametrize("rows", [256 * 49 + 1, 256 * 51 - 31])
+def test_gemm_wide_gated_tile_with_many_tiles_per_pair(rows):
+    """More than four 256 x 256 tiles a CTA pair, where the fp32-out gated form runs with another ring of residual
+    chunks: the bits of the 256 x 128 tile, K blocks fewer and more than its stages, the last rows against
+    the oracle (tolerance as in test_gemm_epilogues) and rows past the end untouched."""
+    N = 1536
+    rng = np.random.default_rng(70 + rows)
+    for K in (64, 448, 832):
+        a_dev, w_dev, b_dev = (to_dev(rand_bf16(rng, s, c)[0]) for s, c in (((rows, K), 1.0), ((N, K), 0.05), ((N,), 0.5)))
+        gate = torch.from_numpy(rng.standard_normal(N, dtype=np.float32)).to(DEV)
+        res = to_dev(rand_bf16(rng, (rows, N))[0])
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+        def run(tile):
+            out = torch.full((rows + 5, N), float("nan"), device=DEV)
+            xb.xema_op_gemm_in_tile(*tile, status=status.data_ptr(), a=a_dev.data_ptr(), lda=K, a_batch_rows=rows,
+                                    w=w_dev.data_ptr(), ldw=K, bias=b_dev.data_ptr(), out=out.data_ptr(), ldo=N,
+                                    out_batch_rows=rows, batch=1, rows=rows, N=N, K=K, epilogue=xb.EPI_GATE_RES_F32,
+                                    resid=res.data_ptr(), ldr=N, resid_batch_rows=rows, gate=gate.data_ptr(), gate_stride=N)
+            return out
+
+        wide, narrow = run((1, 256)), run((1, 128))
+        _sync_status(status)
+        assert torch.equal(wide[:rows], narrow[:rows]) and bool(wide[rows:].isnan().all())
+        c = slice(rows - 300, rows)
+        as64 = lambda t: t.view(torch.bfloat16).double()
+        ref = as64(res[c]) + gate.double() * (as64(a_dev[c]) @ as64(w_dev).T + as64(b_dev))
+        assert_close(wide[c].cpu().numpy(), ref.cpu().numpy(), ("gemm many wide tiles", rows, K), rel=1e-4, cos=0.9999999)
+
+
 def test_gemm_many_tiles_persistent():
     """More tiles than SMs so every CTA runs several tiles through both TMEM accumulators."""
     rng = np.random.default_rng(7)
