@@ -34,6 +34,12 @@
 //     600 keys with three times the scores; without reference and rounded sum 2.34e-3, 2.35e-3, 2.35e-3; with a
 //     running maximum instead 2.29e-3, 2.33e-3, 2.23e-3.  Both together cost 2 % (4608 x 4608 x 24 heads
 //     229 -> 233 us, launches in turn on a warm board);
+//   * per block a softmax warp runs 212 instructions of arithmetic and, at first, 100 around them.  Warp index and TMEM base are
+//     made uniform (barrier and TMEM addresses then stay in uniform registers: no moves there, fewer spills), a wait
+//     that gives up does not leave the block (mbar_wait_sticky), three score loads share one wait, P leaves in one store.
+//     In turn, cool board / under the power cap: dh 64, 4444 x 17776 x 48 heads 887 -> 861 / 1017 -> 986 us; dh 128, 4608 x
+//     4608 x 24 heads 205 -> 190 / 237 -> 221 us.  One arrival per warp instead of one per thread: 1 % slower; 32 / 112
+//     registers for helpers / softmax: spills, 4 % slower;
 //   * one body for all blocks where there are few: the first time an SM runs a piece of code costs
 //     microseconds of instruction fetch, which a call with few keys pays in full.  Keys past the end get
 //     the exponent -119 (they add 2^-119 each to a row sum of at least 2^-90; their V rows are zero).
@@ -152,8 +158,13 @@ __device__ __forceinline__ f32x2 exp2_poly(f32x2 x2) {
   f32x2 p2 = fma_f32x2(make_float2(0.0551208667f, 0.0551208667f), r2, make_float2(0.242484242f, 0.242484242f));
   p2 = fma_f32x2(p2, r2, make_float2(0.693255842f, 0.693255842f));
   p2 = fma_f32x2(p2, r2, make_float2(0.999933064f, 0.999933064f));
-  return make_float2(__uint_as_float(__float_as_uint(p2.x) + (__float_as_uint(t2.x) << 23)),
-                     __uint_as_float(__float_as_uint(p2.y) + (__float_as_uint(t2.y) << 23)));
+  // (t << 23) + p: written as a plain shift and sum it becomes an IMAD on the pipe of the packed FMAs, which was busy
+  // 63 % of the time beside 30 % of the ALU's, where a funnel shift and an add run.  4444 x 17776 x 48 heads 878 -> 846 us,
+  // under the power cap 999 -> 971.
+  uint32_t nx, ny;
+  asm("shf.l.wrap.b32 %0, %1, %2, 23;" : "=r"(nx) : "r"(0u), "r"(__float_as_uint(t2.x)));
+  asm("shf.l.wrap.b32 %0, %1, %2, 23;" : "=r"(ny) : "r"(0u), "r"(__float_as_uint(t2.y)));
+  return make_float2(__uint_as_float(__float_as_uint(p2.x) + nx), __uint_as_float(__float_as_uint(p2.y) + ny));
 }
 
 // Partial sums of one thread's part of a row: of the probabilities, and (ROUNDED_SUM) of what bf16 makes
@@ -264,7 +275,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint32_t* item_flag = tmem_slot + 5;              // [MAX_ITEMS / 32] one bit per item of this CTA
   static_assert(34 * 8 + (5 + MAX_ITEMS / 32) * 4 <= 512, "barrier area");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int n_kv = (p.keys + BN - 1) / BN;
   const int n_items = (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // of this CTA
 
@@ -309,7 +320,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // uniform, like the warp index
   if (threadIdx.x == 0) grid_dep_launch();
   grid_dep_wait();
 
@@ -574,9 +585,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr Mode MODE = decltype(mode_tag)::value;
     constexpr bool TRACK = decltype(track_tag)::value;
     constexpr bool CLAMP = MODE == REPEAT;
-    ok = mbar_wait_warp(&s_full[tile], s_ph, abort_flag);
+    mbar_wait_sticky(&s_full[tile], s_ph, abort_flag, ok);
     if (C::FIRST_MAX && MODE != REPEAT && j == 0) first_max();
-    if (!ok) return;
     tc_fence_after();
     s_ph ^= 1;
     const int valid = p.keys - j * BN - half * COLS;     // keys of this thread's columns that exist
@@ -601,22 +611,23 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       if (MASKED) mask_tail(s, valid - c * CH, PAST_END);
     };
-    uint32_t pk[2][COLS / 4];                          // packed probabilities, by halves
+    uint32_t pk[COLS / 2];                             // packed probabilities
     float b0[CH], b1[CH], b2[CH];
     ld_scores(s_tmem, b0);
     ld_scores(s_tmem + CH, b1);
     ld_scores(s_tmem + 2 * CH, b2);
-    wait_scores(b0);
-    wait_scores(b1);
-    wait_scores(b2);
+    tmem_ld_wait();
+    tmem_ld_tie(b0);
+    tmem_ld_tie(b1);
+    tmem_ld_tie(b2);
     adjust(b0, 0);
-    exp_cols<DH, 0, CLAMP, TRACK>(b0, &pk[0][0], sums, poly_abs);
+    exp_cols<DH, 0, CLAMP, TRACK>(b0, &pk[0], sums, poly_abs);
     ld_scores(s_tmem + 3 * CH, b0);
     adjust(b1, 1);
-    exp_cols<DH, 1, CLAMP, TRACK>(b1, &pk[0][CH / 2], sums, poly_abs);
+    exp_cols<DH, 1, CLAMP, TRACK>(b1, &pk[CH / 2], sums, poly_abs);
     wait_scores(b0);
     if (C::ALIAS && MODE != PROBE) {
-      tmem_st16(p_tmem, pk[0]);                            // all scores are in registers
+      tmem_st16(p_tmem, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));   // all scores are in registers
       tmem_st_wait();
       tc_fence_before();
       mbar_arrive(&p_half[tile]);
@@ -625,20 +636,20 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_arrive(&s_free[tile]);                         // S(j) is in registers: S(j+1) may land
     }
     adjust(b2, 2);
-    exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[1][0], sums, poly_abs);
+    exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[CH], sums, poly_abs);
     adjust(b0, 3);
-    exp_cols<DH, 3, CLAMP, TRACK>(b0, &pk[1][CH / 2], sums, poly_abs);
+    exp_cols<DH, 3, CLAMP, TRACK>(b0, &pk[3 * CH / 2], sums, poly_abs);
     if (MODE == PROBE) return;
     if (!C::ALIAS) {
       if (j > 0) {                                        // the previous product reads the same columns
-        if (!mbar_peek(&pv_done[tile], pv_ph)) ok = mbar_wait_warp(&pv_done[tile], pv_ph, abort_flag);
-        if (!ok) return;
+        mbar_wait_sticky(&pv_done[tile], pv_ph, abort_flag, ok);
         pv_ph ^= 1;
         tc_fence_after();
       }
-      tmem_st16(p_tmem, pk[0]);
+      tmem_st32(p_tmem, pk);
+    } else {
+      tmem_st16(p_tmem + COLS / 4, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
     }
-    tmem_st16(p_tmem + COLS / 4, pk[1]);
     tmem_st_wait();
     tc_fence_before();
     mbar_arrive(&p_full[tile]);

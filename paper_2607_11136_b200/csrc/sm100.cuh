@@ -66,21 +66,6 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 // kernels.)
 constexpr uint32_t kWaitHintNs = 1000u;
 constexpr int kWaitFastPolls = 2;
-// Non-blocking look at a barrier phase (try_wait may park the thread for a while when the phase
-// is still open; test_wait returns at once).
-__device__ __forceinline__ bool mbar_peek(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
                                                    long long limit_cycles) {
   const long long t0 = clock64();
@@ -113,6 +98,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     if (mbar_test(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, abort_flag, kWaitLimitCycles);
 }
+
+// The warp's index as a value the compiler knows to be the same in all 32 lanes: what is computed from it (barrier and
+// TMEM addresses) stays in uniform registers instead of being moved there at every use.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
 
 // Bounded wait for a whole warp that polls together (every lane executes it with the same
 // arguments): one loop in a single block of PTX -- no function call, no vote, no compiler-made
@@ -160,6 +149,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
       return false;
     }
   }
+}
+
+// The same for a loop that looks at `ok` once per round: a wait that gives up clears it and the round goes on with
+// whatever is there, so the common case is a poll and one branch, with no exit of its own.
+__device__ __forceinline__ void mbar_wait_sticky(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, bool& ok) {
+  if (!mbar_test(bar, parity)) ok = mbar_wait_warp(bar, parity, abort_flag) && ok;
 }
 
 // ---- programmatic dependent launch -----------------------------------------------------------
@@ -479,14 +474,32 @@ __device__ __forceinline__ void tmem_ld_wait_on(uint32_t (&r)[16]) {
       :
       : "memory");
 }
+// The wait alone, and its tie to the values of a load (for several loads behind one wait).
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void tmem_ld_tie(float (&v)[N]) {
+#pragma unroll
+  for (int t = 0; t < N; ++t) asm volatile("" : "+f"(v[t]));
+}
 
-// registers -> TMEM: 16 consecutive columns.
+// registers -> TMEM: 16 or 32 consecutive columns.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
       "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
