@@ -570,8 +570,10 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
       if (et < p.head_dim) s_gate[et] = __bfloat162float(p.norm_gain[et]);   // read after the tile's barrier
     }
-    ep.dry = kRehearse<BN, PAIR> && total_tiles > 0;      // the first round is a rehearsal
-    if (!ep.dry) grid_dep_wait();
+    ep.dry = kRehearse<BN, PAIR>;                          // the first round is a rehearsal
+    if constexpr (!kRehearse<BN, PAIR>) {
+      grid_dep_wait();
+    }
     for (int tile = worker; tile < total_tiles;) {
       const bool dry = ep.rehearsing();
       // The four warps meet (the previous tile's bias and gate are no longer read) and agree on going
@@ -631,6 +633,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
       if (++acc == 2) { acc = 0; acc_phase ^= 1; }
       tile += n_workers;
     }
+    grid_dep_wait();                     // (a CTA without tiles has not waited yet)
     if (GATED && !ok) {
       // gave up: the residual chunks already requested must land before the CTA leaves
       for (uint32_t i = ep.asked > (uint32_t)RING ? ep.asked - RING : 0; i < ep.asked; ++i) {
