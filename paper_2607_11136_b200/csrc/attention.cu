@@ -103,6 +103,12 @@ constexpr uint32_t kPolyPairs = DH == 64 ? 0xc358a94au : 0u;
 static_assert(!(kPolyPairs<64> & 1u), "a row's first key goes through the MUFU, which keeps a NaN");
 static_assert(BN == 128 && BM == 128, "the kernel is written for 128-key blocks of 128-row tiles");
 
+// Barriers between softmax threads and issuers per set (s_full to pv_done); the rehearsal uses a second set, none of whose
+// phases completes: a wait for the phase before the first returns at once, an arrival has no effect.
+constexpr int kDry = 5 * TILES;
+constexpr uint32_t kNever = 1u << 19;
+constexpr int kRehearseBlocks = 8;       // key blocks a CTA works on, up to which a launch rehearses (see attention_kernel)
+
 template <int DH>
 struct Cfg {
   static constexpr bool ALIAS = DH == 128;                 // P over S; otherwise P has its own columns
@@ -249,7 +255,12 @@ __device__ __forceinline__ void transpose_4x4(uint4 (&c)[4], int lane) {
 // Sweeps of one item: the pass itself; the scores only (flags and true maxima); the repeat.
 enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
 
-template <int DH, bool SCALED>
+// REHEARSE: a round of the softmax threads' loop before the wait for earlier launches, on whatever TMEM holds and
+// without results, so that the first item does not meet every line of the code in an empty instruction cache.  A launch of
+// few key blocks gains 1 to 2 us by it; the second set of barriers costs the loop 2 %.  us without / with it: block of 288 x 512
+// 48.2 / 46.8, 464 x 1792 160 / 156, two blocks of 630 x 1536 235 / 228, eight of 304 x 2304 1123 / 1099; with 9 key blocks a CTA (1101 x
+// 1536) 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.
+template <int DH, bool SCALED, bool REHEARSE>
 __global__ void __launch_bounds__(THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
@@ -268,12 +279,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint64_t* p_half = bars + 28;    // [TILES] the first half of P(j) is complete in TMEM (ALIAS)
   uint64_t* p_full = bars + 30;    // [TILES] P(j) is complete in TMEM
   uint64_t* pv_done = bars + 32;   // [TILES] O += P(j) V(j) has finished (ALIAS: of an item's last block)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 34);
+  // bars + 34: s_full to pv_done once more, for the rehearsal (kDry)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 44);
   volatile uint32_t* abort_flag = tmem_slot + 1;
   uint32_t* gain_max = tmem_slot + 2;               // [2] bit patterns of max|gain_q|, max|gain_k|
   volatile uint32_t* any_flag = tmem_slot + 4;
   uint32_t* item_flag = tmem_slot + 5;              // [MAX_ITEMS / 32] one bit per item of this CTA
-  static_assert(34 * 8 + (5 + MAX_ITEMS / 32) * 4 <= 512, "barrier area");
+  static_assert((34 + kDry) * 8 + (5 + MAX_ITEMS / 32) * 4 <= 512 && kDry == 10, "barrier area");
 
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int n_kv = (p.keys + BN - 1) / BN;
@@ -304,6 +316,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_init(&p_full[t], BM * TPR);
       mbar_init(&pv_done[t], 1);
     }
+    if (REHEARSE)
+      for (int i = 0; i < kDry; ++i) mbar_init(&s_full[kDry + i], kNever);
     *abort_flag = 0;
     *any_flag = 0;
     gain_max[0] = gain_max[1] = 0;
@@ -322,7 +336,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // uniform, like the warp index
   if (threadIdx.x == 0) grid_dep_launch();
-  grid_dep_wait();
+  // (the wait for earlier launches stands in the roles, behind the moves of registers)
 
   struct Item {
     int row0, h, b;
@@ -540,8 +554,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int r = quad * 32 + lane;                          // query row inside the tile = TMEM lane
   const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + tile * C::TM_TILE;
   const uint32_t s_tmem = t_lane + half * COLS;
-  const uint32_t p_tmem = t_lane + C::TM_P + half * (C::ALIAS ? COLS : COLS / 2);
+  uint32_t p_tmem = t_lane + C::TM_P + half * (C::ALIAS ? COLS : COLS / 2);
   const uint32_t o_tmem = t_lane + C::TM_O + half * (DH / TPR);
+  int set = 0;                 // offset of the barriers in use (kDry: the rehearsal's) ...
+  uint32_t live = 1;           // ... and what their phases advance by
   RowSums sums;
   float poly_abs = 0.f, m_ref = 0.f, m_true = 0.f;
   // The two warps that share 32 rows meet: all of them, with a vote on going on (a warp that gave up
@@ -585,10 +601,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr Mode MODE = decltype(mode_tag)::value;
     constexpr bool TRACK = decltype(track_tag)::value;
     constexpr bool CLAMP = MODE == REPEAT;
-    mbar_wait_sticky(&s_full[tile], s_ph, abort_flag, ok);
+    mbar_wait_sticky(&s_full[set + tile], s_ph, abort_flag, ok);
     if (C::FIRST_MAX && MODE != REPEAT && j == 0) first_max();
     tc_fence_after();
-    s_ph ^= 1;
+    s_ph ^= live;
     const int valid = p.keys - j * BN - half * COLS;     // keys of this thread's columns that exist
     auto adjust = [&](float(&s)[CH], int c) {
       // score -> exponent relative to the row's reference (zero for dh 64 but in the repeat of a flagged row)
@@ -630,10 +646,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       tmem_st16(p_tmem, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));   // all scores are in registers
       tmem_st_wait();
       tc_fence_before();
-      mbar_arrive(&p_half[tile]);
+      mbar_arrive(&p_half[set + tile]);
     } else {
       tc_fence_before();
-      mbar_arrive(&s_free[tile]);                         // S(j) is in registers: S(j+1) may land
+      mbar_arrive(&s_free[set + tile]);                         // S(j) is in registers: S(j+1) may land
     }
     adjust(b2, 2);
     exp_cols<DH, 2, CLAMP, TRACK>(b2, &pk[CH], sums, poly_abs);
@@ -642,8 +658,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (MODE == PROBE) return;
     if (!C::ALIAS) {
       if (j > 0) {                                        // the previous product reads the same columns
-        mbar_wait_sticky(&pv_done[tile], pv_ph, abort_flag, ok);
-        pv_ph ^= 1;
+        mbar_wait_sticky(&pv_done[set + tile], pv_ph, abort_flag, ok);
+        pv_ph ^= live;
         tc_fence_after();
       }
       tmem_st32(p_tmem, pk);
@@ -652,7 +668,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     tmem_st_wait();
     tc_fence_before();
-    mbar_arrive(&p_full[tile]);
+    mbar_arrive(&p_full[set + tile]);
   };
   // Blocks without keys past the end.  With few of them they all take the masking form, so that
   // only one body has to be fetched.
@@ -663,9 +679,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     sums.rounded[0] = sums.rounded[1] = make_float2(0.f, 0.f);
     poly_abs = 0.f;
 #pragma unroll 1
-    for (int j = 0; ok && j < n_plain; ++j) run_block(j, mode_tag, std::false_type{}, track_tag);
+    for (int j = 0; ok && j < (set ? min(n_plain, 1) : n_plain); ++j) run_block(j, mode_tag, std::false_type{}, track_tag);
 #pragma unroll 1
-    for (int j = n_plain; ok && j < n_kv; ++j) run_block(j, mode_tag, std::true_type{}, track_tag);
+    for (int j = n_plain; ok && j < (set ? min(n_kv, n_plain + 1) : n_kv); ++j) run_block(j, mode_tag, std::true_type{}, track_tag);
   };
   using PassT = std::integral_constant<Mode, PASS>;
   using ProbeT = std::integral_constant<Mode, PROBE>;
@@ -690,8 +706,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const float mine = sum_partials(sums.rounded);
       o_row = mine + exchange(mine);
     }
-    ok = mbar_wait_warp(&pv_done[tile], pv_ph, abort_flag);
-    pv_ph ^= 1;
+    ok = mbar_wait_warp(&pv_done[set + tile], pv_ph, abort_flag);
+    pv_ph ^= live;
     if (!ok) return;
     tc_fence_after();
     const int row = it.row0 + tile * BM + r;
@@ -751,6 +767,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // First pass over the CTA's items, then the flagged ones once more in two sweeps.
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_HELPER));
+    grid_dep_wait();
     if (warp == 0) {
       if (lane == 0)
         for (int i = 0; ok && i < n_items; ++i) produce(item_at(i), true);
@@ -834,9 +851,27 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       constexpr float factor = 11.55f * 1.01f;
       bounded = gq * gk * factor < 100.f;    // false for a NaN gain
     }
-    for (int i = 0; i < n_items; ++i) {
-      const Item it = item_at(i);
-      if (!tile_live(it, tile)) continue;
+    // Round -1 is the rehearsal: its rows lie past the end (from a multiple of 128 on, because finish stores groups of four
+    // rows), its probabilities go where the first product overwrites them (P over S would meet the first scores).
+    const uint32_t p_live = p_tmem;
+    if (REHEARSE) {
+      if (C::ALIAS) p_tmem = o_tmem;
+      set = kDry;
+      live = 0;
+      s_ph = pv_ph = 1;
+    } else {
+      grid_dep_wait();
+    }
+    for (int i = REHEARSE ? -1 : 0; i < n_items; ++i) {
+      if (REHEARSE && i == 0) {
+        grid_dep_wait();
+        p_tmem = p_live;
+        set = 0;
+        live = 1;
+        s_ph = pv_ph = 0;
+      }
+      const Item it = i < 0 ? Item{(p.rows + BM - 1) / BM * BM, 0, 0} : item_at(i);
+      if (i >= 0 && !tile_live(it, tile)) continue;
       if (ok) {
         if (bounded) run_blocks(PassT{}, std::false_type{});
         else run_blocks(PassT{}, std::bool_constant<POLY>{});
@@ -845,7 +880,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!ok) break;
       bool flag;
       const float l = row_sum(flag);
-      if (flag) {
+      if (flag && i >= 0) {
         *any_flag = 1;
         atomicOr(&item_flag[i >> 5], 1u << (i & 31));
       }
@@ -883,11 +918,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
 }
 
-template <int DH, bool SCALED>
+template <int DH, bool SCALED, bool REHEARSE>
 int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   using C = Cfg<DH>;
   static PerDeviceInt attr_done;
-  auto kern = attention_kernel<DH, SCALED>;
+  auto kern = attention_kernel<DH, SCALED, REHEARSE>;
   if (int rc = ensure_smem_attr(kern, C::SMEM_BYTES, attr_done)) return rc;
   AttnParams p;
   p.o = (__nv_bfloat16*)a.o;
@@ -916,11 +951,19 @@ int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
 
 int launch_attention(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   if (a.rows == 0 || a.batch == 0) return XEMA_OK;
+  // Behind another launch there is a wait to use, and up to kRehearseBlocks key blocks a CTA the gain is the larger.
+  const long long tiles = (a.rows + BM - 1) / BM * (long long)a.heads * a.batch;
+  const long long rounds = (tiles + 2 * sm_count() - 1) / (2 * sm_count());
+  const bool rehearse = chained && rounds * ((a.keys + BN - 1) / BN) <= kRehearseBlocks;
   const bool scaled = a.q_scale != 1.f;
   if (a.head_dim == 64)
-    return scaled ? launch_attention_t<64, true>(a, stream, chained) : launch_attention_t<64, false>(a, stream, chained);
+    return scaled     ? launch_attention_t<64, true, false>(a, stream, chained)
+           : rehearse ? launch_attention_t<64, false, true>(a, stream, chained)
+                      : launch_attention_t<64, false, false>(a, stream, chained);
   if (a.head_dim == 128)
-    return scaled ? launch_attention_t<128, true>(a, stream, chained) : launch_attention_t<128, false>(a, stream, chained);
+    return scaled     ? launch_attention_t<128, true, false>(a, stream, chained)
+           : rehearse ? launch_attention_t<128, false, true>(a, stream, chained)
+                      : launch_attention_t<128, false, false>(a, stream, chained);
   return XEMA_EINVAL;
 }
 

@@ -1,4 +1,5 @@
-"""Forms that only the short launches of a plan take: the FFN2 product with its K divided over a cluster."""
+"""Forms that only the short launches of a plan take: the FFN2 product with its K divided over a cluster, the attention that
+rehearses."""
 import numpy as np
 import pytest
 import torch
@@ -72,3 +73,24 @@ def test_a_template_of_many_rows_is_not_divided():
                     out=out.data_ptr(), ldo=512, out_batch_rows=1100, resid=res.data_ptr(), ldr=512, resid_batch_rows=1100,
                     gate=gate.data_ptr(), gate_stride=3072, batch=1, rows=1100, N=512, K=2048, epilogue=xb.EPI_GATE_RES_BF16)
     assert torch.equal(out, s.hid_out())
+
+
+# the attention of a plan follows another launch and, up to 8 key blocks a CTA, rehearses; the same call by itself does not
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("tokens,chunks", [(9, 1), (130, 1), (161, 3), (333, 2), (1024, 1), (1030, 1)])
+def test_attention_behind_another_launch_keeps_its_bits(head_dim, tokens, chunks):
+    t = _template(1, tokens, 512, 512, heads=512 // head_dim)
+    s = BlockSession(t, [make_block_weights(t, 5)], chunks=(1, chunks, 1))
+    s.set_inputs(*make_activations(t))
+    stream = torch.cuda.current_stream().cuda_stream
+    s.plan.forward_prefix(8, stream)       # MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN of the first chunk
+    rows = tokens // chunks
+    q, kv = s.view("q0_0", torch.int16, (1, rows, 512)), s.view("kv0", torch.int16, (1, tokens, 1024))
+    got = s.view("o0_0", torch.int16, (1, rows, 512)).clone()
+    lse = s.view("lse0_0", torch.float32, (1, 512 // head_dim, rows)).clone()
+    o, l = torch.empty_like(got), torch.empty_like(lse)
+    xb.xema_op_attention(q.data_ptr(), 512, rows, kv.data_ptr(), kv.data_ptr() + 1024, 1024, tokens, o.data_ptr(), l.data_ptr(),
+                         1, rows, tokens, 512 // head_dim, head_dim, status=s.status.data_ptr(), stream=stream, q_scale=1.0)
+    s.check_status()
+    assert torch.equal(o, got) and torch.equal(l, lse)
+
