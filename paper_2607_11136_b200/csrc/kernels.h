@@ -73,7 +73,7 @@ int launch_kernel(void (*kern)(Params...), dim3 grid, int threads, size_t smem, 
 }
 
 int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream, bool chained = false);
+               cudaStream_t stream, bool chained = false, bool opens = false);
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
                        cudaStream_t stream, bool chained = false);
@@ -81,7 +81,8 @@ int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void*
                         int batch, int rows, int heads, int head_dim, float eps, cudaStream_t stream);
 
 // dst0 <- src0 (n0 bytes) and dst1 <- src1 (n1 bytes); pointers and sizes are multiples of 16 bytes.
-int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream);
+int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream,
+                 bool opens = false);
 
 // ---- TMA descriptors (encoded on the host once per bound tensor) --------------------------
 // bf16 tensor viewed as [batch][rows][cols] with row stride ld and batch stride batch_rows*ld

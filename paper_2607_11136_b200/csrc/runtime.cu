@@ -178,11 +178,13 @@ struct xema_plan {
 };
 
 // `chained`: the launch right before this one in the stream is the op before it (see launch_kernel).
-static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained) {
+// `opens`: it opens a call and may start before the launch ahead of it in the stream has finished (it waits for that
+// one itself before it reads anything).
+static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained, bool opens = false) {
   const xema_config& c = pl->cfg;
   switch (op.kind) {
     case OP_MOD:
-      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained);
+      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained, opens);
     case OP_LN:
       return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale,
                                 6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st, chained);
@@ -199,6 +201,17 @@ static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chaine
   return XEMA_EINVAL;
 }
 
+// Whether a launch that opens a call may start early: not inside a stream capture, where the node ahead of it need not
+// be a kernel.
+static bool may_open(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return status == cudaStreamCaptureStatusNone;
+}
+
 static int run_ops(const xema_plan* pl, size_t first, size_t n, void* stream) {
   if (!pl) return XEMA_EINVAL;
   if (!pl->bound) return XEMA_ESTATE;
@@ -206,7 +219,8 @@ static int run_ops(const xema_plan* pl, size_t first, size_t n, void* stream) {
   n = std::min(n, pl->ops.size());
   bool chained = false;
   for (size_t i = first; i < n; ++i) {
-    int rc = issue(pl, pl->ops[i], st, chained);
+    const bool opens = !chained && pl->ops[i].kind == OP_MOD && may_open(st);
+    int rc = issue(pl, pl->ops[i], st, chained, opens);
     if (rc) return rc;
     chained = chained || pl->ops[i].kind != OP_FUSED;
   }
@@ -608,7 +622,7 @@ int xema_plan_set_inputs(const xema_plan* plan, const void* hid_dev, const void*
       overlaps(hid_dev, hid_bytes, plan->temb_in, temb_bytes) || overlaps(temb_dev, temb_bytes, plan->hid_in, hid_bytes))
     return XEMA_EINVAL;
   if (((reinterpret_cast<uintptr_t>(hid_dev) | reinterpret_cast<uintptr_t>(temb_dev)) & 15) == 0)
-    return launch_copy2(plan->hid_in, hid_dev, hid_bytes, plan->temb_in, temb_dev, temb_bytes, st);
+    return launch_copy2(plan->hid_in, hid_dev, hid_bytes, plan->temb_in, temb_dev, temb_bytes, st, may_open(st));
   cudaError_t e = cudaMemcpyAsync(plan->hid_in, hid_dev, hid_bytes, cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(plan->temb_in, temb_dev, temb_bytes, cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) {

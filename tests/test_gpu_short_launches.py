@@ -1,5 +1,5 @@
 """Forms that only the short launches of a plan take: the FFN2 product with its K divided over a cluster, the attention that
-rehearses."""
+rehearses, the launches that open a call."""
 import numpy as np
 import pytest
 import torch
@@ -94,3 +94,31 @@ def test_attention_behind_another_launch_keeps_its_bits(head_dim, tokens, chunks
     s.check_status()
     assert torch.equal(o, got) and torch.equal(l, lse)
 
+
+
+@pytest.mark.parametrize("tokens", [130, 1030])
+def test_calls_back_to_back_see_their_own_inputs_and_weights(tokens):
+    """The first launches of a call may start while the work ahead of them runs: inputs, and weights that a kernel of the
+    caller writes right before the call, are read only when it has finished."""
+    t = _template(1, tokens, 512, 2048)
+    ws = [make_block_weights(t, seed) for seed in (1, 2)]
+    ins = [make_activations(t, seed) for seed in (3, 4)]
+    want = []
+    for w, (x, temb) in zip(ws, ins):
+        s = BlockSession(t, [w], chunks=(1, 1, 1))
+        s.set_inputs(x, temb)
+        s.forward()
+        want.append(s.output_bits().copy())
+    dev = [{k: torch.from_numpy(v.view(np.int16)).cuda() for k, v in w.items()} for w in ws]
+    src = [[torch.from_numpy(v.view(np.int16)).cuda() for v in pair] for pair in ins]
+    s = BlockSession(t, [{k: v.clone() for k, v in dev[0].items()}], chunks=(1, 1, 1))
+    outs = []
+    for i in (0, 1, 1, 0, 1, 0):
+        x, temb = (v.clone() for v in src[i])
+        s.set_inputs(x, temb, non_blocking=True)
+        for k, v in s.weights[0].items():
+            v.copy_(dev[i][k])
+        s.forward()
+        outs.append((i, s.hid_out().clone()))
+    for i, y in outs:
+        assert np.array_equal(y.cpu().numpy().view(np.uint16), want[i].reshape(y.shape))
