@@ -54,8 +54,8 @@
 //           per tile the two bursts shared the pipe and both ended late (a block 3090 cycles against
 //           2690).  P goes over in two halves, so half of the product runs under the rest of the softmax.
 //
-// Measured (B200, inside the block): dh 64, 4444 x 17776 x 48 heads 933 us (with one CTA per 256 rows and code
-// copies for first and last blocks 970); power-capped 17776-token block 7.28 ms against 7.52.  dh 128, 17776 x
+// Measured (B200): dh 64, 4444 x 17776 x 48 heads 845 us; before the overhead instructions went, inside the block, 933 (with one
+// CTA per 256 rows and code copies for first and last blocks 970); power-capped 17776-token block 7.28 ms against 7.52.  dh 128, 17776 x
 // 17776 x 24 heads 3.38 ms on a warm board (one tile per CTA, two CTAs per SM, 64-key blocks, running maximum:
 // 3.79 in turn with it), 4608 x 4608 x 24 heads 235 us (275).  288 x 288 x 8 heads of 64 10.4 us (14.4).
 //
