@@ -686,9 +686,9 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 // rows and columns do not give every SM a tile.  Every CTA multiplies its share of the K blocks, sends the partial sums
 // of the columns that others own to their shared memory, and finishes its own 128 / S columns: the partials are added
 // in the order of the CTAs, then as in Epilogue.  Roles as in gemm_body.
-// 333 x 1024 x 4096: the K loop takes 3.4 us on 24 x 4 CTAs where 96 CTAs with 128 x 32 tiles took 10.2, the exchange and its
-// wait 2; step of 8 blocks of 333 x 1024 tokens 448 -> 430 us, of 304 x 2304 1165 -> 1134.  A cluster barrier in front of the
-// sums instead of the byte count of a warp's own rows took 0.5 us longer.
+// 333 x 1024 x 4096: the K loop takes 3.4 us on 24 x 4 CTAs where 96 CTAs with 128 x 32 tiles took 10.2, but 3.5 instead of 0.6 pass
+// from its end to the end of the launch; step of 8 blocks of 333 x 1024 tokens 448 -> 429 us, of 304 x 2304 1152 -> 1123.  Plain remote
+// stores and a cluster barrier in front of the sums took the same time as the byte count of a warp's own rows.
 template <int S>
 struct SplitCfg {
   static constexpr int BN = 128, OWN = BN / S;                 // tile columns; columns a CTA finishes
@@ -1072,8 +1072,8 @@ long long pick_tile(GemmLaunch* g) {      // returns its estimate
 
 // How many CTAs share the K of a gated product (1: none): taken where the clusters of every 128 x 128 tile of the whole
 // template run at once (7/8 of the SMs: clusters of four do not fill every GPC) and the estimate -- 265 ns per K block as
-// above, 2000 for the exchange and a later start -- is a tenth below the best whole tile's.  us of FFN2 so / whole: 333 x 1024 x
-// 4096 9.3 / 11.6, 288 x 512 x 2048 7.1 / 7.1; PROJ of the same blocks (K = 1024, 512) would lose 1 and does not get it.
+// above, 2000 for the exchange and a later start -- is a tenth below the best whole tile's.  A block of 333 x 1024 (K = 4096) gains
+// 2.4 us, one of 288 x 512 (K = 2048) nothing; PROJ of the same blocks (K = 1024, 512) fails the estimate.
 int split_for(const GemmLaunch& g, int batch, int rows) {
   GemmLaunch whole = g;
   whole.batch = batch;
