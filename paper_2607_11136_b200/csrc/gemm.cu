@@ -9,7 +9,7 @@
 //           memory fill per SM and every MMA reads 8 KB of operands per SM; the even CTA issues
 //           tcgen05.mma.cta_group::2 (M = 256), which accumulates 128 rows in the TMEM of each CTA.
 //   single  one CTA per 128 x 128, 128 x 64 or (gated epilogues, few rows) 128 x 32 tile.
-// pick_tile says which when.  A second kernel divides the K of a tile among the CTAs of a cluster (see SplitCfg).
+// pick_tile says which when.
 //
 //   warp 0    TMA producer: tiles of A and W into a ring of shared-memory stages (128-byte swizzle)
 //   warp 1    owns TMEM; converged warp, one elected lane issues tcgen05.mma into one of two fp32
@@ -32,8 +32,7 @@
 // end of every launch.
 //
 // A row's result depends only on (row, N, K): every form accumulates K in the same order, 16 at a
-// time, so outputs are bit-identical however rows are chunked and whichever tile is chosen.  The divided form adds
-// S such sums; whether a plan takes it is decided once for its template (gemm_split), not per launch.
+// time, so outputs are bit-identical however rows are chunked and whichever tile is chosen.
 #include <algorithm>
 
 #include "kernels.h"
@@ -209,46 +208,6 @@ struct Epilogue {
     return ring + (used % RING) * BUF_BYTES;
   }
 
-  // resid + gate * v of one chunk, over the residual in the chunk's buffer
-  __device__ __forceinline__ void gate_chunk(uint8_t* buf, const float* chunk_gate, float (&v)[CHUNK]) {
-    const float4* g = reinterpret_cast<const float4*>(chunk_gate);
-    if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
-      // out fp32 = resid(bf16) + gate * v
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 x = *reinterpret_cast<const uint4*>(piece_b16(buf, rlane, q));
-        const float4 g0 = g[2 * q], g1 = g[2 * q + 1];
-        v[8 * q + 0] = fmaf(g0.x, v[8 * q + 0], bf16_lo(x.x));
-        v[8 * q + 1] = fmaf(g0.y, v[8 * q + 1], bf16_hi(x.x));
-        v[8 * q + 2] = fmaf(g0.z, v[8 * q + 2], bf16_lo(x.y));
-        v[8 * q + 3] = fmaf(g0.w, v[8 * q + 3], bf16_hi(x.y));
-        v[8 * q + 4] = fmaf(g1.x, v[8 * q + 4], bf16_lo(x.z));
-        v[8 * q + 5] = fmaf(g1.y, v[8 * q + 5], bf16_hi(x.z));
-        v[8 * q + 6] = fmaf(g1.z, v[8 * q + 6], bf16_lo(x.w));
-        v[8 * q + 7] = fmaf(g1.w, v[8 * q + 7], bf16_hi(x.w));
-      }
-    } else {
-      // out bf16 = resid(fp32) + gate * v
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 x = *reinterpret_cast<const float4*>(piece_f32(buf, rlane, q));
-        const float4 gg = g[q];
-        v[4 * q + 0] = fmaf(gg.x, v[4 * q + 0], x.x);
-        v[4 * q + 1] = fmaf(gg.y, v[4 * q + 1], x.y);
-        v[4 * q + 2] = fmaf(gg.z, v[4 * q + 2], x.z);
-        v[4 * q + 3] = fmaf(gg.w, v[4 * q + 3], x.w);
-      }
-    }
-    __syncwarp();                                    // every lane has read its residual row
-    if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        *reinterpret_cast<float4*>(piece_f32(buf, lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    } else {
-      put_b16(buf, lane, v);
-    }
-  }
-
   __device__ __forceinline__ bool gated_tile(int b, int row0, int n_base, uint32_t t_addr) {
 #pragma unroll 1
     for (int ch = 0; ch < (rehearsing() ? 1 : BN / CHUNK); ++ch) {
@@ -256,7 +215,42 @@ struct Epilogue {
       if (!rehearsing() && !mbar_wait_warp(rbar + used % RING, (used / RING) & 1u, abort_flag)) return false;
       float v[CHUNK];
       load_chunk(t_addr + ch * CHUNK, bias + ch * CHUNK, v);
-      gate_chunk(buf, gate + ch * CHUNK, v);
+      const float4* g = reinterpret_cast<const float4*>(gate + ch * CHUNK);
+      if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
+        // out fp32 = resid(bf16) + gate * v
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 x = *reinterpret_cast<const uint4*>(piece_b16(buf, rlane, q));
+          const float4 g0 = g[2 * q], g1 = g[2 * q + 1];
+          v[8 * q + 0] = fmaf(g0.x, v[8 * q + 0], bf16_lo(x.x));
+          v[8 * q + 1] = fmaf(g0.y, v[8 * q + 1], bf16_hi(x.x));
+          v[8 * q + 2] = fmaf(g0.z, v[8 * q + 2], bf16_lo(x.y));
+          v[8 * q + 3] = fmaf(g0.w, v[8 * q + 3], bf16_hi(x.y));
+          v[8 * q + 4] = fmaf(g1.x, v[8 * q + 4], bf16_lo(x.z));
+          v[8 * q + 5] = fmaf(g1.y, v[8 * q + 5], bf16_hi(x.z));
+          v[8 * q + 6] = fmaf(g1.z, v[8 * q + 6], bf16_lo(x.w));
+          v[8 * q + 7] = fmaf(g1.w, v[8 * q + 7], bf16_hi(x.w));
+        }
+      } else {
+        // out bf16 = resid(fp32) + gate * v
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float4 x = *reinterpret_cast<const float4*>(piece_f32(buf, rlane, q));
+          const float4 gg = g[q];
+          v[4 * q + 0] = fmaf(gg.x, v[4 * q + 0], x.x);
+          v[4 * q + 1] = fmaf(gg.y, v[4 * q + 1], x.y);
+          v[4 * q + 2] = fmaf(gg.z, v[4 * q + 2], x.z);
+          v[4 * q + 3] = fmaf(gg.w, v[4 * q + 3], x.w);
+        }
+      }
+      __syncwarp();                                    // every lane has read its residual row
+      if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(piece_f32(buf, lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      } else {
+        put_b16(buf, lane, v);
+      }
       send(buf, b, row0, n_base + ch * CHUNK);
       // the buffer of the chunk before this one takes the next residual once its store has been read
       if (ch > 0 && ch - 1 + RING < BN / CHUNK) {
@@ -681,250 +675,6 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   gemm_body<EPI, BN, true, DEEP>(map_a, map_w, map_out, map_res, p);
 }
 
-// One tile of 128 x 128 whose K is divided among the S CTAs of a cluster, for gated products that have few rows and a
-// long K (FFN2): a CTA fills shared memory at about 70 B/clk, which bounds them, and K is what is left to divide where
-// rows and columns do not give every SM a tile.  Every CTA multiplies its share of the K blocks, sends the partial sums
-// of the columns that others own to their shared memory, and finishes its own 128 / S columns: the partials are added
-// in the order of the CTAs, then as in Epilogue.  Roles as in gemm_body.
-// 333 x 1024 x 4096: the K loop takes 3.4 us on 24 x 4 CTAs where 96 CTAs with 128 x 32 tiles took 10.2, but 3.5 instead of 0.6 pass
-// from its end to the end of the launch; step of 8 blocks of 333 x 1024 tokens 448 -> 429 us, of 304 x 2304 1152 -> 1123.  Plain remote
-// stores and a cluster barrier in front of the sums took the same time as the byte count of a warp's own rows.
-template <int S>
-struct SplitCfg {
-  static constexpr int BN = 128, OWN = BN / S;                 // tile columns; columns a CTA finishes
-  static constexpr int STAGES = 5;                             // K blocks in flight: 160 KB covers the latency of the fill
-  static constexpr int STAGE_BYTES = A_TILE_BYTES + BN * BK * 2;
-  static constexpr int CHUNKS = OWN / CHUNK;
-  static constexpr int PART_BYTES = BM * OWN * 4;              // one CTA's partial sums of one owner's columns
-  static constexpr int OFF_PART = STAGES * STAGE_BYTES;        // [S - 1] of them
-  static constexpr int OFF_RING = OFF_PART + (S - 1) * PART_BYTES;
-  static constexpr int OFF_BIAS = OFF_RING + 4 * CHUNKS * BUF_BYTES;   // one staging buffer per chunk and warp
-  static constexpr int OFF_GATE = OFF_BIAS + OWN * 4;
-  static constexpr int OFF_BAR = OFF_GATE + OWN * 4;
-  static constexpr int SMEM_BYTES = OFF_BAR + 256;
-  static_assert((2 * STAGES + 1 + 8 + 4) * 8 + 8 <= 256, "barrier area");
-  static_assert(CHUNKS >= 1 && CHUNKS <= 2 && SMEM_BYTES <= 232448, "shared memory of one SM");
-};
-
-template <int EPI, int S>
-__global__ void __cluster_dims__(S, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
-gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                  const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const GemmParams p) {
-  using Cfg = SplitCfg<S>;
-  constexpr int STAGES = Cfg::STAGES, OWN = Cfg::OWN, CHUNKS = Cfg::CHUNKS, RING = 2;
-  static_assert(kGated<EPI> && GemmCfg<EPI, Cfg::BN, false>::RING == RING, "gated epilogues");
-  extern __shared__ __align__(1024) uint8_t smem[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::OFF_BAR);
-  uint64_t* empty = full + STAGES;
-  uint64_t* tmem_full = empty + STAGES;
-  uint64_t* res_full = tmem_full + 1;                // [4][RING]
-  uint64_t* part_full = res_full + 4 * RING;         // [4] the partial sums of a warp's rows have arrived
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(part_full + 4);
-  volatile uint32_t* abort_flag = tmem_slot + 1;
-
-  const int warp = uniform_warp(), lane = threadIdx.x & 31;
-  const int rank = (int)cluster_ctarank();
-  const TileCoord c = tile_coord(blockIdx.x / S, (p.rows + BM - 1) / BM, p.N / Cfg::BN);
-  const int k_blocks = p.K / BK;
-  const int kb0 = rank * k_blocks / S, n_kb = (rank + 1) * k_blocks / S - kb0;   // this CTA's K blocks (at least one)
-  const bool aligned = (smem_u32(smem) & 1023u) == 0;   // the swizzled tiles need a 1024-byte aligned base
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    mbar_init(tmem_full, 1);
-    for (int s = 0; s < 4 * RING; ++s) mbar_init(&res_full[s], 1);
-    for (int s = 0; s < 4; ++s) mbar_init(&part_full[s], 1);
-    *abort_flag = aligned ? 0u : 1u;
-    fence_mbar_init();
-    prefetch_tmap(&map_a);
-    prefetch_tmap(&map_w);
-    prefetch_tmap(&map_out);
-    prefetch_tmap(&map_res);
-  }
-  if (warp == 1) {
-    tmem_alloc(tmem_slot, Cfg::BN);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  cluster_arrive();          // every CTA of the cluster runs, its barriers set, before anything is sent to it
-  cluster_wait();
-  tc_fence_after();
-  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-  if (threadIdx.x == 0) grid_dep_launch();
-
-  bool ok = aligned;
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    auto load_w = [&](int st, int kb) {                // with the stage's expected bytes
-      mbar_expect_tx(&full[st], Cfg::STAGE_BYTES);
-      tma_load_3d(smem + st * Cfg::STAGE_BYTES + A_TILE_BYTES, &map_w, &full[st], (kb0 + kb) * BK, c.nt * Cfg::BN, 0);
-    };
-    auto load_a = [&](int st, int kb) {
-      tma_load_3d(smem + st * Cfg::STAGE_BYTES, &map_a, &full[st], (kb0 + kb) * BK, c.mt * BM, c.b);
-    };
-    const int early = ok ? min(STAGES, n_kb) : 0;      // weights before the wait for earlier launches, activations behind it
-    if (elect_one())
-      for (int kb = 0; kb < early; ++kb) load_w(kb, kb);
-    __syncwarp();
-    grid_dep_wait();
-    if (elect_one())
-      for (int kb = 0; kb < early; ++kb) load_a(kb, kb);
-    __syncwarp();
-    int issued = early;
-    for (; ok && issued < n_kb; ++issued) {
-      const int st = issued % STAGES;
-      if (!(ok = mbar_wait_warp(&empty[st], (issued / STAGES - 1) & 1u, abort_flag))) break;
-      if (elect_one()) {
-        load_w(st, issued);
-        load_a(st, issued);
-      }
-      __syncwarp();
-    }
-    if (!ok && lane == 0) {                            // gave up: copies already issued land before the CTA leaves
-      for (int kb = max(0, issued - STAGES); kb < issued; ++kb) {
-        volatile uint32_t dummy = 0;
-        mbar_wait_slow(&full[kb % STAGES], (uint32_t)(kb / STAGES) & 1u, &dummy, kDrainLimitCycles);
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    constexpr uint32_t idesc = idesc_bf16_f32(BM, Cfg::BN, false, false);
-    const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-    const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + A_TILE_BYTES), 16, 1024);
-    for (int kb = 0; ok && kb < n_kb; ++kb) {
-      const int st = kb % STAGES;
-      if (!(ok = mbar_wait_warp(&full[st], (uint32_t)(kb / STAGES) & 1u, abort_flag))) break;
-      tc_fence_after();
-      if (elect_one()) {
-        const uint64_t soff = (uint64_t)(st * (Cfg::STAGE_BYTES >> 4));
-        const uint64_t da = a_desc0 + soff, db = b_desc0 + soff;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mma_ss(tmem_base, da + 2 * u, db + 2 * u, idesc, kb > 0 || u > 0);
-        mma_commit(&empty[st]);
-      }
-      __syncwarp();
-    }
-    if (ok && elect_one()) mma_commit(tmem_full);
-    __syncwarp();
-  } else {
-    // ---------------- epilogue (thread = row) ----------------
-    const int quad = warp & 3;                         // TMEM lanes [32 * quad, 32 * quad + 32)
-    const int row0 = c.mt * BM + quad * 32;
-    const int n_own = c.nt * Cfg::BN + rank * OWN;     // first column this CTA finishes
-    const bool live = row0 < p.rows;                   // (the same in every CTA of the cluster)
-    float* s_bias = reinterpret_cast<float*>(smem + Cfg::OFF_BIAS);
-    float* s_gate = reinterpret_cast<float*>(smem + Cfg::OFF_GATE);
-    Epilogue<EPI, Cfg::BN, false, false> ep{p, &map_out, &map_res, smem + Cfg::OFF_RING + quad * CHUNKS * BUF_BYTES,
-                                            res_full + quad * RING, s_bias, s_gate, abort_flag, lane, p.resid_rows ? lane : 0};
-    const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-    // partial sums in shared memory: [slot][chunk][quad][4 columns][lane] of 16 bytes, so that a warp moves whole lines
-    auto part_at = [&](int slot, int ch) { return (uint32_t)(slot * Cfg::PART_BYTES + ((ch * 4 + quad) * 8) * 512 + lane * 16); };
-    // The first round is a rehearsal (see kRehearse).
-#pragma unroll 1
-    for (int round = 0; round < 2; ++round) {
-      const bool dry = round == 0;
-      if (!dry) {
-        grid_dep_wait();
-        if (live && ok) {
-#pragma unroll
-          for (int ch = 0; ch < CHUNKS; ++ch) ep.request(c.b, row0, n_own + ch * CHUNK);
-          if (lane == 0) mbar_expect_tx(&part_full[quad], (S - 1) * CHUNKS * 4096);
-        }
-        for (int i = (threadIdx.x - 64) * 2; i < OWN; i += 256) {
-          const uint32_t bb = __ldg(reinterpret_cast<const uint32_t*>(p.bias + n_own + i));
-          *reinterpret_cast<float2*>(s_bias + i) = make_float2(bf16_lo(bb), bf16_hi(bb));
-          *reinterpret_cast<float2*>(s_gate + i) = ld_f2(p.gate + (size_t)c.b * p.gate_stride + n_own + i);
-        }
-        named_barrier(1, 128);
-        ok = ok && mbar_wait_warp(tmem_full, 0, abort_flag);
-        tc_fence_after();
-      }
-      if (!live || !ok) continue;
-      // send the partial sums of the other CTAs' columns
-#pragma unroll 1
-      for (int i = 1; i < S; ++i) {
-        const int to = (rank + i) % S;                 // (every CTA starts with another receiver)
-        const uint32_t dst = mapa_shared(smem_u32(smem + Cfg::OFF_PART), (uint32_t)to);
-        const uint32_t bar = mapa_shared(smem_u32(&part_full[quad]), (uint32_t)to);
-#pragma unroll 1
-        for (int ch = 0; ch < CHUNKS; ++ch) {
-          uint32_t v[32];
-          tmem_ld32(t_addr + to * OWN + ch * CHUNK, v);
-          tmem_ld_wait_on(v);
-          const uint32_t at = dst + part_at(rank < to ? rank : rank - 1, ch);
-          if (!dry) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) st_async_v4(at + q * 512, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3], bar);
-          }
-        }
-      }
-      // finish this CTA's own columns
-      if (!dry) ok = __all_sync(0xffffffffu, mbar_wait_cluster(&part_full[quad], 0, abort_flag));
-#pragma unroll 1
-      for (int ch = 0; ok && ch < CHUNKS; ++ch) {
-        uint32_t own[32];
-        tmem_ld32(t_addr + rank * OWN + ch * CHUNK, own);
-        tmem_ld_wait_on(own);
-        float v[CHUNK];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int r = 0; r < S; ++r) {
-            const int slot = r < rank ? r : r - 1;
-            const float4 x = r == rank ? make_float4(__uint_as_float(own[4 * q]), __uint_as_float(own[4 * q + 1]),
-                                                     __uint_as_float(own[4 * q + 2]), __uint_as_float(own[4 * q + 3]))
-                                       : *reinterpret_cast<const float4*>(smem + Cfg::OFF_PART + part_at(slot, ch) + q * 512);
-            sum.x = r ? sum.x + x.x : x.x;
-            sum.y = r ? sum.y + x.y : x.y;
-            sum.z = r ? sum.z + x.z : x.z;
-            sum.w = r ? sum.w + x.w : x.w;
-          }
-          const float4 bb = reinterpret_cast<const float4*>(s_bias + ch * CHUNK)[q];
-          v[4 * q + 0] = sum.x + bb.x;
-          v[4 * q + 1] = sum.y + bb.y;
-          v[4 * q + 2] = sum.z + bb.z;
-          v[4 * q + 3] = sum.w + bb.w;
-        }
-        uint8_t* buf = ep.ring + ch * BUF_BYTES;
-        if (!dry && !(ok = mbar_wait_warp(ep.rbar + ch, 0, abort_flag))) break;
-        ep.gate_chunk(buf, s_gate + ch * CHUNK, v);
-        if (dry) {
-          fence_proxy_async_smem();                    // before the residual arrives where this wrote
-          __syncwarp();
-          break;
-        }
-        ep.send(buf, c.b, row0, n_own + ch * CHUNK);
-      }
-    }
-    if (!ok) {
-      // gave up: the residual chunks already requested must land before the CTA leaves
-      for (uint32_t i = 0; i < ep.asked; ++i) {
-        volatile uint32_t dummy = 0;
-        mbar_wait_slow(ep.rbar + i, 0, &dummy, kDrainLimitCycles);
-      }
-      for (int i = 0; i < 64; ++i) __nanosleep(1000);  // and so must partial sums on their way
-    }
-    if (lane == 0) bulk_wait<0>();       // this warp's stores are complete
-    __syncwarp();
-  }
-  // No CTA leaves while others may still send to it.
-  tc_fence_before();
-  __syncthreads();
-  cluster_arrive();
-  cluster_wait();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem_base, Cfg::BN);
-  }
-  if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
-}
-
 // ---------------------------------------------------------------------------------------------
 GemmParams make_params(const GemmLaunch& g) {
   GemmParams p;
@@ -998,24 +748,8 @@ int launch_pair(const GemmLaunch& g, cudaStream_t stream, bool chained) {
                        g.map_res, make_params(g));
 }
 
-template <int EPI, int S>
-int launch_split(const GemmLaunch& g, cudaStream_t stream, bool chained) {
-  using Cfg = SplitCfg<S>;
-  static PerDeviceInt attr_done;
-  auto kern = gemm_split_kernel<EPI, S>;
-  if (int rc = ensure_smem_attr(kern, Cfg::SMEM_BYTES, attr_done)) return rc;
-  const long long tiles = (long long)g.batch * ((g.rows + BM - 1) / BM) * (g.N / Cfg::BN);
-  if (tiles > (1ll << 28)) return XEMA_EINVAL;
-  return launch_kernel(kern, dim3((unsigned)(tiles * S)), GEMM_THREADS, Cfg::SMEM_BYTES, stream, chained, g.map_a, g.map_w, g.map_out,
-                       g.map_res, make_params(g));
-}
-
 template <int EPI>
 int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
-  if constexpr (kGated<EPI>) {
-    if (g.split == 4) return launch_split<EPI, 4>(g, stream, chained);
-    if (g.split == 2) return launch_split<EPI, 2>(g, stream, chained);
-  }
   if constexpr (EPI == XEMA_EPI_GATE_RES_F32) {
     // six stages from four tiles a pair on (5.7 of them at 8888 rows x 3072 columns are 3 % faster, 2.9 at 4608 1 % slower)
     const long long tiles = (long long)g.batch * ((g.rows + 2 * BM - 1) / (2 * BM)) * (g.N / 256);
@@ -1051,7 +785,7 @@ bool tile_fits(const GemmLaunch& g, const Tile& t) {
   return g.epilogue != XEMA_EPI_BIAS_NORM_ROPE || t.block_n >= g.head_dim;   // whole heads only
 }
 
-long long pick_tile(GemmLaunch* g) {      // returns its estimate
+void pick_tile(GemmLaunch* g) {
   const long long k_blocks = g->K / BK;
   long long best = 0;
   g->block_n = 0;
@@ -1067,22 +801,6 @@ long long pick_tile(GemmLaunch* g) {      // returns its estimate
       g->pair = t.pair;
     }
   }
-  return best;
-}
-
-// How many CTAs share the K of a gated product (1: none): taken where the clusters of every 128 x 128 tile of the whole
-// template run at once (7/8 of the SMs: clusters of four do not fill every GPC) and the estimate -- 265 ns per K block as
-// above, 2000 for the exchange and a later start -- is a tenth below the best whole tile's.  A block of 333 x 1024 (K = 4096) gains
-// 2.4 us, one of 288 x 512 (K = 2048) nothing; PROJ of the same blocks (K = 1024, 512) fails the estimate.
-int split_for(const GemmLaunch& g, int batch, int rows) {
-  GemmLaunch whole = g;
-  whole.batch = batch;
-  whole.rows = rows;
-  const long long best = pick_tile(&whole), k_blocks = g.K / BK;
-  const long long tiles = (long long)batch * ((rows + BM - 1) / BM) * (g.N / SplitCfg<2>::BN);
-  for (int s = 4; s > 1; s /= 2)
-    if (tiles * s <= sm_count() * 7 / 8 && k_blocks >= s && 10 * ((k_blocks + s - 1) / s * 265 + 2000) < 9 * best) return s;
-  return 1;
 }
 
 // The sizes and flags of a problem, without its pointers.
@@ -1105,11 +823,6 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained) {
     case XEMA_EPI_BIAS_NORM_ROPE: return launch_epi<XEMA_EPI_BIAS_NORM_ROPE>(g, stream, chained);
     default: return XEMA_EINVAL;
   }
-}
-
-int gemm_split(const GemmLaunch& g, int batch, int rows) {
-  const bool gated = g.epilogue == XEMA_EPI_GATE_RES_F32 || g.epilogue == XEMA_EPI_GATE_RES_BF16;
-  return gated && check_shape(g) == XEMA_OK ? split_for(g, batch, rows) : 1;
 }
 
 int gemm_tile(GemmLaunch* g) {
@@ -1141,10 +854,7 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   g->lda = lda;
   g->a_batch_rows = a_batch_rows;
   g->ldw = ldw;
-  if (g->split > 1) {
-    g->pair = 0;
-    g->block_n = SplitCfg<2>::BN;
-  } else if (!tile) {
+  if (!tile) {
     pick_tile(g);
   } else {
     g->block_n = 0;

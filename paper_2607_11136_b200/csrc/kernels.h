@@ -110,7 +110,6 @@ struct GemmLaunch {
   const float* gate;
   long long gate_stride;
   int batch, rows, N, K, epilogue, block_n;
-  int split;           // > 1: gated products whose K is divided among that many CTAs of a cluster (see gemm_split)
   int pair;            // a CTA pair per tile (256 x block_n) or one CTA (128 x block_n)
   const void *a, *w;   // operands as given to gemm_prepare
   long long lda, a_batch_rows, ldw;
@@ -126,9 +125,6 @@ struct GemmLaunch {
 // of the one estimated to be fastest, XEMA_EINVAL where the problem cannot run in it.
 int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_rows, const void* w, long long ldw,
                  const int* tile = nullptr);
-// How many CTAs should share the K of this product in a plan whose template has `batch` x `rows` token rows (1: none).
-// The bits of a result depend on it, so all launches of the product in a plan take the same.
-int gemm_split(const GemmLaunch& g, int batch, int rows);
 // The tile alone, on the host (GemmLaunch as for gemm_prepare): fills pair and block_n.
 int gemm_tile(GemmLaunch* g);
 int launch_gemm(const GemmLaunch& g, cudaStream_t stream, bool chained = false);

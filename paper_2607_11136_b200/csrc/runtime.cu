@@ -487,7 +487,6 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       g.resid = resid; g.ldr = ldr; g.resid_batch_rows = resid_batch_rows;
       g.gate = gate; g.gate_stride = 6 * D;
       g.batch = pc.nb; g.rows = rows; g.N = N; g.K = K; g.epilogue = epi; g.status = status;
-      g.split = gemm_split(g, c.batch, (int)S_all);      // the same for every piece and every shard
       int rc = gemm_prepare(&g, a, lda, a_batch_rows, wt, ldw);
       if (rc) return rc;
       plan->ops.push_back(o);

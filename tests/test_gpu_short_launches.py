@@ -1,4 +1,4 @@
-"""Forms that only the short launches of a plan take: the FFN2 product with its K divided over a cluster, the attention that
+"""What the short launches of a plan do differently, and what they must not: the bits of their products, the attention that
 rehearses, the launches that open a call."""
 import numpy as np
 import pytest
@@ -8,8 +8,6 @@ from paper_2607_11136_b200 import binding as xb
 from paper_2607_11136_b200.session import BlockSession
 from xema_inputs import Template, make_activations, make_block_weights
 
-from gpu_util import assert_bf16_close, from_dev_bf16
-
 pytestmark = pytest.mark.gpu
 
 
@@ -18,61 +16,53 @@ def _template(batch, tokens, hidden, ffn, heads=None):
     return Template("short", batch, 8, 1, 1, tokens - 8, hidden, heads, hidden // heads, ffn)
 
 
-# (batch, tokens, hidden, ffn, CTAs that share K): few rows, both sides of the 128-row tiles, several batch elements, K blocks
-# fewer and more than the stages (8 to 32 a CTA), the most tiles that still share
-@pytest.mark.parametrize("batch,tokens,hidden,ffn,split", [
-    (1, 9, 512, 2048, 4), (1, 128, 512, 2304, 4), (1, 129, 1024, 4096, 4), (2, 255, 512, 4096, 4), (1, 512, 1024, 4096, 4),
-    (1, 577, 1024, 4096, 2), (3, 200, 1024, 4352, 2)])
-def test_ffn2_with_k_divided_over_a_cluster(batch, tokens, hidden, ffn, split):
-    t = _template(batch, tokens, hidden, ffn)
+def _op_gemm(s, tokens, N, K, a, w, bias, resid, gate, epilogue):
+    """The gated product of a plan of whole phases once more, as the stand-alone operator computes it."""
+    t = s.template
+    out = torch.empty((t.batch, tokens, N), dtype=torch.float32 if epilogue == xb.EPI_GATE_RES_F32 else torch.int16, device="cuda")
+    xb.xema_op_gemm(a=a.data_ptr(), lda=K, a_batch_rows=tokens, w=w.data_ptr(), ldw=K, bias=bias.data_ptr(), out=out.data_ptr(),
+                    ldo=N, out_batch_rows=tokens, resid=resid.data_ptr(), ldr=N, resid_batch_rows=tokens, gate=gate.data_ptr(),
+                    gate_stride=6 * N, batch=t.batch, rows=tokens, N=N, K=K, epilogue=epilogue, status=s.status.data_ptr(),
+                    stream=torch.cuda.current_stream().cuda_stream)
+    return out
+
+
+# few rows, widths and K that leave SMs without a tile: one sum over K in order, whatever the plan
+@pytest.mark.parametrize("batch,tokens,hidden,ffn", [
+    (1, 9, 512, 2048), (1, 128, 512, 2304), (1, 129, 1024, 4096), (2, 255, 512, 4096), (1, 333, 1024, 4096), (1, 577, 1024, 4096),
+    (3, 200, 1024, 4352), (1, 256, 2048, 2048), (2, 120, 1536, 1536), (1, 100, 3072, 3072), (1, 1100, 512, 2048)])
+def test_gated_products_of_a_plan_have_the_bits_of_the_operator(batch, tokens, hidden, ffn):
+    s = BlockSession(_template(batch, tokens, hidden, ffn), [make_block_weights(_template(batch, tokens, hidden, ffn), 3)],
+                     chunks=(1, 1, 1))
+    s.set_inputs(*make_activations(s.template))
+    w, rows = s.weights[0], (batch, tokens)
+    mod = s.view("mod0", torch.float32, (batch, 6 * hidden))
+    s.plan.forward_prefix(9, torch.cuda.current_stream().cuda_stream)      # up to PROJ
+    res = s.view("res0", torch.float32, rows + (hidden,))
+    proj = _op_gemm(s, tokens, hidden, hidden, s.view("o0_0", torch.int16, rows + (hidden,)), w["w_o"], w["b_o"],
+                    s.view("hid0", torch.int16, rows + (hidden,)), mod[:, 2 * hidden:], xb.EPI_GATE_RES_F32)
+    assert torch.equal(proj, res)
+    s.forward()                            # (the operands of FFN2 outlive it in the arena)
+    ffn2 = _op_gemm(s, tokens, hidden, ffn, s.view("g0_0", torch.int16, rows + (ffn,)), w["w_2"], w["b_2"], res,
+                    mod[:, 5 * hidden:], xb.EPI_GATE_RES_BF16)
+    assert torch.equal(ffn2, s.hid_out())
+    s.check_status()
+
+
+@pytest.mark.parametrize("tokens,hidden", [(200, 512), (333, 1024)])
+def test_a_request_has_the_same_bits_alone_and_in_a_batch(tokens, hidden):
+    t = _template(3, tokens, hidden, 4 * hidden)
     w = make_block_weights(t, 3)
     x, temb = make_activations(t)
     outs = []
-    for chunks in ((1, 1, 1), (1, 1, min(3, tokens))):
-        s = BlockSession(t, [w], chunks=chunks)
-        s.set_inputs(x, temb)
+    for first, n in ((0, 3), (0, 1), (1, 2), (2, 1)):
+        s = BlockSession(_template(n, tokens, hidden, 4 * hidden), [w], chunks=(1, 1, 1))
+        s.set_inputs(np.ascontiguousarray(x[first:first + n]), np.ascontiguousarray(temb[first:first + n]))
         s.forward()
-        outs.append(s.output_bits().copy())
+        outs.append((first, n, s.output_bits().copy()))
         s.check_status()
-        if chunks[2] > 1:
-            continue
-        # the operands of FFN2 outlive it in the arena
-        g = s.view("g0_0", torch.int16, (batch, tokens, ffn))
-        res = s.view("res0", torch.float32, (batch, tokens, hidden))
-        gate = s.view("mod0", torch.float32, (batch, 6 * hidden))[:, 5 * hidden:]
-        w2, b2 = s.weights[0]["w_2"], s.weights[0]["b_2"]
-        f64 = lambda v: torch.from_numpy(from_dev_bf16(v))
-        want = res.double().cpu() + gate.double().cpu()[:, None] * (f64(g) @ f64(w2).T + f64(b2))
-        # partial sums add fp32 roundings only: the bound of every other form of the product
-        assert_bf16_close(from_dev_bf16(s.hid_out()), want.numpy(), (batch, tokens, hidden, ffn))
-        # the undivided sum differs in its last bits, and in a bf16 rounding here and there
-        out = torch.empty_like(s.hid_out())
-        kw = dict(a=g.data_ptr(), lda=ffn, a_batch_rows=tokens, w=w2.data_ptr(), ldw=ffn, bias=b2.data_ptr(), out=out.data_ptr(),
-                  ldo=hidden, out_batch_rows=tokens, resid=res.data_ptr(), ldr=hidden, resid_batch_rows=tokens,
-                  gate=gate.data_ptr(), gate_stride=6 * hidden, batch=batch, rows=tokens, N=hidden, K=ffn,
-                  epilogue=xb.EPI_GATE_RES_BF16)
-        xb.xema_op_gemm(status=s.status.data_ptr(), stream=torch.cuda.current_stream().cuda_stream, **kw)
-        tiles = batch * -(-tokens // 128) * (hidden // 128)
-        assert tiles * split <= 148 * 7 // 8 and (split == 4 or tiles * 4 > 148 * 7 // 8)
-        if tokens > 100:
-            assert not torch.equal(out, s.hid_out())
-        assert_bf16_close(from_dev_bf16(out), want.numpy(), "undivided")
-    assert np.array_equal(outs[0], outs[1])
-
-
-def test_a_template_of_many_rows_is_not_divided():
-    t = _template(1, 1100, 512, 2048)      # 36 tiles of 128 x 128: its FFN2 keeps the bits of xema_op_gemm
-    s = BlockSession(t, [make_block_weights(t, 3)], chunks=(1, 1, 1))
-    s.set_inputs(*make_activations(t))
-    s.forward()
-    g, res = s.view("g0_0", torch.int16, (1, 1100, 2048)), s.view("res0", torch.float32, (1, 1100, 512))
-    gate = s.view("mod0", torch.float32, (1, 3072))[:, 2560:]
-    out = torch.empty_like(s.hid_out())
-    xb.xema_op_gemm(status=s.status.data_ptr(), stream=torch.cuda.current_stream().cuda_stream, a=g.data_ptr(), lda=2048,
-                    a_batch_rows=1100, w=s.weights[0]["w_2"].data_ptr(), ldw=2048, bias=s.weights[0]["b_2"].data_ptr(),
-                    out=out.data_ptr(), ldo=512, out_batch_rows=1100, resid=res.data_ptr(), ldr=512, resid_batch_rows=1100,
-                    gate=gate.data_ptr(), gate_stride=3072, batch=1, rows=1100, N=512, K=2048, epilogue=xb.EPI_GATE_RES_BF16)
-    assert torch.equal(out, s.hid_out())
+    for first, n, y in outs[1:]:
+        assert np.array_equal(y, outs[0][2][first:first + n]), (first, n)
 
 
 # the attention of a plan follows another launch and, up to 8 key blocks a CTA, rehearses; the same call by itself does not
