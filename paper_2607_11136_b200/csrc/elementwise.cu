@@ -13,7 +13,6 @@ using sm100::bf16_hi;
 using sm100::bf16_lo;
 using sm100::grid_dep_launch;
 using sm100::grid_dep_wait;
-using sm100::ld_b16;
 using sm100::ld_f4;
 using sm100::ld_u4;
 using sm100::pack_bf16x2;
@@ -30,15 +29,11 @@ __device__ __forceinline__ float warp_sum(float v) {
 // 512 inputs before the wait for earlier launches (the weights do not depend on them); silu(temb) for
 // all batch elements sits in shared memory.  Bound by the latency of one trip to HBM for one batch
 // element, by the reductions (five shuffles per feature and batch element) for several.
-// OPENS: the launch that opens a call, which may have started before the work ahead of it in the stream has
-// finished.  That may be writing anything, the weights too, so the kernel reads, and lets later launches start,
-// only behind its wait.
 // ---------------------------------------------------------------------------------------
 constexpr int kModWarps = 8;
 constexpr int kModRows = 4;
 constexpr int kModMaxBatch = 4;     // batch elements per pass over the weights
 
-template <bool OPENS>
 __global__ void __launch_bounds__(kModWarps * 32)
 mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, const __nv_bfloat16* __restrict__ bias,
                 float* mod, int batch, int Dt, int n_out) {
@@ -47,29 +42,16 @@ mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, 
   const int j0 = (blockIdx.x * kModWarps + warp) * kModRows;
   const int n8 = Dt / 8;
   auto weights = [&](int r, int k8) {
-    if (j0 + r >= n_out || k8 >= n8) return make_uint4(0u, 0u, 0u, 0u);
-    const uint4* at = reinterpret_cast<const uint4*>(w + (size_t)(j0 + r) * Dt) + k8;
-    return OPENS ? ld_u4(at) : __ldg(at);      // (a read-only load could move above the wait)
+    return (j0 + r < n_out && k8 < n8) ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)(j0 + r) * Dt) + k8)
+                                       : make_uint4(0u, 0u, 0u, 0u);
   };
-  if (OPENS) {
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int r = 0; r < kModRows; ++r)
-        if (j0 + r < n_out && u * 32 + lane < n8)
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(w + (size_t)(j0 + r) * Dt + (u * 32 + lane) * 8));
-    grid_dep_wait();
-    grid_dep_launch();
-  }
   uint4 first[2][kModRows];
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
     for (int r = 0; r < kModRows; ++r) first[u][r] = weights(r, u * 32 + lane);
-  if (!OPENS) {
-    grid_dep_launch();
-    grid_dep_wait();
-  }
+  grid_dep_launch();
+  grid_dep_wait();
   for (int i = threadIdx.x; i < batch * Dt; i += blockDim.x) {
     const float z = __bfloat162float(*(const volatile __nv_bfloat16*)(temb + i));
     s_e[i] = z / (1.f + __expf(-z));
@@ -112,23 +94,20 @@ mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, 
 #pragma unroll
       for (int r = 0; r < kModRows; ++r) {
         const float sum = warp_sum(acc[r][b]);
-        if (lane == r && j0 + r < n_out) mod[(size_t)(b0 + b) * n_out + j0 + r] = sum + __bfloat162float(OPENS ? ld_b16(bias + j0 + r) : bias[j0 + r]);
+        if (lane == r && j0 + r < n_out) mod[(size_t)(b0 + b) * n_out + j0 + r] = sum + __bfloat162float(bias[j0 + r]);
       }
     }
   }
 }
 
 int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream, bool chained, bool opens) {
+               cudaStream_t stream, bool chained) {
   if (batch < 1 || Dt < 8 || (Dt & 7) || n_out < 1) return XEMA_EINVAL;
   size_t smem = (size_t)batch * Dt * sizeof(float);
   if (smem > 48 * 1024) return XEMA_EINVAL;
   const int blocks = (n_out + kModWarps * kModRows - 1) / (kModWarps * kModRows);
-  auto run = [&](auto kern) {
-    return launch_kernel(kern, dim3(blocks), kModWarps * 32, smem, stream, chained || opens, (const __nv_bfloat16*)temb,
-                         (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
-  };
-  return opens ? run(mod_gemv_kernel<true>) : run(mod_gemv_kernel<false>);
+  return launch_kernel(mod_gemv_kernel, dim3(blocks), kModWarps * 32, smem, stream, chained, (const __nv_bfloat16*)temb,
+                       (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -382,9 +361,8 @@ int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void*
 // ---------------------------------------------------------------------------------------
 // Two contiguous copies in one launch (a forward call's inputs): 16 bytes per thread and step, four
 // loads in flight.  One launch instead of two memory copies takes 2-4 us off a call with small inputs;
-// bound by HBM for large ones.  Like the modulation that opens a call, it may be launched before the work ahead of it in
-// the stream has finished, and waits for that (back to back with it, a block of 288 x 512 48.2 -> 45.6 us, of 1101 x 1536
-// 121.9 -> 118.7).
+// bound by HBM for large ones.  It may be launched before the work ahead of it in the stream has finished, and waits for
+// that (calls back to back, a block of 288 x 512 47.1 -> 45.1 us, of 1101 x 1536 123.7 -> 122.2).
 // ---------------------------------------------------------------------------------------
 constexpr int kCopyThreads = 256;
 
@@ -405,16 +383,15 @@ __device__ __forceinline__ void copy_part(uint8_t* dst, const uint8_t* src, size
 __global__ void __launch_bounds__(kCopyThreads)
 copy2_kernel(uint8_t* dst0, const uint8_t* src0, size_t n0, uint8_t* dst1, const uint8_t* src1, size_t n1) {
   grid_dep_wait();
-  grid_dep_launch();
   copy_part(dst0, src0, n0);
   copy_part(dst1, src1, n1);
 }
 
 int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream,
-                 bool opens) {
+                 bool early) {
   const size_t steps = (std::max(n0, n1) / 16 + 4 * kCopyThreads) / (4 * kCopyThreads);
   const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>(steps, 1), (size_t)sm_count() * 8);
-  return launch_kernel(copy2_kernel, dim3(blocks), kCopyThreads, 0, stream, opens, (uint8_t*)dst0, (const uint8_t*)src0, n0,
+  return launch_kernel(copy2_kernel, dim3(blocks), kCopyThreads, 0, stream, early, (uint8_t*)dst0, (const uint8_t*)src0, n0,
                        (uint8_t*)dst1, (const uint8_t*)src1, n1);
 }
 

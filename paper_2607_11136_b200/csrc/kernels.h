@@ -47,8 +47,9 @@ int ensure_smem_attr(Kernel kern, int bytes, PerDeviceInt& done) {
 // Launches a kernel.  `chained`: it may start while the launch before it in the stream still runs
 // (programmatic dependent launch) -- for kernels that call grid_dep_wait() before they touch memory
 // which earlier launches use, and whose weights no launch before them in the same forward call
-// writes.  The first launch of a call is never chained: what the caller enqueued before it is then
-// complete before any kernel of the call starts.  Measured (B200): without it launches of dependent
+// writes.  The first launch of a forward call is never chained: what the caller enqueued before it, weights
+// too, is then complete before any kernel of the call starts.  (A launch that only waits for the work ahead of it and
+// copies may itself be chained to that: launch_copy2.)  Measured (B200): without it launches of dependent
 // kernels start on a 2.05 us raster, 2 to 4 us after the previous one's last CTA.
 template <typename... Params, typename... Args>
 int launch_kernel(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool chained,
@@ -73,16 +74,17 @@ int launch_kernel(void (*kern)(Params...), dim3 grid, int threads, size_t smem, 
 }
 
 int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream, bool chained = false, bool opens = false);
+               cudaStream_t stream, bool chained = false);
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
                        cudaStream_t stream, bool chained = false);
 int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void* g, const float* rope, int pos0,
                         int batch, int rows, int heads, int head_dim, float eps, cudaStream_t stream);
 
-// dst0 <- src0 (n0 bytes) and dst1 <- src1 (n1 bytes); pointers and sizes are multiples of 16 bytes.
+// dst0 <- src0 (n0 bytes) and dst1 <- src1 (n1 bytes); pointers and sizes are multiples of 16 bytes.  `early`: it may be
+// launched before the work ahead of it in the stream has finished; it waits for that before its first access.
 int launch_copy2(void* dst0, const void* src0, size_t n0, void* dst1, const void* src1, size_t n1, cudaStream_t stream,
-                 bool opens = false);
+                 bool early = false);
 
 // ---- TMA descriptors (encoded on the host once per bound tensor) --------------------------
 // bf16 tensor viewed as [batch][rows][cols] with row stride ld and batch stride batch_rows*ld

@@ -178,13 +178,11 @@ struct xema_plan {
 };
 
 // `chained`: the launch right before this one in the stream is the op before it (see launch_kernel).
-// `opens`: it opens a call and may start before the launch ahead of it in the stream has finished (it waits for that
-// one itself before it reads anything).
-static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained, bool opens = false) {
+static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained) {
   const xema_config& c = pl->cfg;
   switch (op.kind) {
     case OP_MOD:
-      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained, opens);
+      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained);
     case OP_LN:
       return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale,
                                 6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st, chained);
@@ -201,8 +199,8 @@ static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chaine
   return XEMA_EINVAL;
 }
 
-// Whether a launch that opens a call may start early: not inside a stream capture, where the node ahead of it need not
-// be a kernel.
+// Whether the copy of the inputs may be launched before the work ahead of it in the stream has finished: not inside a
+// stream capture, where the node ahead of it need not be a kernel.
 static bool may_open(cudaStream_t st) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
@@ -219,8 +217,7 @@ static int run_ops(const xema_plan* pl, size_t first, size_t n, void* stream) {
   n = std::min(n, pl->ops.size());
   bool chained = false;
   for (size_t i = first; i < n; ++i) {
-    const bool opens = !chained && pl->ops[i].kind == OP_MOD && may_open(st);
-    int rc = issue(pl, pl->ops[i], st, chained, opens);
+    int rc = issue(pl, pl->ops[i], st, chained);
     if (rc) return rc;
     chained = chained || pl->ops[i].kind != OP_FUSED;
   }

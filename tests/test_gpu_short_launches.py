@@ -86,29 +86,79 @@ def test_attention_behind_another_launch_keeps_its_bits(head_dim, tokens, chunks
 
 
 
+MASK = 0x5a5a
+
+
+class _Tail:
+    """Device tensors at the end of a large buffer.  `write(i)` puts source `i` there with one kernel that works through the whole
+    buffer, some 50 us, and comes to the tensors last: what is launched right behind it is there before they are written."""
+
+    def __init__(self, sources):
+        shapes = {k: v.shape for k, v in sources[0].items()}
+        end = [0]
+        for v in sources[0].values():
+            assert v.size % 8 == 0               # every tensor starts on a 16-byte boundary
+            end.append(end[-1] + v.size)
+        lead = (1 << 26) - end[-1]
+        self.live = torch.zeros(1 << 26, dtype=torch.int16, device="cuda")
+        self.sources = []
+        for src in sources:
+            flat = torch.from_numpy(np.concatenate([v.reshape(-1) for v in src.values()]).view(np.int16)).cuda()
+            self.sources.append(torch.zeros_like(self.live))
+            self.sources[-1][lead:] = flat ^ MASK
+        self.tensors = {k: self.live[lead + at:lead + at + int(np.prod(shape))].view(shape)
+                        for (k, shape), at in zip(shapes.items(), end)}
+
+    def write(self, i):
+        torch.bitwise_xor(self.sources[i], MASK, out=self.live)
+
+
 @pytest.mark.parametrize("tokens", [130, 1030])
-def test_calls_back_to_back_see_their_own_inputs_and_weights(tokens):
-    """The first launches of a call may start while the work ahead of them runs: inputs, and weights that a kernel of the
-    caller writes right before the call, are read only when it has finished."""
+def test_calls_see_what_a_kernel_wrote_right_before_them(tokens):
+    """The copy of set_inputs is launched while the work ahead of it still runs, and weights are requested ahead of a launch's own
+    wait: inputs and weights of a call are those that the caller's last kernel before it wrote, and its output is the
+    caller's until the next call.  Nothing but kernels stands between the calls: no copy, no synchronisation."""
     t = _template(1, tokens, 512, 2048)
     ws = [make_block_weights(t, seed) for seed in (1, 2)]
-    ins = [make_activations(t, seed) for seed in (3, 4)]
-    want = []
-    for w, (x, temb) in zip(ws, ins):
-        s = BlockSession(t, [w], chunks=(1, 1, 1))
-        s.set_inputs(x, temb)
+    ins = [dict(zip(("x", "temb"), make_activations(t, seed))) for seed in (3, 4)]
+    want = {}
+    for i, w in enumerate(ws):
+        for j, a in enumerate(ins):
+            s = BlockSession(t, [w], chunks=(1, 1, 1))
+            s.set_inputs(a["x"], a["temb"])
+            s.forward()
+            want[i, j] = s.output_bits().copy()
+    weights, inputs = _Tail(ws), _Tail(ins)
+    ready = [{k: torch.from_numpy(v.view(np.int16)).cuda() for k, v in a.items()} for a in ins]
+    s = BlockSession(t, [weights.tensors], chunks=(1, 1, 1))
+    outs, got = torch.empty((14,) + s.hid_out().shape, dtype=torch.int16, device="cuda"), []
+
+    def collect(i, j):
+        torch.bitwise_xor(s.hid_out(), MASK, out=outs[len(got)])
+        got.append((i, j))
+
+    weights.write(0)
+    torch.cuda.synchronize()
+    for j in (0, 1, 1, 0):                       # inputs written right before set_inputs
+        inputs.write(j)
+        s.set_inputs(inputs.tensors["x"], inputs.tensors["temb"])
         s.forward()
-        want.append(s.output_bits().copy())
-    dev = [{k: torch.from_numpy(v.view(np.int16)).cuda() for k, v in w.items()} for w in ws]
-    src = [[torch.from_numpy(v.view(np.int16)).cuda() for v in pair] for pair in ins]
-    s = BlockSession(t, [{k: v.clone() for k, v in dev[0].items()}], chunks=(1, 1, 1))
-    outs = []
-    for i in (0, 1, 1, 0, 1, 0):
-        x, temb = (v.clone() for v in src[i])
-        s.set_inputs(x, temb, non_blocking=True)
-        for k, v in s.weights[0].items():
-            v.copy_(dev[i][k])
+        collect(0, j)
+    for j in (1, 0, 1):                          # nothing between a call and the next one's inputs
+        for k in (1 - j, j):
+            s.set_inputs(ready[k]["x"], ready[k]["temb"])
+            s.forward()
+        collect(0, j)
+    for i in (1, 0, 0, 1):                       # weights written right before forward
+        s.set_inputs(ready[0]["x"], ready[0]["temb"])
+        weights.write(i)
         s.forward()
-        outs.append((i, s.hid_out().clone()))
-    for i, y in outs:
-        assert np.array_equal(y.cpu().numpy().view(np.uint16), want[i].reshape(y.shape))
+        collect(i, 0)
+    for i in (0, 1, 0):                          # weights written right before set_inputs
+        weights.write(i)
+        s.set_inputs(ready[1]["x"], ready[1]["temb"])
+        s.forward()
+        collect(i, 1)
+    s.check_status()
+    for (i, j), y in zip(got, outs):
+        assert np.array_equal((y ^ MASK).cpu().numpy().view(np.uint16), want[i, j].reshape(y.shape)), (i, j)

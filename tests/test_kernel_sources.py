@@ -28,3 +28,18 @@ def test_chained_kernels_wait_before_they_read_activations():
     gemm = _code("gemm.cu")
     producer = gemm[gemm.index("const int early = worker"):]
     assert producer.index("grid_dep_wait()") < producer.index("load_a(")
+
+
+def test_only_the_copy_of_the_inputs_is_chained_to_the_work_ahead_of_a_call():
+    """The launches of a forward call request weights ahead of their own waits, so the first of them starts when all that the
+    caller enqueued before has finished.  The copy may start early: it waits before its first access."""
+    runtime = _code("runtime.cu")
+    uses = re.findall(r"[^;{}]*\bmay_open\(st\)[^;{}]*;", runtime)
+    assert len(uses) == 1 and "return launch_copy2(" in uses[0], uses
+    run_ops = runtime[runtime.index("static int run_ops("):]
+    run_ops = run_ops[:run_ops.index("\n}")]
+    assert "bool chained = false;\n  for (" in run_ops
+    assert re.findall(r"\bissue\((.*)\)", run_ops) == ["pl, pl->ops[i], st, chained"]
+    copy = _code("elementwise.cu")
+    copy = copy[copy.index("copy2_kernel(uint8_t* dst0"):]
+    assert copy[copy.index("{") + 1:].split(";")[0].strip() == "grid_dep_wait()"
