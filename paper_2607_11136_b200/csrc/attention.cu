@@ -918,8 +918,27 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicExch(p.status, STATUS_TIMEOUT_MBARRIER);
 }
 
+// How a launch is divided: tiles an item, items a head, items, CTAs.
+struct AttnGrid {
+  int tiles, q_items, items, ctas;
+};
+
+int attention_grid(const AttnLaunch& a, AttnGrid* g) {
+  const long long q_tiles = (a.rows + BM - 1) / BM, bh = (long long)a.heads * a.batch;
+  // two tiles per item share their K and V blocks; where every tile can have an SM of its own they
+  // are faster apart
+  g->tiles = q_tiles * bh <= sm_count() ? 1 : TILES;
+  g->q_items = (int)((q_tiles + g->tiles - 1) / g->tiles);
+  const long long items = g->q_items * bh;
+  if (items > (1ll << 30)) return XEMA_EINVAL;
+  g->items = (int)items;
+  // one CTA per SM (each takes all of TMEM); more only where a CTA could not keep a flag per item
+  g->ctas = std::max((int)std::min<long long>(items, sm_count()), (int)((items + MAX_ITEMS - 1) / MAX_ITEMS));
+  return XEMA_OK;
+}
+
 template <int DH, bool SCALED, bool REHEARSE>
-int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
+int launch_attention_t(const AttnLaunch& a, const AttnGrid& g, cudaStream_t stream, bool chained) {
   using C = Cfg<DH>;
   static PerDeviceInt attr_done;
   auto kern = attention_kernel<DH, SCALED, REHEARSE>;
@@ -935,35 +954,29 @@ int launch_attention_t(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   p.status = a.status;
   p.gain_q = (const __nv_bfloat16*)a.gain_q;
   p.gain_k = (const __nv_bfloat16*)a.gain_k;
-  const long long q_tiles = (a.rows + BM - 1) / BM, bh = (long long)a.heads * a.batch;
-  // two tiles per item share their K and V blocks; where every tile can have an SM of its own they
-  // are faster apart
-  p.tiles = q_tiles * bh <= sm_count() ? 1 : TILES;
-  p.q_items = (int)((q_tiles + p.tiles - 1) / p.tiles);
-  const long long items = p.q_items * bh;
-  if (items > (1ll << 30)) return XEMA_EINVAL;
-  p.items = (int)items;
-  // one CTA per SM (each takes all of TMEM); more only where a CTA could not keep a flag per item
-  const int grid = std::max((int)std::min<long long>(items, sm_count()), (int)((items + MAX_ITEMS - 1) / MAX_ITEMS));
-  return launch_kernel(kern, dim3(grid), THREADS, C::SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
+  p.tiles = g.tiles;
+  p.q_items = g.q_items;
+  p.items = g.items;
+  return launch_kernel(kern, dim3(g.ctas), THREADS, C::SMEM_BYTES, stream, chained, a.map_q, a.map_k, a.map_v, p);
 }
 }  // namespace
 
 int launch_attention(const AttnLaunch& a, cudaStream_t stream, bool chained) {
   if (a.rows == 0 || a.batch == 0) return XEMA_OK;
+  AttnGrid g;
+  if (int rc = attention_grid(a, &g)) return rc;
   // Behind another launch there is a wait to use, and up to kRehearseBlocks key blocks a CTA the gain is the larger.
-  const long long tiles = (a.rows + BM - 1) / BM * (long long)a.heads * a.batch;
-  const long long rounds = (tiles + 2 * sm_count() - 1) / (2 * sm_count());
+  const long long rounds = (g.items + g.ctas - 1) / g.ctas;
   const bool rehearse = chained && rounds * ((a.keys + BN - 1) / BN) <= kRehearseBlocks;
   const bool scaled = a.q_scale != 1.f;
   if (a.head_dim == 64)
-    return scaled     ? launch_attention_t<64, true, false>(a, stream, chained)
-           : rehearse ? launch_attention_t<64, false, true>(a, stream, chained)
-                      : launch_attention_t<64, false, false>(a, stream, chained);
+    return scaled     ? launch_attention_t<64, true, false>(a, g, stream, chained)
+           : rehearse ? launch_attention_t<64, false, true>(a, g, stream, chained)
+                      : launch_attention_t<64, false, false>(a, g, stream, chained);
   if (a.head_dim == 128)
-    return scaled     ? launch_attention_t<128, true, false>(a, stream, chained)
-           : rehearse ? launch_attention_t<128, false, true>(a, stream, chained)
-                      : launch_attention_t<128, false, false>(a, stream, chained);
+    return scaled     ? launch_attention_t<128, true, false>(a, g, stream, chained)
+           : rehearse ? launch_attention_t<128, false, true>(a, g, stream, chained)
+                      : launch_attention_t<128, false, false>(a, g, stream, chained);
   return XEMA_EINVAL;
 }
 

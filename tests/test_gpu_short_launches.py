@@ -1,5 +1,7 @@
 """What the short launches of a plan do differently, and what they must not: the bits of their products, the attention that
 rehearses, the launches that open a call."""
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -65,25 +67,46 @@ def test_a_request_has_the_same_bits_alone_and_in_a_batch(tokens, hidden):
         assert np.array_equal(y, outs[0][2][first:first + n]), (first, n)
 
 
-# the attention of a plan follows another launch and, up to 8 key blocks a CTA, rehearses; the same call by itself does not
-@pytest.mark.parametrize("head_dim", [64, 128])
-@pytest.mark.parametrize("tokens,chunks", [(9, 1), (130, 1), (161, 3), (333, 2), (1024, 1), (1030, 1)])
-def test_attention_behind_another_launch_keeps_its_bits(head_dim, tokens, chunks):
-    t = _template(1, tokens, 512, 512, heads=512 // head_dim)
+def _attention_of_a_plan(batch, heads, head_dim, tokens, chunks):
+    """A session that has run up to its first attention launch: MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN."""
+    t = _template(batch, tokens, heads * head_dim, 512, heads=heads)
     s = BlockSession(t, [make_block_weights(t, 5)], chunks=(1, chunks, 1))
     s.set_inputs(*make_activations(t))
-    stream = torch.cuda.current_stream().cuda_stream
-    s.plan.forward_prefix(8, stream)       # MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN of the first chunk
+    s.plan.forward_prefix(8, torch.cuda.current_stream().cuda_stream)
+    return s
+
+
+# The attention of a plan follows another launch and, up to 8 key blocks a CTA, rehearses; the same call by itself does not.
+# One tile per item and two, one item per CTA and two, up to 8 key blocks and beyond.
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("batch,hidden,tokens,chunks", [
+    (1, 512, 9, 1), (1, 512, 130, 1), (1, 512, 161, 3), (1, 512, 333, 2), (1, 512, 1024, 1), (1, 512, 1030, 1),
+    (4, 1536, 257, 1), (8, 1536, 257, 1), (8, 1536, 400, 1), (8, 1536, 500, 4)])
+def test_attention_behind_another_launch_keeps_its_bits(head_dim, batch, hidden, tokens, chunks):
+    heads = hidden // head_dim
+    s = _attention_of_a_plan(batch, heads, head_dim, tokens, chunks)
     rows = tokens // chunks
-    q, kv = s.view("q0_0", torch.int16, (1, rows, 512)), s.view("kv0", torch.int16, (1, tokens, 1024))
-    got = s.view("o0_0", torch.int16, (1, rows, 512)).clone()
-    lse = s.view("lse0_0", torch.float32, (1, 512 // head_dim, rows)).clone()
+    q, kv = s.view("q0_0", torch.int16, (batch, rows, hidden)), s.view("kv0", torch.int16, (batch, tokens, 2 * hidden))
+    got = s.view("o0_0", torch.int16, (batch, rows, hidden)).clone()
+    lse = s.view("lse0_0", torch.float32, (batch, heads, rows)).clone()
     o, l = torch.empty_like(got), torch.empty_like(lse)
-    xb.xema_op_attention(q.data_ptr(), 512, rows, kv.data_ptr(), kv.data_ptr() + 1024, 1024, tokens, o.data_ptr(), l.data_ptr(),
-                         1, rows, tokens, 512 // head_dim, head_dim, status=s.status.data_ptr(), stream=stream, q_scale=1.0)
+    xb.xema_op_attention(q.data_ptr(), hidden, rows, kv.data_ptr(), kv.data_ptr() + 2 * hidden, 2 * hidden, tokens, o.data_ptr(),
+                         l.data_ptr(), batch, rows, tokens, heads, head_dim, status=s.status.data_ptr(),
+                         stream=torch.cuda.current_stream().cuda_stream, q_scale=1.0)
     s.check_status()
     assert torch.equal(o, got) and torch.equal(l, lse)
 
+
+# (batch 8: 192 items over 148 SMs, whether a head has one row tile or two)
+@pytest.mark.parametrize("batch,tokens,chunks,rehearses", [
+    (1, 1024, 1, True), (1, 1025, 1, False), (8, 500, 4, True), (8, 600, 5, False), (8, 512, 2, True), (8, 513, 2, False)])
+def test_attention_rehearses_up_to_eight_key_blocks_a_cta(batch, tokens, chunks, rehearses):
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+        _attention_of_a_plan(batch, 24, 64, tokens, chunks)
+        torch.cuda.synchronize()
+    names = [re.search(r"attention_kernel<([^>]*)>", e.name) for e in prof.events() if "attention_kernel" in e.name]
+    assert len(names) == 1
+    assert names[0].group(1).split(",")[2].strip().replace("(bool)", "") in (("1", "true") if rehearses else ("0", "false"))
 
 
 MASK = 0x5a5a
