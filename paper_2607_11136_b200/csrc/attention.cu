@@ -92,10 +92,10 @@ static_assert(128 * REG_HELPER + SOFTMAX_THREADS * REG_SOFTMAX <= THREADS * 96, 
 // Which of a thread's 32 column pairs evaluate 2^x as a polynomial on the FMA pipe, one bit per pair; the
 // others use the MUFU.  dh 64: without any the MUFU sets the pace, with too many the issue slots do, and
 // where they stand decides how well the compiler interleaves the two pipes -- the placement is the result of
-// a search with this compiler and nothing else: 4444 x 17776 x 48 heads 933 to 1177 us over 125 placements of 6 to
-// 17 bits (this one 933, the next best 945; 9 bits 1000 and more; 24 placements of 12 bits 4.8 to 12.7 % slower
-// inside the block).  Power-capped, the block of 17776 tokens takes 7.28 ms with this placement, 7.39-7.56 with
-// three others.  Accuracy: see exp2_poly; a polynomial of degree 4 costs 10 % of the launch.
+// a search with this compiler and nothing else.  4444 x 17776 x 48 heads, with the overhead instructions that are gone by
+// now: 933 to 1177 us over 125 placements of 6 to 17 bits (this one 933, the next best 945; 9 bits 1000 and more).
+// Without them 845; 44 other placements 5.8 % slower to 0.6 % faster.  Accuracy: see exp2_poly; a polynomial of
+// degree 4 costs 10 % of the launch.
 // dh 128: none.  The MUFU needs no longer for a block than the tensor pipe (2048 cycles each), and 8 pairs on the
 // FMA pipe were 2 % slower in turn with none (4608 x 4608 x 24 heads 231 against 226 us).
 template <int DH>
