@@ -257,9 +257,10 @@ enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
 
 // REHEARSE: a round of the softmax threads' loop before the wait for earlier launches, on whatever TMEM holds and
 // without results, so that the first item does not meet every line of the code in an empty instruction cache.  A launch of
-// few key blocks gains 1 to 2 us by it; the second set of barriers costs the loop 2 %.  us without / with it: block of 288 x 512
-// 48.2 / 46.8, 464 x 1792 160 / 156, two blocks of 630 x 1536 235 / 228, eight of 304 x 2304 1123 / 1099; with 9 key blocks a CTA (1101 x
-// 1536) 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.
+// few key blocks gains 0.5 to 3 us by it; the second set of barriers costs the loop 2 %.  us without / with it: block of 288 x 512
+// 45.8 / 45.3, 464 x 1792 100.3 / 97.1 (dh 128 105.7 / 101.9), two blocks of 630 x 1536 184.2 / 179.6, eight of 304 x 2304 859.7 /
+// 833.7, eight of 333 x 1024 470.9 / 468.7; with 9 key blocks a CTA (1101 x 1536)
+// 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.
 template <int DH, bool SCALED, bool REHEARSE>
 __global__ void __launch_bounds__(THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
