@@ -287,7 +287,7 @@ def main():
     sess = BlockSession(t, weights, chunks=forced, budget_bytes=budget, device=dev,
                         per_phase=not args.uniform_chunks)
     n_launch = sess.plan.n_ops            # logical ops of the trace (fused ones launch nothing)
-    n_kernels = sess.plan.launch_count()  # kernels actually launched per step
+    n_kernels = sess.plan.forward_launches()  # kernels actually launched per step
     ops = [sess.plan.op(i) for i in range(n_launch)]
     flops = block_flops(t)
     stream = torch.cuda.current_stream(dev)

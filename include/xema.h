@@ -340,8 +340,10 @@ int xema_block_forward_static(const xema_config* cfg, int32_t chunks, const xema
                               const float* rope_dev, const void* hid_in_dev, const void* temb_dev,
                               void* hid_out_dev, void* status_dev, void* stream);
 
-/* Number of kernel launches one forward call enqueues (0 if unbound). */
+/* Number of operators that launch a kernel (0 if unbound), and of the launches that one xema_block_forward or
+ * xema_step_forward enqueues: neighbouring operators of a call may share one. */
 int xema_plan_launch_count(const xema_plan* plan);
+int xema_plan_forward_launches(const xema_plan* plan);
 
 /* Debug aid: enqueue only the first n_logical_ops logical ops of the trace order. */
 int xema_forward_prefix(const xema_plan* plan, uint32_t n_logical_ops, void* stream);

@@ -26,7 +26,7 @@ EXPORTS = (
     "xema_plan_tensor_at", "xema_plan_bind", "xema_plan_set_inputs", "xema_block_forward", "xema_step_forward",
     "xema_block_forward_static",
     "xema_shard_rows", "xema_trace_sharded", "xema_plan_create_sharded", "xema_plan_shard", "xema_plan_gather_point", "xema_plan_create_guarded", "xema_plan_guard_bytes",
-    "xema_plan_launch_count", "xema_forward_host", "xema_forward_prefix", "xema_forward_range", "xema_plan_op", "xema_op_mod", "xema_op_ln_modulate",
+    "xema_plan_launch_count", "xema_plan_forward_launches", "xema_forward_host", "xema_forward_prefix", "xema_forward_range", "xema_plan_op", "xema_op_mod", "xema_op_ln_modulate",
     "xema_op_rmsnorm_rope", "xema_op_gemm", "xema_gemm_tile", "xema_op_gemm_in_tile", "xema_op_attention", "xema_strerror",
     "xema_last_cuda_error", "xema_version", "xema_selftest_wait_timeout",
     "xema_pluggable_malloc", "xema_pluggable_free", "xema_pluggable_mode", "xema_pluggable_recorded",
@@ -130,6 +130,7 @@ def lib() -> C.CDLL:
             "xema_forward_host": [vp, vp, vp, vp, vp],
             "xema_block_forward_static": [P(xema_config), i32, P(xema_block_weights), vp, vp, vp, vp, vp, vp],
             "xema_plan_launch_count": [vp],
+            "xema_plan_forward_launches": [vp],
             "xema_forward_prefix": [vp, u32, vp],
             "xema_forward_range": [vp, u32, u32, vp],
             "xema_plan_op": [vp, u32, C.c_char_p, P(i32), P(i32), P(C.c_double), P(C.c_double)],
@@ -448,6 +449,9 @@ class Plan:
 
     def launch_count(self) -> int:
         return lib().xema_plan_launch_count(self._h)
+
+    def forward_launches(self) -> int:
+        return lib().xema_plan_forward_launches(self._h)
 
     def set_inputs(self, hid: int, temb: int, stream: int = 0):
         """Device pointers of the block input and the timestep embedding, copied into the arena."""

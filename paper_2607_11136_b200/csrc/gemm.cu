@@ -74,8 +74,8 @@ struct GemmCfg {
   static constexpr int STAGES = BN == 256 ? (kGated<EPI> && !DEEP ? 5 : 6) : 196608 / STAGE_BYTES;
   static constexpr int OFF_RING = STAGES * STAGE_BYTES;
   static constexpr int OFF_BIAS = OFF_RING + RING_BYTES;       // float [BN]: bias
-  static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [128]: RMSNorm gain
-  static constexpr int OFF_BAR = OFF_GATE + (kGated<EPI> ? BN * 4 : 512);
+  static constexpr int OFF_GATE = OFF_BIAS + BN * 4;           // float [BN]: gate, or [2][128]: RMSNorm gains
+  static constexpr int OFF_BAR = OFF_GATE + (kGated<EPI> ? BN * 4 : 1024);
   static constexpr int SMEM_BYTES = OFF_BAR + 384;
   static constexpr int TMEM_COLS = 2 * BN;   // a power of two from 32 on
   static_assert((2 * STAGES + 4 + 4 * RING) * 8 + 8 <= 384, "barrier area");
@@ -95,6 +95,10 @@ struct GemmParams {
   const float* rope;                // [token][head_dim/2][cos, sin]
   int rope_pos0, head_dim, norm_cols;
   float rms_eps, norm_out_scale;
+  // the first cols2 columns: another result (map_res), gain and factor
+  const __nv_bfloat16* norm_gain2;
+  float norm_out_scale2;
+  int cols2;
 };
 
 __device__ __forceinline__ float gelu_tanh_f(float z) {
@@ -167,16 +171,18 @@ struct Epilogue {
   using Cfg = GemmCfg<EPI, BN, PAIR, DEEP>;
   static constexpr int RING = Cfg::RING;
   const GemmParams& p;
-  const CUtensorMap* map_out;
+  const CUtensorMap* map_out;   // of the tile's result
   const CUtensorMap* map_res;
   uint8_t* ring;          // [RING][BUF_BYTES]
   uint64_t* rbar;         // [RING] residual chunk has arrived
   const float* bias;      // [BN], shared memory
-  const float* gate;      // [BN] (gated) or the RMSNorm gain
+  const float* gate;      // [BN] (gated) or the tile's RMSNorm gain
   volatile uint32_t* abort_flag;
   int lane;
   int rlane;              // row of a residual chunk that belongs to this lane
   bool dry = false;       // rehearsal
+  float out_scale = 1.f;  // factor of the tile's normalised heads
+  int col0 = 0;           // column of the product that is column 0 of the tile's result
   uint32_t used = 0;      // chunks worked on so far (buffer = used % RING)
   uint32_t asked = 0;     // residual chunks requested so far
 
@@ -196,7 +202,7 @@ struct Epilogue {
     __syncwarp();
     if (rehearsing()) return;
     if (lane == 0) {
-      tma_store_3d(map_out, buf, n0, row0, b);
+      tma_store_3d(map_out, buf, n0 - col0, row0, b);
       bulk_commit();
     }
     ++used;
@@ -302,7 +308,7 @@ struct Epilogue {
           s3 = fmaf(v[t + 3], v[t + 3], s3);
         }
       }
-      const float r = rsqrtf(((s0 + s1) + (s2 + s3)) * (1.f / DH) + p.rms_eps) * p.norm_out_scale;
+      const float r = rsqrtf(((s0 + s1) + (s2 + s3)) * (1.f / DH) + p.rms_eps) * out_scale;
 #pragma unroll
       for (int i = 0; i < 4; ++i) rstd[i] = h == i ? r : rstd[i];
     }
@@ -389,7 +395,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     prefetch_tmap(&map_a);
     prefetch_tmap(&map_w);
     prefetch_tmap(&map_out);
-    if (GATED) prefetch_tmap(&map_res);
+    if (GATED || p.cols2) prefetch_tmap(&map_res);
   }
   if (warp == 1) {
     if (PAIR) {
@@ -568,7 +574,10 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
     uint32_t acc_phase = 0;
     bool ok = true;
     if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
-      if (et < p.head_dim) s_gate[et] = __bfloat162float(p.norm_gain[et]);   // read after the tile's barrier
+      if (et < p.head_dim) {                           // read after the tile's barrier
+        s_gate[et] = __bfloat162float(p.norm_gain[et]);
+        if (p.cols2) s_gate[128 + et] = __bfloat162float(p.norm_gain2[et]);
+      }
     }
     ep.dry = kRehearse<BN, PAIR>;                          // the first round is a rehearsal
     if constexpr (!kRehearse<BN, PAIR>) {
@@ -592,6 +601,11 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
       }
       float4 cs[8];
       if constexpr (EPI == XEMA_EPI_BIAS_NORM_ROPE) {
+        const bool second = n_base < p.cols2;
+        ep.map_out = second ? &map_res : &map_out;
+        ep.gate = second ? s_gate + 128 : s_gate;
+        ep.out_scale = second ? p.norm_out_scale2 : p.norm_out_scale;
+        ep.col0 = second ? 0 : p.cols2;
         if (live && n_base < p.norm_cols && !dry) {
           const int row = min(row0 + lane, p.rows - 1);
           ep.load_angles(reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * p.head_dim), cs);
@@ -695,6 +709,9 @@ GemmParams make_params(const GemmLaunch& g) {
   p.norm_cols = g.norm_cols;
   p.rms_eps = g.rms_eps;
   p.norm_out_scale = g.norm_out_scale > 0.f ? g.norm_out_scale : 1.f;
+  p.norm_gain2 = (const __nv_bfloat16*)g.norm_gain2;
+  p.norm_out_scale2 = g.norm_out_scale2 > 0.f ? g.norm_out_scale2 : 1.f;
+  p.cols2 = g.cols2;
   return p;
 }
 
@@ -807,7 +824,8 @@ void pick_tile(GemmLaunch* g) {
 int check_shape(const GemmLaunch& g) {
   if (g.batch < 1 || g.rows < 0 || g.N < 128 || (g.N % 128) || g.K < 64 || (g.K % 64)) return XEMA_EINVAL;
   if (g.epilogue < XEMA_EPI_BIAS || g.epilogue > XEMA_EPI_BIAS_NORM_ROPE) return XEMA_EINVAL;
-  if (g.epilogue != XEMA_EPI_BIAS_NORM_ROPE) return XEMA_OK;
+  if (g.epilogue != XEMA_EPI_BIAS_NORM_ROPE) return g.cols2 ? XEMA_EINVAL : XEMA_OK;
+  if (g.cols2 < 0 || g.cols2 % 256 || g.cols2 >= g.N) return XEMA_EINVAL;    // whole tiles for either result
   if (g.head_dim != 64 && g.head_dim != 128) return XEMA_EINVAL;
   return g.norm_cols < 0 || g.norm_cols > g.N || g.norm_cols % g.head_dim || g.N % 256 || g.rope_pos0 < 0 ? XEMA_EINVAL : XEMA_OK;
 }
@@ -840,10 +858,15 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   if (g->epilogue == XEMA_EPI_BIAS_NORM_ROPE) {
     if (!g->norm_gain || !g->rope) return XEMA_EINVAL;
     if ((reinterpret_cast<uintptr_t>(g->norm_gain) & 15) || (reinterpret_cast<uintptr_t>(g->rope) & 15)) return XEMA_EALIGN;
+    if (g->cols2) {
+      if (!g->out2 || !g->norm_gain2 || g->ldo2 < g->cols2) return XEMA_EINVAL;
+      if ((g->ldo2 & 7) || (reinterpret_cast<uintptr_t>(g->out2) & 15)) return XEMA_EALIGN;
+    }
   }
   // Result rows lie behind one another; residual rows may be shared (ldr = 0: one row for all,
   // resid_batch_rows = 0: the same rows for every batch element).
-  if ((g->rows > 1 && g->ldo < g->N) || (g->batch > 1 && (g->ldo < 1 || g->out_batch_rows < 1))) return XEMA_EINVAL;
+  const long long out_cols = g->N - g->cols2;
+  if ((g->rows > 1 && g->ldo < out_cols) || (g->batch > 1 && (g->ldo < 1 || g->out_batch_rows < 1))) return XEMA_EINVAL;
   if (gated && (g->ldr < 0 || g->resid_batch_rows < 0)) return XEMA_EINVAL;
   if ((lda & 7) || (ldw & 7) || (g->ldo & 7) || (gated && (g->ldr & 7))) return XEMA_EALIGN;
   auto mis = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) != 0; };
@@ -872,8 +895,10 @@ int gemm_prepare(GemmLaunch* g, const void* a, long long lda, long long a_batch_
   rc = encode_tmap_bf16(&g->map_w, w, g->K, g->N, 1, ldw, g->N, g->pair ? g->block_n / 2 : g->block_n);
   if (rc) return rc;
   // results leave, and residuals arrive, as boxes of 32 columns x 32 rows
-  rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, g->N, rows, g->batch, g->ldo,
+  rc = encode_tmap_box32(&g->map_out, g->out, g->epilogue == XEMA_EPI_GATE_RES_F32, out_cols, rows, g->batch, g->ldo,
                          g->out_batch_rows * g->ldo);
+  if (!rc && g->cols2)
+    rc = encode_tmap_box32(&g->map_res, g->out2, false, g->cols2, rows, g->batch, g->ldo2, g->out2_batch_rows * g->ldo2);
   if (rc || !gated) return rc;
   const long long resid_stride = g->resid_batch_rows * g->ldr;
   return encode_tmap_box32(&g->map_res, g->resid, g->epilogue == XEMA_EPI_GATE_RES_BF16, g->N, g->ldr ? rows : 1,

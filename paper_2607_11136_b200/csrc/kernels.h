@@ -103,7 +103,7 @@ struct GemmLaunch {
   CUtensorMap map_a;   // [batch][rows][K], box 64 x 128
   CUtensorMap map_w;   // [1][N][K],       box 64 x block_n (a pair: each CTA half of it)
   CUtensorMap map_out; // [batch][rows][N], box 32 x 32
-  CUtensorMap map_res; // the same for the residual (gated epilogues)
+  CUtensorMap map_res; // the same for the residual (gated epilogues) or for out2
   const void* bias;    // bf16 [N]
   void* out;
   long long ldo, out_batch_rows;
@@ -122,6 +122,13 @@ struct GemmLaunch {
   int rope_pos0, head_dim, norm_cols;
   float rms_eps;
   float norm_out_scale;   // the normalised, rotated heads are multiplied by this before rounding (1 = as they are)
+  // ... and a second result: with cols2 > 0 the first cols2 columns of the product go to out2, normalised with gain2 and
+  // multiplied by norm_out_scale2, the others to column 0 on of out (norm_cols counts from the product's first column)
+  void* out2;
+  long long ldo2, out2_batch_rows;
+  const void* norm_gain2;
+  float norm_out_scale2;
+  int cols2;
 };
 // Fills the descriptors and the tile (pair, block_n) from plain pointers.  `tile`: {pair, block_n} to take instead
 // of the one estimated to be fastest, XEMA_EINVAL where the problem cannot run in it.

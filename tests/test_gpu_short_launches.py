@@ -67,6 +67,30 @@ def test_a_request_has_the_same_bits_alone_and_in_a_batch(tokens, hidden):
         assert np.array_equal(y, outs[0][2][first:first + n]), (first, n)
 
 
+# One tile form after the other: single 64, pair 128 and pair 256, rows at and beside their edges, both head sizes, a shard.
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("batch,hidden,tokens,shard", [
+    (1, 512, 9, None), (1, 512, 128, None), (2, 512, 129, None), (3, 1024, 200, None), (1, 1536, 1025, None), (1, 2048, 1280, None),
+    (1, 3072, 2561, None), (1, 512, 300, (1, 2))])
+def test_keys_values_and_queries_in_one_launch_have_the_bits_of_two(head_dim, batch, hidden, tokens, shard):
+    t = _template(batch, tokens, hidden, 512, heads=hidden // head_dim)
+    s = BlockSession(t, [make_block_weights(t, 7)], chunks=(1, 1, 1), shard=shard)
+    assert s.plan.forward_launches() == s.plan.launch_count() - 1
+    x, temb = make_activations(t)
+    r0, rows = (0, tokens) if shard is None else (s.plan.row0, s.plan.rows)
+    stream = torch.cuda.current_stream().cuda_stream
+    got = []
+    for ends in (range(1, 8), [7]):              # MOD, LN1A, KV, KROPE, LN1B, Q, QROPE one by one, and in one call
+        s.arena.fill_(0x5A)
+        s.set_inputs(np.ascontiguousarray(x[:, r0:r0 + rows]), temb)
+        for first, end in zip([0] + list(ends), ends):
+            s.plan.forward_range(first, end, stream)
+        got.append((s.view("q0_0", torch.int16, (batch, rows, hidden)).clone(),
+                    s.view("kv0", torch.int16, (batch, tokens, 2 * hidden)).clone()))
+        s.check_status()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 def _attention_of_a_plan(batch, heads, head_dim, tokens, chunks):
     """A session that has run up to its first attention launch: MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN."""
     t = _template(batch, tokens, heads * head_dim, 512, heads=heads)
