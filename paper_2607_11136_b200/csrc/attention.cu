@@ -365,7 +365,17 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   auto q_next = [&]() { if (++q_st == QBUF) { q_st = 0; q_ph ^= 1; } };
 
   // One item in one sweep, in the roles of the single-warp loops.
-  auto produce = [&](const Item& it, bool with_v) {   // warp 0, one lane
+  auto load_q = [&](const Item& it) {
+    for (int t = 0; t < p.tiles; ++t)
+#pragma unroll
+      for (int a = 0; a < C::ATOMS; ++a)
+        tma_load_3d(smem + C::OFF_Q + (q_st * TILES + t) * C::TILE_BYTES + a * ATOM_BYTES, &map_q, &q_full[q_st],
+                    it.h * DH + a * 64, it.row0 + t * BM, it.b);
+    ++q_issued;
+    q_next();
+  };
+  // `asked`: the item's queries and first keys are on their way
+  auto produce = [&](const Item& it, bool with_v, bool asked) {   // warp 0, one lane
     auto load = [&](uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int row0) {
       mbar_expect_tx(bar, C::TILE_BYTES);
 #pragma unroll
@@ -377,16 +387,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       ++k_issued;
       k_next();
     };
-    load_k(0);
-    if (!ok || !(ok = mbar_wait(&q_empty[q_st], q_ph ^ 1, abort_flag))) return;
-    mbar_expect_tx(&q_full[q_st], p.tiles * C::TILE_BYTES);
-    for (int t = 0; t < p.tiles; ++t)
-#pragma unroll
-      for (int a = 0; a < C::ATOMS; ++a)
-        tma_load_3d(smem + C::OFF_Q + (q_st * TILES + t) * C::TILE_BYTES + a * ATOM_BYTES, &map_q, &q_full[q_st],
-                    it.h * DH + a * 64, it.row0 + t * BM, it.b);
-    ++q_issued;
-    q_next();
+    if (!asked) {
+      load_k(0);
+      if (!ok || !(ok = mbar_wait(&q_empty[q_st], q_ph ^ 1, abort_flag))) return;
+      mbar_expect_tx(&q_full[q_st], p.tiles * C::TILE_BYTES);
+      load_q(it);
+    }
     for (int j = 0; ok && j < n_kv; ++j) {
       if (j + 1 < n_kv) load_k(j + 1);
       if (!ok) return;
@@ -462,21 +468,36 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint32_t s_free_ph[TILES] = {0, 0}, p_full_ph[TILES] = {0, 0}, p_half_ph[TILES] = {0, 0};
   bool s_pending[TILES] = {false, false};     // scores issued whose release has not been waited for yet
 
-  // dh 64, and the score-only sweep: a warp for the scores ...
+  // dh 64, and the score-only sweep: a warp for the scores (it shares an issue port with four softmax warps; with the tiles'
+  // checks out of the loop and one election a tile, 4444 x 17776 x 48 heads 857 -> 852 us) ...
   auto issue_scores = [&](const Item& it) {
+    const bool two = tile_live(it, 1);
     for (int j = 0; j < n_kv; ++j) {
       wait_k(j == 0);
-#pragma unroll
-      for (int t = 0; t < TILES; ++t) {
-        if (!ok) return;
-        if (!tile_live(it, t)) continue;
-        if (s_pending[t]) wait_phase(&s_free[t], s_free_ph[t]);
-        if (!ok) return;
-        if (elect_one()) mma_scores(t);
-        __syncwarp();
-        s_pending[t] = true;
+      if (!ok) return;
+      if (s_pending[0]) wait_phase(&s_free[0], s_free_ph[0]);
+      if (!ok) return;
+      if (elect_one()) {
+        mma_scores(0);
+        if (!two) {
+          mma_commit(&k_empty[k_st]);
+          if (j == n_kv - 1) mma_commit(&q_empty[q_st]);
+        }
       }
-      k_done(j == n_kv - 1);
+      __syncwarp();
+      s_pending[0] = true;
+      if (two) {
+        if (s_pending[1]) wait_phase(&s_free[1], s_free_ph[1]);
+        if (!ok) return;
+        if (elect_one()) {
+          mma_scores(1);
+          mma_commit(&k_empty[k_st]);
+          if (j == n_kv - 1) mma_commit(&q_empty[q_st]);
+        }
+        __syncwarp();
+        s_pending[1] = true;
+      }
+      k_next();
     }
     q_next();
   };
@@ -768,17 +789,32 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // First pass over the CTA's items, then the flagged ones once more in two sweeps.
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_HELPER));
+    // The first loads stand right behind the wait, with all that they need worked out: in `produce`, whose code is met for the
+    // first time, they came 1.5 to 3.3 us after it, now 0.5 to 1.3.  us: block of 288 x 512 41.2 -> 39.9, of 1101 x 1536 115.0 ->
+    // 113.4; one tile an item and few blocks gain the most.
+    const Item first = item_at(0);
+    if (threadIdx.x == 0) {
+      mbar_expect_tx(&k_full[0], C::TILE_BYTES);
+      mbar_expect_tx(&q_full[0], p.tiles * C::TILE_BYTES);
+    }
     grid_dep_wait();
     if (warp == 0) {
-      if (lane == 0)
-        for (int i = 0; ok && i < n_items; ++i) produce(item_at(i), true);
+      if (lane == 0) {
+#pragma unroll
+        for (int a = 0; a < C::ATOMS; ++a)
+          tma_load_3d(smem + C::OFF_K + a * ATOM_BYTES, &map_k, &k_full[0], first.h * DH + a * 64, 0, first.b);
+        load_q(first);
+        ++k_issued;
+        k_next();
+        for (int i = 0; ok && i < n_items; ++i) produce(i ? item_at(i) : first, true, i == 0);
+      }
       __syncwarp();
       const bool again = second_pass();
       if (lane == 0) {
         if (again)
           for_flagged([&](const Item& it) {
 #pragma unroll 1
-            for (int with_v = 0; ok && with_v < 2; ++with_v) produce(it, with_v != 0);
+            for (int with_v = 0; ok && with_v < 2; ++with_v) produce(it, with_v != 0, false);
           });
         if (!ok) {
           // gave up: let the copies already issued land before the CTA leaves (the latest fill of
