@@ -27,56 +27,80 @@ __device__ __forceinline__ float warp_sum(float v) {
 // mod[b, j] = sum_k silu(temb[b,k]) * w[j,k] + bias[j]
 // A warp takes kModRows output features at once: their weight rows are requested together, for up to
 // 512 inputs before the wait for earlier launches (the weights do not depend on them); silu(temb) for
-// all batch elements sits in shared memory.  Bound by the latency of one trip to HBM for one batch
-// element, by the reductions (five shuffles per feature and batch element) for several.
+// all batch elements sits in shared memory, loaded 16 bytes at a time.  Bound by the latency of one trip to HBM for one
+// batch element (which has an instance of its own: 80 registers instead of 128, so that three blocks fit an SM, and half of the
+// code to fetch), by the products and reductions for several.  us back to back, before these two, the wide load and the
+// six-shuffle reduction / with them: 1 x 6144 features 4.7 / 4.2 (as short as launches follow one another), 1 x 9216 5.2 /
+// 4.2, 1 x 18432 7.2 / 6.2, 3 x 12288 10.0 / 8.3, 4 x 18432 12.4 / 10.3, 7 x 3072 10.3 / 6.5.
 // ---------------------------------------------------------------------------------------
 constexpr int kModWarps = 8;
 constexpr int kModRows = 4;
-constexpr int kModMaxBatch = 4;     // batch elements per pass over the weights
 
-__global__ void __launch_bounds__(kModWarps * 32)
-mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, const __nv_bfloat16* __restrict__ bias,
-                float* mod, int batch, int Dt, int n_out) {
+// A load of weights that stays where it stands: an __ldg the compiler may move down to its use, behind the wait.
+__device__ __forceinline__ uint4 ld_weights(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// Features [j_first, j_end) of block `tile` of WARPS * kModRows of them, BATCH batch elements per pass over the weights.
+template <int WARPS, int BATCH>
+__device__ __forceinline__ void mod_features(const ModArgs& a, int tile) {
   extern __shared__ float s_e[];  // [batch][Dt]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j0 = (blockIdx.x * kModWarps + warp) * kModRows;
-  const int n8 = Dt / 8;
+  const int j0 = a.j_first + (tile * WARPS + warp) * kModRows;
+  const int n8 = a.Dt / 8;
+  const __nv_bfloat16* w = static_cast<const __nv_bfloat16*>(a.w);
   auto weights = [&](int r, int k8) {
-    return (j0 + r < n_out && k8 < n8) ? __ldg(reinterpret_cast<const uint4*>(w + (size_t)(j0 + r) * Dt) + k8)
-                                       : make_uint4(0u, 0u, 0u, 0u);
+    return (j0 + r < a.j_end && k8 < n8) ? ld_weights(reinterpret_cast<const uint4*>(w + (size_t)(j0 + r) * a.Dt) + k8)
+                                         : make_uint4(0u, 0u, 0u, 0u);
   };
   uint4 first[2][kModRows];
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
     for (int r = 0; r < kModRows; ++r) first[u][r] = weights(r, u * 32 + lane);
+  // the feature whose sum this lane ends up with, and its bias as it comes (a conversion here would wait for it)
+  const int j_own = j0 + lane / 8;
+  const unsigned short bias = j_own < a.j_end ? __ldg(static_cast<const unsigned short*>(a.bias) + j_own) : (unsigned short)0;
   grid_dep_launch();
   grid_dep_wait();
-  for (int i = threadIdx.x; i < batch * Dt; i += blockDim.x) {
-    const float z = __bfloat162float(*(const volatile __nv_bfloat16*)(temb + i));
-    s_e[i] = z / (1.f + __expf(-z));
+  for (int i = threadIdx.x; i < a.batch * n8; i += WARPS * 32) {
+    float e[8];
+    if ((reinterpret_cast<uintptr_t>(a.temb) & 15) == 0) {
+      const uint4 t = ld_u4(static_cast<const uint4*>(a.temb) + i);
+      e[0] = bf16_lo(t.x); e[1] = bf16_hi(t.x); e[2] = bf16_lo(t.y); e[3] = bf16_hi(t.y);
+      e[4] = bf16_lo(t.z); e[5] = bf16_hi(t.z); e[6] = bf16_lo(t.w); e[7] = bf16_hi(t.w);
+    } else {                          // (the operator takes any address; a plan's slot is aligned)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) e[k] = __bfloat162float(*(static_cast<const volatile __nv_bfloat16*>(a.temb) + i * 8 + k));
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) e[k] = e[k] / (1.f + __expf(-e[k]));
+    *reinterpret_cast<float4*>(s_e + i * 8) = make_float4(e[0], e[1], e[2], e[3]);
+    *reinterpret_cast<float4*>(s_e + i * 8 + 4) = make_float4(e[4], e[5], e[6], e[7]);
   }
   __syncthreads();
-  for (int b0 = 0; b0 < batch; b0 += kModMaxBatch) {
-    float acc[kModRows][kModMaxBatch];
+  for (int b0 = 0; b0 < (BATCH == 1 ? 1 : a.batch); b0 += BATCH) {
+    float acc[kModRows][BATCH];
 #pragma unroll
     for (int r = 0; r < kModRows; ++r)
 #pragma unroll
-      for (int b = 0; b < kModMaxBatch; ++b) acc[r][b] = 0.f;
+      for (int b = 0; b < BATCH; ++b) acc[r][b] = 0.f;
     auto add = [&](const uint4 (&v)[kModRows], int k8) {
 #pragma unroll
-      for (int b = 0; b < kModMaxBatch; ++b) {
-        if (b0 + b >= batch || k8 >= n8) continue;
-        const float4 e0 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * Dt + k8 * 8);
-        const float4 e1 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * Dt + k8 * 8 + 4);
+      for (int b = 0; b < BATCH; ++b) {
+        if ((BATCH > 1 && b0 + b >= a.batch) || k8 >= n8) continue;
+        const float4 e0 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * a.Dt + k8 * 8);
+        const float4 e1 = *reinterpret_cast<const float4*>(s_e + (size_t)(b0 + b) * a.Dt + k8 * 8 + 4);
 #pragma unroll
         for (int r = 0; r < kModRows; ++r) {
-          float a = acc[r][b];
-          a = fmaf(bf16_lo(v[r].x), e0.x, a); a = fmaf(bf16_hi(v[r].x), e0.y, a);
-          a = fmaf(bf16_lo(v[r].y), e0.z, a); a = fmaf(bf16_hi(v[r].y), e0.w, a);
-          a = fmaf(bf16_lo(v[r].z), e1.x, a); a = fmaf(bf16_hi(v[r].z), e1.y, a);
-          a = fmaf(bf16_lo(v[r].w), e1.z, a); a = fmaf(bf16_hi(v[r].w), e1.w, a);
-          acc[r][b] = a;
+          float c = acc[r][b];
+          c = fmaf(bf16_lo(v[r].x), e0.x, c); c = fmaf(bf16_hi(v[r].x), e0.y, c);
+          c = fmaf(bf16_lo(v[r].y), e0.z, c); c = fmaf(bf16_hi(v[r].y), e0.w, c);
+          c = fmaf(bf16_lo(v[r].z), e1.x, c); c = fmaf(bf16_hi(v[r].z), e1.y, c);
+          c = fmaf(bf16_lo(v[r].w), e1.z, c); c = fmaf(bf16_hi(v[r].w), e1.w, c);
+          acc[r][b] = c;
         }
       }
     };
@@ -89,25 +113,40 @@ mod_gemv_kernel(const __nv_bfloat16* temb, const __nv_bfloat16* __restrict__ w, 
       add(v, k8);
     }
 #pragma unroll
-    for (int b = 0; b < kModMaxBatch; ++b) {
-      if (b0 + b >= batch) continue;
+    for (int b = 0; b < BATCH; ++b) {
+      if (BATCH > 1 && b0 + b >= a.batch) continue;
+      // The four features' sums over the warp at once: after each of the first two steps a lane holds half as many of them.
+      // Six shuffles instead of twenty; the values that are added are those of warp_sum, so are the bits.
+      static_assert(kModRows == 4, "two halving steps");
+      const bool hi = lane & 16, hi2 = lane & 8;
+      float u0 = hi ? acc[2][b] : acc[0][b], u1 = hi ? acc[3][b] : acc[1][b];
+      u0 += __shfl_xor_sync(0xffffffffu, hi ? acc[0][b] : acc[2][b], 16);
+      u1 += __shfl_xor_sync(0xffffffffu, hi ? acc[1][b] : acc[3][b], 16);
+      float sum = hi2 ? u1 : u0;
+      sum += __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 8);
 #pragma unroll
-      for (int r = 0; r < kModRows; ++r) {
-        const float sum = warp_sum(acc[r][b]);
-        if (lane == r && j0 + r < n_out) mod[(size_t)(b0 + b) * n_out + j0 + r] = sum + __bfloat162float(bias[j0 + r]);
-      }
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if ((lane & 7) == 0 && j_own < a.j_end) a.mod[(size_t)(b0 + b) * a.n_out + j_own] = sum + __uint_as_float((uint32_t)bias << 16);
     }
   }
 }
 
-int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream, bool chained) {
-  if (batch < 1 || Dt < 8 || (Dt & 7) || n_out < 1) return XEMA_EINVAL;
-  size_t smem = (size_t)batch * Dt * sizeof(float);
-  if (smem > 48 * 1024) return XEMA_EINVAL;
-  const int blocks = (n_out + kModWarps * kModRows - 1) / (kModWarps * kModRows);
-  return launch_kernel(mod_gemv_kernel, dim3(blocks), kModWarps * 32, smem, stream, chained, (const __nv_bfloat16*)temb,
-                       (const __nv_bfloat16*)w_mod, (const __nv_bfloat16*)b_mod, mod, batch, Dt, n_out);
+template <int BATCH>
+__global__ void __launch_bounds__(kModWarps * 32, 2) mod_gemv_kernel(const ModArgs a) {
+  mod_features<kModWarps, BATCH>(a, blockIdx.x);
+}
+
+constexpr size_t kModSmemLimit = 48 * 1024;
+static int check_mod(const ModArgs& a) {
+  if (a.batch < 1 || a.Dt < 8 || (a.Dt & 7) || a.n_out < 1 || a.j_first < 0 || a.j_first >= a.j_end || a.j_end > a.n_out)
+    return XEMA_EINVAL;
+  return (size_t)a.batch * a.Dt * sizeof(float) > kModSmemLimit ? XEMA_EINVAL : XEMA_OK;
+}
+
+int launch_mod(const ModArgs& a, cudaStream_t stream, bool chained) {
+  if (int rc = check_mod(a)) return rc;
+  const int blocks = (a.j_end - a.j_first + kModWarps * kModRows - 1) / (kModWarps * kModRows);
+  return launch_kernel(a.batch == 1 ? mod_gemv_kernel<1> : mod_gemv_kernel<4>, dim3(blocks), kModWarps * 32, (size_t)a.batch * a.Dt * sizeof(float), stream, chained, a);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -73,8 +73,13 @@ int launch_kernel(void (*kern)(Params...), dim3 grid, int threads, size_t smem, 
   return XEMA_OK;
 }
 
-int launch_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int batch, int Dt, int n_out,
-               cudaStream_t stream, bool chained = false);
+// Features [j_first, j_end) of mod[b, j] = sum_k silu(temb[b, k]) * w[j, k] + bias[j] (mod has n_out features a row).
+struct ModArgs {
+  const void *temb, *w, *bias;
+  float* mod;
+  int batch, Dt, n_out, j_first, j_end;
+};
+int launch_mod(const ModArgs& a, cudaStream_t stream, bool chained = false);
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
                        cudaStream_t stream, bool chained = false);

@@ -179,12 +179,16 @@ struct xema_plan {
   }
 };
 
+static ModArgs mod_args(const xema_config& c, const Op& op, int j_first, int j_end) {
+  return ModArgs{op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, j_first, j_end};
+}
+
 // `chained`: the launch right before this one in the stream is the op before it (see launch_kernel).
 static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained) {
   const xema_config& c = pl->cfg;
   switch (op.kind) {
     case OP_MOD:
-      return launch_mod(op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, st, chained);
+      return launch_mod(mod_args(c, op, 0, 6 * c.hidden), st, chained);
     case OP_LN:
       return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale,
                                 6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st, chained);
@@ -973,7 +977,7 @@ int xema_plan_forward_launches(const xema_plan* plan) {
 int xema_op_mod(const void* temb, const void* w_mod, const void* b_mod, float* mod, int32_t batch, int32_t temb_dim,
                 int32_t n_out, void* stream) {
   if (!temb || !w_mod || !b_mod || !mod) return XEMA_EINVAL;
-  return launch_mod(temb, w_mod, b_mod, mod, batch, temb_dim, n_out, reinterpret_cast<cudaStream_t>(stream));
+  return launch_mod(ModArgs{temb, w_mod, b_mod, mod, batch, temb_dim, n_out, 0, n_out}, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int xema_op_ln_modulate(const void* in, int32_t in_is_f32, int64_t in_batch_rows, void* out, const float* shift,

@@ -33,6 +33,24 @@ def test_mod_gemv():
         assert_close(out.cpu().numpy(), ref, "mod", rel=1e-4, cos=0.999999)
 
 
+# one element and several (a pass takes four), features and inputs beside the warps' and lanes' shares, an odd address
+@pytest.mark.parametrize("B,Dt,n_out,shift", [(1, 512, 1, 0), (1, 8, 33, 0), (1, 1032, 257, 1), (2, 520, 31, 1), (4, 512, 64, 0), (5, 1032, 130, 3)])
+def test_mod_gemv_edges(B, Dt, n_out, shift):
+    rng = np.random.default_rng(B * Dt + n_out)
+    tb, tf = rand_bf16(rng, (B, Dt))
+    wb, wf = rand_bf16(rng, (n_out, Dt), 0.02)
+    bb, bf = rand_bf16(rng, (n_out,), 0.02)
+    out = torch.full((B * n_out + 1,), 7.0, dtype=torch.float32, device=DEV)
+    room = torch.empty(B * Dt + shift, dtype=torch.int16, device=DEV)
+    room[shift:] = to_dev(tb).reshape(-1)
+    w_dev, b_dev = to_dev(wb), to_dev(bb)
+    xb.xema_op_mod(room.data_ptr() + 2 * shift, w_dev.data_ptr(), b_dev.data_ptr(), out.data_ptr(), B, Dt, n_out)
+    torch.cuda.synchronize()
+    ref = ob.linear(ob.silu(tf), wf, bf)
+    assert_close(out[:-1].view(B, n_out).cpu().numpy(), ref, "mod", rel=1e-4, cos=0.999999)
+    assert out[-1].item() == 7.0
+
+
 @pytest.mark.parametrize("D,in_f32", [(512, 0), (512, 1), (3072, 0), (3072, 1), (768, 0), (1280, 1)])
 def test_ln_modulate(D, in_f32):
     rng = np.random.default_rng(1)
