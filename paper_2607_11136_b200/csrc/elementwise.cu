@@ -218,18 +218,25 @@ struct LnIo {
   }
 };
 
-template <bool IN_F32, int NV>
+// CARRY > 0: the first mod_blocks blocks work out features of a modulation (that many batch elements a pass) beside the rows.
+template <bool IN_F32, int NV, int CARRY>
 __global__ void __launch_bounds__(kLnWarps * 32)
 ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, const float* shift, const float* scale,
-                   long long mod_stride, int batch, int rows, int D, float eps) {
+                   long long mod_stride, int batch, int rows, int D, float eps, const ModArgs mod, int mod_blocks) {
   using Io = LnIo<IN_F32>;
   constexpr int EPV = Io::EPV;
+  if constexpr (CARRY > 0) {
+    if ((int)blockIdx.x < mod_blocks) {
+      mod_features<kLnWarps, CARRY>(mod, blockIdx.x);
+      return;
+    }
+  }
   grid_dep_launch();
   grid_dep_wait();
   const int lane = threadIdx.x & 31;
   const long long total = (long long)batch * rows;
   const float inv_d = 1.f / (float)D;
-  const long long r = (long long)blockIdx.x * kLnWarps + (threadIdx.x >> 5);
+  const long long r = (long long)(blockIdx.x - (CARRY > 0 ? mod_blocks : 0)) * kLnWarps + (threadIdx.x >> 5);
   if (r >= total) return;
   const int b = (int)(r / rows);
   const int i = (int)(r - (long long)b * rows);
@@ -294,31 +301,46 @@ ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, 
 
 template <bool IN_F32>
 static int launch_ln_t(const void* in, long long in_batch_rows, void* out, const float* shift, const float* scale,
-                       long long mod_stride, int batch, int rows, int D, float eps, cudaStream_t stream, bool chained) {
+                       long long mod_stride, int batch, int rows, int D, float eps, cudaStream_t stream, bool chained,
+                       const ModArgs* mod) {
   constexpr int PER = IN_F32 ? 2 : 1;                  // steps per 256 columns
   const long long total = (long long)batch * rows;
   const unsigned blocks = (unsigned)((total + kLnWarps - 1) / kLnWarps);
+  const int per_block = kLnWarps * kModRows;
+  const int mod_blocks = mod ? (mod->j_end - mod->j_first + per_block - 1) / per_block : 0;
+  const size_t smem = mod ? (size_t)mod->batch * mod->Dt * sizeof(float) : 0;
   auto run = [&](auto kern) {
-    return launch_kernel(kern, dim3(blocks), kLnWarps * 32, 0, stream, chained, in, in_batch_rows, (__nv_bfloat16*)out, shift,
-                         scale, mod_stride, batch, rows, D, eps);
+    return launch_kernel(kern, dim3(blocks + mod_blocks), kLnWarps * 32, smem, stream, chained, in, in_batch_rows,
+                         (__nv_bfloat16*)out, shift, scale, mod_stride, batch, rows, D, eps, mod ? *mod : ModArgs{}, mod_blocks);
   };
+  if (mod) {
+    if (int rc = check_mod(*mod)) return rc;
+    switch (D / 256) {
+#define XEMA_LN_CASE(N) \
+  case N: return mod->batch == 1 ? run(ln_modulate_kernel<IN_F32, N * PER, 1>) : run(ln_modulate_kernel<IN_F32, N * PER, 4>);
+      XEMA_LN_CASE(1) XEMA_LN_CASE(2) XEMA_LN_CASE(3) XEMA_LN_CASE(4) XEMA_LN_CASE(5) XEMA_LN_CASE(6)
+      XEMA_LN_CASE(7) XEMA_LN_CASE(8) XEMA_LN_CASE(9) XEMA_LN_CASE(10) XEMA_LN_CASE(11) XEMA_LN_CASE(12)
+#undef XEMA_LN_CASE
+      default: return XEMA_EINVAL;
+    }
+  }
   switch (D / 256) {
-#define XEMA_LN_CASE(N) case N: return run(ln_modulate_kernel<IN_F32, N * PER>);
+#define XEMA_LN_CASE(N) case N: return run(ln_modulate_kernel<IN_F32, N * PER, 0>);
     XEMA_LN_CASE(1) XEMA_LN_CASE(2) XEMA_LN_CASE(3) XEMA_LN_CASE(4) XEMA_LN_CASE(5) XEMA_LN_CASE(6)
     XEMA_LN_CASE(7) XEMA_LN_CASE(8) XEMA_LN_CASE(9) XEMA_LN_CASE(10) XEMA_LN_CASE(11) XEMA_LN_CASE(12)
     XEMA_LN_CASE(13) XEMA_LN_CASE(14) XEMA_LN_CASE(15) XEMA_LN_CASE(16)
 #undef XEMA_LN_CASE
-    default: return run(ln_modulate_kernel<IN_F32, 0>);
+    default: return run(ln_modulate_kernel<IN_F32, 0, 0>);
   }
 }
 
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
-                       cudaStream_t stream, bool chained) {
+                       cudaStream_t stream, bool chained, const ModArgs* mod) {
   if (batch < 1 || rows < 0 || D < 256 || (D % 256)) return XEMA_EINVAL;
-  if (rows == 0) return XEMA_OK;
-  return in_is_f32 ? launch_ln_t<true>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained)
-                   : launch_ln_t<false>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained);
+  if (rows == 0) return mod ? launch_mod(*mod, stream, chained) : XEMA_OK;
+  return in_is_f32 ? launch_ln_t<true>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained, mod)
+                   : launch_ln_t<false>(in, in_batch_rows, out, shift, scale, mod_stride, batch, rows, D, eps, stream, chained, mod);
 }
 
 // ---------------------------------------------------------------------------------------

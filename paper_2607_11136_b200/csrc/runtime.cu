@@ -131,10 +131,13 @@ struct Op {
   int rows;
   int batch;          // batch elements this launch covers (OP_LN, OP_ROPE)
   bool reads_ln1a;    // OP_GEMM Q: its input is LN1A's output (LN1B elided)
+  size_t mod_op;      // OP_LN LN2, last piece: the next block's MOD op, and LN1A, first piece: its own, where launches may carry it; or 0
   size_t q_op;        // OP_GEMM KV: the Q op that may share its launch (xema_plan::qkv), or 0
   GemmLaunch gemm;
   AttnLaunch attn;
 };
+
+constexpr long long kCarryRows = 8192;   // rows of an LN launch up to which it may carry a modulation
 
 // One step of xema_forward_host: a launch, or the arrival / departure of a piece of the block input /
 // output (`rows` x `width` bytes at byte offset `offset` of the tensor, rows `pitch` apart).
@@ -183,6 +186,11 @@ static ModArgs mod_args(const xema_config& c, const Op& op, int j_first, int j_e
   return ModArgs{op.temb, op.w_mod, op.b_mod, op.mod, c.batch, c.temb_dim, 6 * c.hidden, j_first, j_end};
 }
 
+static int launch_ln(const xema_config& c, const Op& op, cudaStream_t st, bool chained, const ModArgs* mod = nullptr) {
+  return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale, 6LL * c.hidden, op.batch,
+                            op.rows, c.hidden, c.ln_eps, st, chained, mod);
+}
+
 // `chained`: the launch right before this one in the stream is the op before it (see launch_kernel).
 static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chained) {
   const xema_config& c = pl->cfg;
@@ -190,8 +198,7 @@ static int issue(const xema_plan* pl, const Op& op, cudaStream_t st, bool chaine
     case OP_MOD:
       return launch_mod(mod_args(c, op, 0, 6 * c.hidden), st, chained);
     case OP_LN:
-      return launch_ln_modulate(op.ln_in, op.ln_in_f32, op.ln_in_batch_rows, op.ln_out, op.shift, op.scale,
-                                6LL * c.hidden, op.batch, op.rows, c.hidden, c.ln_eps, st, chained);
+      return launch_ln(c, op, st, chained);
     case OP_ROPE:
       return launch_rmsnorm_rope(op.rope_x, op.rope_ld, op.rope_batch_rows, op.rope_g, pl->rope, op.pos0, op.batch,
                                  op.rows, c.heads, c.head_dim, c.rms_eps, st);
@@ -222,14 +229,21 @@ static int run_ops(const xema_plan* pl, size_t first, size_t n, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   n = std::min(n, pl->ops.size());
   size_t done = 0;              // the Q op that a launch of KV took along
+  size_t carried = 0;           // the MOD op whose first half the LN2 before it took along
   bool chained = false;
   for (size_t i = first; i < n; ++i) {
-    if (done && i == done) continue;
-    const size_t q_op = pl->ops[i].q_op;
+    if ((done && i == done) || (carried && i == carried)) continue;
+    const size_t q_op = pl->ops[i].q_op, mod_op = pl->ops[i].mod_op;
     int rc;
     if (q_op && q_op < n) {
       rc = launch_gemm(pl->qkv[pl->ops[i].block], st, chained);
       done = q_op;
+    } else if (mod_op && (mod_op > i ? mod_op + 1 < n : mod_op == carried)) {
+      // the shift, scale and gate of the attention half with LN2 of the block before, those of the feed-forward half with LN1A
+      const int half = 3 * pl->cfg.hidden;
+      const ModArgs mod = mod_args(pl->cfg, pl->ops[mod_op], mod_op > i ? 0 : half, mod_op > i ? half : 2 * half);
+      rc = launch_ln(pl->cfg, pl->ops[i], st, chained, &mod);
+      carried = mod_op;
     } else {
       rc = issue(pl, pl->ops[i], st, chained);
     }
@@ -636,6 +650,29 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
     }
   }
   if (plan->ops.size() != plan->n_ops) return XEMA_EINVAL;
+  // The modulation of a later block needs the timestep embedding and the slot of the block before, of which the attention half
+  // (shift, scale, gate) has been read when LN2 starts and the rest when the next LN1A does: the blocks of those two launches
+  // that have no row work it out, and its own launch falls away.  Where mod<m> lies over nothing but mod<m - 1> from LN2 to
+  // MOD and nothing takes the embedding's bytes until LN1A.  Eight blocks of 333 x 1024 in a graph 401.7 -> 385.0 us; from some
+  // thousand rows on MOD is a thousandth of a block, and the larger instance of LN has fewer warps an SM.
+  const size_t per_block = 1 + 3 * (size_t)CA + 5 * (size_t)CB + 3 * (size_t)CC;
+  for (int m = 1; m < c.n_blocks; ++m) {
+    const size_t mod_op = m * per_block, ln1 = mod_op + 1, ln2 = mod_op - 3;
+    const size_t im = plan->index.at("mod" + std::to_string(m)), ib = plan->index.at("mod" + std::to_string(m - 1));
+    const size_t it = plan->index.at("temb");
+    const long long rows = std::max((long long)plan->ops[ln1].batch * plan->ops[ln1].rows, (long long)plan->ops[ln2].batch * plan->ops[ln2].rows);
+    bool free = D <= kLnMaxCarryCols && rows <= kCarryRows;
+    auto overlap = [&](size_t i, size_t j) {
+      return plan->offsets[i] < plan->offsets[j] + plan->tensors[j].bytes && plan->offsets[j] < plan->offsets[i] + plan->tensors[i].bytes;
+    };
+    for (size_t i = 0; i < plan->tensors.size() && free; ++i) {
+      const xema_tensor& t = plan->tensors[i];
+      if (t.death <= ln2 || t.birth > ln1) continue;
+      if (i != im && overlap(i, im) && t.birth <= mod_op) free = i == ib && plan->offsets[ib] == plan->offsets[im];
+      if (i != it && overlap(i, it)) free = false;
+    }
+    if (free) plan->ops[ln2].mod_op = plan->ops[ln1].mod_op = mod_op;
+  }
   plan->hid_in = at("hid", 0, -1);
   plan->temb_in = at("temb", -1, -1);
   plan->own_rows = S;
@@ -970,7 +1007,7 @@ int xema_plan_launch_count(const xema_plan* plan) {
 int xema_plan_forward_launches(const xema_plan* plan) {
   if (!plan || !plan->bound) return 0;
   int n = xema_plan_launch_count(plan);
-  for (const Op& o : plan->ops) n -= o.q_op != 0;
+  for (const Op& o : plan->ops) n -= (o.q_op != 0) + (o.mod_op != 0 && !std::strcmp(o.name, "LN2"));
   return n;
 }
 

@@ -91,6 +91,37 @@ def test_keys_values_and_queries_in_one_launch_have_the_bits_of_two(head_dim, ba
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
 
 
+# One and several batch elements, whole and cut phases, a width without an instance that carries a modulation, a shard.
+@pytest.mark.parametrize("batch,hidden,tokens,chunks,shard,carried", [
+    (1, 512, 9, (1, 1, 1), None, 2), (3, 768, 130, (1, 1, 1), None, 2), (5, 512, 33, (2, 1, 3), None, 2), (1, 3072, 40, (1, 2, 2), None, 2),
+    (1, 3328, 40, (1, 1, 1), None, 0), (2, 512, 100, (1, 1, 1), (1, 2), 2)])
+def test_a_step_has_the_same_bits_wherever_it_is_cut(batch, hidden, tokens, chunks, shard, carried):
+    """Launches that take a neighbouring operator along (Q beside KV, a later block's modulation beside LN2 and LN1A) do so only
+    where the call covers all that is involved."""
+    t = _template(batch, tokens, hidden, 512)
+    t = Template(t.name, *[getattr(t, f) for f in ("batch", "s_text", "grid_t", "grid_h", "grid_w", "hidden", "heads", "head_dim", "ffn")],
+                 n_blocks=3)
+    s = BlockSession(t, [make_block_weights(t, seed) for seed in range(3)], chunks=chunks, shard=shard)
+    joint = 3 if chunks[:2] == (1, 1) else 0
+    assert s.plan.forward_launches() == s.plan.launch_count() - joint - carried
+    x, temb = make_activations(t)
+    r0, rows = (0, tokens) if shard is None else (s.plan.row0, s.plan.rows)
+    x = torch.from_numpy(np.ascontiguousarray(x[:, r0:r0 + rows]).view(np.int16)).cuda()
+    temb = torch.from_numpy(temb.view(np.int16)).cuda()
+    n, stream = s.plan.n_ops, torch.cuda.current_stream().cuda_stream
+    outs = []
+    for cuts in [range(1, n)] + [[]] + [[c] for c in range(1, n)]:
+        s.arena.fill_(0)             # (a shard's missing keys)
+        s.set_inputs(x, temb)
+        for first, end in zip([0] + list(cuts), list(cuts) + [n]):
+            s.plan.forward_range(first, end, stream)
+        outs.append(s.hid_out().clone())
+    s.check_status()
+    assert len(outs) == n + 1 and outs[0].any()
+    for cut, y in enumerate(outs[1:]):
+        assert torch.equal(y, outs[0]), cut
+
+
 def _attention_of_a_plan(batch, heads, head_dim, tokens, chunks):
     """A session that has run up to its first attention launch: MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN."""
     t = _template(batch, tokens, heads * head_dim, 512, heads=heads)
