@@ -49,6 +49,7 @@ constexpr int GROUP_M = 8;
 constexpr int A_TILE_BYTES = BM * BK * 2;
 constexpr int CHUNK = 32;        // columns per epilogue step
 constexpr int BUF_BYTES = 4096;  // one staging buffer: 32 rows x 32 columns of fp32, or of bf16 in its first half
+constexpr int HALF_BUF = BUF_BYTES / 2;
 
 template <int EPI>
 constexpr bool kGated = EPI == XEMA_EPI_GATE_RES_F32 || EPI == XEMA_EPI_GATE_RES_BF16;
@@ -211,7 +212,9 @@ struct Epilogue {
   __device__ __forceinline__ uint8_t* next_buf() {
     if (lane == 0) bulk_wait_read<RING - 1>();
     __syncwarp();
-    return ring + (used % RING) * BUF_BYTES;
+    // RMSNorm + RoPE: results in the first half of the ring, angles in the second
+    static_assert(EPI != XEMA_EPI_BIAS_NORM_ROPE || RING == 2, "two results and one block of angles");
+    return ring + (used % RING) * (EPI == XEMA_EPI_BIAS_NORM_ROPE ? HALF_BUF : BUF_BYTES);
   }
 
   __device__ __forceinline__ bool gated_tile(int b, int row0, int n_base, uint32_t t_addr) {
@@ -280,10 +283,25 @@ struct Epilogue {
     send(buf, b, row0, n_base + col);
   }
 
-  // 16 angles (32 columns) of one row of the rotation table
-  __device__ __forceinline__ void load_angles(const float4* rp, float4 (&cs)[8]) {
+  // The angles of the warp's 32 rows for 32 columns from column c of a head on, 16 per row.  A warp reads four rows of 128 bytes at a
+  // time; own_angles hands every lane its row through shared memory.  With a row per lane each load met 32 lines, and the epilogue
+  // of the K | V | Q products was bound by that: 8000 rows x 3072 columns, K = 1024, heads of 128, 54.2 -> 48.6 us with 256 x 256
+  // tiles, 63.3 -> 58.1 with 128 x 128, heads of 64 48.5 -> 45.8 and 51.0 -> 52.2, with 128 x 64 83.9 -> 72.4.
+  __device__ __forceinline__ void load_angles(int row0, int c, float4 (&cs)[8]) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) cs[q] = __ldg(rp + q);
+    for (int q = 0; q < 8; ++q) {
+      const int row = min(row0 + 4 * q + (lane >> 3), p.rows - 1);
+      cs[q] = __ldg(reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * p.head_dim + c) + (lane & 7));
+    }
+  }
+  __device__ __forceinline__ void own_angles(float4 (&cs)[8]) {
+    uint8_t* buf = ring + BUF_BYTES;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) *reinterpret_cast<float4*>(piece_f32(buf, 4 * q + (lane >> 3), lane & 7)) = cs[q];
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) cs[q] = *reinterpret_cast<const float4*>(piece_f32(buf, lane, q));
+    __syncwarp();
   }
   // acc + bias, RMSNorm over each head, gain, rotation of adjacent pairs by the token's angles.
   // First the head norms from a pass over the accumulator, then 32 columns of every head per
@@ -312,16 +330,15 @@ struct Epilogue {
 #pragma unroll
       for (int i = 0; i < 4; ++i) rstd[i] = h == i ? r : rstd[i];
     }
-    const int row = min(row0 + lane, p.rows - 1);
-    const float4* rp = reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * DH);
 #pragma unroll 1
     for (int c = 0; c < DH; c += CHUNK) {
+      if (norm_heads > 0) own_angles(cs);
       // the angles of the next step are requested before this one's heads, which hide the trip to global memory
       // (with the warp index uniform, a step of 8 blocks of 333 x 1024 tokens 483 -> 450 us, a block of 1101 x 1536 129 -> 123,
       // one of 288 x 512 52.6 -> 50.2)
       float4 ahead[8];
       const bool more = c + CHUNK < DH && norm_heads > 0 && !rehearsing();
-      if (more) load_angles(rp + (c + CHUNK) / 4, ahead);
+      if (more) load_angles(row0, c + CHUNK, ahead);
 #pragma unroll 1
       for (int h = 0; h < HEADS; ++h) {
         const int col = h * DH + c;
@@ -606,10 +623,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap& map_a, const CUtens
         ep.gate = second ? s_gate + 128 : s_gate;
         ep.out_scale = second ? p.norm_out_scale2 : p.norm_out_scale;
         ep.col0 = second ? 0 : p.cols2;
-        if (live && n_base < p.norm_cols && !dry) {
-          const int row = min(row0 + lane, p.rows - 1);
-          ep.load_angles(reinterpret_cast<const float4*>(p.rope + (size_t)(p.rope_pos0 + row) * p.head_dim), cs);
-        }
+        if (live && n_base < p.norm_cols && !dry) ep.load_angles(row0, 0, cs);
       }
       for (int i = dry ? BN : et * 2; i < BN; i += 256) {
         const uint32_t bb = __ldg(reinterpret_cast<const uint32_t*>(p.bias + n_base + i));
