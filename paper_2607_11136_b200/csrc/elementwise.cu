@@ -14,6 +14,7 @@ using sm100::bf16_lo;
 using sm100::grid_dep_launch;
 using sm100::grid_dep_wait;
 using sm100::ld_f4;
+using sm100::ld_f8;
 using sm100::ld_u4;
 using sm100::pack_bf16x2;
 
@@ -196,11 +197,21 @@ struct LnIo {
     if constexpr (!IN_F32) s += fmaf(f[4], f[4], f[5] * f[5]) + fmaf(f[6], f[6], f[7] * f[7]);
     return s;
   }
-  // scale and shift of one step
+  // Scale and shift of one step.  A lane of the bf16 form needs 32 bytes of each: by two 16-byte loads a warp met every line twice,
+  // and the L1 was busy with scale and shift for four fifths of a row's time.  `wide`: both rows start on a 32-byte boundary, and
+  // one load takes all of it.  us, launches chained: 1101 x 1536 5.1 -> 4.2, 2040 x 2048 6.2 -> 4.8, 4608 x 3072 14.9 -> 12.9, 8888 x 1024
+  // 8.5 -> 7.5, 17776 x 2048 31.1 -> 28.5, x 3072 44.3 -> 41.2.
   struct Mod {
     float4 a[EPV / 4], c[EPV / 4];
   };
-  __device__ static __forceinline__ void load_mod(const float* sc, const float* sh, int idx, Mod& m) {
+  __device__ static __forceinline__ void load_mod(const float* sc, const float* sh, int idx, bool wide, Mod& m) {
+    if constexpr (!IN_F32) {
+      if (wide) {
+        ld_f8(sc + idx * EPV, m.a[0], m.a[1]);
+        ld_f8(sh + idx * EPV, m.c[0], m.c[1]);
+        return;
+      }
+    }
 #pragma unroll
     for (int q = 0; q < EPV / 4; ++q) {
       m.a[q] = ld_f4(sc + idx * EPV + 4 * q);
@@ -219,10 +230,12 @@ struct LnIo {
 };
 
 // CARRY > 0: the first mod_blocks blocks work out features of a modulation (that many batch elements a pass) beside the rows.
+// (Four blocks an SM for 2816 and 3072 columns, where the compiler would take 167 registers, three blocks, and be 15 % slower; for
+// fewer it stays within 128 by itself, and does worse when told to.)
 template <bool IN_F32, int NV, int CARRY>
-__global__ void __launch_bounds__(kLnWarps * 32)
+__global__ void __launch_bounds__(kLnWarps * 32, !IN_F32 && !CARRY && (NV == 11 || NV == 12) ? 4 : 0)
 ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, const float* shift, const float* scale,
-                   long long mod_stride, int batch, int rows, int D, float eps, const ModArgs mod, int mod_blocks) {
+                   long long mod_stride, int batch, int rows, int D, float eps, bool wide, const ModArgs mod, int mod_blocks) {
   using Io = LnIo<IN_F32>;
   constexpr int EPV = Io::EPV;
   if constexpr (CARRY > 0) {
@@ -251,7 +264,7 @@ ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, 
 #pragma unroll
     for (int v = 0; v < NV; ++v) raw[v] = Io::load(src, v * 32 + lane);
     typename Io::Mod m[2];
-    Io::load_mod(sc, sh, lane, m[0]);
+    Io::load_mod(sc, sh, lane, wide, m[0]);
     float f[EPV];
     float s = 0.f;
 #pragma unroll
@@ -269,7 +282,7 @@ ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, 
     const float rstd = rsqrtf(warp_sum(q) * inv_d + eps);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      if (v + 1 < NV) Io::load_mod(sc, sh, (v + 1) * 32 + lane, m[(v + 1) & 1]);
+      if (v + 1 < NV) Io::load_mod(sc, sh, (v + 1) * 32 + lane, wide, m[(v + 1) & 1]);
       Io::unpack(raw[v], f);
       Io::modulate(f, mean, rstd, m[v & 1]);
       Io::store(dst, v * 32 + lane, f);
@@ -292,7 +305,7 @@ ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, 
     for (int v = 0; v < nv; ++v) {
       typename Io::Mod m;
       Io::unpack(Io::load(src, v * 32 + lane), f);
-      Io::load_mod(sc, sh, v * 32 + lane, m);
+      Io::load_mod(sc, sh, v * 32 + lane, wide, m);
       Io::modulate(f, mean, rstd, m);
       Io::store(dst, v * 32 + lane, f);
     }
@@ -306,12 +319,13 @@ static int launch_ln_t(const void* in, long long in_batch_rows, void* out, const
   constexpr int PER = IN_F32 ? 2 : 1;                  // steps per 256 columns
   const long long total = (long long)batch * rows;
   const unsigned blocks = (unsigned)((total + kLnWarps - 1) / kLnWarps);
+  const bool wide = ((reinterpret_cast<uintptr_t>(shift) | reinterpret_cast<uintptr_t>(scale)) & 31) == 0 && (batch == 1 || mod_stride % 8 == 0);
   const int per_block = kLnWarps * kModRows;
   const int mod_blocks = mod ? (mod->j_end - mod->j_first + per_block - 1) / per_block : 0;
   const size_t smem = mod ? (size_t)mod->batch * mod->Dt * sizeof(float) : 0;
   auto run = [&](auto kern) {
     return launch_kernel(kern, dim3(blocks + mod_blocks), kLnWarps * 32, smem, stream, chained, in, in_batch_rows,
-                         (__nv_bfloat16*)out, shift, scale, mod_stride, batch, rows, D, eps, mod ? *mod : ModArgs{}, mod_blocks);
+                         (__nv_bfloat16*)out, shift, scale, mod_stride, batch, rows, D, eps, wide, mod ? *mod : ModArgs{}, mod_blocks);
   };
   if (mod) {
     if (int rc = check_mod(*mod)) return rc;

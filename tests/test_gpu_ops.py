@@ -51,6 +51,29 @@ def test_mod_gemv_edges(B, Dt, n_out, shift):
     assert out[-1].item() == 7.0
 
 
+# scale and shift on a 32-byte boundary in every row, in the first only, and in none; widths with a row in registers and beyond
+@pytest.mark.parametrize("D", [256, 2048, 2816, 3072, 4352])
+def test_ln_modulate_wide_loads_change_nothing(D):
+    gen = torch.Generator(device=DEV).manual_seed(D)
+    B, rows = 2, 37
+    x = torch.randn(B, rows, D, device=DEV, generator=gen).to(torch.bfloat16)
+    vals = torch.randn(B, 2, D, device=DEV, generator=gen)
+    outs = []
+    for first, stride in ((0, 2 * D), (0, 2 * D + 4), (4, 2 * D)):
+        mod = torch.zeros(first + 2 * stride + 2 * D, device=DEV)
+        for b in range(B):
+            mod[first + b * stride:first + b * stride + 2 * D] = vals[b].reshape(-1)
+        out = torch.empty(B, rows, D, dtype=torch.bfloat16, device=DEV)
+        at = mod.data_ptr() + 4 * first
+        xb.xema_op_ln_modulate(x.data_ptr(), 0, rows, out.data_ptr(), at, at + 4 * D, stride, B, rows, D, 1e-6)
+        outs.append(out)
+    f = x.double()
+    f = (f - f.mean(-1, keepdim=True)) / torch.sqrt(f.var(-1, unbiased=False, keepdim=True) + 1e-6)
+    want = f * (1 + vals[:, 1:2].double()) + vals[:, :1].double()
+    assert_bf16_close(outs[0].double().cpu().numpy(), want.cpu().numpy(), "LN")
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
 @pytest.mark.parametrize("D,in_f32", [(512, 0), (512, 1), (3072, 0), (3072, 1), (768, 0), (1280, 1)])
 def test_ln_modulate(D, in_f32):
     rng = np.random.default_rng(1)
