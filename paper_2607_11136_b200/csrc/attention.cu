@@ -260,7 +260,9 @@ enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
 // few key blocks gains 0.5 to 3 us by it; the second set of barriers costs the loop 2 %.  us without / with it: block of 288 x 512
 // 45.8 / 45.3, 464 x 1792 100.3 / 97.1 (dh 128 105.7 / 101.9), two blocks of 630 x 1536 184.2 / 179.6, eight of 304 x 2304 859.7 /
 // 833.7, eight of 333 x 1024 470.9 / 468.7; with 9 key blocks a CTA (1101 x 1536)
-// 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.
+// 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.  A CTA that starts when the launch
+// before it ends has no time to rehearse in: its scores came 1.8 us after the wait and found the softmax threads at it until 4.8.
+// Where an item has one tile the idle warps of the second do it instead: eight of 333 x 1024 382.0 -> 367.4.
 template <int DH, bool SCALED, bool REHEARSE>
 __global__ void __launch_bounds__(THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -908,7 +910,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         s_ph = pv_ph = 0;
       }
       const Item it = i < 0 ? Item{(p.rows + BM - 1) / BM * BM, 0, 0} : item_at(i);
-      if (i >= 0 && !tile_live(it, tile)) continue;
+      // (with one tile an item the second tile's warps, which have nothing else to do, rehearse while the first's go ahead)
+      if (i < 0 ? p.tiles == 1 && tile == 0 : !tile_live(it, tile)) continue;
       if (ok) {
         if (bounded) run_blocks(PassT{}, std::false_type{});
         else run_blocks(PassT{}, std::bool_constant<POLY>{});
