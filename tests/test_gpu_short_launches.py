@@ -240,3 +240,26 @@ def test_calls_see_what_a_kernel_wrote_right_before_them(tokens):
     s.check_status()
     for (i, j), y in zip(got, outs):
         assert np.array_equal((y ^ MASK).cpu().numpy().view(np.uint16), want[i, j].reshape(y.shape)), (i, j)
+
+
+# rows of several waves of tiles; the output over h2 of the first chunk, four rows behind it and apart from it; batch elements
+@pytest.mark.parametrize("batch,tokens,hidden,chunks,over", [
+    (1, 6930, 3072, (1, 1, 1), "at"), (1, 13000, 3072, (1, 1, 2), "at"), (1, 17776, 3072, (1, 1, 3), "behind"), (3, 2500, 2048, (1, 1, 1), "at"),
+    (2, 4800, 1536, (1, 1, 2), "at")])
+def test_forward_host_cuts_the_first_feed_forward_chunk(batch, tokens, hidden, chunks, over):
+    t = _template(batch, tokens, hidden, 12288 if over == "behind" else 1024)
+    s = BlockSession(t, [make_block_weights(t, 2)], chunks=chunks)
+    (out, _), (h2, _) = s.plan.tensor("hid1"), s.plan.tensor("h20_0")
+    assert (out == h2) == (over == "at") and (out > h2) == (over == "behind")
+    x, temb = (torch.from_numpy(a.view(np.int16)) for a in make_activations(t))
+    s.set_inputs(x, temb)
+    s.forward()
+    want = s.hid_out().cpu()
+    x, temb = x.pin_memory(), temb.pin_memory()
+    y = torch.empty_like(x).pin_memory()
+    for fill in (0xFF, 0x00):
+        s.arena.fill_(fill)
+        s.plan.forward_host(x.data_ptr(), temb.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        s.check_status()
+        assert torch.equal(y, want), fill
