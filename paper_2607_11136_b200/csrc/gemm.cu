@@ -65,7 +65,7 @@ struct GemmCfg {
   static constexpr int W_TILE_BYTES = W_ROWS * BK * 2;
   // K blocks of 64 per stage.  The K block of a smaller tile is short (128 to 256 cycles of MMA), and
   // with a stage per block the barrier round of each one takes longer than that: 8888 x 12288 x 3072 with
-  // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block, 72 B/clk of fill).
+  // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block).
   static constexpr int KSUB = BN == 256 ? 1 : 2;
   static constexpr int STAGE_BYTES = KSUB * (A_TILE_BYTES + W_TILE_BYTES);
   static constexpr int OFF_W = KSUB * A_TILE_BYTES;            // in a stage
@@ -798,12 +798,13 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // Tile for a problem: the one with the shortest estimated time, waves x K blocks x nanoseconds per K
 // block plus what its last tile's epilogue adds.  Measured (B200, shapes from 288 x 512 x 2048 to 8888 x 12288 x
 // 3072): a K block takes 370-385 ns with 256 x 256 pair tiles, 212-270 with 256 x 128 pair tiles, 255-290 with
-// 128 x 128 and 172-211 with 128 x 64 -- a CTA fills shared memory at about 70 B/clk whatever its tile -- so a
+// 128 x 128 and 172-211 with 128 x 64 -- an MMA of 16 along K takes about 26 + operand bytes / 170 clocks (128 x 32 55, 128 x 64 62,
+// 128 x 128 73, pairs of 256 x 128 69, without any loads the same), and with every SM at it 57 B/clk of fill are the limit -- so a
 // smaller tile is slower per flop and pays only where the larger one leaves SMs idle.  us for 256 x 256 /
 // 256 x 128 / 128 x 128 / 128 x 64: 333 x 1024 x 4096 28.8 / 20.2 / 21.9 / 16.5, 1101 x 1536 x 6144 39.1 / 27.3 / 30.9 /
 // 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.  128 x 32 exists for the
 // gated epilogues, whose products are narrow: 288 x 512 x 2048 12.1 -> 10.4 us, a step of 8 blocks of 333 tokens
-// x 1024 521 -> 500.
+// x 1024 521 -> 500.  (Shorter tiles -- 32, 64 or 96 of the 128 rows filled -- are no faster: the MMAs are the same.)
 // The 256 x 256 figure was taken under the power cap, as launches that need it run, the small tiles' at full clock, as
 // theirs do.  Pairs are counted as SMs / 2, all of which are resident on a B200 (74); where fewer fit, the launch
 // takes those and only the estimate is off.  The bits of a row do not depend on the choice.
