@@ -805,13 +805,18 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.  128 x 32 exists for the
 // gated epilogues, whose products are narrow: 288 x 512 x 2048 12.1 -> 10.4 us, a step of 8 blocks of 333 tokens
 // x 1024 521 -> 500.  (Shorter tiles -- 32, 64 or 96 of the 128 rows filled -- are no faster: the MMAs are the same.)
+// A pair's ends cost 700 ns more than its epilogue alone (its clusters start and end together): with them counted the pick takes 1.010
+// times the best form, without them 1.023, over 447 products back to back (widths 512 to 3072, 170 to 6700 rows; 287 others 1.010 and
+// 1.016), and single tiles of 128 x 128 get what is close to a wave either way.  us without / with: eight blocks of 333 x 1024 366.8 /
+// 363.8, 1055 x 1280 129.6 / 125.6, 4251 x 768 225.6 / 216.2, two blocks of 4706 x 1280 810 / 800.  (Fitted freely the figures give
+// 1.005, but 2.8 % more time for eight blocks of 847 x 2816, whose weights do not stay in L2.)
 // The 256 x 256 figure was taken under the power cap, as launches that need it run, the small tiles' at full clock, as
 // theirs do.  Pairs are counted as SMs / 2, all of which are resident on a B200 (74); where fewer fit, the launch
 // takes those and only the estimate is off.  The bits of a row do not depend on the choice.
 struct Tile {
   int pair, block_n, block_ns, epilogue_ns;
 };
-constexpr Tile kTiles[] = {{1, 256, 372, 3000}, {1, 128, 230, 1500}, {0, 128, 265, 1000}, {0, 64, 180, 500}, {0, 32, 150, 400}};
+constexpr Tile kTiles[] = {{1, 256, 372, 3700}, {1, 128, 230, 2200}, {0, 128, 265, 1000}, {0, 64, 180, 500}, {0, 32, 150, 400}};
 
 bool tile_fits(const GemmLaunch& g, const Tile& t) {
   if (g.N % t.block_n) return false;
