@@ -44,8 +44,9 @@ __device__ __forceinline__ uint4 ld_weights(const uint4* p) {
   return v;
 }
 
-// Features [j_first, j_end) of block `tile` of WARPS * kModRows of them, BATCH batch elements per pass over the weights.
-template <int WARPS, int BATCH>
+// Features [j_first, j_end) of block `tile` of WARPS * kModRows of them, BATCH batch elements per pass over the weights (ONE_PASS: there
+// are no more of them).
+template <int WARPS, int BATCH, bool ONE_PASS>
 __device__ __forceinline__ void mod_features(const ModArgs& a, int tile) {
   extern __shared__ float s_e[];  // [batch][Dt]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -82,7 +83,7 @@ __device__ __forceinline__ void mod_features(const ModArgs& a, int tile) {
     *reinterpret_cast<float4*>(s_e + i * 8 + 4) = make_float4(e[4], e[5], e[6], e[7]);
   }
   __syncthreads();
-  for (int b0 = 0; b0 < (BATCH == 1 ? 1 : a.batch); b0 += BATCH) {
+  for (int b0 = 0; b0 < (ONE_PASS ? 1 : a.batch); b0 += BATCH) {
     float acc[kModRows][BATCH];
 #pragma unroll
     for (int r = 0; r < kModRows; ++r)
@@ -134,7 +135,7 @@ __device__ __forceinline__ void mod_features(const ModArgs& a, int tile) {
 
 template <int BATCH>
 __global__ void __launch_bounds__(kModWarps * 32, 2) mod_gemv_kernel(const ModArgs a) {
-  mod_features<kModWarps, BATCH>(a, blockIdx.x);
+  mod_features<kModWarps, BATCH, BATCH == 1>(a, blockIdx.x);
 }
 
 constexpr size_t kModSmemLimit = 48 * 1024;
@@ -229,18 +230,21 @@ struct LnIo {
   }
 };
 
-// CARRY > 0: the first mod_blocks blocks work out features of a modulation (that many batch elements a pass) beside the rows.
-// (Four blocks an SM for 2816 and 3072 columns, where the compiler would take 167 registers, three blocks, and be 15 % slower; for
-// fewer it stays within 128 by itself, and does worse when told to.)
+// CARRY > 0: the first mod_blocks blocks work out features of a modulation (that many batch elements a pass) beside the rows.  For 1 and
+// 2 elements one pass is all there is, and the instance needs no more registers than the rows alone or 80.  The instance for 4 loops
+// over passes and takes 156: in one pass it needs 80 too, but then its four sums follow one another and few rows wait for it (8
+// blocks of 4 x 250 x 1024 462 us with 156 registers, 483 with 80).
+// Four blocks an SM for 2816 and 3072 bf16 columns (128 registers, of which 16 and 52 bytes a thread go to local memory), where the
+// compiler would take 167, three blocks, and be 15 % slower; fewer columns stay within 128 by themselves.
 template <bool IN_F32, int NV, int CARRY>
-__global__ void __launch_bounds__(kLnWarps * 32, !IN_F32 && !CARRY && (NV == 11 || NV == 12) ? 4 : 0)
+__global__ void __launch_bounds__(kLnWarps * 32, !IN_F32 && (NV == 11 || NV == 12) ? 4 : 0)
 ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, const float* shift, const float* scale,
                    long long mod_stride, int batch, int rows, int D, float eps, bool wide, const ModArgs mod, int mod_blocks) {
   using Io = LnIo<IN_F32>;
   constexpr int EPV = Io::EPV;
   if constexpr (CARRY > 0) {
     if ((int)blockIdx.x < mod_blocks) {
-      mod_features<kLnWarps, CARRY>(mod, blockIdx.x);
+      mod_features<kLnWarps, CARRY, CARRY <= 2>(mod, blockIdx.x);
       return;
     }
   }
@@ -330,10 +334,12 @@ static int launch_ln_t(const void* in, long long in_batch_rows, void* out, const
   if (mod) {
     if (int rc = check_mod(*mod)) return rc;
     switch (D / 256) {
-#define XEMA_LN_CASE(N) \
-  case N: return mod->batch == 1 ? run(ln_modulate_kernel<IN_F32, N * PER, 1>) : run(ln_modulate_kernel<IN_F32, N * PER, 4>);
-      XEMA_LN_CASE(1) XEMA_LN_CASE(2) XEMA_LN_CASE(3) XEMA_LN_CASE(4) XEMA_LN_CASE(5) XEMA_LN_CASE(6)
-      XEMA_LN_CASE(7) XEMA_LN_CASE(8) XEMA_LN_CASE(9) XEMA_LN_CASE(10) XEMA_LN_CASE(11) XEMA_LN_CASE(12)
+#define XEMA_LN_CASE(N, MOST) \
+  case N: return mod->batch == 1   ? run(ln_modulate_kernel<IN_F32, N * PER, 1>) \
+                 : mod->batch == 2 ? run(ln_modulate_kernel<IN_F32, N * PER, 2>) \
+                 : MOST > 2        ? run(ln_modulate_kernel<IN_F32, N * PER, MOST>) : XEMA_EINVAL;
+      XEMA_LN_CASE(1, 4) XEMA_LN_CASE(2, 4) XEMA_LN_CASE(3, 4) XEMA_LN_CASE(4, 4) XEMA_LN_CASE(5, 4) XEMA_LN_CASE(6, 4)
+      XEMA_LN_CASE(7, 4) XEMA_LN_CASE(8, 4) XEMA_LN_CASE(9, 2) XEMA_LN_CASE(10, 2) XEMA_LN_CASE(11, 2) XEMA_LN_CASE(12, 2)
 #undef XEMA_LN_CASE
       default: return XEMA_EINVAL;
     }

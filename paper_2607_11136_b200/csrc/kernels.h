@@ -83,7 +83,7 @@ int launch_mod(const ModArgs& a, cudaStream_t stream, bool chained = false);
 int launch_ln_modulate(const void* in, int in_is_f32, long long in_batch_rows, void* out, const float* shift,
                        const float* scale, long long mod_stride, int batch, int rows, int D, float eps,
                        cudaStream_t stream, bool chained = false, const ModArgs* mod = nullptr);   // mod: beside the rows
-constexpr int kLnMaxCarryCols = 3072;   // widths that have an instance for that
+constexpr int kLnMaxCarryCols = 3072, kLnMaxCarryCols4 = 2048;   // widths that have an instance for that: 1 and 2 batch elements, more
 int launch_rmsnorm_rope(void* x, long long ld, long long batch_rows, const void* g, const float* rope, int pos0,
                         int batch, int rows, int heads, int head_dim, float eps, cudaStream_t stream);
 

@@ -137,7 +137,24 @@ struct Op {
   AttnLaunch attn;
 };
 
-constexpr long long kCarryRows = 8192;   // rows of an LN launch up to which it may carry a modulation
+// Whether LN launches of up to `rows` rows (batch elements counted) may carry a modulation of `batch` elements.  One launch falls
+// away, two get longer by half of its work each.  Speed of stacks of 3 or 8 blocks with it over the same with MOD as a launch of its own
+// (the same build twice: within 0.01):
+//   1 and 2 elements, whose carrying instances need hardly more registers than the rows: up to 2000 rows 0.99 to 1.07 at every width (8
+//   blocks of 1 x 300 x 1024 1.05, of 2 x 500 x 1280 1.05, of 2 x 1000 x 512 1.04, of 2 x 500 x 3072 1.00), at 4000 0.99 to 1.01, at
+//   8000 0.98 to 1.01.
+//   3 to 6, whose instance takes 156 registers, so that fewer blocks of rows fit an SM: 768 and 1024 columns 0.99 to 1.05 up to 2000 rows,
+//   0.98 to 1.00 at 3000 and 4000; 1280 and 1536 1.01 to 1.09 up to 640, 1.00 to 1.03 at 1000, 0.98 to 1.01 at 2000; 1792 and 2048 1.01
+//   to 1.07 at 300, 0.99 to 1.04 at 500, 0.99 at 640; 2560 0.98 at 300.
+//   512 columns and fewer, where MOD by itself is short: 3 and 4 elements 0.99 to 1.03 from 800 to 2000 rows, 0.92 to 1.02 below, 5 and 6
+//   0.90 to 1.02; at 512 columns and under 100 rows 3 to 5 elements 0.99 to 1.02.
+//   7 and 8, in two passes over the weights: 512 0.93 to 1.01, 1024 0.98 to 1.01, 1536 and 2048 0.97 to 1.02.
+static bool ln_may_carry(int batch, long long rows, int D) {
+  if (batch <= 2) return D <= kLnMaxCarryCols && rows <= 4096;
+  if (batch > 6) return false;
+  if (D <= 512) return rows < 800 ? D == 512 && batch <= 5 && rows < 100 : batch <= 4 && rows <= 2048;
+  return rows <= (D <= 1024 ? 2048 : D <= 1536 ? 1024 : D <= kLnMaxCarryCols4 ? 512 : 0);
+}
 
 // One step of xema_forward_host: a launch, or the arrival / departure of a piece of the block input /
 // output (`rows` x `width` bytes at byte offset `offset` of the tensor, rows `pitch` apart).
@@ -653,15 +670,15 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
   // The modulation of a later block needs the timestep embedding and the slot of the block before, of which the attention half
   // (shift, scale, gate) has been read when LN2 starts and the rest when the next LN1A does: the blocks of those two launches
   // that have no row work it out, and its own launch falls away.  Where mod<m> lies over nothing but mod<m - 1> from LN2 to
-  // MOD and nothing takes the embedding's bytes until LN1A.  Eight blocks of 333 x 1024 in a graph 401.7 -> 385.0 us; from some
-  // thousand rows on MOD is a thousandth of a block, and the larger instance of LN has fewer warps an SM.
+  // MOD and nothing takes the embedding's bytes until LN1A, and where it is faster (ln_may_carry).  Eight blocks of 333 x 1024 in a graph
+  // 401.7 -> 385.0 us.
   const size_t per_block = 1 + 3 * (size_t)CA + 5 * (size_t)CB + 3 * (size_t)CC;
   for (int m = 1; m < c.n_blocks; ++m) {
     const size_t mod_op = m * per_block, ln1 = mod_op + 1, ln2 = mod_op - 3;
     const size_t im = plan->index.at("mod" + std::to_string(m)), ib = plan->index.at("mod" + std::to_string(m - 1));
     const size_t it = plan->index.at("temb");
     const long long rows = std::max((long long)plan->ops[ln1].batch * plan->ops[ln1].rows, (long long)plan->ops[ln2].batch * plan->ops[ln2].rows);
-    bool free = D <= kLnMaxCarryCols && rows <= kCarryRows;
+    bool free = ln_may_carry(c.batch, rows, (int)D);
     auto overlap = [&](size_t i, size_t j) {
       return plan->offsets[i] < plan->offsets[j] + plan->tensors[j].bytes && plan->offsets[j] < plan->offsets[i] + plan->tensors[i].bytes;
     };

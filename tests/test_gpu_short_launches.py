@@ -122,6 +122,30 @@ def test_a_step_has_the_same_bits_wherever_it_is_cut(batch, hidden, tokens, chun
         assert torch.equal(y, outs[0]), cut
 
 
+# Both sides of every line of the rule; a launch that carries, and one of many rows, has the bits of the launches apart.
+@pytest.mark.parametrize("batch,hidden,tokens,carried", [
+    (1, 512, 4096, 1), (1, 512, 4097, 0), (1, 3072, 300, 1), (1, 3328, 300, 0), (2, 512, 2048, 1), (2, 512, 2049, 0), (2, 2816, 65, 1),
+    (4, 512, 24, 1), (4, 512, 100, 0), (4, 512, 200, 1), (4, 512, 513, 0), (5, 512, 200, 0), (3, 1024, 682, 1), (3, 1024, 683, 0),
+    (4, 1280, 256, 1), (4, 1280, 257, 0), (6, 2048, 85, 1), (6, 2048, 86, 0), (3, 2304, 20, 0), (7, 1024, 40, 0), (1, 512, 8193, 0)])
+def test_a_modulation_is_carried_where_that_is_faster(batch, hidden, tokens, carried):
+    t = _template(batch, tokens, hidden, 256)
+    t = Template(t.name, *[getattr(t, f) for f in ("batch", "s_text", "grid_t", "grid_h", "grid_w", "hidden", "heads", "head_dim", "ffn")],
+                 n_blocks=2)
+    w = [make_block_weights(t, 1), make_block_weights(t, 2)]
+    s = BlockSession(t, w, chunks=(1, 1, 1))
+    assert s.plan.forward_launches() == s.plan.launch_count() - 2 - carried       # (both blocks' Q goes with KV)
+    x, temb = (torch.from_numpy(a.view(np.int16)).cuda() for a in make_activations(t))
+    stream, outs = torch.cuda.current_stream().cuda_stream, []
+    for ends in ([s.plan.n_ops], range(1, s.plan.n_ops + 1)):
+        s.arena.fill_(0x5A)
+        s.set_inputs(x, temb)
+        for first, end in zip([0] + list(ends), ends):
+            s.plan.forward_range(first, end, stream)
+        outs.append(s.hid_out().clone())
+    s.check_status()
+    assert torch.equal(outs[0], outs[1])
+
+
 def _attention_of_a_plan(batch, heads, head_dim, tokens, chunks):
     """A session that has run up to its first attention launch: MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN."""
     t = _template(batch, tokens, heads * head_dim, 512, heads=heads)
