@@ -201,7 +201,10 @@ struct LnIo {
   // Scale and shift of one step.  A lane of the bf16 form needs 32 bytes of each: by two 16-byte loads a warp met every line twice,
   // and the L1 was busy with scale and shift for four fifths of a row's time.  `wide`: both rows start on a 32-byte boundary, and
   // one load takes all of it.  us, launches chained: 1101 x 1536 5.1 -> 4.2, 2040 x 2048 6.2 -> 4.8, 4608 x 3072 14.9 -> 12.9, 8888 x 1024
-  // 8.5 -> 7.5, 17776 x 2048 31.1 -> 28.5, x 3072 44.3 -> 41.2.
+  // 8.5 -> 7.5, 17776 x 2048 31.1 -> 28.5, x 3072 44.3 -> 41.2, x 3328 51.3 -> 46.7, x 3840 57.7 -> 52.5.  It is slower where its registers
+  // cost a wave (2961 to 3552 rows of 1536 columns 5.6 -> 6.0, 2000 of 3840 10.4 -> 11.0) and, in LN launches that follow one another
+  // with a block an SM or less, by 0.1 (1792 columns) to 1 us (4096) -- not in plans: with narrow loads up to 592 rows, stacks of 1792 to
+  // 3072 columns and 68 to 500 rows a launch took 0.99 to 1.01 of the time that they take with wide ones.
   struct Mod {
     float4 a[EPV / 4], c[EPV / 4];
   };
@@ -235,9 +238,13 @@ struct LnIo {
 // over passes and takes 156: in one pass it needs 80 too, but then its four sums follow one another and few rows wait for it (8
 // blocks of 4 x 250 x 1024 462 us with 156 registers, 483 with 80).
 // Four blocks an SM for 2816 and 3072 bf16 columns (128 registers, of which 16 and 52 bytes a thread go to local memory), where the
-// compiler would take 167, three blocks, and be 15 % slower; fewer columns stay within 128 by themselves.
+// compiler would take 167, three blocks, and be 15 % slower; three for 4096 (168 registers and 16 bytes), where it would take 247,
+// two blocks: us 1200 x 4096 10.3 -> 6.8, 3500 16.6 -> 14.2, 8888 36.5 -> 31.4, 17776 64.6 -> 55.8 (by narrow loads, 166 registers:
+// 7.2, 15.3, 34.5, 60.5).  3328 to 3840 columns take 153 to 166 by themselves and are 5 to 22 % slower when told so, fewer than 2816
+// stay within 128; told to be six blocks (80 registers) 1536 columns gain 15 % at 3500 rows, which then are one wave, and lose 8 % at
+// 1200.
 template <bool IN_F32, int NV, int CARRY>
-__global__ void __launch_bounds__(kLnWarps * 32, !IN_F32 && (NV == 11 || NV == 12) ? 4 : 0)
+__global__ void __launch_bounds__(kLnWarps * 32, IN_F32 ? 0 : NV == 11 || NV == 12 ? 4 : NV == 16 ? 3 : 0)
 ln_modulate_kernel(const void* in, long long in_batch_rows, __nv_bfloat16* out, const float* shift, const float* scale,
                    long long mod_stride, int batch, int rows, int D, float eps, bool wide, const ModArgs mod, int mod_blocks) {
   using Io = LnIo<IN_F32>;

@@ -1,4 +1,5 @@
 """Per-kernel parity against the oracle's operator definitions, through the C ABI (GPU)."""
+import json
 import math
 
 import numpy as np
@@ -72,6 +73,27 @@ def test_ln_modulate_wide_loads_change_nothing(D):
     want = f * (1 + vals[:, 1:2].double()) + vals[:, :1].double()
     assert_bf16_close(outs[0].double().cpu().numpy(), want.cpu().numpy(), "LN")
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+# Every width whose rows stay in registers: four blocks of 128 threads an SM up to 3072 columns, three up to 4096, in 65536 registers.
+def test_ln_modulate_leaves_room_for_other_blocks(tmp_path):
+    widths, rows = range(256, 4097, 256), 5
+    gen = torch.Generator(device=DEV).manual_seed(7)
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+        for D in widths:
+            x = torch.randn(rows, D, device=DEV, generator=gen).to(torch.bfloat16)
+            mod = torch.randn(2, D, device=DEV, generator=gen)
+            out = torch.empty_like(x)
+            xb.xema_op_ln_modulate(x.data_ptr(), 0, rows, out.data_ptr(), mod.data_ptr(), mod.data_ptr() + 4 * D, 0, 1, rows, D, 1e-6)
+            f = x.double()
+            f = (f - f.mean(-1, keepdim=True)) / torch.sqrt(f.var(-1, unbiased=False, keepdim=True) + 1e-6)
+            assert_bf16_close(out.double().cpu().numpy(), (f * (1 + mod[1].double()) + mod[0].double()).cpu().numpy(), "LN %d" % D)
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    events = [e for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if "ln_modulate_kernel" in e.get("name", "")]
+    assert len(events) == len(widths)
+    for D, e in zip(widths, sorted(events, key=lambda e: e["ts"])):
+        assert e["args"]["registers per thread"] <= (128 if D <= 3072 else 168), (D, e["args"])
 
 
 @pytest.mark.parametrize("D,in_f32", [(512, 0), (512, 1), (3072, 0), (3072, 1), (768, 0), (1280, 1)])
