@@ -311,7 +311,8 @@ def main():
         op); the ops between two events go out in one call.  An event between two kernels costs
         about a microsecond of idle GPU, so the headline leg brackets only the dominant kernel
         (its duration is what the roofline needs) and the table of all ops comes from a pass of
-        its own.  Returns (total ms, sorted per-step ms, restore ms, per-op dict of the bracketed
+        its own, in which every op is a launch of its own (in the headline leg neighbours may share
+        one: KV and Q do).  Returns (total ms, sorted per-step ms, restore ms, per-op dict of the bracketed
         ops, clocks)."""
         marks = set(range(n_launch)) if bracket is None else set(bracket)
         cuts = sorted({0, n_launch} | marks | {i + 1 for i in marks})
@@ -379,7 +380,8 @@ def main():
         sustained = {"steps": n_sus, "preheat_seconds": 2.0, "ms_per_step": s_total / n_sus,
                      "ms_median": s_steps[len(s_steps) // 2], "value": whole_job_tflops(flops, world, s_total / n_sus),
                      "clocks": s_clk, "per_op_raw": s_ops, "dom_raw": s_dom,
-                     "per_op_pass": {"steps": n_tab, "ms_per_step": s_tab_total / n_tab, "clocks": s_tab_clk}}
+                     "per_op_pass": {"steps": n_tab, "ms_per_step": s_tab_total / n_tab, "gpu_launches_per_step": sess.plan.launch_count(),
+                                     "clocks": s_tab_clk}}
         if s_clk.get("sm_mhz"):       # time x median clock: how the step depends on the clock it ran at
             sustained["sm_mcycles_per_step"] = sustained["ms_per_step"] * s_clk["sm_mhz"] / 1e3
 
@@ -566,7 +568,8 @@ def main():
         "per_op": breakdown,
         # the per-op table comes from a second pass of the same K steps with an event around every op;
         # the timed region of `value` carries events only around each step and the dominant kernel
-        "per_op_pass": {"steps": args.steps, "ms_per_step": per_op_total_ms / args.steps, "clocks": per_op_clocks},
+        "per_op_pass": {"steps": args.steps, "ms_per_step": per_op_total_ms / args.steps, "gpu_launches_per_step": sess.plan.launch_count(),
+                        "clocks": per_op_clocks},
         "sustained": sustained,
         "cpu_baseline": cpu,
     }

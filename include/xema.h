@@ -347,8 +347,9 @@ int xema_plan_forward_launches(const xema_plan* plan);
 
 /* Debug aid: enqueue only the first n_logical_ops logical ops of the trace order. */
 int xema_forward_prefix(const xema_plan* plan, uint32_t n_logical_ops, void* stream);
-/* Enqueue logical ops [first_op, end_op) of the trace order (one launch each); lets a caller
- * put its own events between ops to time them. */
+/* Enqueue logical ops [first_op, end_op) of the trace order; lets a caller put its own events between
+ * ops to time them.  A range of one op is that op's own launch; neighbours that lie in the same range may
+ * share one, as in xema_block_forward. */
 int xema_forward_range(const xema_plan* plan, uint32_t first_op, uint32_t end_op, void* stream);
 /* Describes launch i of a bound plan: name8 (host, 8 bytes) receives "MOD", "LN1A", "KV",
  * "KROPE", "LN1B", "Q", "QROPE", "ATTN", "PROJ", "LN2", "FFN1" or "FFN2"; *flops the algorithmic

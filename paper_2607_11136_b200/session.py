@@ -194,7 +194,8 @@ class BlockSession:
         so call this after set_inputs) and checked after every op for as long as the tensor
         lives.  Returns the violations as (op index, op name, tensor name, damaged bytes): a
         kernel that writes past the end of its tensor is caught at the op that did it.  An empty
-        list means every band stayed intact.  `exchange(block)`: as in forward_sharded."""
+        list means every band stayed intact.  Every op runs in a launch of its own here, also those that
+        share one with a neighbour in `forward`.  `exchange(block)`: as in forward_sharded."""
         if not self.plan.guard_bytes:
             raise ValueError("the session was not created with guard_bytes")
         st = stream or torch.cuda.current_stream(self.device)

@@ -146,6 +146,43 @@ def test_a_modulation_is_carried_where_that_is_faster(batch, hidden, tokens, car
     assert torch.equal(outs[0], outs[1])
 
 
+@pytest.mark.parametrize("batch,hidden,tokens,chunks", [(1, 512, 200, (1, 1, 1)), (2, 768, 130, (1, 1, 3)), (3, 1024, 77, (1, 1, 1))])
+def test_launches_that_take_a_neighbour_along_write_their_results_and_nothing_else(batch, hidden, tokens, chunks):
+    """Over an arena with 4 KiB free behind every tensor: the calls that run KV .. Q in one launch and LN2 .. LN1A with the next
+    block's modulation inside change bytes of their operators' results only, neither other tensors nor what lies between them."""
+    t = _template(batch, tokens, hidden, 512)
+    t = Template(t.name, *[getattr(t, f) for f in ("batch", "s_text", "grid_t", "grid_h", "grid_w", "hidden", "heads", "head_dim", "ffn")],
+                 n_blocks=3)
+    s = BlockSession(t, [make_block_weights(t, seed) for seed in range(3)], chunks=chunks, guard_bytes=4096)
+    assert s.plan.forward_launches() == s.plan.launch_count() - 5
+    names = [s.plan.op(k)["name"] for k in range(s.plan.n_ops)]
+    calls = []                                   # (first op, end, tensors that they write)
+    for l, kv in enumerate(k for k, name in enumerate(names) if name == "KV"):
+        assert names[kv:kv + 4] == ["KV", "KROPE", "LN1B", "Q"]
+        calls.append((kv, kv + 4, ["kv%d" % l, "q%d_0" % l]))
+    for l, mod in enumerate((k for k, name in enumerate(names) if name == "MOD" and k), start=1):
+        assert names[mod - 3:mod + 2] == ["LN2", "FFN1", "FFN2", "MOD", "LN1A"]
+        last = chunks[2] - 1
+        calls.append((mod - 3, mod + 2, ["h2%d_%d" % (l - 1, last), "g%d_%d" % (l - 1, last), "hid%d" % l, "mod%d" % l, "h1a%d_0" % l]))
+    stream, at = torch.cuda.current_stream().cuda_stream, 0
+    s.arena.fill_(0xA5)
+    s.set_inputs(*make_activations(t))
+    for first, end, written in sorted(calls):
+        s.plan.forward_range(at, first, stream)
+        before = s.arena.clone()
+        s.plan.forward_range(first, end, stream)
+        changed = s.arena != before
+        for name in written:
+            off, nbytes = s.plan.tensor(name)
+            assert changed[off:off + nbytes].any(), (first, name)
+        for name in written:
+            off, nbytes = s.plan.tensor(name)
+            changed[off:off + nbytes] = False
+        assert not changed.any(), (first, changed.nonzero()[:4].tolist())
+        at = end
+    s.check_status()
+
+
 def _attention_of_a_plan(batch, heads, head_dim, tokens, chunks):
     """A session that has run up to its first attention launch: MOD, LN1A, KV, KROPE, LN1B, Q, QROPE, ATTN."""
     t = _template(batch, tokens, heads * head_dim, 512, heads=heads)
@@ -287,3 +324,28 @@ def test_forward_host_cuts_the_first_feed_forward_chunk(batch, tokens, hidden, c
         torch.cuda.synchronize()
         s.check_status()
         assert torch.equal(y, want), fill
+
+
+# LN2 launches of the call: of a first chunk that is cut and, where a piece of the output would end behind h2's rows that are still to
+# come, of one that is not (the output four rows behind h2; two row chunks of three batch elements)
+@pytest.mark.parametrize("batch,tokens,hidden,ffn,chunks,launches", [
+    (1, 6930, 3072, 1024, (1, 1, 1), [4]), (1, 17776, 3072, 12288, (1, 1, 3), [1, 4, 4]), (2, 4800, 1536, 1024, (1, 1, 2), [2, 2]),
+    (3, 3200, 1536, 1024, (1, 1, 2), [1, 3])])
+def test_forward_host_leaves_a_first_chunk_whole_where_its_pieces_would_meet(batch, tokens, hidden, ffn, chunks, launches):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the pieces are counted for 148 SMs")
+    t = _template(batch, tokens, hidden, ffn)
+    s = BlockSession(t, [make_block_weights(t, 2)], chunks=chunks)
+    x, temb = (torch.from_numpy(a.view(np.int16)) for a in make_activations(t))
+    s.set_inputs(x, temb)
+    s.forward()
+    want = s.hid_out().cpu()
+    x, temb = x.pin_memory(), temb.pin_memory()
+    y = torch.empty_like(x).pin_memory()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+        s.plan.forward_host(x.data_ptr(), temb.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+    s.check_status()
+    assert torch.equal(y, want)
+    ln2 = [e for e in prof.events() if re.search(r"ln_modulate_kernel<(\(bool\))?(1|true),", e.name)]     # (float32 rows)
+    assert len(ln2) == sum(launches)
