@@ -263,6 +263,8 @@ enum Mode { PASS = 0, PROBE = 1, REPEAT = 2 };
 // 121.8 / 122.5, with 16 (ragged batch of 3) 799 / 814, with 417 (17776 x 3072) 7129 / 7263.  A CTA that starts when the launch
 // before it ends has no time to rehearse in: its scores came 1.8 us after the wait and found the softmax threads at it until 4.8.
 // Where an item has one tile the idle warps of the second do it instead: eight of 333 x 1024 382.0 -> 367.4.
+// (Registers are given out by the role: what the compiler sees as 96 is short by 4 to 20 bytes a thread in five of the six instances, 20 in
+// the plain one of dh 64, which had 8 before the first loads stood behind the wait: 17776 x 3072 7026 / 7052, no difference.)
 template <int DH, bool SCALED, bool REHEARSE>
 __global__ void __launch_bounds__(THREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,

@@ -65,7 +65,7 @@ struct GemmCfg {
   static constexpr int W_TILE_BYTES = W_ROWS * BK * 2;
   // K blocks of 64 per stage.  The K block of a smaller tile is short (128 to 256 cycles of MMA), and
   // with a stage per block the barrier round of each one takes longer than that: 8888 x 12288 x 3072 with
-  // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block).
+  // 64-column tiles 936 us, with two blocks per stage 769 (335 cycles per K block, 73 B/clk of fill).
   static constexpr int KSUB = BN == 256 ? 1 : 2;
   static constexpr int STAGE_BYTES = KSUB * (A_TILE_BYTES + W_TILE_BYTES);
   static constexpr int OFF_W = KSUB * A_TILE_BYTES;            // in a stage
@@ -286,7 +286,10 @@ struct Epilogue {
   // The angles of the warp's 32 rows for 32 columns from column c of a head on, 16 per row.  A warp reads four rows of 128 bytes at a
   // time; own_angles hands every lane its row through shared memory.  With a row per lane each load met 32 lines, and the epilogue
   // of the K | V | Q products was bound by that: 8000 rows x 3072 columns, K = 1024, heads of 128, 54.2 -> 48.6 us with 256 x 256
-  // tiles, 63.3 -> 58.1 with 128 x 128, heads of 64 48.5 -> 45.8 and 51.0 -> 52.2, with 128 x 64 83.9 -> 72.4.
+  // tiles, 63.3 -> 58.1 with 128 x 128, heads of 64 48.5 -> 45.8 and 51.0 -> 52.2, with 128 x 64 83.9 -> 72.4.  Heads of 64 in 128 x 128
+  // tiles are the one form that can lose: launches chained, 5200 x 2304 x 768 22.5 -> 23.3, 2200 x 2048 x 1024 12.2 -> 12.5, 4650 x 3072 x
+  // 1024 29.3 -> 29.9, from K = 1280 on 1 to 3 % faster (3650 x 3840 x 1280 35.1 -> 34.2, 1100 x 6144 x 2048 28.5 -> 28.1).  A row per lane for
+  // that form alone gives 22.9, 12.4, 29.6, 35.2 and 27.6: not kept.  The epilogue takes 245 to 249 of 255 registers (226 to 232 before).
   __device__ __forceinline__ void load_angles(int row0, int c, float4 (&cs)[8]) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -798,8 +801,8 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // Tile for a problem: the one with the shortest estimated time, waves x K blocks x nanoseconds per K
 // block plus what its last tile's epilogue adds.  Measured (B200, shapes from 288 x 512 x 2048 to 8888 x 12288 x
 // 3072): a K block takes 370-385 ns with 256 x 256 pair tiles, 212-270 with 256 x 128 pair tiles, 255-290 with
-// 128 x 128 and 172-211 with 128 x 64 -- an MMA of 16 along K takes about 26 + operand bytes / 170 clocks (128 x 32 55, 128 x 64 62,
-// 128 x 128 73, pairs of 256 x 128 69, without any loads the same), and with every SM at it 57 B/clk of fill are the limit -- so a
+// 128 x 128 and 172-211 with 128 x 64 -- of a single CTA an MMA of 16 along K takes about 26 + operand bytes / 170 clocks (128 x 32 55,
+// 128 x 64 62, 128 x 128 73; pairs of 256 x 128 69; without any loads the same) -- so a
 // smaller tile is slower per flop and pays only where the larger one leaves SMs idle.  us for 256 x 256 /
 // 256 x 128 / 128 x 128 / 128 x 64: 333 x 1024 x 4096 28.8 / 20.2 / 21.9 / 16.5, 1101 x 1536 x 6144 39.1 / 27.3 / 30.9 /
 // 37.7, 2222 x 3072 x 3072 41.1 / 37.0 / 43.2 / 56.2, 4444 x 3072 x 3072 58.0 / 65.7 / 78.0 / 104.  128 x 32 exists for the
@@ -809,7 +812,8 @@ int launch_epi(const GemmLaunch& g, cudaStream_t stream, bool chained) {
 // times the best form, without them 1.023, over 447 products back to back (widths 512 to 3072, 170 to 6700 rows; 287 others 1.010 and
 // 1.016), and single tiles of 128 x 128 get what is close to a wave either way.  us without / with: eight blocks of 333 x 1024 366.8 /
 // 363.8, 1055 x 1280 129.6 / 125.6, 4251 x 768 225.6 / 216.2, two blocks of 4706 x 1280 810 / 800.  (Fitted freely the figures give
-// 1.005, but 2.8 % more time for eight blocks of 847 x 2816, whose weights do not stay in L2.)
+// 1.005, but 2.8 % more time for eight blocks of 847 x 2816, whose weights do not stay in L2.)  With every SM at it loads can take
+// over: 3 x 680 x 2048 x 8192 52.0 us with 256 x 256 tiles, 44.6 without loads in the steady state (57 B/clk of fill a CTA).
 // The 256 x 256 figure was taken under the power cap, as launches that need it run, the small tiles' at full clock, as
 // theirs do.  Pairs are counted as SMs / 2, all of which are resident on a B200 (74); where fewer fit, the launch
 // takes those and only the estimate is off.  The bits of a row do not depend on the choice.

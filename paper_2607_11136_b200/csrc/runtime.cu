@@ -605,9 +605,12 @@ int xema_plan_bind(xema_plan* plan, void* arena_dev, uint64_t arena_bytes, const
       if (rc) return rc;
       plan->ops.back().reads_ln1a = q_follows_kv;     // ops: LN1A, KV, KROPE (fused), LN1B (elided), Q
       // Q then multiplies the same rows with the weight rows in front of KV's, by the same epilogue: one launch does both where
-      // nothing that lives between the two ops lies in q's bytes.  It needs as many waves of tiles as the two together or
-      // fewer, and one start and end less.  us apart / together: block of 288 x 512 45.3 / 40.7, eight of 333 x 1024 443.5 /
-      // 404.8, 1101 x 1536 121.1 / 114.4, 4608 x 3072 1083 / 1068, 17776 x 3072 6883 / 6896 (no difference).
+      // nothing that lives between the two ops lies in q's bytes.  It has one start and end less.  The tile is picked for the 3 D
+      // columns, and the product by itself can take longer than the two (by the rule's own figures up to 0.7 us, at 535 to 680 rows of 1280
+      // columns, where one wave of 256 x 256 pairs stands against one of 128 x 128 and one of 128 x 64); the saved launch is worth more.  us
+      // apart / together, blocks: 640 x 1280 74.8 / 73.7, 879 x 1280 77.5 / 75.7, 796 x 1024 67.1 / 63.8, 1028 x 768 63.4 / 61.6, 535 x 3072
+      // 197.1 / 188.8, 2072 x 2816 480.4 / 478.3 (the sizes where the rule's figures speak most against it); 288 x 512 45.3 / 40.7, eight of 333 x
+      // 1024 443.5 / 404.8, 1101 x 1536 121.1 / 114.4, 4608 x 3072 and 17776 x 3072 no difference.
       if (q_follows_kv) {
         const size_t q_op = plan->ops.size() - 1;
         const size_t iq = plan->index.at(std::string("q") + std::to_string(l) + "_0");
