@@ -74,17 +74,17 @@ def whole_job_tflops(flops_per_replica: float, world: int, ms: float) -> float:
     return world * flops_per_replica / (ms * 1e-3) / 1e12
 
 
-# DRAM traffic of one attention launch (dram__bytes_read.sum + dram__bytes_write.sum under ncu).  Captured inside
-# this bench at the full 17776 query rows: 422.9 MB (329.0 read + 93.9 written; algorithmic 440.3 -- q is still
-# in L2 from the Q projection), with an earlier kernel that read and wrote the same tensors; the present one alone:
-# 425.1 (329.2 + 95.9).  Captured alone at 2222 rows: 266.6 MB (present kernel 259.2; algorithmic 246.2), of
+# DRAM traffic of one attention launch (dram__bytes_read.sum + dram__bytes_write.sum under ncu).  Captured in the
+# block at the full 17776 query rows: 421.0 MB (328.5 read + 92.5 written; algorithmic 440.3 -- q is still
+# in L2 from the K | V | Q product); alone 425.1 (329.2 + 95.9).  At 2222 rows alone, with an
+# earlier kernel that read and wrote the same tensors: 266.6 MB (the present one 259.2; algorithmic 246.2), of
 # which k and v (4*S*D bytes, independent of the number of query rows) are read once and the rest scales with
 # the query rows; other row counts are scaled from that capture.  Not measured in the timed run.
 def attention_traffic_bytes(t, rows: int) -> float:
     if (t.seq, t.hidden, t.head_dim) != (17776, 3072, 64):
         return None
     if rows == t.seq:
-        return 422.9e6
+        return 421.0e6
     kv = 4.0 * t.seq * t.hidden
     return kv + (266.6e6 - kv) * rows / 2222.0
 
@@ -484,8 +484,8 @@ def main():
         r["traffic"] = None
         if dom == "ATTN":
             r["traffic"] = attention_traffic_bytes(t, t.seq * t.n_blocks // d["launches"])
-            r["traffic_source"] = ("not measured in this run: dram__bytes_read.sum + dram__bytes_write.sum of ncu captures of an "
-                                   "earlier kernel (the present one is within 3 % of them)" if r["traffic"] else None)
+            r["traffic_source"] = ("not measured in this run: dram__bytes_read.sum + dram__bytes_write.sum of an ncu capture of the "
+                                   "block (17776 query rows; other row counts from an earlier kernel's, within 3 %)" if r["traffic"] else None)
         return r
 
     def breakdown_of(ops_t, step_ms_):
