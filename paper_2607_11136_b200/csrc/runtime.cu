@@ -139,16 +139,16 @@ struct Op {
 
 // Whether LN launches of up to `rows` rows (batch elements counted) may carry a modulation of `batch` elements.  One launch falls
 // away, two get longer by half of its work each.  Speed of stacks of 3 or 8 blocks with it over the same with MOD as a launch of its own
-// (the same build twice: within 0.01):
+// (repeats differ by 0.01, few by 0.02):
 //   1 and 2 elements, whose carrying instances need hardly more registers than the rows: up to 2000 rows 0.99 to 1.07 at every width (8
 //   blocks of 1 x 300 x 1024 1.05, of 2 x 500 x 1280 1.05, of 2 x 1000 x 512 1.04, of 2 x 500 x 3072 1.00), at 4000 0.99 to 1.01, at
 //   8000 0.98 to 1.01.
-//   3 to 6, whose instance takes 156 registers, so that fewer blocks of rows fit an SM: 768 and 1024 columns 0.99 to 1.05 up to 2000 rows,
+//   3 to 6 (5 and more in two passes over the weights), whose instance takes 156 registers, so that fewer blocks of rows fit an SM: 768 and 1024 columns 0.99 to 1.05 up to 2000 rows,
 //   0.98 to 1.00 at 3000 and 4000; 1280 and 1536 1.01 to 1.09 up to 640, 1.00 to 1.03 at 1000, 0.98 to 1.01 at 2000; 1792 and 2048 1.01
 //   to 1.07 at 300, 0.99 to 1.04 at 500, 0.99 at 640; 2560 0.98 at 300.
 //   512 columns and fewer, where MOD by itself is short: 3 and 4 elements 0.99 to 1.03 from 800 to 2000 rows, 0.92 to 1.02 below, 5 and 6
 //   0.90 to 1.02; at 512 columns and under 100 rows 3 to 5 elements 0.99 to 1.02.
-//   7 and 8, in two passes over the weights: 512 0.93 to 1.01, 1024 0.98 to 1.01, 1536 and 2048 0.97 to 1.02.
+//   7 and 8: 512 0.93 to 1.01, 1024 0.98 to 1.01, 1536 and 2048 0.97 to 1.02.
 static bool ln_may_carry(int batch, long long rows, int D) {
   if (batch <= 2) return D <= kLnMaxCarryCols && rows <= 4096;
   if (batch > 6) return false;
